@@ -16,20 +16,20 @@
 //                (the second form avoids the cancellation of S_{r+1} - 1 when S_{r+1} is near 1)
 //                dl/du_c  = dl/dlq_r * sigmoid(-u_c);  du/da = s x_f / tau, du/dt = -s / tau,
 //                du/db = -s x_g / tau.
-// Everything is evaluated in float32 in the log domain, which keeps 1 - q_r and the products of
-// many sigmoids representable where the linear form underflows. A float32 log-probability of
-// magnitude L is only known to about L * 2^-24, and at large margins (fine-tuned coefficients)
-// L reaches thousands while the probabilities that make up the gradient are ratios of such
-// values: a 64-sample group in which some sample's log p_y exceeds SOFT_FF_LIMIT in magnitude
-// (or is not finite) is evaluated again in float-float arithmetic (about 48 significant bits),
-// with the margins formed exactly, 1 - q_r taken as a log-sum-exp of -u_c when q_r rounds to 1,
-// and each d ell / d u_c formed in the exponent (soft_group_ff). Other groups keep the float path.
+// These are the formulas in logs; the float kernels evaluate them as products and sums of positive
+// numbers in the linear domain (see "the float path" below), whose relative errors do not grow with the
+// margins, and a group of samples in which some sample's p_y is below e^-64 (or is not a number) is
+// evaluated again in float-float logs (about 48 significant bits), with the margins formed exactly,
+// 1 - q_r taken as a log-sum-exp of -u_c when q_r rounds to 1, and each d ell / d u_c formed in the
+// exponent (soft_group_ff): there a probability comes near float32's range, and the exponentials of
+// margins of that size carry their rounding.
 //
-// Work: one warp owns a (rule set, sample chunk) pair and walks the chunk 64 samples at a time
-// (two per lane), so each partial sum has a fixed summation order. The forward keeps lu_r per
-// rule and sample; the adjoint computes lq_r again from the conditions. Chunks are a function of N
-// only; partial losses and gradients per chunk are reduced in a second kernel in a fixed order,
-// which makes results bit-reproducible run to run and independent of scheduling.
+// Work: one warp owns a (rule set, sample chunk) pair and walks the chunk in groups of 64 or 128
+// samples (two or four neighbouring ones per lane), so each partial sum has a fixed summation order.
+// The forward keeps U_r per rule and sample; the adjoint computes q_r again from the conditions.
+// Chunks are a function of the call's shape only; partial losses and gradients per chunk are reduced
+// in a second kernel in a fixed order, which makes results bit-reproducible run to run and
+// independent of scheduling.
 #include "rs_internal.cuh"
 #include "soft_step.cuh"
 #include "block_scan.cuh"
@@ -45,6 +45,9 @@ constexpr int SOFT_MAX_CONDS = 512;       // conditions per set accumulated in s
 constexpr int SOFT_MAX_CHUNKS = 128;
 constexpr int SOFT_V = 2;                 // samples per lane; a group is 32 * SOFT_V samples
 constexpr int SOFT_G = 32 * SOFT_V;
+// the call's counters: tasks taken, [1..2] most rules / conditions of a set, length of the
+// float-float list, list items taken
+constexpr int SOFT_NEXT_FF_LEN = 3, SOFT_NEXT_FF = 4, SOFT_NEXT_N = 8;
 
 // Floats of a warp's shared arrays: lu [maxR + 1][G], acc [maxC][4], and lq [maxR][G] when the
 // class probabilities are written.
@@ -63,7 +66,7 @@ struct __align__(16) SoftRec {
 __global__ void k_pack_soft(BatchDev b, int F, int K, SoftRec *recs, uint32_t *status, int32_t *work_counter)
 {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c == 0) *work_counter = 0;            // the soft kernel's task counter
+    if (c == 0) work_counter[0] = work_counter[SOFT_NEXT_FF_LEN] = work_counter[SOFT_NEXT_FF] = 0;
     if (b.dR) { b.R = *b.dR; b.C = *b.dC; }
     if (c >= b.C) return;
     const int f = b.cond_f[c], g = b.cond_g[c], op = b.cond_op[c];
@@ -159,16 +162,14 @@ __device__ __forceinline__ float log1p_unit(float e)
     return e * p;
 }
 
-// The float path's exponentials of non-positive arguments use the hardware approximation
-// (__expf: ex2.approx of x log2(e)); for the arguments that occur here (|x| up to about 100,
-// beyond which the float-float pass takes over for the terms that matter) its relative error
-// stays below a few 1e-6, within the soft tolerance. Logarithms stay accurate (the hardware lg2
-// has an absolute error near 1 that is too large relative to log1p of small arguments); the
-// float-float pass keeps expf.
+// The hardware exponential (ex2.approx of x log2(e)) of a non-positive argument: for |x| up to about
+// 100 its relative error stays below a few 1e-6. Used by log1m_exp and by the class probabilities of
+// the float-float pass.
 __device__ __forceinline__ float exp_np(float x) { return __expf(x); }
 
 // log(1 - e^s) for s <= 0: the log-probability that a rule whose conditions hold with
-// probability q = e^s does not fire. Both pieces are evaluated and one is selected (a warp's
+// probability q = e^s does not fire (rs_selftest_log1m_exp; the kernels' float path works in the
+// linear domain). Both pieces are evaluated and one is selected (a warp's
 // samples fall on both sides):
 // * q <= e^(-1/2): log1p(-q) = -q a(q), a the degree-10 polynomial of least maximum relative
 //   error against -log1p(-q) / q on [0, e^(-1/2)] (Remez exchange; within 2 ulp given q). q comes
@@ -217,19 +218,6 @@ __global__ void k_selftest_soft_math(const float *in, int n, float *out, int whi
         out[i] = which == 0 ? log1p_unit(in[i]) : log1m_exp(in[i]);
 }
 
-__device__ __forceinline__ float log_sigmoid(float u)
-{
-    // log(1/(1+e^-u)) = -(max(-u,0) + log1p(e^-|u|))
-    const float e = exp_np(-fabsf(u));
-    return -(fmaxf(-u, 0.f) + log1p_unit(e));
-}
-
-__device__ __forceinline__ float sigmoid_neg(float u)     // 1/(1+e^u)
-{
-    const float e = exp_np(-fabsf(u));
-    return __fdividef(u >= 0.f ? e : 1.f, 1.f + e);
-}
-
 __device__ __forceinline__ float log_add(float a, float b)
 {
     if (a == -INFINITY) return b;
@@ -273,14 +261,18 @@ struct SoftKArgs {
     float *part_ga, *part_gbt;       // [nchunks][C]
     float *probs;                    // [P*N*K] or null
     int32_t backward;
-    int32_t *next;                   // work counter
+    int32_t *next;                   // [8] counters (SOFT_NEXT_*)
     int32_t maxR, maxC;              // shared-memory capacity per warp (rules, conditions)
     int64_t Ccap;                    // row stride of the gradient partials
     const uint32_t *status;          // no work if non-zero (malformed batch)
     const int32_t *order;            // sets by decreasing size (schedule only; results do not depend on it)
-    uint8_t *ffmark;                 // [nchunks][P]: the task left groups to the float-float pass
+    int32_t *fflist;                 // [nchunks * P]: tasks (ch * P + p) with groups left to the float-float pass
     uint32_t *ffbits;                // [nchunks][P][ff_wpt]: bit g of a task: its group g is one of them
     int32_t ff_wpt;                  // words per task (groups per chunk / 32, rounded up)
+    int32_t group;                   // samples per group of the main kernel (a bit of ffbits)
+    int32_t pslots;                  // class-probability slots per warp (0: not written)
+    int32_t teams;                   // teams per CTA (staged-tile kernel)
+    uint32_t tm_cols;                // tensor-memory columns of a CTA (staged-tile adjoint)
 };
 
 // Feature access for one group of 64 samples: the lane's first sample column either in global
@@ -292,110 +284,6 @@ struct XView {
     // x[f] of the lane's sample v (32 v samples after its first)
     __device__ __forceinline__ float operator()(int f, int v) const { return col[(int64_t)f * stride + 32 * v]; }
 };
-
-// The lane's sample v: (d ell / d a, d ell / d b or d t) of condition rc, given d ell / d log q of
-// its rule.
-__device__ __forceinline__ float2 cond_grad(const SoftKArgs &a, const SoftRec &rc, const XView &x, int v, float gq)
-{
-    const float xf = x(rc.f, v);
-    const bool pair = rc.meta & 1u;
-    const float xg = pair ? x(rc.g, v) : 0.f;
-    const float lhs = rc.a * xf;
-    const float rhs = pair ? rc.bt * xg : rc.bt;
-    const float sg = (rc.meta & 2u) ? -1.f : 1.f;
-    const float u = sg * (lhs - rhs) * a.inv_tau;
-    const float du = gq * sigmoid_neg(u) * sg * a.inv_tau;
-    return make_float2(du * xf, pair ? -du * xg : -du);
-}
-
-// log q of one rule (its conditions [c0, c1)) for the lane's V samples: the sum of the
-// conditions' log-sigmoids (membership tests: 0 or -inf). The forward and the adjoint both call it.
-template <bool CAT, int V>
-__device__ __forceinline__ void rule_logq(const SoftKArgs &a, int c0, int c1, const XView &x, float (&s)[V])
-{
-#pragma unroll
-    for (int v = 0; v < V; ++v) s[v] = 0.f;
-#pragma unroll 2
-    for (int c = c0; c < c1; ++c) {
-        const SoftRec rc = a.recs[c];
-        if (CAT && (rc.meta & 4u)) {   // membership: its exact indicator, a factor 1 or 0 of q_r
-#pragma unroll
-            for (int v = 0; v < V; ++v)
-                if (!category_member(x(rc.f, v), __float_as_uint(rc.a), __float_as_uint(rc.bt))) s[v] = -INFINITY;
-            continue;
-        }
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            const float lhs = rc.a * x(rc.f, v);
-            const float rhs = (rc.meta & 1u) ? rc.bt * x(rc.g, v) : rc.bt;
-            float u = (lhs - rhs) * a.inv_tau;
-            if (rc.meta & 2u) u = -u;
-            s[v] += log_sigmoid(u);
-        }
-    }
-}
-
-// rule_logq for the adjoint, which also keeps u and e^-|u| of the rule's first SOFT_CACHE
-// conditions (same arithmetic and order, so the same log q) for their gradients.
-constexpr int SOFT_CACHE = 4;
-template <bool CAT, int V>
-__device__ __forceinline__ void rule_logq_cached(const SoftKArgs &a, int c0, int c1, const XView &x, float (&s)[V],
-                                                 float (&cu)[SOFT_CACHE][V], float (&ce)[SOFT_CACHE][V])
-{
-#pragma unroll
-    for (int v = 0; v < V; ++v) s[v] = 0.f;
-#pragma unroll
-    for (int k = 0; k < SOFT_CACHE; ++k) {
-        if (c0 + k >= c1) break;
-        const SoftRec rc = a.recs[c0 + k];
-        if (CAT && (rc.meta & 4u)) {
-#pragma unroll
-            for (int v = 0; v < V; ++v)
-                if (!category_member(x(rc.f, v), __float_as_uint(rc.a), __float_as_uint(rc.bt))) s[v] = -INFINITY;
-            continue;
-        }
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            const float lhs = rc.a * x(rc.f, v);
-            const float rhs = (rc.meta & 1u) ? rc.bt * x(rc.g, v) : rc.bt;
-            float u = (lhs - rhs) * a.inv_tau;
-            if (rc.meta & 2u) u = -u;
-            const float e = exp_np(-fabsf(u));
-            cu[k][v] = u;
-            ce[k][v] = e;
-            s[v] += -(fmaxf(-u, 0.f) + log1p_unit(e));
-        }
-    }
-#pragma unroll 2
-    for (int c = c0 + SOFT_CACHE; c < c1; ++c) {
-        const SoftRec rc = a.recs[c];
-        if (CAT && (rc.meta & 4u)) {
-#pragma unroll
-            for (int v = 0; v < V; ++v)
-                if (!category_member(x(rc.f, v), __float_as_uint(rc.a), __float_as_uint(rc.bt))) s[v] = -INFINITY;
-            continue;
-        }
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            const float lhs = rc.a * x(rc.f, v);
-            const float rhs = (rc.meta & 1u) ? rc.bt * x(rc.g, v) : rc.bt;
-            float u = (lhs - rhs) * a.inv_tau;
-            if (rc.meta & 2u) u = -u;
-            s[v] += log_sigmoid(u);
-        }
-    }
-}
-
-// cond_grad from the condition's u (already signed) and e = e^-|u|.
-__device__ __forceinline__ float2 cond_grad_cached(const SoftKArgs &a, const SoftRec &rc, const XView &x, int v,
-                                                   float gq, float u, float e)
-{
-    const float xf = x(rc.f, v);
-    const bool pair = rc.meta & 1u;
-    const float sg = (rc.meta & 2u) ? -1.f : 1.f;
-    const float du = gq * __fdividef(u >= 0.f ? e : 1.f, 1.f + e) * sg * a.inv_tau;
-    return make_float2(du * xf, pair ? -du * x(rc.g, v) : -du);
-}
 
 // ------------------------------------------------------------------ float-float arithmetic
 // A value held as the unevaluated sum hi + lo of two floats (Dekker, "A floating-point technique
@@ -575,8 +463,6 @@ __device__ __forceinline__ void write_probs(const SoftKArgs &a, int p, int rb, i
     }
 }
 
-constexpr float SOFT_FF_LIMIT = 32.f;    // |log p_y| beyond which a group is evaluated in float-float
-
 // soft_group in float-float arithmetic, one sample of each lane at a time (all lanes walk the same
 // rules and conditions, so the gradient butterflies stay warp-wide). Forward: log q_r and
 // log(1 - q_r) of every rule, lu and log p_y accumulated in float-float. Adjoint: lu_r recovered
@@ -655,148 +541,532 @@ __device__ __forceinline__ void soft_group_ff(const SoftKArgs &a, int p, int rb,
     }
 }
 
-// Forward of set p over one group of 32 * V samples (lane l holds samples n0 + l + 32 v; bit v
-// of valid: the sample exists): the rules' log "no earlier rule fired" into lu (and log q into
-// lq when class probabilities are written), the labels yn and log p_y. Returns true when some
-// sample's log p_y is beyond SOFT_FF_LIMIT in magnitude or not finite (warp-uniform).
-template <bool CAT, int V>
-__device__ __forceinline__ bool soft_forward(const SoftKArgs &a, int rb, int R, int deflt, int64_t n0, uint32_t valid,
-                                             const XView &x, float (*lq)[32 * V], float (*lu)[32 * V], int lane,
-                                             int (&yn)[V], float (&lpy)[V])
+// ------------------------------------------------------------------ the float path
+// A condition with margin u has sigmoid(u) = 1 / (1 + E), E = e^-u. Over the conditions of a rule,
+// with D = prod (1 + E) and z = D - 1,
+//     q = 1 / D,    1 - q = z / D    (taken as 1 - q itself where q < 1/2),
+// and z follows its own recursion z' = z + E D of positive terms, so that 1 - q keeps its relative
+// accuracy where q rounds to 1. D beyond 1.6e38 counts as q = 0 (an infinite D that meets an E of 0,
+// a margin beyond 87, turns into a NaN, and its group takes the float-float pass, as one does whose
+// margins are not numbers).
+// Everything after it is a sum of products of positive numbers as well: U_r = prod_{j<r} (1 - q_j),
+// p_y and 1 - p_y over the rules, S_r and T_r backwards (S_r = [same] q + (1 - q) S_{r+1}, T_r with
+// the other rules), and d ell / d log q_r = q_r U_r (S_{r+1} or -T_{r+1}) / p_y. No logarithm and no
+// log-sum-exp is left: per condition and sample one ex2 forward, and an ex2 and a reciprocal in the
+// adjoint, against two ex2, two degree-8 polynomials and a division before; relative errors grow
+// by a rounding per factor instead of an ulp of the log-probability. Underflow only meets terms
+// below 2^-126 of a sample whose p_y is at least e^-64 (others take the float-float pass).
+// A rule of more than SOFT_SEG conditions is taken in pieces, q = q1 q2, 1 - q = w1 + q1 w2.
+//
+// What bounds it: instruction issue. A lane holds 2 NV neighbouring samples, so that a feature is one
+// 8- or 16-byte load, the products and sums are packed two-lane instructions, and reading a record
+// is shared by all of them; records, with the sign of '<' folded into the coefficients, and rule
+// ends sit in the warp's shared memory; U_r is parked in tensor memory by the staged-tile kernel
+// (2 NV columns a rule, which leaves shared memory to twice the warps). Gradient sums of 16
+// conditions are gathered in a 16 x 32 shared table and summed by all lanes at once: a condition
+// costs one store and about two instructions of summing, where a warp butterfly per two conditions
+// cost about 13 with its accumulator update. Forward + adjoint of 1024 sets x 32 rules x 4 conditions
+// on 262,144 samples: 139.7 ms in the log domain with two samples a lane (238 warp instructions per
+// condition and 64 samples), 70.3 ms so with U_r in tensor memory (123), 45.6 ms with E = e^-u in
+// place of e^-|u| and its sign and four samples a lane (72, issue slots 68 % busy at 16 warps an SM),
+// 44.6 ms with the caps taken off the forward's E.
+constexpr int SOFT_SEG = 32;               // conditions per piece of a rule
+constexpr float SOFT_D_MAX = 1.6e38f;      // D from which q is 0 (above 2^126: its reciprocal is subnormal)
+constexpr float SOFT_E_MAX = 1e38f;        // E above which 1 / (1 + E) would come out 0
+constexpr int SOFT_NV_TILE = 2, SOFT_NV = 1;    // float2 per lane: staged-tile and per-warp kernel
+constexpr int SOFT_CACHE = 4;              // conditions of a rule whose e the adjoint keeps in registers
+constexpr int SOFT_GROWS = 16;             // conditions per gradient table
+constexpr int SOFT_GPITCH = 288;           // bytes per table row: 32 lanes x 8, + 32 against bank conflicts
+constexpr float SOFT_P_MIN = 1.60381e-28f;   // e^-64: p_y below which a group is evaluated in float-float
+constexpr int32_t SREC_THR = -1, SREC_SET = -2;  // SoftRec4.g of a threshold / membership record
+
+// A record staged for the warp's set: v = s (a x[f] - rhs) = a' x[f] + n' (x[g] for a pair).
+struct __align__(16) SoftRec4 {
+    uint32_t f;        // feature (staged tile: byte offset of its row)
+    int32_t g;         // the same for a pair's second feature, SREC_THR, SREC_SET
+    float a, n;        // s a and -s t or -s b; a membership test's set words
+};
+
+// One warp's shared memory.
+struct SoftWarp {
+    SoftRec4 *recs;    // [maxC]
+    uint32_t *rules;   // [maxR] end of the rule's conditions (set-relative) | class << 16
+    float4 *acc;       // [maxC] Kahan sums of d/da (x, y) and d/d(b or t) (z, w), without s / tau (adjoint)
+    char *gtab;        // gradient table (adjoint)
+    float2 *u;         // [maxR][NV][32] U_r of the lane's samples (per-warp kernel's adjoint)
+    float2 *pc;        // [min(K, maxR + 1)][NV][32] class (or rule) probabilities (class probabilities)
+};
+
+__host__ __device__ constexpr size_t soft_main_bytes(int maxR, int maxC, bool bwd, bool tile, int pslots)
 {
-#pragma unroll
-    for (int v = 0; v < V; ++v) yn[v] = ((valid >> v) & 1u) ? a.y[n0 + lane + 32 * v] : -1;
-    float lu_r[V];
-#pragma unroll
-    for (int v = 0; v < V; ++v) { lu_r[v] = 0.f; lpy[v] = -INFINITY; }
-    for (int j = 0; j < R; ++j) {
-        const int r = rb + j;
-        const int c0 = a.rule_cond_off[r], c1 = a.rule_cond_off[r + 1];
-        float s[V];
-        rule_logq<CAT, V>(a, c0, c1, x, s);
-        const int cls = a.rule_class[r];
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            if (lq) lq[j][lane + 32 * v] = s[v];      // kept only for the class probabilities
-            lu[j][lane + 32 * v] = lu_r[v];
-            if (cls == yn[v]) lpy[v] = log_add(lpy[v], s[v] + lu_r[v]);
-            lu_r[v] += log1m_exp(s[v]);
-        }
-    }
-    bool big = false;
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-        lu[R][lane + 32 * v] = lu_r[v];
-        if (deflt == yn[v]) lpy[v] = log_add(lpy[v], lu_r[v]);
-        if (((valid >> v) & 1u) && !(fabsf(lpy[v]) <= SOFT_FF_LIMIT)) big = true;
-    }
-    return __any_sync(FULL, big);
+    return (size_t)maxC * sizeof(SoftRec4) + ((size_t)maxR * 4 + 15) / 16 * 16 +
+           (bwd ? (size_t)maxC * sizeof(float4) + SOFT_GROWS * SOFT_GPITCH : 0) +
+           (bwd && !tile ? (size_t)maxR * SOFT_NV * 32 * sizeof(float2) : 0) +
+           (size_t)pslots * (tile ? SOFT_NV_TILE : SOFT_NV) * 32 * sizeof(float2);
 }
 
-// Forward (and adjoint) of set p over one group of 32 * V samples: lane l holds samples
-// n0 + l + 32 v (v < V; bit v of valid: the sample exists), whose independent chains interleave.
-// lu: the warp's per-rule log-probabilities that no earlier rule fired [rule][32 V]; lq: the
-// rules' log q, kept only when class probabilities are written (null otherwise: the adjoint
-// computes them again); acc: the per-condition gradient sums.
-// CAT: the batch may hold membership conditions. Returns true, having added nothing, when some
-// sample's log p_y is beyond SOFT_FF_LIMIT: the task is then marked, and k_soft_ff evaluates the
-// group in float-float after this kernel.
-template <bool BWD, bool CAT, int V>
-__device__ __forceinline__ bool soft_group(const SoftKArgs &a, int p, int rb, int R, int cb, int deflt,
-                                           int64_t n0, uint32_t valid, const XView &x,
-                                           float (*lq)[32 * V], float (*lu)[32 * V], float (*acc)[4], int lane,
-                                           float &loss_s, float &loss_c)
+__device__ __forceinline__ SoftWarp soft_warp(char *base, int maxR, int maxC, bool bwd, bool tile)
 {
-    int yn[V];
-    float lpy[V];
-    if (soft_forward<CAT, V>(a, rb, R, deflt, n0, valid, x, lq, lu, lane, yn, lpy)) return true;
-#pragma unroll
-    for (int v = 0; v < V; ++v)
-        if (((valid >> v) & 1u)) kadd_loss(loss_s, loss_c, -lpy[v]);
-    if (a.probs) {
-#pragma unroll
-        for (int v = 0; v < V; ++v)
-            if ((valid >> v) & 1u) write_probs<V>(a, p, rb, R, deflt, n0, lane + 32 * v, lq, lu);
+    SoftWarp m{};
+    m.recs = reinterpret_cast<SoftRec4 *>(base);
+    base += (size_t)maxC * sizeof(SoftRec4);
+    m.rules = reinterpret_cast<uint32_t *>(base);
+    base += ((size_t)maxR * 4 + 15) / 16 * 16;
+    if (bwd) {
+        m.acc = reinterpret_cast<float4 *>(base);
+        base += (size_t)maxC * sizeof(float4);
+        m.gtab = base;
+        base += SOFT_GROWS * SOFT_GPITCH;
+        if (!tile) { m.u = reinterpret_cast<float2 *>(base); base += (size_t)maxR * SOFT_NV * 32 * sizeof(float2); }
     }
-    if (!BWD) return false;
-    // ---------------- adjoint
-    float lS[V], lT[V];
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-        lS[v] = (deflt == yn[v]) ? 0.f : -INFINITY;
-        lT[v] = (deflt == yn[v]) ? -INFINITY : 0.f;
+    m.pc = reinterpret_cast<float2 *>(base);
+    return m;
+}
+
+// The lane's 2 NV samples of some value, two to a register pair.
+template <int NV>
+struct Vec {
+    float2 v[NV];
+};
+
+// The lane's samples of a feature, from the staged tile (o: the row's byte offset) or from global
+// memory (o: the feature).
+template <bool TILE, int NV>
+struct XPair {
+    const char *base;
+    int64_t row;       // bytes per feature row (global form)
+    __device__ __forceinline__ Vec<NV> operator()(uint32_t o) const
+    {
+        const char *p = TILE ? base + o : base + (int64_t)o * row;
+        Vec<NV> r;
+        if constexpr (NV == 2) {
+            const float4 t = *reinterpret_cast<const float4 *>(p);
+            r.v[0] = make_float2(t.x, t.y);
+            r.v[1] = make_float2(t.z, t.w);
+        } else {
+            r.v[0] = *reinterpret_cast<const float2 *>(p);
+        }
+        return r;
     }
-    for (int j = R - 1; j >= 0; --j) {
-        const int r = rb + j;
-        const int cls = a.rule_class[r];
-        const int c0 = a.rule_cond_off[r], c1 = a.rule_cond_off[r + 1];
-        float lqr[V], cu[SOFT_CACHE][V], ce[SOFT_CACHE][V];
-        rule_logq_cached<CAT, V>(a, c0, c1, x, lqr, cu, ce);   // log q again: cheaper than keeping it
-        float gq[V];
+};
+
+__device__ __forceinline__ float ex2_ftz(float x)
+{
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+__device__ __forceinline__ float rcp_ftz(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+__device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
+
+// Tensor memory as a per-warp array of Vec (2 NV columns each; a warp reaches its own 32 lanes).
+template <int NV>
+__device__ __forceinline__ void tmem_put(uint32_t at, const Vec<NV> &u)
+{
+    if constexpr (NV == 2)
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at),
+                     "r"(__float_as_uint(u.v[0].x)), "r"(__float_as_uint(u.v[0].y)), "r"(__float_as_uint(u.v[1].x)),
+                     "r"(__float_as_uint(u.v[1].y))
+                     : "memory");
+    else
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};" ::"r"(at), "r"(__float_as_uint(u.v[0].x)),
+                     "r"(__float_as_uint(u.v[0].y))
+                     : "memory");
+}
+// The load's registers hold the values only after tmem_wait_get on them.
+template <int NV>
+__device__ __forceinline__ void tmem_get(uint32_t at, uint32_t (&r)[2 * NV])
+{
+    if constexpr (NV == 2)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                     : "r"(at)
+                     : "memory");
+    else
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(at) : "memory");
+}
+template <int NV>
+__device__ __forceinline__ void tmem_wait_get(uint32_t (&r)[2 * NV])
+{
+    if constexpr (NV == 2)
+        asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3])::"memory");
+    else
+        asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0]), "+r"(r[1])::"memory");
+}
+__device__ __forceinline__ void tmem_wait_put() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// min that keeps a NaN.
+__device__ __forceinline__ float min_nan(float a, float b)
+{
+    float r;
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+
+// E = e^-u of the lane's samples under record rc. nc = -log2(e) / tau.
+template <bool TILE, int NV>
+__device__ __forceinline__ Vec<NV> cond_e(const SoftRec4 &rc, const XPair<TILE, NV> &x, float nc)
+{
+    const Vec<NV> xf = x(rc.f);
+    Vec<NV> t;
+    if (rc.g >= 0) {
+        const Vec<NV> xg = x((uint32_t)rc.g);
 #pragma unroll
-        for (int v = 0; v < V; ++v) {
-            const float lqj = lqr[v], luj = lu[j][lane + 32 * v];
-            const bool same = cls == yn[v];
-            const float g = exp_np(lqj + luj + (same ? lT[v] : lS[v]) - lpy[v]);
-            gq[v] = ((valid >> v) & 1u) ? (same ? -g : g) : 0.f;
-            // log(1 - q_j): the forward's step from lu_j to lu_{j+1}. Where lu_j is -inf (an earlier
-            // rule certainly fired) the value does not matter (every later term is multiplied by
-            // exp(lu) = 0 and lS, lT only meet it through lu): any finite value keeps them finite.
-            const float lun = lu[j + 1][lane + 32 * v];
-            const float l1q = luj == -INFINITY ? 0.f : lun - luj;
-            // one of the two recursions adds q_j (the one of the sample's label class or not), the
-            // other only carries the factor 1 - q_j
-            const float grow = log_add(lqj, l1q + (same ? lS[v] : lT[v]));
-            const float carry = l1q + (same ? lT[v] : lS[v]);
-            lS[v] = same ? grow : carry;
-            lT[v] = same ? carry : grow;
+        for (int i = 0; i < NV; ++i) t.v[i] = __ffma2_rn(f2(rc.a), xf.v[i], __fmul2_rn(f2(rc.n), xg.v[i]));
+    } else {
+#pragma unroll
+        for (int i = 0; i < NV; ++i) t.v[i] = __ffma2_rn(f2(rc.a), xf.v[i], f2(rc.n));
+    }
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+        t.v[i] = __fmul2_rn(t.v[i], f2(nc));
+        t.v[i] = make_float2(ex2_ftz(t.v[i].x), ex2_ftz(t.v[i].y));
+    }
+    return t;
+}
+
+// D and z of a rule's piece so far, for the lane's samples.
+template <int NV>
+struct SoftProd {
+    float2 D[NV], z[NV];
+    uint32_t dead = 0;                               // bit i: a membership test of sample i failed
+    __device__ __forceinline__ SoftProd()
+    {
+#pragma unroll
+        for (int i = 0; i < NV; ++i) { D[i] = f2(1.f); z[i] = f2(0.f); }
+    }
+    __device__ __forceinline__ void add(const Vec<NV> &e)
+    {
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            z[i] = __ffma2_rn(e.v[i], D[i], z[i]);
+            D[i] = __ffma2_rn(e.v[i], D[i], D[i]);
         }
-        // conditions two at a time: the four sums (d/da, d/db-or-dt of both, over all 32 V samples)
-        // share one butterfly; the first SOFT_CACHE conditions reuse u and e^-|u| from above
+    }
+    // a membership test: its exact indicator
+    template <bool TILE>
+    __device__ __forceinline__ void member(const SoftRec4 &rc, const XPair<TILE, NV> &x)
+    {
+        const Vec<NV> v = x(rc.f);
+        const uint32_t lo = __float_as_uint(rc.a), hi = __float_as_uint(rc.n);
 #pragma unroll
-        for (int k = 0; k < SOFT_CACHE; k += 2) {
-            const int c = c0 + k;
-            if (c >= c1) break;
-            const bool has1 = c + 1 < c1;
-            const SoftRec r0 = a.recs[c];
-            const SoftRec r1 = a.recs[has1 ? c + 1 : c];
-            const bool use0 = !(CAT && (r0.meta & 4u)), use1 = has1 && !(CAT && (r1.meta & 4u));
-            float2 g0 = make_float2(0.f, 0.f), g1 = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-                if (use0) {
-                    const float2 t = cond_grad_cached(a, r0, x, v, gq[v], cu[k][v], ce[k][v]);
-                    g0.x += t.x; g0.y += t.y;
-                }
-                if (use1) {
-                    const float2 t = cond_grad_cached(a, r1, x, v, gq[v], cu[k + 1][v], ce[k + 1][v]);
-                    g1.x += t.x; g1.y += t.y;
-                }
-            }
-            reduce_pair(g0, g1, c - cb, has1, acc, lane);
+        for (int i = 0; i < NV; ++i) {
+            if (!category_member(v.v[i].x, lo, hi)) dead |= 1u << (2 * i);
+            if (!category_member(v.v[i].y, lo, hi)) dead |= 2u << (2 * i);
         }
+    }
+    template <bool CAT>
+    __device__ __forceinline__ void close(Vec<NV> &q, Vec<NV> &w) const
+    {
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            // beyond SOFT_D_MAX the reciprocal is subnormal and comes out 0, which the Newton step keeps
+            const float2 d = make_float2(min_nan(D[i].x, SOFT_D_MAX), min_nan(D[i].y, SOFT_D_MAX));
+            float2 r = make_float2(rcp_ftz(d.x), rcp_ftz(d.y));
+            r = __ffma2_rn(r, __ffma2_rn(__fmul2_rn(d, f2(-1.f)), r, f2(1.f)), r);
+            if (CAT && ((dead >> (2 * i)) & 1u)) r.x = 0.f;
+            if (CAT && ((dead >> (2 * i)) & 2u)) r.y = 0.f;
+            q.v[i] = r;
+            // 1 - q rounded once where q < 1/2, else the quotient, which keeps a small 1 - q
+            w.v[i] = __fmul2_rn(z[i], r);
+            const float2 v = __ffma2_rn(r, f2(-1.f), f2(1.f));
+            if (r.x < 0.5f) w.v[i].x = v.x;
+            if (r.y < 0.5f) w.v[i].y = v.y;
+        }
+    }
+};
+
+// The conditions [c, c1) of a rule into (q, w), a piece of SOFT_SEG at a time; (q, w) holds the rule
+// so far.
+template <bool CAT, bool TILE, int NV>
+__device__ __forceinline__ void rule_more(const SoftRec4 *recs, int c, int c1, const XPair<TILE, NV> &x, float nc,
+                                       Vec<NV> &q, Vec<NV> &w)
+{
+    while (c < c1) {
+        const int end = min(c1, c + SOFT_SEG);
+        SoftProd<NV> d;
+        for (; c < end; ++c) {
+            const SoftRec4 rc = recs[c];
+            if (CAT && rc.g == SREC_SET) d.member(rc, x);
+            else d.add(cond_e(rc, x, nc));
+        }
+        Vec<NV> q2, w2;
+        d.template close<CAT>(q2, w2);
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            w.v[i] = __ffma2_rn(q.v[i], w2.v[i], w.v[i]);
+            q.v[i] = __fmul2_rn(q.v[i], q2.v[i]);
+        }
+    }
+}
+
+// Sum a block of the gradient table (rows of conditions [16 blk, 16 blk + 16) of the set) over the
+// warp into their accumulators: lane 2 s + h adds half of row s (16-byte pieces 2 i + h: eight lanes
+// of a phase fall on distinct banks), the halves meet, and lane 2 s + h keeps component h.
+__device__ __forceinline__ void grad_block(const SoftWarp &m, int blk, int nc, int lane)
+{
+    __syncwarp();
+    const char *row = m.gtab + (lane >> 1) * SOFT_GPITCH + (lane & 1) * 16;
+    float2 s0 = f2(0.f), s1 = f2(0.f);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const float4 t = *reinterpret_cast<const float4 *>(row + 32 * i);
+        s0 = __fadd2_rn(s0, make_float2(t.x, t.y));
+        s1 = __fadd2_rn(s1, make_float2(t.z, t.w));
+    }
+    s0 = __fadd2_rn(s0, s1);
+    const bool odd = lane & 1;
+    const float other = __shfl_xor_sync(FULL, odd ? s0.x : s0.y, 1);
+    const float v = (odd ? s0.y : s0.x) + other;
+    const int ci = blk * SOFT_GROWS + (lane >> 1);
+    if (ci < nc) {
+        float2 *p = reinterpret_cast<float2 *>(m.acc + ci) + (lane & 1);
+        float2 k = *p;
+        kadd(k.x, k.y, v);
+        *p = k;
+    }
+    __syncwarp();
+}
+
+// The lane's part of condition ci's two gradient sums into the table; the table is summed after the
+// block's first condition (conditions arrive in descending order).
+template <bool CAT, bool TILE, int NV>
+__device__ __forceinline__ void cond_grads(const SoftWarp &m, int ci, int nconds, const Vec<NV> &e, const Vec<NV> &G,
+                                           const XPair<TILE, NV> &x, int lane)
+{
+    const SoftRec4 rc = m.recs[ci];
+    float2 g = f2(0.f);
+    if (!(CAT && rc.g == SREC_SET)) {
+        float2 h[NV];
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {        // sigmoid(-u) = E / (1 + E)
+            const float2 c = make_float2(fminf(e.v[i].x, SOFT_E_MAX), fminf(e.v[i].y, SOFT_E_MAX));
+            const float2 d = __fadd2_rn(c, f2(1.f));
+            h[i] = __fmul2_rn(__fmul2_rn(G.v[i], c), make_float2(rcp_ftz(d.x), rcp_ftz(d.y)));
+        }
+        const Vec<NV> xf = x(rc.f);
+        float2 ga = __fmul2_rn(h[0], xf.v[0]), gb = h[0];
+#pragma unroll
+        for (int i = 1; i < NV; ++i) ga = __ffma2_rn(h[i], xf.v[i], ga);
+        if (rc.g >= 0) {
+            const Vec<NV> xg = x((uint32_t)rc.g);
+            gb = __fmul2_rn(h[0], xg.v[0]);
+#pragma unroll
+            for (int i = 1; i < NV; ++i) gb = __ffma2_rn(h[i], xg.v[i], gb);
+        } else {
+#pragma unroll
+            for (int i = 1; i < NV; ++i) gb = __fadd2_rn(gb, h[i]);
+        }
+        g = make_float2(ga.x + ga.y, gb.x + gb.y);
+    }
+    *reinterpret_cast<float2 *>(m.gtab + (ci & (SOFT_GROWS - 1)) * SOFT_GPITCH + lane * 8) = g;
+    if ((ci & (SOFT_GROWS - 1)) == 0) grad_block(m, ci / SOFT_GROWS, nconds, lane);
+}
+
+// Forward (and adjoint) of a set of R rules over one group of 64 NV samples: lane l holds samples
+// n0 + 2 NV l + i (bit i of valid: the sample exists). tm: the warp's tensor-memory base
+// (staged-tile adjoint). Returns true, having added nothing, when some sample's p_y is below e^-64
+// (or not a number): the group's bit is then set, and k_soft_ff evaluates it in float-float after
+// this kernel.
+template <bool BWD, bool CAT, bool TILE, int NV>
+__device__ __forceinline__ bool soft_group(const SoftKArgs &a, const SoftWarp &m, int p, int R, int nconds, int deflt,
+                                           int64_t n0, uint32_t valid, const XPair<TILE, NV> &x, float nc, uint32_t tm,
+                                           int lane, float &loss_s, float &loss_c)
+{
+    const int64_t n = n0 + 2 * NV * lane;
+    int y[2 * NV];
+#pragma unroll
+    for (int i = 0; i < 2 * NV; ++i) y[i] = ((valid >> i) & 1u) ? a.y[n + i] : -1;
+    const bool by_class = a.K <= a.maxR + 1;
+    float2 *const pc = m.pc + lane;
+    Vec<NV> U, py, po;
+#pragma unroll
+    for (int i = 0; i < NV; ++i) { U.v[i] = f2(1.f); py.v[i] = f2(0.f); po.v[i] = f2(0.f); }
+    if (!BWD && a.probs && by_class)
+        for (int k = 0; k < a.K * NV; ++k) pc[k * 32] = f2(0.f);
+    const auto add_class = [&](int cls, const Vec<NV> &pr) {
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            if (cls == y[2 * i]) py.v[i].x += pr.v[i].x; else po.v[i].x += pr.v[i].x;
+            if (cls == y[2 * i + 1]) py.v[i].y += pr.v[i].y; else po.v[i].y += pr.v[i].y;
+        }
+    };
+    int c0 = 0;
+    for (int j = 0; j < R; ++j) {
+        const uint32_t ru = m.rules[j];
+        const int c1 = ru & 0xFFFFu, cls = ru >> 16;
+        Vec<NV> q, w;
+        {
+            SoftProd<NV> d;
+            const int end = min(c1, c0 + SOFT_SEG);
 #pragma unroll 2
-        for (int c = c0 + SOFT_CACHE; c < c1; c += 2) {
-            const bool has1 = c + 1 < c1;
-            const SoftRec r0 = a.recs[c];
-            const SoftRec r1 = a.recs[has1 ? c + 1 : c];
-            const bool use0 = !(CAT && (r0.meta & 4u)), use1 = has1 && !(CAT && (r1.meta & 4u));
-            float2 g0 = make_float2(0.f, 0.f), g1 = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-                if (use0) { const float2 t = cond_grad(a, r0, x, v, gq[v]); g0.x += t.x; g0.y += t.y; }
-                if (use1) { const float2 t = cond_grad(a, r1, x, v, gq[v]); g1.x += t.x; g1.y += t.y; }
+            for (int c = c0; c < end; ++c) {
+                const SoftRec4 rc = m.recs[c];
+                if (CAT && rc.g == SREC_SET) d.member(rc, x);
+                else d.add(cond_e(rc, x, nc));
             }
-            reduce_pair(g0, g1, c - cb, has1, acc, lane);
+            d.template close<CAT>(q, w);
+            if (end < c1) rule_more<CAT>(m.recs, end, c1, x, nc, q, w);
         }
+        if (BWD) {
+            if constexpr (TILE) tmem_put<NV>(tm + 2 * NV * j, U);
+            else
+#pragma unroll
+                for (int i = 0; i < NV; ++i) m.u[(j * NV + i) * 32 + lane] = U.v[i];
+        }
+        Vec<NV> pr;
+#pragma unroll
+        for (int i = 0; i < NV; ++i) pr.v[i] = __fmul2_rn(q.v[i], U.v[i]);
+        add_class(cls, pr);
+        if (!BWD && a.probs) {
+#pragma unroll
+            for (int i = 0; i < NV; ++i) {
+                float2 *s = pc + ((by_class ? cls : j) * NV + i) * 32;
+                *s = by_class ? __fadd2_rn(*s, pr.v[i]) : pr.v[i];
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < NV; ++i) U.v[i] = __fmul2_rn(U.v[i], w.v[i]);
+        c0 = c1;
+    }
+    add_class(deflt, U);
+    // every q_r went into p_y or 1 - p_y: a NaN anywhere shows in one of them
+    bool big = false;
+#pragma unroll
+    for (int i = 0; i < NV; ++i)
+        big |= (((valid >> (2 * i)) & 1u) && !(py.v[i].x >= SOFT_P_MIN && po.v[i].x >= 0.f)) ||
+               (((valid >> (2 * i + 1)) & 1u) && !(py.v[i].y >= SOFT_P_MIN && po.v[i].y >= 0.f));
+    if (BWD && TILE) tmem_wait_put();
+    if (__any_sync(FULL, big)) return true;
+    // -log p_y; near 1 from 1 - p_y, which is its own sum of positive terms
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+        if ((valid >> (2 * i)) & 1u) kadd_loss(loss_s, loss_c, py.v[i].x < 0.5f ? -logf(py.v[i].x) : -log1pf(-po.v[i].x));
+        if ((valid >> (2 * i + 1)) & 1u)
+            kadd_loss(loss_s, loss_c, py.v[i].y < 0.5f ? -logf(py.v[i].y) : -log1pf(-po.v[i].y));
+    }
+    if (!BWD) {
+        if (a.probs) {
+            int64_t o[2 * NV];
+#pragma unroll
+            for (int i = 0; i < 2 * NV; ++i) o[i] = ((valid >> i) & 1u) ? ((int64_t)p * a.N + a.perm[n + i]) * a.K : -1;
+            for (int k = 0; k < a.K; ++k) {
+#pragma unroll
+                for (int i = 0; i < NV; ++i) {
+                    float2 v = f2(0.f);
+                    if (by_class) v = pc[(k * NV + i) * 32];
+                    else
+                        for (int j = 0; j < R; ++j)
+                            if ((int)(m.rules[j] >> 16) == k) v = __fadd2_rn(v, pc[(j * NV + i) * 32]);
+                    if (k == deflt) v = __fadd2_rn(v, U.v[i]);
+                    if (o[2 * i] >= 0) a.probs[o[2 * i] + k] = v.x;
+                    if (o[2 * i + 1] >= 0) a.probs[o[2 * i + 1] + k] = v.y;
+                }
+            }
+        }
+        return false;
+    }
+    // ---------------- adjoint
+    __syncwarp();
+    Vec<NV> rp, S, T;
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+        rp.v[i] = make_float2(((valid >> (2 * i)) & 1u) ? 1.f / py.v[i].x : 0.f,
+                              ((valid >> (2 * i + 1)) & 1u) ? 1.f / py.v[i].y : 0.f);
+        S.v[i] = make_float2(deflt == y[2 * i] ? 1.f : 0.f, deflt == y[2 * i + 1] ? 1.f : 0.f);
+        T.v[i] = make_float2(1.f - S.v[i].x, 1.f - S.v[i].y);
+    }
+    uint32_t ru = R > 0 ? m.rules[R - 1] : 0u;
+    for (int j = R - 1; j >= 0; --j) {
+        const int c1 = ru & 0xFFFFu, cls = ru >> 16;
+        ru = j > 0 ? m.rules[j - 1] : 0u;
+        const int b0 = ru & 0xFFFFu;                 // the rule's first condition
+        uint32_t ur[2 * NV];
+        if constexpr (TILE) tmem_get<NV>(tm + 2 * NV * j, ur);
+        Vec<NV> q, w, ce[SOFT_CACHE];
+        {
+            SoftProd<NV> d;
+#pragma unroll
+            for (int k = 0; k < SOFT_CACHE; ++k) {
+                if (b0 + k >= c1) break;
+                const SoftRec4 rc = m.recs[b0 + k];
+                if (CAT && rc.g == SREC_SET) d.member(rc, x);
+                else {
+                    ce[k] = cond_e(rc, x, nc);
+                    d.add(ce[k]);
+                }
+            }
+            const int end = min(c1, b0 + SOFT_SEG);
+            for (int c = b0 + SOFT_CACHE; c < end; ++c) {
+                const SoftRec4 rc = m.recs[c];
+                if (CAT && rc.g == SREC_SET) d.member(rc, x);
+                else d.add(cond_e(rc, x, nc));
+            }
+            d.template close<CAT>(q, w);
+            if (end < c1) rule_more<CAT>(m.recs, end, c1, x, nc, q, w);
+        }
+        if constexpr (TILE) tmem_wait_get<NV>(ur);
+        Vec<NV> G;
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            float2 Uj;
+            if constexpr (TILE) Uj = make_float2(__uint_as_float(ur[2 * i]), __uint_as_float(ur[2 * i + 1]));
+            else Uj = m.u[(j * NV + i) * 32 + lane];
+            const bool s0 = cls == y[2 * i], s1 = cls == y[2 * i + 1];
+            const float2 pr = __fmul2_rn(__fmul2_rn(Uj, rp.v[i]), q.v[i]);
+            G.v[i] = __fmul2_rn(pr, make_float2(s0 ? -T.v[i].x : S.v[i].x, s1 ? -T.v[i].y : S.v[i].y));
+            S.v[i] = __ffma2_rn(w.v[i], S.v[i], make_float2(s0 ? q.v[i].x : 0.f, s1 ? q.v[i].y : 0.f));
+            T.v[i] = __ffma2_rn(w.v[i], T.v[i], make_float2(s0 ? 0.f : q.v[i].x, s1 ? 0.f : q.v[i].y));
+        }
+        for (int c = c1 - 1; c >= b0 + SOFT_CACHE; --c) {
+            const SoftRec4 rc = m.recs[c];
+            Vec<NV> e = {};
+            if (!(CAT && rc.g == SREC_SET)) e = cond_e(rc, x, nc);
+            cond_grads<CAT>(m, c, nconds, e, G, x, lane);
+        }
+#pragma unroll
+        for (int k = SOFT_CACHE - 1; k >= 0; --k)
+            if (b0 + k < c1) cond_grads<CAT>(m, b0 + k, nconds, ce[k], G, x, lane);
     }
     return false;
 }
 
-// Write a task's chunk partials (loss; gradient sums when BWD).
+// Stage a set's records and rule ends for the warp (row: bytes of a staged feature row, or 1 for
+// plain feature numbers) and clear its accumulators. Returns the number of conditions.
 template <bool BWD>
-__device__ __forceinline__ void soft_flush(const SoftKArgs &a, int p, int ch, int cb, int ce, float loss_s,
-                                           float (*acc)[4], int lane)
+__device__ __forceinline__ int soft_stage(const SoftKArgs &a, const SoftWarp &m, int rb, int R, uint32_t row, int lane)
+{
+    const int cb = a.rule_cond_off[rb], nc = a.rule_cond_off[rb + R] - cb;
+    __syncwarp();
+    for (int i = lane; i < nc; i += 32) {
+        const SoftRec r = a.recs[cb + i];
+        const bool pair = r.meta & 1u, lt = r.meta & 2u, set = r.meta & 4u;
+        SoftRec4 o;
+        o.f = r.f * row;
+        o.g = set ? SREC_SET : (pair ? (int32_t)(r.g * row) : SREC_THR);
+        o.a = set ? r.a : (lt ? -r.a : r.a);
+        o.n = set ? r.bt : (lt ? r.bt : -r.bt);
+        m.recs[i] = o;
+        if (BWD) m.acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    for (int j = lane; j < R; j += 32)
+        m.rules[j] = (uint32_t)(a.rule_cond_off[rb + j + 1] - cb) | (uint32_t)a.rule_class[rb + j] << 16;
+    __syncwarp();
+    return nc;
+}
+
+// Write a task's chunk partials (loss; gradient sums when BWD, with the factor s / tau of
+// du/da = s x / tau and -s / tau of du/dt that the table's sums leave out).
+template <bool BWD>
+__device__ __forceinline__ void soft_flush(const SoftKArgs &a, const SoftWarp &m, int p, int ch, int cb, int nc,
+                                           float loss_s, int lane)
 {
     float ls = loss_s;
 #pragma unroll
@@ -804,28 +1074,33 @@ __device__ __forceinline__ void soft_flush(const SoftKArgs &a, int p, int ch, in
     if (lane == 0) a.part_loss[(int64_t)ch * a.P + p] = ls;
     if (BWD) {
         __syncwarp();
-        for (int i = lane; i < (ce - cb); i += 32) {
-            a.part_ga[(int64_t)ch * a.Ccap + cb + i] = acc[i][0];
-            a.part_gbt[(int64_t)ch * a.Ccap + cb + i] = acc[i][2];
+        for (int i = lane; i < nc; i += 32) {
+            const float sc = (a.recs[cb + i].meta & 2u) ? -a.inv_tau : a.inv_tau;
+            const float4 g = m.acc[i];
+            a.part_ga[(int64_t)ch * a.Ccap + cb + i] = g.x * sc;
+            a.part_gbt[(int64_t)ch * a.Ccap + cb + i] = -g.z * sc;
         }
         __syncwarp();
     }
 }
 
-template <bool BWD, bool CAT>
-__global__ void __maxnreg__(96) k_soft(SoftKArgs a)     // launched with SOFT_W warps
+constexpr float LOG2E = 1.44269504f;
+
+// Bit i: the lane's sample i exists, `left` samples being left from its first one on.
+template <int NV>
+__device__ __forceinline__ uint32_t valid_mask(int64_t left)
 {
-    // per warp: lu[maxR+1][G], acc[maxC][4] (ga sum/comp, gbt sum/comp), lq[maxR][G] (probabilities)
-    extern __shared__ __align__(16) float sm[];
+    return left >= 2 * NV ? (1u << (2 * NV)) - 1u : (left <= 0 ? 0u : (1u << (int)left) - 1u);
+}
+
+template <bool BWD, bool CAT>
+__global__ void __launch_bounds__(SOFT_W * 32) k_soft(SoftKArgs a)
+{
+    extern __shared__ __align__(16) char smc[];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t tasks = (int64_t)a.P * a.nchunks;
-    const size_t per_warp = soft_per_warp(a.maxR, a.maxC, a.probs != nullptr);
-    float *base_w = sm + per_warp * w;
-    float(*lu)[SOFT_G] = reinterpret_cast<float(*)[SOFT_G]>(base_w);
-    float(*acc)[4] = reinterpret_cast<float(*)[4]>(base_w + (size_t)(a.maxR + 1) * SOFT_G);
-    float(*lq)[SOFT_G] = a.probs ? reinterpret_cast<float(*)[SOFT_G]>(base_w + (size_t)(a.maxR + 1) * SOFT_G +
-                                                                    (size_t)a.maxC * 4)
-                                 : nullptr;
+    const SoftWarp m = soft_warp(smc + soft_main_bytes(a.maxR, a.maxC, BWD, false, a.pslots) * w, a.maxR, a.maxC, BWD, false);
+    const float nc = -a.inv_tau * LOG2E;
     if (*a.status) return;
 
     while (true) {
@@ -835,8 +1110,185 @@ __global__ void __maxnreg__(96) k_soft(SoftKArgs a)     // launched with SOFT_W 
         if (task >= tasks) break;
         const int p = a.order[task / a.nchunks];
         const int ch = (int)(task % a.nchunks);
+        const int rb = a.set_rule_off[p], R = a.set_rule_off[p + 1] - rb;
+        const int nconds = soft_stage<BWD>(a, m, rb, R, 1u, lane);
+        float loss_s = 0.f, loss_c = 0.f;
+        const int64_t s0 = (int64_t)ch * a.chunk;
+        const int64_t s1 = min(s0 + a.chunk, a.N);
+        uint32_t *fbits = a.ffbits + ((int64_t)ch * a.P + p) * a.ff_wpt;
+        uint32_t fw = 0, ff = 0;
+        int gi = 0;
+        for (int64_t nb = s0; nb < s1; nb += 64 * SOFT_NV, ++gi) {
+            const int64_t n = nb + 2 * SOFT_NV * lane;
+            const uint32_t valid = valid_mask<SOFT_NV>(s1 - n);
+            // the dataset is padded to a multiple of 256 samples: every read stays inside it
+            const XPair<false, SOFT_NV> x{reinterpret_cast<const char *>(a.Xt + n), a.n_pad * (int64_t)sizeof(float)};
+            if (soft_group<BWD, CAT, false, SOFT_NV>(a, m, p, R, nconds, a.set_default[p], nb, valid, x, nc, 0u, lane, loss_s,
+                                            loss_c))
+                fw |= 1u << (gi & 31);
+            if ((gi & 31) == 31 || nb + 64 * SOFT_NV >= s1) {
+                if (lane == 0) fbits[gi >> 5] = fw;
+                ff |= fw;
+                fw = 0;
+            }
+        }
+        soft_flush<BWD>(a, m, p, ch, a.rule_cond_off[rb], nconds, loss_s, lane);
+        if (lane == 0 && ff) a.fflist[atomicAdd(a.next + SOFT_NEXT_FF_LEN, 1)] = (int32_t)((int64_t)ch * a.P + p);
+    }
+}
+
+// The same evaluation with the warps of a team on as many neighbouring sets (in size order) over
+// the same chunk: the features of each 64-sample group are staged once per team in shared memory
+// (double-buffered asynchronous copies), so condition loads are shared-memory reads. Per-set
+// results are identical to k_soft (same per-sample arithmetic and summation order).
+constexpr int SOFT_TW_MIN = 4, SOFT_TW_MAX = 16;   // warps per CTA (and sets per team) of the staged-tile kernel
+constexpr int SOFT_GT = 64 * SOFT_NV_TILE;    // samples per group of the staged-tile kernel
+constexpr int SOFT_TILE_STATIC = 256;   // bytes kept for the kernel's static shared memory
+
+__device__ __forceinline__ void stage_group(float *dst, const float *Xt, int64_t n_pad, int F, int64_t nb, int thread,
+                                            int threads)
+{
+    // F rows x G samples, 16-byte pieces
+    constexpr int PR = SOFT_GT / 4;   // pieces per row
+    for (int i = thread; i < F * PR; i += threads) {
+        const int f = i / PR, q = i % PR;
+        const float *src = Xt + (int64_t)f * n_pad + nb + 4 * q;
+        const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst + f * SOFT_GT + 4 * q);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// A CTA is a.teams teams of TW warps, each taking tasks of its own with its own buffers and named
+// barrier (a kernel that allocates tensor memory runs one CTA per SM: teams take the place of
+// further CTAs; the forward, which needs none, runs one team per CTA). The adjoint's CTA allocates
+// a.tm_cols tensor-memory columns for U_r: warp w holds rule r of its set at columns
+// (w / 4) 2 NV maxR + 2 NV r of its own 32 lanes. One barrier per group: a warp that has passed it is done
+// with the buffer that is restaged after it.
+template <bool BWD, bool CAT>
+__global__ void __maxnreg__(128) k_soft_tile(SoftKArgs a, int F)
+{
+    extern __shared__ __align__(16) char smc[];
+    __shared__ int64_t s_tasks[SOFT_TW_MAX / SOFT_TW_MIN];
+    __shared__ uint32_t s_tm;
+    const int lane = threadIdx.x & 31;
+    const int TW = (int)(blockDim.x >> 5) / a.teams;  // sets per team
+    const int team = (int)(threadIdx.x >> 5) / TW, w = (int)(threadIdx.x >> 5) - team * TW;
+    const int64_t set_groups = (a.P + TW - 1) / TW;
+    const int64_t tasks = set_groups * a.nchunks;
+    const size_t per_warp = soft_main_bytes(a.maxR, a.maxC, BWD, true, a.pslots);
+    char *const team_sm = smc + (per_warp * TW + sizeof(float) * 2 * SOFT_GT * (size_t)F) * team;
+    const SoftWarp m = soft_warp(team_sm + per_warp * w, a.maxR, a.maxC, BWD, true);
+    float *xbuf = reinterpret_cast<float *>(team_sm + per_warp * TW);     // [2][F][G]
+    const float nc = -a.inv_tau * LOG2E;
+    const auto team_sync = [&] { asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(TW * 32) : "memory"); };
+    if (*a.status) return;
+    uint32_t tm = 0;
+    if (BWD) {
+        const uint32_t cw = threadIdx.x >> 5;
+        if (cw == 0) {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                             (uint32_t)__cvta_generic_to_shared(&s_tm)),
+                         "r"(a.tm_cols)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        tm = s_tm + ((cw & 3u) << 21) + (cw >> 2) * (2u * SOFT_NV_TILE) * (uint32_t)a.maxR;
+    }
+
+    while (true) {
+        team_sync();
+        if (w == 0 && lane == 0) s_tasks[team] = atomicAdd(a.next, 1);
+        team_sync();
+        const int64_t task = s_tasks[team];
+        if (task >= tasks) break;
+        const int g = (int)(task / a.nchunks);
+        const int ch = (int)(task % a.nchunks);
+        const int64_t s0 = (int64_t)ch * a.chunk;
+        const int64_t s1 = min(s0 + a.chunk, a.N);
+        stage_group(xbuf, a.Xt, a.n_pad, F, s0, w * 32 + lane, TW * 32);
+        // the CTA's warps move through the chunk in step: sets of one group have similar sizes
+        const bool active = g * TW + w < a.P;
+        const int p = active ? a.order[g * TW + w] : 0;
+        int rb = 0, R = 0, nconds = 0, deflt = 0;
+        if (active) {
+            rb = a.set_rule_off[p];
+            R = a.set_rule_off[p + 1] - rb;
+            deflt = a.set_default[p];
+            nconds = soft_stage<BWD>(a, m, rb, R, SOFT_GT * (uint32_t)sizeof(float), lane);
+        }
+        float loss_s = 0.f, loss_c = 0.f;
+        uint32_t fw = 0, ff = 0;
+        const int ngroups = (int)((s1 - s0 + SOFT_GT - 1) / SOFT_GT);
+        uint32_t *fbits = a.ffbits + ((int64_t)ch * a.P + p) * a.ff_wpt;
+        for (int gi = 0; gi < ngroups; ++gi) {
+            const int64_t nb = s0 + SOFT_GT * (int64_t)gi;
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            team_sync();
+            if (gi + 1 < ngroups)
+                stage_group(xbuf + ((gi + 1) & 1) * F * SOFT_GT, a.Xt, a.n_pad, F, nb + SOFT_GT, w * 32 + lane, TW * 32);
+            if (active) {
+                constexpr int NV = SOFT_NV_TILE;
+                const uint32_t valid = valid_mask<NV>(s1 - nb - 2 * NV * lane);
+                const XPair<true, NV> x{reinterpret_cast<const char *>(xbuf + (gi & 1) * F * SOFT_GT + 2 * NV * lane), 0};
+                if (soft_group<BWD, CAT, true, NV>(a, m, p, R, nconds, deflt, nb, valid, x, nc, tm, lane, loss_s, loss_c))
+                    fw |= 1u << (gi & 31);
+                if ((gi & 31) == 31 || gi + 1 == ngroups) {
+                    if (lane == 0) fbits[gi >> 5] = fw;
+                    ff |= fw;
+                    fw = 0;
+                }
+            }
+        }
+        if (active) {
+            soft_flush<BWD>(a, m, p, ch, a.rule_cond_off[rb], nconds, loss_s, lane);
+            if (lane == 0 && ff) a.fflist[atomicAdd(a.next + SOFT_NEXT_FF_LEN, 1)] = (int32_t)((int64_t)ch * a.P + p);
+        }
+    }
+    if (BWD) {
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (threadIdx.x < 32)
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tm), "r"(a.tm_cols));
+    }
+}
+
+// The float-float pass: the CTAs take the (set, chunk) tasks that the main kernel listed, SOFT_W warps
+// to a task: warp i evaluates every SOFT_W-th of the groups whose bits the main kernel set (those it
+// left out) in float-float (soft_group_ff), its loss and gradient sums Kahan-summed in group order;
+// the warps' sums are added to the task's partials in warp order, so that results do not depend on
+// the order of the list. Runs after the main kernel on the same stream; features are read from
+// global memory.
+template <bool BWD, bool CAT>
+__global__ void __launch_bounds__(SOFT_W * 32) k_soft_ff(SoftKArgs a)
+{
+    extern __shared__ __align__(16) float sm[];
+    __shared__ int s_item;
+    __shared__ float s_loss[SOFT_W];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (*a.status) return;
+    const int items = a.next[SOFT_NEXT_FF_LEN];
+    const size_t per_warp = soft_per_warp(a.maxR, a.maxC, a.probs != nullptr);
+    float *base_w = sm + per_warp * w;
+    float(*lu)[SOFT_G] = reinterpret_cast<float(*)[SOFT_G]>(base_w);
+    float(*acc)[4] = reinterpret_cast<float(*)[4]>(base_w + (size_t)(a.maxR + 1) * SOFT_G);
+    float(*lq)[SOFT_G] = a.probs ? reinterpret_cast<float(*)[SOFT_G]>(base_w + (size_t)(a.maxR + 1) * SOFT_G +
+                                                                    (size_t)a.maxC * 4)
+                                 : nullptr;
+    while (true) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_item = atomicAdd(a.next + SOFT_NEXT_FF, 1);
+        __syncthreads();
+        if (s_item >= items) break;
+        const int64_t task = a.fflist[s_item];         // ch * P + p
+        const int p = (int)(task % a.P), ch = (int)(task / a.P);
         const int rb = a.set_rule_off[p], re = a.set_rule_off[p + 1];
         const int cb = a.rule_cond_off[rb], ce = a.rule_cond_off[re];
+        const int deflt = a.set_default[p];
         if (BWD) {
             for (int i = lane; i < (ce - cb); i += 32) {
                 acc[i][0] = 0.f; acc[i][1] = 0.f; acc[i][2] = 0.f; acc[i][3] = 0.f;
@@ -846,191 +1298,43 @@ __global__ void __maxnreg__(96) k_soft(SoftKArgs a)     // launched with SOFT_W 
         float loss_s = 0.f, loss_c = 0.f;
         const int64_t s0 = (int64_t)ch * a.chunk;
         const int64_t s1 = min(s0 + a.chunk, a.N);
-        uint32_t *fbits = a.ffbits + ((int64_t)ch * a.P + p) * a.ff_wpt;
-        uint32_t fw = 0, ff = 0;
-        int gi = 0;
-        for (int64_t nb = s0; nb < s1; nb += SOFT_G, ++gi) {
+        const uint32_t *fbits = a.ffbits + task * a.ff_wpt;
+        uint32_t fw = 0;
+        int k = 0;                                     // 64-sample groups of marked groups so far
+        for (int64_t nb = s0; nb < s1; nb += SOFT_G) {
+            const int gi = (int)((nb - s0) / a.group);
+            if ((nb - s0) % (32 * a.group) == 0) fw = fbits[gi >> 5];
+            if (!((fw >> (gi & 31)) & 1u)) continue;
+            if ((k++ & (SOFT_W - 1)) != w) continue;
             uint32_t valid = 0;
 #pragma unroll
             for (int v = 0; v < SOFT_V; ++v) valid |= (nb + lane + 32 * v < s1 ? 1u : 0u) << v;
-            // the dataset is padded to a multiple of 128 samples: every read stays inside it
             const XView x{a.Xt + nb + lane, a.n_pad};
-            if (soft_group<BWD, CAT, SOFT_V>(a, p, rb, re - rb, cb, a.set_default[p], nb, valid, x, lq, lu, acc,
-                                             lane, loss_s, loss_c))
-                fw |= 1u << (gi & 31);
-            if ((gi & 31) == 31 || nb + SOFT_G >= s1) {
-                if (lane == 0) fbits[gi >> 5] = fw;
-                ff |= fw;
-                fw = 0;
-            }
+            soft_group_ff<BWD, CAT, SOFT_V>(a, p, rb, re - rb, cb, deflt, nb, valid, x, lq, lu, acc, lane, loss_s,
+                                            loss_c);
         }
-        soft_flush<BWD>(a, p, ch, cb, ce, loss_s, acc, lane);
-        if (lane == 0) a.ffmark[(int64_t)ch * a.P + p] = ff != 0;
-    }
-}
-
-// The same evaluation with the warps of a CTA on as many neighbouring sets (in size order) over
-// the same chunk: the features of each 64-sample group are staged once per CTA in shared memory
-// (double-buffered asynchronous copies), so condition loads are shared-memory reads. Per-set
-// results are identical to k_soft (same per-sample arithmetic and summation order).
-constexpr int SOFT_TW_MIN = 4, SOFT_TW_MAX = 24;   // warps (sets) per CTA of the staged-tile kernel
-constexpr int SOFT_TILE_STATIC = 256;   // bytes kept for the kernel's static shared memory
-
-__device__ __forceinline__ void stage_group(float *dst, const float *Xt, int64_t n_pad, int F, int64_t nb)
-{
-    // F rows x G samples, 16-byte pieces
-    constexpr int PR = SOFT_G / 4;   // pieces per row
-    for (int i = threadIdx.x; i < F * PR; i += blockDim.x) {
-        const int f = i / PR, q = i % PR;
-        const float *src = Xt + (int64_t)f * n_pad + nb + 4 * q;
-        const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst + f * SOFT_G + 4 * q);
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-}
-
-// Launched with at most SOFT_TW_MAX warps: 96 registers per thread keep the two samples' chains
-// of the adjoint in registers and fit 512 threads (a launch bound of 512 capped it at 64 and spilled).
-template <bool BWD, bool CAT>
-__global__ void __maxnreg__(96) k_soft_tile(SoftKArgs a, int F)
-{
-    extern __shared__ __align__(16) float sm[];
-    __shared__ int64_t s_task;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int TW = blockDim.x >> 5;                   // sets per CTA group
-    const int64_t set_groups = (a.P + TW - 1) / TW;
-    const int64_t tasks = set_groups * a.nchunks;
-    const size_t per_warp = soft_per_warp(a.maxR, a.maxC, a.probs != nullptr);
-    float *base_w = sm + per_warp * w;
-    float(*lu)[SOFT_G] = reinterpret_cast<float(*)[SOFT_G]>(base_w);
-    float(*acc)[4] = reinterpret_cast<float(*)[4]>(base_w + (size_t)(a.maxR + 1) * SOFT_G);
-    float(*lq)[SOFT_G] = a.probs ? reinterpret_cast<float(*)[SOFT_G]>(base_w + (size_t)(a.maxR + 1) * SOFT_G +
-                                                                    (size_t)a.maxC * 4)
-                                 : nullptr;
-    float *xbuf = sm + per_warp * TW;                 // [2][F][G]
-    if (*a.status) return;
-
-    while (true) {
+        float ls = loss_s;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) ls += __shfl_xor_sync(FULL, ls, o);
+        if (lane == 0) s_loss[w] = ls;
         __syncthreads();
-        if (threadIdx.x == 0) s_task = atomicAdd(a.next, 1);
-        __syncthreads();
-        const int64_t task = s_task;
-        if (task >= tasks) break;
-        const int g = (int)(task / a.nchunks);
-        const int ch = (int)(task % a.nchunks);
-        // the CTA's warps move through the chunk in step: sets of one group have similar sizes
-        const bool active = g * TW + w < a.P;
-        const int p = active ? a.order[g * TW + w] : 0;
-        int rb = 0, R = 0, cb = 0, ce = 0, deflt = 0;
-        if (active) {
-            rb = a.set_rule_off[p];
-            const int re = a.set_rule_off[p + 1];
-            R = re - rb;
-            cb = a.rule_cond_off[rb];
-            ce = a.rule_cond_off[re];
-            deflt = a.set_default[p];
-            if (BWD) {
-                for (int i = lane; i < (ce - cb); i += 32) {
-                    acc[i][0] = 0.f; acc[i][1] = 0.f; acc[i][2] = 0.f; acc[i][3] = 0.f;
+        if (threadIdx.x == 0) {
+            float t = s_loss[0];
+            for (int i = 1; i < SOFT_W; ++i) t += s_loss[i];
+            a.part_loss[task] += t;
+        }
+        if (BWD) {
+            const float(*acc0)[4] = reinterpret_cast<const float(*)[4]>(sm + (size_t)(a.maxR + 1) * SOFT_G);
+            for (int i = threadIdx.x; i < (ce - cb); i += SOFT_W * 32) {
+                float ga = 0.f, gbt = 0.f;
+                for (int v = 0; v < SOFT_W; ++v) {
+                    const float *t = reinterpret_cast<const float *>(acc0) + per_warp * v + 4 * (size_t)i;
+                    ga += t[0];
+                    gbt += t[2];
                 }
-                __syncwarp();
+                a.part_ga[(int64_t)ch * a.Ccap + cb + i] += ga;
+                a.part_gbt[(int64_t)ch * a.Ccap + cb + i] += gbt;
             }
-        }
-        float loss_s = 0.f, loss_c = 0.f;
-        uint32_t fw = 0, ff = 0;
-        const int64_t s0 = (int64_t)ch * a.chunk;
-        const int64_t s1 = min(s0 + a.chunk, a.N);
-        const int ngroups = (int)((s1 - s0 + SOFT_G - 1) / SOFT_G);
-        uint32_t *fbits = a.ffbits + ((int64_t)ch * a.P + p) * a.ff_wpt;
-        stage_group(xbuf, a.Xt, a.n_pad, F, s0);
-        for (int gi = 0; gi < ngroups; ++gi) {
-            const int64_t nb = s0 + SOFT_G * (int64_t)gi;
-            if (gi + 1 < ngroups) {
-                stage_group(xbuf + ((gi + 1) & 1) * F * SOFT_G, a.Xt, a.n_pad, F, nb + SOFT_G);
-                asm volatile("cp.async.wait_group 1;" ::: "memory");
-            } else {
-                asm volatile("cp.async.wait_group 0;" ::: "memory");
-            }
-            __syncthreads();
-            if (active) {
-                uint32_t valid = 0;
-#pragma unroll
-                for (int v = 0; v < SOFT_V; ++v) valid |= (nb + lane + 32 * v < s1 ? 1u : 0u) << v;
-                const XView x{xbuf + (gi & 1) * F * SOFT_G + lane, SOFT_G};
-                if (soft_group<BWD, CAT, SOFT_V>(a, p, rb, R, cb, deflt, nb, valid, x, lq, lu, acc, lane, loss_s,
-                                                 loss_c))
-                    fw |= 1u << (gi & 31);
-                if ((gi & 31) == 31 || gi + 1 == ngroups) {
-                    if (lane == 0) fbits[gi >> 5] = fw;
-                    ff |= fw;
-                    fw = 0;
-                }
-            }
-            __syncthreads();              // the buffer is restaged two groups later
-        }
-        if (active) {
-            soft_flush<BWD>(a, p, ch, cb, ce, loss_s, acc, lane);
-            if (lane == 0) a.ffmark[(int64_t)ch * a.P + p] = ff != 0;
-        }
-    }
-}
-
-// The float-float pass: one warp per (set, chunk) task that the main kernel marked. The warp
-// evaluates, in group order, the groups whose bits the main kernel set (those it left out) in
-// float-float (soft_group_ff); their loss and gradient sums, Kahan-summed in group order, are
-// added to the task's partials. Runs after the main kernel on the same stream; features are read
-// from global memory.
-template <bool BWD, bool CAT>
-__global__ void __launch_bounds__(SOFT_W * 32) k_soft_ff(SoftKArgs a)
-{
-    extern __shared__ __align__(16) float sm[];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t task = (int64_t)blockIdx.x * SOFT_W + w;
-    if (*a.status || task >= (int64_t)a.P * a.nchunks) return;
-    const int p = (int)(task % a.P);
-    const int ch = (int)(task / a.P);
-    if (!a.ffmark[(int64_t)ch * a.P + p]) return;
-    const size_t per_warp = soft_per_warp(a.maxR, a.maxC, a.probs != nullptr);
-    float *base_w = sm + per_warp * w;
-    float(*lu)[SOFT_G] = reinterpret_cast<float(*)[SOFT_G]>(base_w);
-    float(*acc)[4] = reinterpret_cast<float(*)[4]>(base_w + (size_t)(a.maxR + 1) * SOFT_G);
-    float(*lq)[SOFT_G] = a.probs ? reinterpret_cast<float(*)[SOFT_G]>(base_w + (size_t)(a.maxR + 1) * SOFT_G +
-                                                                    (size_t)a.maxC * 4)
-                                 : nullptr;
-    const int rb = a.set_rule_off[p], re = a.set_rule_off[p + 1];
-    const int cb = a.rule_cond_off[rb], ce = a.rule_cond_off[re];
-    const int deflt = a.set_default[p];
-    if (BWD) {
-        for (int i = lane; i < (ce - cb); i += 32) {
-            acc[i][0] = 0.f; acc[i][1] = 0.f; acc[i][2] = 0.f; acc[i][3] = 0.f;
-        }
-        __syncwarp();
-    }
-    float loss_s = 0.f, loss_c = 0.f;
-    const int64_t s0 = (int64_t)ch * a.chunk;
-    const int64_t s1 = min(s0 + a.chunk, a.N);
-    const uint32_t *fbits = a.ffbits + ((int64_t)ch * a.P + p) * a.ff_wpt;
-    uint32_t fw = 0;
-    int gi = 0;
-    for (int64_t nb = s0; nb < s1; nb += SOFT_G, ++gi) {
-        if ((gi & 31) == 0) fw = fbits[gi >> 5];
-        if (!((fw >> (gi & 31)) & 1u)) continue;
-        uint32_t valid = 0;
-#pragma unroll
-        for (int v = 0; v < SOFT_V; ++v) valid |= (nb + lane + 32 * v < s1 ? 1u : 0u) << v;
-        const XView x{a.Xt + nb + lane, a.n_pad};
-        soft_group_ff<BWD, CAT, SOFT_V>(a, p, rb, re - rb, cb, deflt, nb, valid, x, lq, lu, acc, lane, loss_s,
-                                        loss_c);
-    }
-    float ls = loss_s;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ls += __shfl_xor_sync(FULL, ls, o);
-    if (lane == 0) a.part_loss[(int64_t)ch * a.P + p] += ls;
-    if (BWD) {
-        __syncwarp();
-        for (int i = lane; i < (ce - cb); i += 32) {
-            a.part_ga[(int64_t)ch * a.Ccap + cb + i] += acc[i][0];
-            a.part_gbt[(int64_t)ch * a.Ccap + cb + i] += acc[i][2];
         }
     }
 }
@@ -1106,23 +1410,55 @@ static void set_soft_attributes(Ctx *ctx)
 {
     cudaFuncSetAttribute(k_soft<true, CAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->smem_optin);
     cudaFuncSetAttribute(k_soft<false, CAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->smem_optin);
-    // the staged-tile kernel has a little static shared memory of its own
+    // the staged-tile and float-float kernels have a little static shared memory of their own
     cudaFuncSetAttribute(k_soft_tile<true, CAT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)ctx->smem_optin - SOFT_TILE_STATIC);
     cudaFuncSetAttribute(k_soft_tile<false, CAT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)ctx->smem_optin - SOFT_TILE_STATIC);
-    cudaFuncSetAttribute(k_soft_ff<true, CAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->smem_optin);
-    cudaFuncSetAttribute(k_soft_ff<false, CAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ctx->smem_optin);
+    cudaFuncSetAttribute(k_soft_ff<true, CAT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)ctx->smem_optin - SOFT_TILE_STATIC);
+    cudaFuncSetAttribute(k_soft_ff<false, CAT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)ctx->smem_optin - SOFT_TILE_STATIC);
     cudaGetLastError();
 }
 
-// Resident CTAs per SM of the staged-tile kernel with tw warps and per-warp arrays of
-// per_warp bytes (0 when it does not fit).
-template <bool BWD, bool CAT>
-static int soft_tile_per_sm(Ctx *ctx, int tw, size_t per_warp, int F)
+// Tensor-memory columns of a staged-tile CTA of tw warps: U_r takes 2 NV per rule and group of four
+// warps; allocations are powers of two from 32 to the SM's 512.
+constexpr int TMEM_COLS = 512;
+static int soft_tm_cols(int tw, int maxR)
 {
-    const size_t bytes = per_warp * tw + sizeof(float) * 2 * SOFT_G * (size_t)F;
+    const int need = (tw + 3) / 4 * 2 * SOFT_NV_TILE * maxR;
+    int cols = 32;
+    while (cols < need) cols *= 2;
+    return cols;
+}
+
+// Launch shape of the soft kernel: warps per team and teams per CTA (staged-tile form), resident CTAs
+// per SM.
+struct SoftShape {
+    int tw = SOFT_TW_MIN;
+    int teams = 1;
+    int per_sm = 1;
+};
+
+// Shared memory of a team of tw warps: the warps' arrays and two feature tiles.
+static size_t soft_team_bytes(int tw, size_t per_warp, int F)
+{
+    return per_warp * tw + sizeof(float) * 2 * SOFT_GT * (size_t)F;
+}
+
+// Resident teams per SM of the staged-tile kernel with tw warps to a team (0 when one does not fit):
+// CTAs of one team in the forward, teams of one CTA in the adjoint (tensor memory: one CTA per SM).
+template <bool BWD, bool CAT>
+static int soft_teams_per_sm(Ctx *ctx, int tw, size_t per_warp, int F, int maxR)
+{
+    const size_t bytes = soft_team_bytes(tw, per_warp, F);
     if (bytes + SOFT_TILE_STATIC > ctx->smem_optin) return 0;
+    if (BWD) {
+        int n = std::min(SOFT_TW_MAX / tw, (int)((ctx->smem_optin - SOFT_TILE_STATIC) / bytes));
+        while (n > 0 && (n * tw + 3) / 4 * 2 * SOFT_NV_TILE * maxR > TMEM_COLS) --n;
+        return n;
+    }
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_soft_tile<BWD, CAT>, tw * 32, bytes) != cudaSuccess) {
         cudaGetLastError();
@@ -1131,27 +1467,26 @@ static int soft_tile_per_sm(Ctx *ctx, int tw, size_t per_warp, int F)
     return per_sm;
 }
 
-// Launch shape of the soft kernel: warps per CTA (staged-tile form) and resident CTAs per SM.
-struct SoftShape {
-    int tw = SOFT_TW_MIN;
-    int per_sm = 1;
-};
-
-// The staged-tile form takes the number of warps per CTA that keeps the most warps resident for
-// this batch's per-warp arrays (ties: fewer warps per CTA, so that a CTA's sets are closer in
-// size); small populations keep at most P / 8 warps per CTA, since a CTA walks its sets in step
-// and a wide CTA over few sets of uneven size waits for the longest.
+// The staged-tile form takes the number of warps per team that keeps the most warps resident for
+// this batch's per-warp arrays (ties: fewer warps per team, so that a team's sets are closer in
+// size); small populations keep at most P / 8 warps per team, since a team walks its sets in step
+// and a wide one over few sets of uneven size waits for the longest.
 template <bool CAT>
-static SoftShape soft_shape(Ctx *ctx, bool tiled, bool bwd, int F, size_t smem, size_t per_warp, int P)
+static SoftShape soft_shape(Ctx *ctx, bool tiled, bool bwd, int F, size_t smem, size_t per_warp, int P, int maxR)
 {
     SoftShape sh;
     if (tiled) {
         int best = 0;
         const int tw_max = std::max(SOFT_TW_MIN, std::min(SOFT_TW_MAX, P / 8));
         for (int t = SOFT_TW_MIN; t <= tw_max; ++t) {
-            const int c = bwd ? soft_tile_per_sm<true, CAT>(ctx, t, per_warp, F)
-                              : soft_tile_per_sm<false, CAT>(ctx, t, per_warp, F);
-            if (c * t > best) { best = c * t; sh.tw = t; sh.per_sm = c; }
+            const int c = bwd ? soft_teams_per_sm<true, CAT>(ctx, t, per_warp, F, maxR)
+                              : soft_teams_per_sm<false, CAT>(ctx, t, per_warp, F, maxR);
+            if (c * t > best) {
+                best = c * t;
+                sh.tw = t;
+                sh.teams = bwd ? c : 1;
+                sh.per_sm = bwd ? 1 : c;
+            }
         }
     } else {
         if (bwd) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&sh.per_sm, k_soft<true, CAT>, SOFT_W * 32, smem);
@@ -1169,9 +1504,9 @@ static void launch_soft_kernel(Ctx *ctx, const SoftKArgs &k, bool tiled, bool bw
 {
     const int grid = ctx->sm_count * sh.per_sm;
     if (tiled) {
-        const size_t smem_tile = per_warp * sh.tw + sizeof(float) * 2 * SOFT_G * (size_t)F;
-        if (bwd) k_soft_tile<true, CAT><<<grid, sh.tw * 32, smem_tile, stream>>>(k, F);
-        else k_soft_tile<false, CAT><<<grid, sh.tw * 32, smem_tile, stream>>>(k, F);
+        const size_t smem_tile = soft_team_bytes(sh.tw, per_warp, F) * sh.teams;
+        if (bwd) k_soft_tile<true, CAT><<<grid, sh.tw * sh.teams * 32, smem_tile, stream>>>(k, F);
+        else k_soft_tile<false, CAT><<<grid, sh.tw * sh.teams * 32, smem_tile, stream>>>(k, F);
     } else {
         if (bwd) k_soft<true, CAT><<<grid, SOFT_W * 32, smem, stream>>>(k);
         else k_soft<false, CAT><<<grid, SOFT_W * 32, smem, stream>>>(k);
@@ -1187,9 +1522,9 @@ static size_t ff_words(int P, int64_t N)
 
 // Scratch layout of one soft call: records [C], order [P], per-chunk losses [chunks][P], the work
 // counter and maxima [4], per-chunk gradient sums [chunks][C] twice (adjoint only), the tasks'
-// float-float marks [chunks][P] and group bits.
+// float-float list [chunks * P] and group bits.
 struct SoftScratchLayout {
-    size_t recs, order, part_loss, next, part_ga, part_gbt, ffmark, ffbits, total;
+    size_t recs, order, part_loss, next, part_ga, part_gbt, fflist, ffbits, total;
 };
 
 static SoftScratchLayout soft_layout(int64_t C, int P, int nchunks, bool bwd, int64_t N)
@@ -1203,7 +1538,7 @@ static SoftScratchLayout soft_layout(int64_t C, int P, int nchunks, bool bwd, in
     L.next = o; o += 256;
     L.part_ga = o; o += bwd ? up(sizeof(float) * (size_t)nchunks * C) : 0;
     L.part_gbt = o; o += bwd ? up(sizeof(float) * (size_t)nchunks * C) : 0;
-    L.ffmark = o; o += up((size_t)nchunks * P);
+    L.fflist = o; o += up(sizeof(int32_t) * (size_t)nchunks * P);
     L.ffbits = o; o += up(sizeof(uint32_t) * ff_words(P, N));
     L.total = o;
     return L;
@@ -1236,9 +1571,9 @@ static rs_status soft_run(Ctx *ctx, const SoftArgs &s, int known_maxR, int known
 
     SoftRec *recs = nullptr;
     float *part_loss = nullptr, *part_ga = nullptr, *part_gbt = nullptr;
-    int32_t *next = nullptr;   // [0] work counter, [1..2] max rules / conditions per set
+    int32_t *next = nullptr;   // the call's counters (SOFT_NEXT_*)
     int32_t *order = nullptr;
-    uint8_t *ffmark = nullptr;
+    int32_t *fflist = nullptr;
     uint32_t *ffbits = nullptr;
     const bool bwd = s.dloss != nullptr;
     cudaError_t ae = cudaSuccess;
@@ -1250,28 +1585,28 @@ static rs_status soft_run(Ctx *ctx, const SoftArgs &s, int known_maxR, int known
         next = reinterpret_cast<int32_t *>(pre + L.next);
         part_ga = bwd ? reinterpret_cast<float *>(pre + L.part_ga) : nullptr;
         part_gbt = bwd ? reinterpret_cast<float *>(pre + L.part_gbt) : nullptr;
-        ffmark = reinterpret_cast<uint8_t *>(pre + L.ffmark);
+        fflist = reinterpret_cast<int32_t *>(pre + L.fflist);
         ffbits = reinterpret_cast<uint32_t *>(pre + L.ffbits);
     } else {
         ae = dev_alloc_async(&recs, sizeof(SoftRec) * Ccap, stream);
         if (ae == cudaSuccess) ae = dev_alloc_async(&order, sizeof(int32_t) * (size_t)P, stream);
         if (ae == cudaSuccess) ae = dev_alloc_async(&part_loss, sizeof(float) * (size_t)nchunks * P, stream);
-        if (ae == cudaSuccess) ae = dev_alloc_async(&next, sizeof(int32_t) * 4, stream);
+        if (ae == cudaSuccess) ae = dev_alloc_async(&next, sizeof(int32_t) * SOFT_NEXT_N, stream);
         if (ae == cudaSuccess && bwd) ae = dev_alloc_async(&part_ga, sizeof(float) * (size_t)nchunks * Ccap, stream);
         if (ae == cudaSuccess && bwd) ae = dev_alloc_async(&part_gbt, sizeof(float) * (size_t)nchunks * Ccap, stream);
-        if (ae == cudaSuccess) ae = dev_alloc_async(&ffmark, (size_t)nchunks * P, stream);
+        if (ae == cudaSuccess) ae = dev_alloc_async(&fflist, sizeof(int32_t) * (size_t)nchunks * P, stream);
         if (ae == cudaSuccess) ae = dev_alloc_async(&ffbits, sizeof(uint32_t) * ff_words(P, s.N), stream);
     }
     if (ae != cudaSuccess) {         // release what was taken before the failure
         for (void *q : {(void *)recs, (void *)order, (void *)part_loss, (void *)next, (void *)part_ga, (void *)part_gbt,
-                        (void *)ffmark, (void *)ffbits})
+                        (void *)fflist, (void *)ffbits})
             if (q) cudaFreeAsync(q, stream);
         return cuda_fail(ae, "soft scratch");
     }
     const bool known = known_maxR > 0;
     repeat = repeat && pre && known;
     if (!repeat) {
-        RS_CUDA(cudaMemsetAsync(next, 0, sizeof(int32_t) * 4, stream));
+        RS_CUDA(cudaMemsetAsync(next, 0, sizeof(int32_t) * SOFT_NEXT_N, stream));
         k_check_sets_soft<<<(P + 255) / 256, 256, 0, stream>>>(b, s.K, s.status, next + 1,
                                                                known ? known_maxR : SOFT_MAX_RULES,
                                                                known ? known_maxC : SOFT_MAX_CONDS);
@@ -1304,7 +1639,7 @@ static rs_status soft_run(Ctx *ctx, const SoftArgs &s, int known_maxR, int known
     k.part_ga = part_ga;
     k.part_gbt = part_gbt;
     k.order = order;
-    k.ffmark = ffmark;
+    k.fflist = fflist;
     k.ffbits = ffbits;
     k.probs = s.probs;
     k.backward = bwd;
@@ -1329,12 +1664,14 @@ static rs_status soft_run(Ctx *ctx, const SoftArgs &s, int known_maxR, int known
             set_error("soft evaluation rejected the batch: %s", status_text(*hs).c_str());
         }
     }
-    const size_t per_warp = sizeof(float) * soft_per_warp(k.maxR, k.maxC, k.probs != nullptr);
-    const size_t smem = per_warp * SOFT_W;
-    // the staged-tile kernel when its per-CTA footprint (8 warps + two feature tiles) fits
-    const size_t smem_tile = per_warp * SOFT_TW_MIN + sizeof(float) * 2 * SOFT_G * (size_t)s.F;
+    k.pslots = k.probs ? std::min(k.K, k.maxR + 1) : 0;
+    const size_t smem_ff = sizeof(float) * soft_per_warp(k.maxR, k.maxC, k.probs != nullptr) * SOFT_W;
+    const size_t smem = soft_main_bytes(k.maxR, k.maxC, bwd, false, k.pslots) * SOFT_W;
+    const size_t per_warp = soft_main_bytes(k.maxR, k.maxC, bwd, true, k.pslots);
+    // the staged-tile kernel when its smallest per-CTA footprint (and two feature tiles) fits
+    const size_t smem_tile = soft_team_bytes(SOFT_TW_MIN, per_warp, s.F);
     const bool tiled = s.F <= 128 && smem_tile + SOFT_TILE_STATIC <= ctx->smem_optin;
-    if (rc == RS_OK && smem > ctx->smem_optin) {
+    if (rc == RS_OK && (smem > ctx->smem_optin || smem_ff > ctx->smem_optin)) {
         rc = RS_ERR_TOO_LARGE;
         set_error("soft evaluation: sets too large for shared memory");
     }
@@ -1344,21 +1681,22 @@ static rs_status soft_run(Ctx *ctx, const SoftArgs &s, int known_maxR, int known
             set_soft_attributes<false>(ctx);
             set_soft_attributes<true>(ctx);
         });
-        const SoftShape sh = b.cond_set ? soft_shape<true>(ctx, tiled, bwd, s.F, smem, per_warp, P)
-                                        : soft_shape<false>(ctx, tiled, bwd, s.F, smem, per_warp, P);
+        const SoftShape sh = b.cond_set ? soft_shape<true>(ctx, tiled, bwd, s.F, smem, per_warp, P, k.maxR)
+                                        : soft_shape<false>(ctx, tiled, bwd, s.F, smem, per_warp, P, k.maxR);
         if (tiled) {
             // The staged-tile kernel's CTAs take (set group, chunk) tasks until none is left. When
             // the tasks make only a few rounds of the resident CTAs, the last round decides the
             // time: take the chunk count (at most the one chosen above, whose partial sums the
             // scratch holds) that minimises rounds x samples per chunk, preferring more chunks.
             const int64_t set_groups = (P + sh.tw - 1) / sh.tw;
-            const int64_t workers = (int64_t)ctx->sm_count * sh.per_sm;
+            const int64_t workers = (int64_t)ctx->sm_count * sh.per_sm * sh.teams;
             int64_t best_cost = INT64_MAX;
             for (int n = 1; n <= k.nchunks; ++n) {
                 int64_t ch = (s.N + n - 1) / n;
-                ch = (ch + SOFT_G - 1) / SOFT_G * SOFT_G;
+                ch = (ch + SOFT_GT - 1) / SOFT_GT * SOFT_GT;
                 const int64_t nc = (s.N + ch - 1) / ch;
-                const int64_t cost = (set_groups * nc + workers - 1) / workers * ch;
+                // one round more for the tail: the sets of a group are alike, the groups are not
+                const int64_t cost = ((set_groups * nc + workers - 1) / workers + 1) * ch;
                 if (cost < best_cost || (cost == best_cost && nc > nchunks)) {
                     best_cost = cost;
                     nchunks = (int)nc;
@@ -1368,20 +1706,23 @@ static rs_status soft_run(Ctx *ctx, const SoftArgs &s, int known_maxR, int known
             k.nchunks = nchunks;
             k.chunk = (int32_t)chunk;
         }
-        k.ff_wpt = (int32_t)(((k.chunk + SOFT_G - 1) / SOFT_G + 31) / 32);
+        k.teams = sh.teams;
+        k.tm_cols = (uint32_t)soft_tm_cols(sh.tw * sh.teams, k.maxR);
+        k.group = tiled ? SOFT_GT : 64 * SOFT_NV;
+        k.ff_wpt = (int32_t)(((k.chunk + k.group - 1) / k.group + 31) / 32);
         {
             TimedLaunch tl(ctx, TK_SOFT, stream);
             if (b.cond_set) launch_soft_kernel<true>(ctx, k, tiled, bwd, s.F, smem, per_warp, sh, stream);
             else launch_soft_kernel<false>(ctx, k, tiled, bwd, s.F, smem, per_warp, sh, stream);
         }
         {   // groups beyond float32's resolution (usually none: the kernel's warps exit at once)
-            const unsigned ffgrid = (unsigned)(((int64_t)P * k.nchunks + SOFT_W - 1) / SOFT_W);
+            const unsigned ffgrid = (unsigned)std::min<int64_t>((int64_t)P * k.nchunks, (int64_t)ctx->sm_count * 4);
             if (b.cond_set) {
-                if (bwd) k_soft_ff<true, true><<<ffgrid, SOFT_W * 32, smem, stream>>>(k);
-                else k_soft_ff<false, true><<<ffgrid, SOFT_W * 32, smem, stream>>>(k);
+                if (bwd) k_soft_ff<true, true><<<ffgrid, SOFT_W * 32, smem_ff, stream>>>(k);
+                else k_soft_ff<false, true><<<ffgrid, SOFT_W * 32, smem_ff, stream>>>(k);
             } else {
-                if (bwd) k_soft_ff<true, false><<<ffgrid, SOFT_W * 32, smem, stream>>>(k);
-                else k_soft_ff<false, false><<<ffgrid, SOFT_W * 32, smem, stream>>>(k);
+                if (bwd) k_soft_ff<true, false><<<ffgrid, SOFT_W * 32, smem_ff, stream>>>(k);
+                else k_soft_ff<false, false><<<ffgrid, SOFT_W * 32, smem_ff, stream>>>(k);
             }
             count_launch(ctx);
         }
@@ -1403,7 +1744,7 @@ static rs_status soft_run(Ctx *ctx, const SoftArgs &s, int known_maxR, int known
         cudaFreeAsync(part_loss, stream);
         cudaFreeAsync(next, stream);
         if (bwd) { cudaFreeAsync(part_ga, stream); cudaFreeAsync(part_gbt, stream); }
-        cudaFreeAsync(ffmark, stream);
+        cudaFreeAsync(fflist, stream);
         cudaFreeAsync(ffbits, stream);
     }
     return rc;

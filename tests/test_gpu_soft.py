@@ -362,3 +362,28 @@ def test_log1m_exp_against_float64(ctx):
     o = np.empty_like(sp)
     rs.check(rs.lib().rs_selftest_log1m_exp(ctx.h, rs._ptr(sp), 3, rs._ptr(o)))
     assert o[0] == -np.inf and o[1] == -np.inf and o[2] == 0.0
+
+
+@pytest.mark.parametrize("N,F,P,R,C,K,tau", [
+    (127, 3, 5, (2, 4), (31, 70), 2, 2.0),       # rules longer than one 32-condition piece
+    (129, 129, 9, (2, 12), (1, 9), 3, 0.1),      # the per-warp kernel, one sample past its second group
+    (257, 128, 40, (2, 64), (1, 8), 2, 0.1),     # widest staged tile, full tensor-memory columns (64 rules)
+    (1000, 5, 200, (2, 3), (1, 5), 2, 0.02),     # margins up to a few hundred: D and E leave float32's range
+    (130, 4, 3, (5, 9), (1, 2), 40, 0.5),        # more classes than rules
+    (64, 1, 1, (2, 2), (1, 1), 2, 0.1),          # one group, one set
+])
+def test_soft_linear_domain_edges(ctx, orc, N, F, P, R, C, K, tau):
+    """The float path at the edges of its pieces, groups, kernels and ranges, and its class
+    probabilities, against the float64 oracle."""
+    X, y = synth.gaussian_mixture(N, F, K, 17)
+    if K > 2:
+        y = (y % 2).astype(np.int32)             # labels that every set can reach
+    b = reachable(synth.random_rulesets(synth.quantile_table(X), K, P, R, C, 17, pair_prob=0.3 if F > 1 else 0.0))
+    r0 = b.set_rule_off[:-1]
+    b.rule_class[r0], b.rule_class[r0 + 1] = 0, 1
+    dl = np.random.default_rng(17).uniform(0.5, 2, b.P)
+    got = soft_gpu(ctx, X, y, K, b, tau, dl, probs=True)
+    ref = orc.soft(X, y, K, b, tau, dloss=dl, want_probs=True, want_mag=True)
+    check_against_oracle(got, ref)
+    assert np.allclose(got["probs"], ref["probs"], rtol=RTOL, atol=1e-30)
+    assert np.array_equal(got["loss_fwd"], got["loss"])
