@@ -15,19 +15,19 @@ template <int W, bool CAT>
 __global__ void __launch_bounds__(W * 32, 1) k_hard5(const __grid_constant__ CUtensorMap tmx,
                                                   const __grid_constant__ CUtensorMap tmr, HardArgs a)
 {
-    extern __shared__ __align__(128) unsigned char smem[];
+    extern __shared__ __align__(512) unsigned char smem[];
     const int F = a.F;
     const int Fb = F < 256 ? F : 256;
     const int nbox = (F + Fb - 1) / Fb;
     const int Frows = nbox * Fb;
     unsigned char *xs = smem;                                         // float [Frows][T]
-    unsigned char *rs = xs + (size_t)Frows * T * 4;                   // u8 [Frows][T], then reversed
+    float *ones = reinterpret_cast<float *>(xs + (size_t)Frows * T * 4);  // [T] of 1.0 (products)
+    unsigned char *rs = reinterpret_cast<unsigned char *>(ones + T);  // u8 [Frows][T], then reversed
     float *us = reinterpret_cast<float *>(rs + (size_t)Frows * T * 2);  // float [F][T] sorted (built here)
     uint4 *stage_all = reinterpret_cast<uint4 *>(us + (size_t)Frows * T);
     constexpr int VS = vslots<W>();
     uint32_t *vrows = reinterpret_cast<uint32_t *>(stage_all + W * 32);     // [W][VS][32]
-    float *ones = reinterpret_cast<float *>(vrows + W * VS * 32);             // [T] of 1.0 (products)
-    uint64_t *bar = reinterpret_cast<uint64_t *>(ones + T);
+    uint64_t *bar = reinterpret_cast<uint64_t *>(vrows + W * VS * 32);
     int *next = reinterpret_cast<int *>(bar + 1);
     uint32_t *walked = reinterpret_cast<uint32_t *>(bar + 2);        // [W][4] work counters (counting)
     const uint4 *recs = reinterpret_cast<const uint4 *>(a.recs);
@@ -62,13 +62,12 @@ __global__ void __launch_bounds__(W * 32, 1) k_hard5(const __grid_constant__ CUt
         return;
     }
     const uint32_t rev_off = (uint32_t)Frows * T;
-    build_tile_tables(reinterpret_cast<const float *>(xs), rs, rev_off, us, F, Frows);
+    build_tile_tables(reinterpret_cast<float *>(xs), rs, rev_off, us, F);
     if (threadIdx.x < T) ones[threadIdx.x] = 1.f;
     __syncthreads();
 
     const unsigned char *rl = rs + lane * 4;       // this lane's four rank bytes of row 0
-    const unsigned char *xl = xs + lane * 16;      // this lane's four floats of row 0
-    const uint32_t ones_off = (uint32_t)(reinterpret_cast<unsigned char *>(ones) - xs);
+    const uint32_t ones_off = (uint32_t)Frows * T * 4;
     const int count = (a.P - group + G - 1) / G;
     uint4 *st = stage_all + warp * 32;
 
@@ -89,11 +88,12 @@ __global__ void __launch_bounds__(W * 32, 1) k_hard5(const __grid_constant__ CUt
         uint32_t *vr = vrows + warp * VS * 32;
         const uint32_t vr_off = (uint32_t)(reinterpret_cast<unsigned char *>(vr) - rs);
         WalkCount wc;
+        int more;
         const uint32_t hit =
-            uniform ? walk_set<true, VS, CAT>(st, vr, vr_off, lane, recs, rb, nrec, us, rev_off, F, kmin, rl, xl,
-                                              ones_off, yl, claimed0, si.deflt, wc)
-                    : walk_set<false, VS, CAT>(st, vr, vr_off, lane, recs, rb, nrec, us, rev_off, F, -2, rl, xl,
-                                               ones_off, yl, claimed0, si.deflt, wc);
+            uniform ? walk_set<true, VS, CAT>(st, vr, vr_off, lane, recs, rb, nrec, us, rev_off, F, kmin, rl, xs,
+                                              ones_off, yl, claimed0, si.deflt, wc, more)
+                    : walk_set<false, VS, CAT>(st, vr, vr_off, lane, recs, rb, nrec, us, rev_off, F, -2, rl, xs,
+                                               ones_off, yl, claimed0, si.deflt, wc, more);
         if (a.walked && lane == 0) {           // the warp's own slots: no atomics
             uint32_t *wk = walked + 4 * warp;
             wk[0] += wc.records;
@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(W * 32, 1) k_hard5(const __grid_constant__ CUt
             wk[2] += wc.ends;
             wk[3] += 1;
         }
-        const int hits = __reduce_add_sync(FULL, __popc(hit));
+        const int hits = __reduce_add_sync(FULL, __popc(hit) + more);
         if (lane == 0 && hits) atomicAdd(&a.correct[p], hits);
         if (a.per_class) {
             if (uniform) {

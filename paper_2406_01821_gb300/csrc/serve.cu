@@ -110,7 +110,7 @@ __device__ __forceinline__ void serve_unit_ranked(const ReqDesc &d, int tile, in
         reinterpret_cast<uint4 *>(rs)[i] = *reinterpret_cast<const uint4 *>(d.Rk + (int64_t)f * d.n_pad + col0 + 16 * c16);
     }
     __syncthreads();
-    build_tile_tables(reinterpret_cast<const float *>(xs), rs, (uint32_t)F * T, us, F, F);
+    build_tile_tables(reinterpret_cast<float *>(xs), rs, (uint32_t)F * T, us, F);
     const int32_t *yl = d.y + col0 + lane * 4;
     const int64_t t_last = min(col0 + T, d.N) - 1;
     const int kmin = d.y[col0], kmax = d.y[t_last];
@@ -118,7 +118,7 @@ __device__ __forceinline__ void serve_unit_ranked(const ReqDesc &d, int tile, in
     const uint32_t claimed0 = class_bytes(yl, -1);
     const uint32_t rev_off = (uint32_t)F * T;
     const uint32_t vr_off = (uint32_t)(reinterpret_cast<unsigned char *>(vr) - rs);
-    const unsigned char *rl = rs + lane * 4, *xl = xs + lane * 16;
+    const unsigned char *rl = rs + lane * 4;
     __syncthreads();
     while (true) {
         int m = 0;
@@ -135,17 +135,18 @@ __device__ __forceinline__ void serve_unit_ranked(const ReqDesc &d, int tile, in
                              : t.y - t.x;
         uint32_t hit;
         rank::WalkCount wc;                 // not reported by the serving kernel
+        int more;
         if (d.cat)
             hit = uniform ? walk_set<true, SVS, true>(st, vr, vr_off, lane, d.recs, rb, nrec, us, rev_off, F, kmin,
-                                                      rl, xl, ones_off, yl, claimed0, deflt, wc)
+                                                      rl, xs, ones_off, yl, claimed0, deflt, wc, more)
                           : walk_set<false, SVS, true>(st, vr, vr_off, lane, d.recs, rb, nrec, us, rev_off, F, -2,
-                                                       rl, xl, ones_off, yl, claimed0, deflt, wc);
+                                                       rl, xs, ones_off, yl, claimed0, deflt, wc, more);
         else
             hit = uniform ? walk_set<true, SVS, false>(st, vr, vr_off, lane, d.recs, rb, nrec, us, rev_off, F, kmin,
-                                                       rl, xl, ones_off, yl, claimed0, deflt, wc)
+                                                       rl, xs, ones_off, yl, claimed0, deflt, wc, more)
                           : walk_set<false, SVS, false>(st, vr, vr_off, lane, d.recs, rb, nrec, us, rev_off, F, -2,
-                                                        rl, xl, ones_off, yl, claimed0, deflt, wc);
-        const int hits = __reduce_add_sync(FULL, __popc(hit));
+                                                        rl, xs, ones_off, yl, claimed0, deflt, wc, more);
+        const int hits = __reduce_add_sync(FULL, __popc(hit) + more);
         if (lane == 0 && hits) atomicAdd(&d.correct[p], hits);
         if (d.per_class) {
             if (uniform) {

@@ -541,3 +541,54 @@ def test_measured_pipe_rates():
     nominal = prop.multi_processor_count * 128 * 2.1e9
     assert 0.5 * nominal < r["ffma"] <= 1.05 * nominal, r
     assert all(v > 0 for v in r.values()), r
+
+
+@pytest.mark.parametrize("F,K,cat", [(3, 2, False), (9, 40, False), (128, 5, False), (16, 3, True)])
+def test_sparse_tail_of_the_rank_coded_walk(orc, F, K, cat):
+    """Sets whose first rules leave 0 to 40 samples of a 128-sample tile unclaimed, followed by rules
+    that straddle the 32-record windows (up to 100 conditions), with pairs, ties, both
+    comparisons, products and membership tests, on tiles of one label and of several."""
+    import torch
+    from paper_2406_01821_gb300 import build, rs
+    build.build()
+    rng = np.random.default_rng([F, K])
+    N = 3000
+    X = np.round(rng.standard_normal((N, F)) * 4).astype(np.float32) / 4          # ties
+    y = rng.integers(0, K, N).astype(np.int32)
+    X[:, 0] = rng.permutation(N).astype(np.float32) / N
+    if cat:
+        X[:, -4:] = rng.integers(0, 48, (N, 4))
+
+    def cond():
+        f, g = (int(v) for v in rng.integers(0, F, 2))
+        op = int(rng.integers(0, 2))
+        if cat and f >= F - 4:
+            return (f, -1, synth.IN, 0.0, 0.0, 0.0, sorted({int(v) for v in rng.integers(0, 48, 24)}))
+        kind = rng.random()
+        if kind < 0.25:
+            return (f, g, op, float(rng.uniform(-1, 1)), float(rng.uniform(-1, 1)), 0.0)
+        if kind < 0.3:
+            return (f, -1, op, 0.0, 0.0, float(rng.uniform(-1, 0.5)))                  # a product: 0 x > t
+        a = float(rng.choice([-1.0, 1.0, 0.5]))
+        return (f, -1, op, a, 0.0, float(np.float32(a) * rng.choice(X[:, f])))
+
+    sets = []
+    for keep in (0, 1, 5, 12, 19, 20, 21, 40):
+        for tail in (1, 4, 31, 32, 33, 100):
+            head = [(int(rng.integers(0, K)), [(0, -1, synth.GT, 1.0, 0.0, keep / 128.0)])]
+            easy = [(0, -1, synth.LT, 1.0, 0.0, 2.0)]                                  # always holds
+            rules = [(int(rng.integers(0, K)), [cond() for _ in range(int(rng.integers(1, 4)))]) for _ in range(14)]
+            long_rule = (int(rng.integers(0, K)), easy * (tail - 1) + [cond()])
+            sets.append(head + rules[:7] + [long_rule] + rules[7:])
+    b = synth.from_lists(sets, rng.integers(0, K, len(sets)).tolist())
+    oc, opc, _ = orc.eval_hard(X, y, K, b)
+    with rs.Context(0) as ctx:
+        ds = ctx.dataset(X, y, K)
+        for tile in (21, 22):
+            ctx.set_tile_config(tile)
+            c, pc, _ = ctx.eval_hard(ds, rs.DeviceBatch.from_host(b), K)
+            torch.cuda.synchronize()
+            assert np.array_equal(c.cpu().numpy(), oc) and np.array_equal(pc.cpu().numpy(), opc)
+        t = ctx.submit(ds, rs.HostBatch(b))
+        c, pc, _ = ctx.poll(t, b.P, K, timeout_us=30_000_000)
+        assert np.array_equal(c, oc) and np.array_equal(pc, opc)
