@@ -1,6 +1,7 @@
 // Device building blocks shared by evaluators that process one rule set at a time per warp on a
 // shared-memory feature tile (record format v2, margin-minimum conjunction).
 #pragma once
+#include "eval_sparse.cuh"
 #include "rs_internal.cuh"
 
 namespace rs {
@@ -91,7 +92,7 @@ __device__ void eval_set(const uint4 *recs, int rb, int re, uint4 *st, const flo
         const uint4 *rp = st + (rel - 32 * ck);
         const uint4 r0 = rp[0];
         const int nc = max(1, (int)((r0.x >> LEN_SHIFT) & 0xFFFu));   // >= 1: progress
-        const int cls = (int)(r0.y >> CLS_SHIFT);
+        const int cls = (int)((r0.y >> CLS_SHIFT) & 0xFFFu);
         float mn[V];
 #pragma unroll
         for (int v = 0; v < V; ++v) mn[v] = unc[v] ? __uint_as_float(0x7F800000u) : -1.f;
@@ -121,11 +122,12 @@ constexpr uint32_t SIGN = 0x80000000u;
 
 // acc[v] |= sign-bearing margin of this condition (record format v4): the sign stays clear iff
 // the condition holds. Cut conditions: m = fma(+-1, x, -c') exactly; others: an ordinary compare.
+// xs: the float tile with permuted rows (eval_sparse.cuh); lb: the lane's byte offset in a row.
 template <int V>
-__device__ __forceinline__ void cond_mask(const uint4 r, const float *xl, uint32_t (&acc)[V])
+__device__ __forceinline__ void cond_mask(const uint4 r, const unsigned char *xs, uint32_t lb, uint32_t (&acc)[V])
 {
     float x[V];
-    load_vec<V>(xl + (r.x & OFF_MASK) * 4, x);
+    load_vec<V>(reinterpret_cast<const float *>(xs + ((r.x & OFF_MASK) << 4 ^ lb)), x);
     const float v0 = __uint_as_float(r.z), v1 = __uint_as_float(r.w);
     if (!(r.x & (PAIR_BIT | GENERAL_BIT))) {
         const float2 s2 = make_float2(v0, v0), c2 = make_float2(v1, v1);
@@ -137,7 +139,7 @@ __device__ __forceinline__ void cond_mask(const uint4 r, const float *xl, uint32
         }
     } else if (r.x & PAIR_BIT) {
         float z[V];
-        load_vec<V>(xl + (r.y & OFF_MASK) * 4, z);
+        load_vec<V>(reinterpret_cast<const float *>(xs + ((r.y & OFF_MASK) << 4 ^ lb)), z);
 #pragma unroll
         for (int v = 0; v < V; ++v)
             acc[v] |= (__fmul_rn(v0, x[v]) > __fmul_rn(v1, z[v])) ? 0u : SIGN;
@@ -147,16 +149,58 @@ __device__ __forceinline__ void cond_mask(const uint4 r, const float *xl, uint32
     }
 }
 
-// Evaluate one set (records [rb, re), format v4) on this lane's V samples. hit[v] gets its sign
-// bit set when the sample's prediction equals its label: in a tile of one label (`uniform`, label
-// kmin) only rules of that class count; otherwise the per-sample label y[v] decides. y[v] < 0
-// marks padding. All lanes of the warp call this together.
+// A record of format v4 on the sparse tail. A cut's margin fma(+-1, x, -c') keeps its sign clear
+// exactly where +-x >= c', that is +-x > the float below c'.
+struct Decode4 {
+    uint32_t ones_off;
+    __device__ __forceinline__ sparse::Rec operator()(const uint4 raw) const
+    {
+        const bool pair = raw.x & PAIR_BIT, general = raw.x & GENERAL_BIT;
+        const float v1 = __uint_as_float(raw.w);
+        sparse::Rec r;
+        r.xo = (raw.x & OFF_MASK) << 4;
+        r.zo = pair ? (raw.y & OFF_MASK) << 4 : ones_off;
+        r.A = __uint_as_float(raw.z);
+        r.B = pair || general ? v1 : nextafterf(-v1, __uint_as_float(0xFF800000u));
+        r.inv = r.set = r.row = false;
+        r.end = raw.y & END4_BIT;
+        r.cls = (int)((raw.y >> CLS_SHIFT) & 0xFFFu);
+        return r;
+    }
+};
+
+// Permute the rows [F][32 V] of a float tile in place (eval_sparse.cuh), by the whole block.
 template <int V>
-__device__ void eval_set_sign(const uint4 *recs, int rb, int re, uint4 *st, const float *xl, int lane,
-                              int deflt, const int (&y)[V], bool uniform, int kmin, uint32_t (&hit)[V])
+__device__ __forceinline__ void permute_rows(float *xs, int F)
+{
+    constexpr int PIECES = 8 * V, ROWS = 32 / PIECES;     // 16-byte pieces of a row; rows per warp step
+    const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+    const int piece = lane % PIECES, sub = lane / PIECES;
+    for (int f0 = (threadIdx.x >> 5) * ROWS; f0 < F; f0 += warps * ROWS) {
+        const int f = f0 + sub;
+        float4 *row = reinterpret_cast<float4 *>(xs) + (size_t)f * PIECES;
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (f < F) x = row[piece];
+        __syncwarp();
+        if (f < F) row[piece ^ (f & 7)] = x;
+    }
+}
+
+// Evaluate one set (records [rb, re), format v4) on this lane's V samples (xs: the tile with permuted
+// rows). hit[v] gets its sign bit set when the sample's prediction equals its label: in a tile of one
+// label (`uniform`, label kmin) only rules of that class count; otherwise the per-sample label y[v]
+// (yl in memory) decides. y[v] < 0 marks padding. Once at most sparse::MAX samples are unclaimed, as
+// seen when a new 32-record chunk is reached, the rest of the set takes the sparse tail, whose
+// hits in a one-label tile come back as the lane's count `more`. The stage `st` (64 records) is at
+// a multiple of 512 bytes from xs. All lanes of the warp call this together.
+template <int V>
+__device__ void eval_set_sign(const uint4 *recs, int rb, int re, uint4 *st, const unsigned char *xs, int lane, int deflt,
+                              const int (&y)[V], const int32_t *yl, bool uniform, int kmin, uint32_t (&hit)[V], int &more)
 {
     const uint4 zero4 = make_uint4(0, 0, 0, 0);
+    const uint32_t lb = (uint32_t)lane * (4u * V);
     uint32_t claimed[V];
+    more = 0;
 #pragma unroll
     for (int v = 0; v < V; ++v) {
         claimed[v] = y[v] >= 0 ? 0u : SIGN;
@@ -174,6 +218,29 @@ __device__ void eval_set_sign(const uint4 *recs, int rb, int re, uint4 *st, cons
     int rel = 0;
     const int nrec = re - rb;
     while (rel < nrec) {
+        if ((rel >> 5) > ck) {
+            int open = 0;
+#pragma unroll
+            for (int v = 0; v < V; ++v) open += claimed[v] ? 0 : 1;
+            if (__reduce_add_sync(FULL, open) <= sparse::MAX) {
+                uint32_t cw = 0, hw = 0;
+#pragma unroll
+                for (int v = 0; v < V; ++v) cw |= claimed[v] >> (24 - 8 * v);
+                __syncwarp();
+                st[32 + lane] = make_uint4(0x3F800000u, 0x3F800000u, 0x3F800000u, 0x3F800000u);   // a row of 1.0
+                const Decode4 dec{(uint32_t)(reinterpret_cast<unsigned char *>(st + 32) - xs)};
+                sparse::WalkCount wc;
+                uint32_t *list = reinterpret_cast<uint32_t *>(st);
+                if (uniform)
+                    more = sparse::tail<V, true, false>(list, recs, rb, rel, nrec, lane, kmin, xs, yl, cw, deflt, hw, wc, dec);
+                else
+                    sparse::tail<V, false, false>(list, recs, rb, rel, nrec, lane, kmin, xs, yl, cw, deflt, hw, wc, dec);
+#pragma unroll
+                for (int v = 0; v < V; ++v) hit[v] |= (hw << (24 - 8 * v)) & SIGN;
+                __syncwarp();
+                return;
+            }
+        }
         while ((rel >> 5) > ck) {
             const uint4 keep = st[32 + lane];
             __syncwarp();
@@ -187,16 +254,16 @@ __device__ void eval_set_sign(const uint4 *recs, int rb, int re, uint4 *st, cons
         const uint4 *rp = st + (rel - 32 * ck);
         const uint4 r0 = rp[0];
         const int nc = max(1, (int)((r0.x >> LEN_SHIFT) & 0xFFFu));   // >= 1: progress
-        const int cls = (int)(r0.y >> CLS_SHIFT);
+        const int cls = (int)((r0.y >> CLS_SHIFT) & 0xFFFu);
         uint32_t acc[V];
 #pragma unroll
         for (int v = 0; v < V; ++v) acc[v] = claimed[v];
-        cond_mask<V>(r0, xl, acc);
+        cond_mask<V>(r0, xs, lb, acc);
         if (nc <= 33) {
 #pragma unroll 2
-            for (int k = 1; k < nc; ++k) cond_mask<V>(rp[k], xl, acc);
+            for (int k = 1; k < nc; ++k) cond_mask<V>(rp[k], xs, lb, acc);
         } else {
-            for (int k = 1; k < nc; ++k) cond_mask<V>(__ldcg(recs + rb + rel + k), xl, acc);
+            for (int k = 1; k < nc; ++k) cond_mask<V>(__ldcg(recs + rb + rel + k), xs, lb, acc);
         }
         uint32_t all = SIGN;
         if (uniform) {

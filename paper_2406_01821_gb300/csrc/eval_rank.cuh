@@ -22,11 +22,13 @@
 // to the lane's sample v). A set's records are one flat stream (each rule's conditions, the last
 // one flagged) walked 32 records at a time. Predictions are not produced here.
 #pragma once
+#include "eval_sparse.cuh"
 #include "rs_internal.cuh"
 
 namespace rs {
 namespace rank {
 
+using sparse::WalkCount;
 constexpr uint32_t FULL = 0xFFFFFFFFu;
 constexpr uint32_t HIGH = 0x80808080u;          // bit 7 of every byte
 constexpr uint32_t ONES = 0x01010101u;
@@ -47,21 +49,12 @@ __device__ __forceinline__ int count_below(const float *row, int sw, float c)
     return pos;
 }
 
-// Unclaimed samples up to which the rest of a set is walked sample by sample (sparse_tail). 4096 ragged
-// sets on 2^20 x 128: 53.4 ms without it, 46.5 / 45.0 / 45.2 / 45.4 ms with a limit of 8 / 16 / 24 /
-// 32; ten evolution generations of 10,000 sets of up to 32 rules on 100,000 x 32: 100.0 and 93.2 /
-// 92.2 / 92.5 / 92.5 ms.
-constexpr int SPARSE_MAX = 20;
-
 // pass rows per warp for pair / product conditions of one chunk
 template <int W> __host__ __device__ constexpr int vslots() { return W >= 32 ? 12 : 16; }
 constexpr uint32_t NOOP_K = 127u * ONES;     // constant - rank never has bit 7 set: never fails
 
-// 16-byte piece of a feature's row in the shared float tile that holds samples 4 l .. 4 l + 3: pieces
-// are permuted by l ^ (f & 7), so that one sample's values of 32 features fall on eight groups of
-// banks instead of one (the sparse walk reads them so); a warp reading whole rows is unaffected. A
-// staged row offset carries (f & 7) << 4, and a lane's piece is at (offset ^ (lane << 4)).
-__device__ __forceinline__ uint32_t row_off(uint32_t f) { return f * (T * 4u) | (f & 7u) << 4; }
+// A staged row offset of the float tile (eval_sparse.cuh).
+__device__ __forceinline__ uint32_t row_off(uint32_t f) { return sparse::row_off<T * 4>(f); }
 
 // The per-tile tables built in shared memory by the whole block once the tile's features xs
 // [F][T] and rank bytes rs [Frows][T] have landed: the reversed ranks (127 - rank) at rs + rev_off,
@@ -175,107 +168,28 @@ __device__ __forceinline__ void group4(const uint32_t (&e)[4], const uint32_t *s
 // chunk's pairs that the lanes build in parallel; padding records are no-ops. The chunk is then one
 // straight run of identical steps, with the first-fire claim applied after each rule's last record
 // (a warp vote gives their positions); the all-claimed exit is tested once per chunk.
-//
-// Sparse tail. The first rules claim most samples (each of the ragged workload's claims an eighth of
-// what is left), so that a set's last chunks are walked for a handful of samples: once at most
-// SPARSE_MAX samples are unclaimed, the roles turn (sparse_tail). The unclaimed samples are listed, one
-// per lane; each lane keeps one record of the chunk, and for one sample after another every lane tests
-// its condition (the original compare on the float tile: no cut search, no pass rows, no stage) and a
-// vote hands the 32 outcomes to the sample's lane. Each lane then finds its sample's first firing
-// rule with one addition.
-// Work a walk did: records, pair / product / membership conditions and rule ends (profiling counters).
-struct WalkCount {
-    uint32_t records = 0, rows = 0, ends = 0;
-};
-
-// The rest of a walk from record c0 (a rule's first) on, for at most 32 unclaimed samples of the tile.
-// With P the outcomes of a window's records on a sample, E the ends and S the first records of its
-// rules, (P & ~E) + S carries into a rule's end exactly when all records before it hold. A window
-// ends with a rule's last record; in a rule of more than 32 records a lane remembers that its sample
-// has failed (over). About 12 instructions and 10 shared-memory wavefronts a sample and 80
-// instructions a window, against about 500 and 140 for a dense chunk. Returns the lane's hits (UNI);
-// otherwise they go to the samples' words.
-template <bool UNI, bool CAT>
-__device__ __forceinline__ int sparse_tail(uint32_t *list, const uint4 *recs, int rb, int c0, int nrec, int lane, int F,
-                                           int kmine, const unsigned char *xs, uint32_t ones_off, const int32_t *yl,
-                                           uint32_t claimed, int deflt, uint32_t &hit, WalkCount &wc)
-{
-    const uint32_t below = (1u << lane) - 1u;
-    uint4 raw = c0 + lane < nrec ? __ldcg(recs + rb + c0 + lane) : make_uint4(0u, 0u, 0u, 0u);
-    // list the samples: entry i in lane i, the byte offset 4 n of sample n in a (permuted) row
-    int n = 0;
-    __syncwarp();
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-        const bool mine = ((claimed >> (8 * v)) & 0x80u) == 0u;
-        const uint32_t b = __ballot_sync(FULL, mine);
-        if (mine) list[n + __popc(b & below)] = (uint32_t)lane << 4 | (uint32_t)v << 2;
-        n += __popc(b);
-    }
-    __syncwarp();
-    uint32_t at = lane < n ? list[lane] : 0u;
-    int hits = 0;
-    bool over = false;
-    const auto give_back = [&](uint32_t b) {           // the samples of lanes b have hit
-        for (; b; b &= b - 1u) {
-            const uint32_t a = __shfl_sync(FULL, at, __ffs(b) - 1);
-            if (lane == (int)(a >> 4)) hit |= 0x80u << (2u * (a & 12u));
-        }
-    };
-    while (c0 < nrec && n) {
+// A record of format v5 on the sparse tail: fl(A x) > fl(B z), z = 1 but for pairs; a '<=' cut is the
+// negation of x > c.
+struct Decode5 {
+    int F;
+    uint32_t ones_off;
+    __device__ __forceinline__ sparse::Rec operator()(const uint4 raw) const
+    {
         const uint32_t tag = raw.x >> R5_TAG_SHIFT;
-        const uint32_t E = __ballot_sync(FULL, (raw.x & R5_END_BIT) != 0u);   // records from nrec on are 0
-        const int cnt = E ? 32 - __clz(E) : 32;
-        const bool cut = tag == R5_CUT_GT || tag == R5_CUT_LT, none = tag == R5_NONE, set = CAT && tag == R5_SET;
-        const uint32_t xo = row_off(min(raw.x & R5_F_MASK, (uint32_t)(F - 1)));
-        const uint32_t zo = tag == R5_PAIR ? row_off(min(raw.y, (uint32_t)(F - 1))) : ones_off;
-        // fl(A x) > fl(B z), z = 1 but for pairs; a '<=' cut is the negation of x > c (I)
-        const float A = cut ? 1.f : (none ? 0.f : __uint_as_float(raw.z));
-        const float B = cut ? __uint_as_float(raw.z) : (none ? -1.f : __uint_as_float(raw.w));
-        const uint32_t lo = raw.z, hi = raw.w;
-        const uint32_t I = __ballot_sync(FULL, tag == R5_CUT_LT);
-        const int cls = (int)((raw.x >> R5_CLS_SHIFT) & 0xFFFu);
-        const uint32_t K = UNI ? __ballot_sync(FULL, (raw.x & R5_END_BIT) != 0u && cls == kmine) : 0u;
-        c0 += cnt;
-        wc.records += min(cnt, nrec - c0 + cnt);
-        wc.rows += __popc(__ballot_sync(FULL, lane < cnt && tag >= R5_PAIR));
-        wc.ends += __popc(E);
-        raw = c0 + lane < nrec ? __ldcg(recs + rb + c0 + lane) : make_uint4(0u, 0u, 0u, 0u);
-        uint32_t P = 0;
-#pragma unroll 2
-        for (int i = 0; i < n; ++i) {
-            const uint32_t ai = __shfl_sync(FULL, at, i);
-            const float x = *reinterpret_cast<const float *>(xs + (xo ^ ai));
-            const float z = *reinterpret_cast<const float *>(xs + (zo ^ ai));
-            bool holds = __fmul_rn(A, x) > __fmul_rn(B, z);
-            if (CAT && set) holds = category_member(x, lo, hi);
-            const uint32_t v = __ballot_sync(FULL, holds);
-            if (lane == i) P = v;
-        }
-        P ^= I;
-        if (over) P &= ~1u;
-        const uint32_t fired = lane < n ? ((P & ~E) + (E << 1 | 1u)) & E & P : 0u;
-        const uint32_t first = fired & (0u - fired);
-        over = !E && (over || P != FULL);
-        if (UNI) {
-            if (first & K) ++hits;
-        } else {
-            const int k = __shfl_sync(FULL, cls, fired ? __ffs(first) - 1 : 0);
-            give_back(__ballot_sync(FULL, fired != 0u && k == __ldg(yl - 4 * lane + (at >> 2))));
-        }
-        const uint32_t stay = __ballot_sync(FULL, lane < n && fired == 0u);
-        if (__popc(stay) != n) {                       // close the list's gaps
-            n = __popc(stay);
-            if (fired == 0u && (stay >> lane & 1u)) list[__popc(stay & below)] = at;
-            __syncwarp();
-            at = lane < n ? list[lane] : 0u;
-            __syncwarp();
-        }
+        const bool cut = tag == R5_CUT_GT || tag == R5_CUT_LT, none = tag == R5_NONE;
+        sparse::Rec r;
+        r.xo = row_off(min(raw.x & R5_F_MASK, (uint32_t)(F - 1)));
+        r.zo = tag == R5_PAIR ? row_off(min(raw.y, (uint32_t)(F - 1))) : ones_off;
+        r.A = cut ? 1.f : (none ? 0.f : __uint_as_float(raw.z));
+        r.B = cut ? __uint_as_float(raw.z) : (none ? -1.f : __uint_as_float(raw.w));
+        r.inv = tag == R5_CUT_LT;
+        r.set = tag == R5_SET;
+        r.row = tag >= R5_PAIR;
+        r.end = (raw.x & R5_END_BIT) != 0u;
+        r.cls = (int)((raw.x >> R5_CLS_SHIFT) & 0xFFFu);
+        return r;
     }
-    if (UNI) return hits + (lane < n && deflt == kmine ? 1 : 0);
-    give_back(__ballot_sync(FULL, lane < n && deflt == __ldg(yl - 4 * lane + (at >> 2))));
-    return 0;
-}
+};
 
 // Returns the hit bits; `more` receives the lane's hits of the sparse tail that are not in them.
 template <bool UNI, int VS, bool CAT>
@@ -370,11 +284,11 @@ __device__ __forceinline__ uint32_t walk_set(uint4 *st, uint32_t *vrow, uint32_t
         wc.rows += __popc(pm | sm);
         wc.ends += __popc(ends);
         if (!live) break;
-        if (live <= SPARSE_MAX && ends && c0 < nrec) {      // from the first rule not finished yet
+        if (live <= sparse::MAX && ends && c0 < nrec) {      // from the first rule not finished yet
             const int tail = cnt - (32 - __clz(ends));
             wc.records += c0 - tail;
-            more = sparse_tail<UNI, CAT>(sw, recs, rb, c0 - tail, nrec, lane, F, kmine, xs, ones_off, yl, claimed, deflt,
-                                          hit, wc);
+            more = sparse::tail<4, UNI, CAT>(sw, recs, rb, c0 - tail, nrec, lane, kmine, xs, yl, claimed, deflt, hit, wc,
+                                             Decode5{F, ones_off});
             return hit;
         }
     }

@@ -11,7 +11,9 @@
 //
 // Per-class counting uses the label grouping of the dataset: in a tile holding one label k, only
 // rules of class k (and the default, if it is k) can add hits, decided once per rule for the whole
-// warp. Predictions are not produced here (the caller then uses the general evaluator).
+// warp, and the walk of a set ends after the last rule that can. The last few unclaimed samples are
+// walked one by one (eval_sparse.cuh; the tile's rows are permuted for it after they land).
+// Predictions are not produced here (the caller then uses the general evaluator).
 #include "rs_internal.cuh"
 #include "eval_core.cuh"
 #include "tma.cuh"
@@ -59,15 +61,18 @@ __global__ void __launch_bounds__(W * 32) k_hard4(const __grid_constant__ CUtens
     const int kmin = a.y[(int64_t)tile * S], kmax = a.y[t_last];
     const bool uniform = kmin == kmax;
 
-    if (!mbar_wait_bounded(bar, 0, TMA_WAIT_LIMIT_NS)) {
+    const bool landed = mbar_wait_bounded(bar, 0, TMA_WAIT_LIMIT_NS);
+    if (!__syncthreads_and(landed)) {
         if (threadIdx.x == 0) atomicOr(a.status, ST_WAIT_TIMEOUT);
-        mbar_wait_bounded(bar, 0, TMA_WAIT_LIMIT_NS);
+        mbar_wait_bounded(bar, 0, TMA_WAIT_LIMIT_NS);   // copies still in flight land first
         return;
     }
+    core::permute_rows<V>(xs, F);
+    __syncthreads();
 
     const int count = (a.P - group + G - 1) / G;
     uint4 *st = stage_all + warp * 64;
-    const float *xl = xs + lane * V;
+    const int32_t *yl = a.y + n0;
 
     while (true) {
         int m = 0;
@@ -76,11 +81,16 @@ __global__ void __launch_bounds__(W * 32) k_hard4(const __grid_constant__ CUtens
         if (m >= count) break;
         const int p = a.order[group + m * G];
         const SetInfo si = a.sets[p];
-        const int rb = si.rec_begin, re = si.rec_end;
+        const int rb = si.rec_begin;
+        // one label k in the tile: records after the set's last rule of class k (default of another
+        // class) or of any other class (default k) cannot change its count
+        const int re = (uniform && a.last_end) ? min(rb + a.last_end[(int64_t)p * a.K + kmin], si.rec_end) : si.rec_end;
 
         uint32_t hit[V];
-        core::eval_set_sign<V>(recs, rb, re, st, xl, lane, si.deflt, y, uniform, kmin, hit);
-        int hits = 0;
+        int more;
+        core::eval_set_sign<V>(recs, rb, re, st, reinterpret_cast<const unsigned char *>(xs), lane, si.deflt, y, yl,
+                               uniform, kmin, hit, more);
+        int hits = __reduce_add_sync(FULL, more);
 #pragma unroll
         for (int v = 0; v < V; ++v) hits += __popc(__ballot_sync(FULL, hit[v] != 0u));
         if (lane == 0 && hits) atomicAdd(&a.correct[p], hits);

@@ -132,6 +132,7 @@ __global__ void k_pack_rules2(BatchDev b, int F, int K, int S, int form, Rec *re
     uint4 *out = reinterpret_cast<uint4 *>(recs_out);
     const uint32_t len = (uint32_t)(c1 - c0);
     const uint32_t row16 = (uint32_t)S / 4;   // 16-byte units per feature row
+    const auto row = [&](int f) { return (uint32_t)f * row16 | (form == 4 ? (uint32_t)f & 7u : 0u); };
     for (int c = c0; c < c1; ++c) {
         const int f = b.cond_f[c], g = b.cond_g[c], op = b.cond_op[c];
         uint32_t w0 = len << LEN_SHIFT, w1 = (uint32_t)cls << CLS_SHIFT;
@@ -149,17 +150,18 @@ __global__ void k_pack_rules2(BatchDev b, int F, int K, int S, int form, Rec *re
             if (kind == KIND_GT) { v0 = 1.f; v1 = -nextafterf(c0, pinf); }
             else if (kind == KIND_LT) { v0 = -1.f; v1 = -nextafterf(-c0, pinf); }
             else { rewrite_lin(b.cond_a[c], b.cond_t[c], op, v0, v1); w0 |= GENERAL_BIT; }
-            w0 |= (uint32_t)f * row16;
+            w0 |= row(f);
         } else if (g < 0) {
             rewrite_lin(b.cond_a[c], b.cond_t[c], op, v0, v1);
-            w0 |= (uint32_t)f * row16;
+            w0 |= row(f);
         } else {
             const int lf = op == 0 ? f : g, rg = op == 0 ? g : f;
             v0 = op == 0 ? b.cond_a[c] : b.cond_b[c];
             v1 = op == 0 ? b.cond_b[c] : b.cond_a[c];
-            w0 |= ((uint32_t)lf * row16) | PAIR_BIT;
-            w1 |= (uint32_t)rg * row16;
+            w0 |= row(lf) | PAIR_BIT;
+            w1 |= row(rg);
         }
+        if (form == 4 && c == c1 - 1) w1 |= END4_BIT;
         out[c] = make_uint4(w0, w1, __float_as_uint(v0), __float_as_uint(v1));
     }
 }

@@ -86,6 +86,8 @@ constexpr int LEN_SHIFT = 19;
 constexpr int CLS_SHIFT = 18;
 // v4 only: a threshold condition that is not a +-1 cut (zero or infinite coefficient, never true)
 constexpr uint32_t GENERAL_BIT = 1u << 31;
+// v4 only, in w1: the last record of its rule. v4 row offsets carry the row's permutation (f & 7).
+constexpr uint32_t END4_BIT = 1u << 31;
 
 // Record format v5 (rank-coded evaluator): per rule its threshold cuts, its pair conditions and
 // its remaining product conditions, one record per condition (same positions as the conditions).

@@ -261,7 +261,8 @@ __global__ void __launch_bounds__(SW * 32, 1) k_serve(ServeArgs a)
         const int nvec = d.F * (SS / 4);
         for (int i = threadIdx.x; i < nvec; i += blockDim.x) {
             const int f = i / (SS / 4), c4 = i % (SS / 4);
-            reinterpret_cast<float4 *>(xs)[i] =
+            // the sign-mask form reads permuted rows (eval_sparse.cuh), the general form plain ones
+            reinterpret_cast<float4 *>(xs)[d.finite ? i ^ (f & 7) : i] =
                 *reinterpret_cast<const float4 *>(d.Xt + (int64_t)f * d.n_pad + col0 + 4 * c4);
         }
         const int64_t n0 = col0 + lane * SV;
@@ -289,10 +290,14 @@ __global__ void __launch_bounds__(SW * 32, 1) k_serve(ServeArgs a)
                 si.rec_begin = t.x; si.rec_end = t.y; si.deflt = t.z; si.cost = t.w;
             }
             bool hit[SV];
+            int more = 0;
             if (d.finite) {
                 uint32_t h[SV];
-                core::eval_set_sign<SV>(d.recs, si.rec_begin, si.rec_end, st, xl, lane, si.deflt, y,
-                                        uniform, kmin, h);
+                int re = si.rec_end;
+                if (uniform && d.last_end)
+                    re = min(si.rec_begin + __ldcg(d.last_end + (int64_t)p * d.K + kmin), re);
+                core::eval_set_sign<SV>(d.recs, si.rec_begin, re, st, smem, lane, si.deflt, y, d.y + n0, uniform, kmin, h,
+                                        more);
 #pragma unroll
                 for (int v = 0; v < SV; ++v) hit[v] = h[v] != 0u;
             } else {
@@ -301,7 +306,7 @@ __global__ void __launch_bounds__(SW * 32, 1) k_serve(ServeArgs a)
 #pragma unroll
                 for (int v = 0; v < SV; ++v) hit[v] = pred[v] == y[v];
             }
-            int hits = 0;
+            int hits = __reduce_add_sync(core::FULL, more);
 #pragma unroll
             for (int v = 0; v < SV; ++v) hits += __popc(__ballot_sync(core::FULL, hit[v]));
             if (lane == 0 && hits) atomicAdd(&d.correct[p], hits);

@@ -544,10 +544,11 @@ def test_measured_pipe_rates():
 
 
 @pytest.mark.parametrize("F,K,cat", [(3, 2, False), (9, 40, False), (128, 5, False), (16, 3, True)])
-def test_sparse_tail_of_the_rank_coded_walk(orc, F, K, cat):
+def test_sparse_tail_of_the_walks(orc, F, K, cat):
     """Sets whose first rules leave 0 to 40 samples of a 128-sample tile unclaimed, followed by rules
     that straddle the 32-record windows (up to 100 conditions), with pairs, ties, both
-    comparisons, products and membership tests, on tiles of one label and of several."""
+    comparisons, products and membership tests, on tiles of one label and of several: the
+    rank-coded and the sign-mask forms and the serving units."""
     import torch
     from paper_2406_01821_gb300 import build, rs
     build.build()
@@ -584,7 +585,7 @@ def test_sparse_tail_of_the_rank_coded_walk(orc, F, K, cat):
     oc, opc, _ = orc.eval_hard(X, y, K, b)
     with rs.Context(0) as ctx:
         ds = ctx.dataset(X, y, K)
-        for tile in (21, 22):
+        for tile in (16, 17, 18, 19, 20, 21, 22):
             ctx.set_tile_config(tile)
             c, pc, _ = ctx.eval_hard(ds, rs.DeviceBatch.from_host(b), K)
             torch.cuda.synchronize()
