@@ -279,12 +279,13 @@ __device__ __forceinline__ uint32_t walk_set(uint4 *st, uint32_t *vrow, uint32_t
 #undef RS_GROUP4
             }
         }
-        const int live = __reduce_add_sync(FULL, __popc(~claimed & HIGH));    // 0: the set is decided
         c0 += cnt;
         wc.rows += __popc(pm | sm);
         wc.ends += __popc(ends);
+        if (c0 >= nrec) break;
+        const int live = __reduce_add_sync(FULL, __popc(~claimed & HIGH));    // 0: the set is decided
         if (!live) break;
-        if (live <= sparse::MAX && ends && c0 < nrec) {      // from the first rule not finished yet
+        if (live <= sparse::MAX && ends) {                   // from the first rule not finished yet
             const int tail = cnt - (32 - __clz(ends));
             wc.records += c0 - tail;
             more = sparse::tail<4, UNI, CAT>(sw, recs, rb, c0 - tail, nrec, lane, kmine, xs, yl, claimed, deflt, hit, wc,

@@ -12,7 +12,9 @@
 // Per-class counting uses the label grouping of the dataset: in a tile holding one label k, only
 // rules of class k (and the default, if it is k) can add hits, decided once per rule for the whole
 // warp, and the walk of a set ends after the last rule that can. The last few unclaimed samples are
-// walked one by one (eval_sparse.cuh; the tile's rows are permuted for it after they land).
+// walked one by one (eval_sparse.cuh; the tile's rows are permuted for it after they land): 600 ragged
+// sets on 150,001 x 233, 2.54 -> 1.95 ms. The walk itself is bound by instruction issue and the
+// shared-memory pipe together (a 16-byte row read per condition and lane).
 // Predictions are not produced here (the caller then uses the general evaluator).
 #include "rs_internal.cuh"
 #include "eval_core.cuh"
