@@ -409,7 +409,8 @@ rs_status rs_tile_config_info(int32_t id, int32_t *samples_per_tile, int32_t *wa
 /* Evaluator form of configuration `id`: 1 condition at a time; 2 rule at a time; 3 rule at a
  * time with the margin minimum; 4 sign-mask conjunction (finite datasets, else runs as 3);
  * 5 rank-coded cuts (datasets with rank tables: finite and at most 160 features; else runs as
- * 4, then 3). Forms 4 and 5 produce counts only: a call that asks for predictions runs as 3.
+ * 4, then 3). Form 4 produces counts only, form 5 predictions too for up to 256 classes: other
+ * calls that ask for predictions run as 3.
  * The other configurations stage a feature tile in shared memory and need F small enough for
  * it; configuration 23 (form 1) reads the features from global memory and takes any F. */
 rs_status rs_tile_config_form(int32_t id, int32_t *form);

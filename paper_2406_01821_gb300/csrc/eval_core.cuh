@@ -232,9 +232,9 @@ __device__ void eval_set_sign(const uint4 *recs, int rb, int re, uint4 *st, cons
                 sparse::WalkCount wc;
                 uint32_t *list = reinterpret_cast<uint32_t *>(st);
                 if (uniform)
-                    more = sparse::tail<V, true, false>(list, recs, rb, rel, nrec, lane, kmin, xs, yl, cw, deflt, hw, wc, dec);
+                    more = sparse::tail<V, true, false, false>(list, recs, rb, rel, nrec, lane, kmin, xs, yl, cw, deflt, hw, wc, dec);
                 else
-                    sparse::tail<V, false, false>(list, recs, rb, rel, nrec, lane, kmin, xs, yl, cw, deflt, hw, wc, dec);
+                    sparse::tail<V, false, false, false>(list, recs, rb, rel, nrec, lane, kmin, xs, yl, cw, deflt, hw, wc, dec);
 #pragma unroll
                 for (int v = 0; v < V; ++v) hit[v] |= (hw << (24 - 8 * v)) & SIGN;
                 __syncwarp();

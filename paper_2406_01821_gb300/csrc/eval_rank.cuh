@@ -20,7 +20,7 @@
 // and product conditions are compared on the float tile and packed into the same byte layout.
 // Claims, per-class hits and the all-claimed exit work on these words (bit 7 of byte v belongs
 // to the lane's sample v). A set's records are one flat stream (each rule's conditions, the last
-// one flagged) walked 32 records at a time. Predictions are not produced here.
+// one flagged) walked 32 records at a time.
 #pragma once
 #include "eval_sparse.cuh"
 #include "rs_internal.cuh"
@@ -135,7 +135,8 @@ __device__ __forceinline__ uint32_t set_row(uint4 q, const unsigned char *xs, ui
 }
 
 // One group of four staged records with end-of-rule flags M (bit u: record u ends its rule).
-template <uint32_t M, bool UNI>
+// PRED: the class words are the class in every byte, and hit holds the predicted classes, a byte a sample.
+template <uint32_t M, bool UNI, bool PRED>
 __device__ __forceinline__ void group4(const uint32_t (&e)[4], const uint32_t *sw, const int32_t *yl,
                                        uint32_t &fail, uint32_t &claimed, uint32_t &hit)
 {
@@ -148,7 +149,11 @@ __device__ __forceinline__ void group4(const uint32_t (&e)[4], const uint32_t *s
         if (M & (1u << u)) {
             const uint32_t w = ws[u];
             const uint32_t newly = ~fail & HIGH;
-            if (UNI) hit |= newly & w;
+            if (PRED) {
+                uint32_t m;                                              // bit 7 spread over its byte
+                asm("prmt.b32 %0, %1, 0, 0xBA98;" : "=r"(m) : "r"(newly));
+                hit = (w & m) | (hit & ~m);
+            } else if (UNI) hit |= newly & w;
             else hit |= newly & class_bytes(yl, (int)w);
             claimed |= newly;
             fail = claimed;
@@ -168,6 +173,8 @@ __device__ __forceinline__ void group4(const uint32_t (&e)[4], const uint32_t *s
 // chunk's pairs that the lanes build in parallel; padding records are no-ops. The chunk is then one
 // straight run of identical steps, with the first-fire claim applied after each rule's last record
 // (a warp vote gives their positions); the all-claimed exit is tested once per chunk.
+// PRED: instead of hits, the predicted class of each of the lane's samples, a byte each (classes below
+// 256), the default where no rule fires.
 // A record of format v5 on the sparse tail: fl(A x) > fl(B z), z = 1 but for pairs; a '<=' cut is the
 // negation of x > c.
 struct Decode5 {
@@ -192,7 +199,7 @@ struct Decode5 {
 };
 
 // Returns the hit bits; `more` receives the lane's hits of the sparse tail that are not in them.
-template <bool UNI, int VS, bool CAT>
+template <bool UNI, int VS, bool CAT, bool PRED = false>
 __device__ __forceinline__ uint32_t walk_set(uint4 *st, uint32_t *vrow, uint32_t vrow_off, int lane,
                                              const uint4 *recs, int rb, int nrec, const float *us,
                                              uint32_t rev_off, int F, int kmine, const unsigned char *rl,
@@ -205,7 +212,7 @@ __device__ __forceinline__ uint32_t walk_set(uint4 *st, uint32_t *vrow, uint32_t
     uint2 *s8 = reinterpret_cast<uint2 *>(st);            // staged {offset, constant}, 32 entries
     uint32_t *sw = reinterpret_cast<uint32_t *>(st) + 64;  // end-of-rule class mask / class
     uint4 pf = lane < nrec ? __ldcg(recs + rb + lane) : zero4;
-    uint32_t hit = 0, fail = claimed;
+    uint32_t hit = PRED ? (uint32_t)deflt * ONES : 0u, fail = claimed;
     more = 0;
     int c0 = 0;
     while (c0 < nrec) {
@@ -228,7 +235,7 @@ __device__ __forceinline__ uint32_t walk_set(uint4 *st, uint32_t *vrow, uint32_t
         // every lane runs the cut search (branch-free staging); other records then take their form.
         // A pair or product condition gets a pass-row slot and a pair-table entry.
         const uint32_t cls = (raw.x >> R5_CLS_SHIFT) & 0xFFFu;
-        const uint32_t ew = UNI ? ((int)cls == kmine ? 0xFFFFFFFFu : 0u) : cls;
+        const uint32_t ew = PRED ? cls * ONES : (UNI ? ((int)cls == kmine ? 0xFFFFFFFFu : 0u) : cls);
         uint2 sr = stage_cut(raw, us, rev_off, F);
         const int np = __popc(pm);
         if ((pm >> lane) & 1u) {
@@ -272,7 +279,7 @@ __device__ __forceinline__ uint32_t walk_set(uint4 *st, uint32_t *vrow, uint32_t
             const uint32_t e[4] = {e0, e1, e2, e3};
             const uint32_t *swg = sw + g;
             switch ((ends >> g) & 0xFu) {
-#define RS_GROUP4(M) case M: group4<M, UNI>(e, swg, yl, fail, claimed, hit); break;
+#define RS_GROUP4(M) case M: group4<M, UNI, PRED>(e, swg, yl, fail, claimed, hit); break;
             RS_GROUP4(0) RS_GROUP4(1) RS_GROUP4(2) RS_GROUP4(3) RS_GROUP4(4) RS_GROUP4(5) RS_GROUP4(6)
             RS_GROUP4(7) RS_GROUP4(8) RS_GROUP4(9) RS_GROUP4(10) RS_GROUP4(11) RS_GROUP4(12)
             RS_GROUP4(13) RS_GROUP4(14) RS_GROUP4(15)
@@ -288,12 +295,13 @@ __device__ __forceinline__ uint32_t walk_set(uint4 *st, uint32_t *vrow, uint32_t
         if (live <= sparse::MAX && ends) {                   // from the first rule not finished yet
             const int tail = cnt - (32 - __clz(ends));
             wc.records += c0 - tail;
-            more = sparse::tail<4, UNI, CAT>(sw, recs, rb, c0 - tail, nrec, lane, kmine, xs, yl, claimed, deflt, hit, wc,
+            more = sparse::tail<4, UNI, CAT, PRED>(sw, recs, rb, c0 - tail, nrec, lane, kmine, xs, yl, claimed, deflt, hit, wc,
                                              Decode5{F, ones_off});
             return hit;
         }
     }
     wc.records += c0;
+    if (PRED) return hit;
     const uint32_t left = ~claimed & HIGH;
     if (UNI) hit |= (deflt == kmine) ? left : 0u;
     else hit |= left & class_bytes(yl, deflt);

@@ -47,8 +47,9 @@ struct Rec {
 // ends with a rule's last record; in a rule of more than 32 records a lane remembers that its sample
 // has failed (over). About 12 instructions and 10 shared-memory wavefronts a sample and 80
 // instructions a window, against about 500 and 140 for a dense chunk. Returns the lane's hits (UNI);
-// otherwise they go to the samples' words.
-template <int V, bool UNI, bool CAT, class Decode>
+// otherwise they go to the samples' words. PRED (four samples a lane): `hit` holds the predicted
+// classes, a byte a sample, and receives those of the tail through 32 words after the list.
+template <int V, bool UNI, bool CAT, bool PRED, class Decode>
 __device__ __forceinline__ int tail(uint32_t *list, const uint4 *recs, int rb, int c0, int nrec, int lane, int kmine,
                                     const unsigned char *xs, const int32_t *yl, uint32_t claimed, int deflt,
                                     uint32_t &hit, WalkCount &wc, const Decode &decode)
@@ -67,6 +68,11 @@ __device__ __forceinline__ int tail(uint32_t *list, const uint4 *recs, int rb, i
     }
     __syncwarp();
     uint32_t at = lane < n ? list[lane] : 0u;
+    static_assert(!PRED || V == 4, "a word of four classes per lane");
+    if (PRED) {
+        list[32 + lane] = hit;
+        __syncwarp();
+    }
     int hits = 0;
     bool over = false;
     const auto give_back = [&](uint32_t b) {           // the samples of lanes b have hit
@@ -103,7 +109,10 @@ __device__ __forceinline__ int tail(uint32_t *list, const uint4 *recs, int rb, i
         const uint32_t fired = lane < n ? ((P & ~E) + (E << 1 | 1u)) & E & P : 0u;
         const uint32_t first = fired & (0u - fired);
         over = !E && (over || P != FULL);
-        if (UNI) {
+        if (PRED) {
+            const int k = __shfl_sync(FULL, r.cls, fired ? __ffs(first) - 1 : 0);
+            if (fired) reinterpret_cast<unsigned char *>(list + 32)[at >> 2] = (unsigned char)k;
+        } else if (UNI) {
             if (first & K) ++hits;
         } else {
             const int k = __shfl_sync(FULL, r.cls, fired ? __ffs(first) - 1 : 0);
@@ -117,6 +126,12 @@ __device__ __forceinline__ int tail(uint32_t *list, const uint4 *recs, int rb, i
             at = lane < n ? list[lane] : 0u;
             __syncwarp();
         }
+    }
+    if (PRED) {
+        __syncwarp();
+        hit = list[32 + lane];
+        __syncwarp();
+        return 0;
     }
     if (UNI) return hits + (lane < n && deflt == kmine ? 1 : 0);
     give_back(__ballot_sync(FULL, lane < n && deflt == __ldg(yl - V * lane + (at >> 2))));

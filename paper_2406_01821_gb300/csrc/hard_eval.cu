@@ -279,8 +279,11 @@ int tile_config_count() { return kNumConfigs; }
 
 int effective_version(const TileConfig &tc, const Dataset &ds, bool preds)
 {
-    if (tc.ver >= 4 && (preds || !ds.finite)) return 3;   // same V and W exist for version 3
-    if (tc.ver == 5 && (!ds.ranked || hard5_smem_bytes(ds.F, tc.W) > 227 * 1024)) return 4;
+    if (tc.ver >= 4 && !ds.finite) return 3;              // same V and W exist for version 3
+    const bool ranked = tc.ver == 5 && ds.ranked && hard5_smem_bytes(ds.F, tc.W) <= 227 * 1024;
+    // the rank-coded form writes predictions as bytes; the sign-mask form writes none
+    if (tc.ver >= 4 && preds && !(ranked && ds.K <= 256)) return 3;
+    if (tc.ver == 5 && !ranked) return 4;
     return tc.ver;
 }
 

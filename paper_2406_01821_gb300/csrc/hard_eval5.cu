@@ -11,7 +11,11 @@ namespace {
 using namespace rank;
 constexpr uint64_t TMA_WAIT_LIMIT_NS = 2000000000ull;
 
-template <int W, bool CAT>
+// PRED: every sample's prediction is written (class counts up to 256), in the caller's sample order:
+// four scattered 4-byte stores a lane, which L2 gathers (the store adds 10 to 20 us to 200 sets on
+// 100,000 samples). The predicted classes of a lane's samples are the bytes of one word; the walk has
+// no class-tail stop, and hits are the bytes equal to the label's.
+template <int W, bool CAT, bool PRED>
 __global__ void __launch_bounds__(W * 32, 1) k_hard5(const __grid_constant__ CUtensorMap tmx,
                                                   const __grid_constant__ CUtensorMap tmr, HardArgs a)
 {
@@ -30,6 +34,7 @@ __global__ void __launch_bounds__(W * 32, 1) k_hard5(const __grid_constant__ CUt
     uint64_t *bar = reinterpret_cast<uint64_t *>(vrows + W * VS * 32);
     int *next = reinterpret_cast<int *>(bar + 1);
     uint32_t *walked = reinterpret_cast<uint32_t *>(bar + 2);        // [W][4] work counters (counting)
+    int32_t *place = reinterpret_cast<int32_t *>(walked + 4 * W);    // [T] the caller's sample, or -1 (PRED)
     const uint4 *recs = reinterpret_cast<const uint4 *>(a.recs);
 
     const int tile = blockIdx.x, group = blockIdx.y, G = gridDim.y;
@@ -63,13 +68,22 @@ __global__ void __launch_bounds__(W * 32, 1) k_hard5(const __grid_constant__ CUt
     }
     const uint32_t rev_off = (uint32_t)Frows * T;
     build_tile_tables(reinterpret_cast<float *>(xs), rs, rev_off, us, F);
-    if (threadIdx.x < T) ones[threadIdx.x] = 1.f;
+    if (threadIdx.x < T) {
+        ones[threadIdx.x] = 1.f;
+        const int64_t n = (int64_t)tile * T + threadIdx.x;
+        if (PRED) place[threadIdx.x] = n < a.N ? a.perm[n] : -1;
+    }
     __syncthreads();
 
     const unsigned char *rl = rs + lane * 4;       // this lane's four rank bytes of row 0
     const uint32_t ones_off = (uint32_t)Frows * T * 4;
     const int count = (a.P - group + G - 1) / G;
     uint4 *st = stage_all + warp * 32;
+    uint32_t label4 = 0;                           // the labels of the lane's samples, a byte each
+    if (PRED) {
+        const int4 y = *reinterpret_cast<const int4 *>(yl);
+        label4 = (uint32_t)(y.x & 0xFF) | (uint32_t)(y.y & 0xFF) << 8 | (uint32_t)(y.z & 0xFF) << 16 | (uint32_t)(y.w & 0xFF) << 24;
+    }
 
     while (true) {
         int m = 0;
@@ -81,7 +95,7 @@ __global__ void __launch_bounds__(W * 32, 1) k_hard5(const __grid_constant__ CUt
         const int rb = si.rec_begin;
         // one label k in the tile: records after the set's last rule of class k (default of another
         // class) or of any other class (default k) cannot change its count
-        const int nrec = (uniform && a.last_end)
+        const int nrec = (!PRED && uniform && a.last_end)
                              ? min(a.last_end[(int64_t)p * a.K + kmin], si.rec_end - si.rec_begin)
                              : si.rec_end - si.rec_begin;
 
@@ -89,11 +103,25 @@ __global__ void __launch_bounds__(W * 32, 1) k_hard5(const __grid_constant__ CUt
         const uint32_t vr_off = (uint32_t)(reinterpret_cast<unsigned char *>(vr) - rs);
         WalkCount wc;
         int more;
-        const uint32_t hit =
-            uniform ? walk_set<true, VS, CAT>(st, vr, vr_off, lane, recs, rb, nrec, us, rev_off, F, kmin, rl, xs,
-                                              ones_off, yl, claimed0, si.deflt, wc, more)
-                    : walk_set<false, VS, CAT>(st, vr, vr_off, lane, recs, rb, nrec, us, rev_off, F, -2, rl, xs,
-                                               ones_off, yl, claimed0, si.deflt, wc, more);
+        uint32_t hit;
+        if (PRED) {
+            const uint32_t pred = walk_set<false, VS, CAT, true>(st, vr, vr_off, lane, recs, rb, nrec, us, rev_off, F, -2, rl,
+                                                                 xs, ones_off, yl, claimed0, si.deflt, wc, more);
+            const int4 to = *reinterpret_cast<const int4 *>(place + 4 * lane);
+            int32_t *out = a.preds + (int64_t)p * a.N;
+            if (to.x >= 0) out[to.x] = (int32_t)(pred & 0xFFu);
+            if (to.y >= 0) out[to.y] = (int32_t)(pred >> 8 & 0xFFu);
+            if (to.z >= 0) out[to.z] = (int32_t)(pred >> 16 & 0xFFu);
+            if (to.w >= 0) out[to.w] = (int32_t)(pred >> 24);
+            const uint32_t d = pred ^ label4;      // a byte of 0: a hit
+            hit = ~(((d & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | d) & HIGH & ~claimed0;
+        } else if (uniform) {
+            hit = walk_set<true, VS, CAT>(st, vr, vr_off, lane, recs, rb, nrec, us, rev_off, F, kmin, rl, xs, ones_off, yl,
+                                          claimed0, si.deflt, wc, more);
+        } else {
+            hit = walk_set<false, VS, CAT>(st, vr, vr_off, lane, recs, rb, nrec, us, rev_off, F, -2, rl, xs, ones_off, yl,
+                                           claimed0, si.deflt, wc, more);
+        }
         if (a.walked && lane == 0) {           // the warp's own slots: no atomics
             uint32_t *wk = walked + 4 * warp;
             wk[0] += wc.records;
@@ -124,10 +152,10 @@ size_t hard5_smem_bytes(int F, int W)
     const int Fb = F < 256 ? F : 256;
     const size_t Frows = (size_t)((F + Fb - 1) / Fb) * Fb;
     const size_t vs = W >= 32 ? vslots<32>() : vslots<16>();
-    return Frows * T * (4 + 2 + 4) + (size_t)W * 32 * 16 + (size_t)W * vs * 32 * 4 + T * 4 + 16 + (size_t)W * 16;
+    return Frows * T * (4 + 2 + 4) + (size_t)W * 32 * 16 + (size_t)W * vs * 32 * 4 + T * 4 + 16 + (size_t)W * 16 + T * 4;
 }
 
-template <int W, bool CAT>
+template <int W, bool CAT, bool PRED>
 static rs_status launch5_t(Ctx *ctx, Dataset *ds, const HardArgs &a, cudaStream_t stream)
 {
     const size_t smem = hard5_smem_bytes(a.F, W);
@@ -135,7 +163,7 @@ static rs_status launch5_t(Ctx *ctx, Dataset *ds, const HardArgs &a, cudaStream_
     static std::once_flag once;
     static cudaError_t attr_err = cudaSuccess;
     std::call_once(once, [&] {
-        attr_err = cudaFuncSetAttribute(k_hard5<W, CAT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        attr_err = cudaFuncSetAttribute(k_hard5<W, CAT, PRED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)ctx->smem_optin);
     });
     if (attr_err != cudaSuccess) return cuda_fail(attr_err, "cudaFuncSetAttribute(k_hard5)");
@@ -146,7 +174,7 @@ static rs_status launch5_t(Ctx *ctx, Dataset *ds, const HardArgs &a, cudaStream_
     dim3 grid(tiles, a.groups);
     {
         TimedLaunch tl(ctx, TK_HARD, stream);
-        k_hard5<W, CAT><<<grid, W * 32, smem, stream>>>(*tmx, *tmr, a);
+        k_hard5<W, CAT, PRED><<<grid, W * 32, smem, stream>>>(*tmx, *tmr, a);
     }
     RS_CUDA(cudaGetLastError());
     count_launch(ctx);
@@ -156,8 +184,12 @@ static rs_status launch5_t(Ctx *ctx, Dataset *ds, const HardArgs &a, cudaStream_
 rs_status launch_hard5(Ctx *ctx, Dataset *ds, int W, const HardArgs &a, cudaStream_t stream)
 {
     if (a.P == 0) return RS_OK;
-    if (W == 16) return a.cat ? launch5_t<16, true>(ctx, ds, a, stream) : launch5_t<16, false>(ctx, ds, a, stream);
-    if (W == 32) return a.cat ? launch5_t<32, true>(ctx, ds, a, stream) : launch5_t<32, false>(ctx, ds, a, stream);
+    if (a.preds) {
+        if (W == 16) return a.cat ? launch5_t<16, true, true>(ctx, ds, a, stream) : launch5_t<16, false, true>(ctx, ds, a, stream);
+        if (W == 32) return a.cat ? launch5_t<32, true, true>(ctx, ds, a, stream) : launch5_t<32, false, true>(ctx, ds, a, stream);
+    }
+    if (W == 16) return a.cat ? launch5_t<16, true, false>(ctx, ds, a, stream) : launch5_t<16, false, false>(ctx, ds, a, stream);
+    if (W == 32) return a.cat ? launch5_t<32, true, false>(ctx, ds, a, stream) : launch5_t<32, false, false>(ctx, ds, a, stream);
     return RS_ERR_INVALID;
 }
 
@@ -166,10 +198,14 @@ rs_status launch_hard5(Ctx *ctx, Dataset *ds, int W, const HardArgs &a, cudaStre
 void preload_hard5_kernels()
 {
     cudaFuncAttributes fa;
-    cudaFuncGetAttributes(&fa, k_hard5<16, false>);
-    cudaFuncGetAttributes(&fa, k_hard5<16, true>);
-    cudaFuncGetAttributes(&fa, k_hard5<32, false>);
-    cudaFuncGetAttributes(&fa, k_hard5<32, true>);
+    cudaFuncGetAttributes(&fa, k_hard5<16, false, false>);
+    cudaFuncGetAttributes(&fa, k_hard5<16, false, true>);
+    cudaFuncGetAttributes(&fa, k_hard5<16, true, false>);
+    cudaFuncGetAttributes(&fa, k_hard5<16, true, true>);
+    cudaFuncGetAttributes(&fa, k_hard5<32, false, false>);
+    cudaFuncGetAttributes(&fa, k_hard5<32, false, true>);
+    cudaFuncGetAttributes(&fa, k_hard5<32, true, false>);
+    cudaFuncGetAttributes(&fa, k_hard5<32, true, true>);
 }
 
 }  // namespace rs
