@@ -112,18 +112,31 @@ static std::string tune_key(const Dataset &ds, const rs_batch *b)
     return k.str();
 }
 
-static int heuristic_tile(const Dataset &ds)
+static int heuristic_tile(const Dataset &ds, int P, bool cat)
 {
-    // The rank-coded evaluator with 32 warps (it runs as the sign-mask form on datasets without
-    // rank tables and as the margin-minimum form on non-finite data), then smaller tiles for wide
-    // data, and for data too wide for any shared tile the configuration reading global memory.
+    // Datasets with rank tables: the rank-coded evaluator. Two CTAs of 16 warps where both fit an SM
+    // (up to 63 features): one stages its tile while the other walks (46 sets on 470,000 x 30: 201 us
+    // against 256 with one CTA of 32 warps; 800 sets: 1859 and 1873). Wider: one CTA of 32 warps,
+    // or of 16 where the tables leave no room for 32 (129 < F < 155: 800 sets on 100,000 x 150, 721 us
+    // against 760 with the sign-mask form). A few sets cannot pay for the tables of wide tiles: up
+    // to 32, the sign-mask form in small CTAs (16 sets on 470,000 x 106: 190 us against 257; at 46 sets
+    // 306 and 296).
+    if (ds.ranked) {
+        const size_t s16 = hard5_smem_bytes(ds.F, 16), s32 = hard5_smem_bytes(ds.F, 32), most = 227 * 1024;
+        if (2 * (s16 + 1024) <= most + 1024) return 21;
+        if (P <= 32 && !cat && tile_config_fits(tile_config(16), ds.F)) return 16;
+        if (s32 <= most) return 22;
+        if (s16 <= most) return 21;
+    }
+    // Else the 32-warp sign-mask form (margin-minimum form on non-finite data), then smaller tiles for
+    // wide data, and for data too wide for any shared tile the configuration reading global memory.
     static const int prefs[] = {22, 21, 18, 16, 20, 3, 5, 23};
     for (int id : prefs)
         if (tile_config_fits(tile_config(id), ds.F)) return id;
     return 5;
 }
 
-int heuristic_tile_for(const Dataset &ds) { return heuristic_tile(ds); }
+int heuristic_tile_for(const Dataset &ds, int P, bool cat) { return heuristic_tile(ds, P, cat); }
 
 static int pick_tile(Ctx *ctx, const Dataset &ds, const rs_batch *b)
 {
@@ -135,7 +148,7 @@ static int pick_tile(Ctx *ctx, const Dataset &ds, const rs_batch *b)
         if (it != ctx->tune_table.end() && tile_config_fits(tile_config(it->second), ds.F))
             return it->second;
     }
-    return heuristic_tile(ds);
+    return heuristic_tile(ds, b->P, b->cond_set != nullptr);
 }
 
 // Strict reader of the cache file written by save_tune_table: {"key": id, ...} with ids of

@@ -50,7 +50,7 @@ __device__ __forceinline__ int count_below(const float *row, int sw, float c)
 }
 
 // pass rows per warp for pair / product conditions of one chunk
-template <int W> __host__ __device__ constexpr int vslots() { return W >= 32 ? 12 : 16; }
+constexpr int VSLOTS = 12;
 constexpr uint32_t NOOP_K = 127u * ONES;     // constant - rank never has bit 7 set: never fails
 
 // A staged row offset of the float tile (eval_sparse.cuh).

@@ -641,7 +641,7 @@ rs_status evolve_run(Ctx *ctx, uint64_t ds_h, const rs_evolve_config *cfg, rs_po
     // a configuration forced on the context (rs_set_tile_config) applies here too, else the heuristic
     const TileConfig &tc = tile_config(ctx->forced_tile >= 0 && tile_config_fits(tile_config(ctx->forced_tile), ds.F)
                                            ? ctx->forced_tile
-                                           : heuristic_tile_for(ds));
+                                           : heuristic_tile_for(ds, P, false));
     auto evaluate = [&](int nsub, int32_t *out_fit, cudaStream_t st) -> rs_status {
         BatchDev bd{};
         bd.P = nsub;

@@ -42,7 +42,8 @@ __global__ void __launch_bounds__(W * 32) k_hard4(const __grid_constant__ CUtens
     int *next = reinterpret_cast<int *>(bar + 1);
     const uint4 *recs = reinterpret_cast<const uint4 *>(a.recs);
 
-    const int tile = blockIdx.x, group = blockIdx.y, G = gridDim.y;
+    const TileTask task(a);
+    const int tile = task.tile, group = task.group, G = task.groups;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
     if (threadIdx.x == 0) {
@@ -114,7 +115,7 @@ __global__ void __launch_bounds__(W * 32) k_hard4(const __grid_constant__ CUtens
 }  // namespace
 
 template <int V, int W>
-rs_status launch4_t(Ctx *ctx, Dataset *ds, const HardArgs &a, cudaStream_t stream)
+rs_status launch4_t(Ctx *ctx, Dataset *ds, HardArgs a, cudaStream_t stream)
 {
     const int Fb = a.F < 256 ? a.F : 256;
     const int Frows = ((a.F + Fb - 1) / Fb) * Fb;
@@ -129,8 +130,9 @@ rs_status launch4_t(Ctx *ctx, Dataset *ds, const HardArgs &a, cudaStream_t strea
     if (attr_err != cudaSuccess) return cuda_fail(attr_err, "cudaFuncSetAttribute(k_hard4)");
     const CUtensorMap *tm = dataset_tmap(ds, 32 * V);
     if (!tm) return RS_ERR_DEVICE;
-    const int tiles = (int)((a.N + 32 * V - 1) / (32 * V));
-    dim3 grid(tiles, a.groups);
+    int resident = 1;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, k_hard4<V, W>, W * 32, smem);
+    const int grid = split_tiles(ctx, a.N, a.F, a.P, 32 * V, W, resident, a);
     {
         TimedLaunch tl(ctx, TK_HARD, stream);
         k_hard4<V, W><<<grid, W * 32, smem, stream>>>(*tm, a);

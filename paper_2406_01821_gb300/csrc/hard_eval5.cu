@@ -16,7 +16,7 @@ constexpr uint64_t TMA_WAIT_LIMIT_NS = 2000000000ull;
 // 100,000 samples). The predicted classes of a lane's samples are the bytes of one word; the walk has
 // no class-tail stop, and hits are the bytes equal to the label's.
 template <int W, bool CAT, bool PRED>
-__global__ void __launch_bounds__(W * 32, 1) k_hard5(const __grid_constant__ CUtensorMap tmx,
+__global__ void __launch_bounds__(W * 32, 32 / W) k_hard5(const __grid_constant__ CUtensorMap tmx,
                                                   const __grid_constant__ CUtensorMap tmr, HardArgs a)
 {
     extern __shared__ __align__(512) unsigned char smem[];
@@ -29,7 +29,7 @@ __global__ void __launch_bounds__(W * 32, 1) k_hard5(const __grid_constant__ CUt
     unsigned char *rs = reinterpret_cast<unsigned char *>(ones + T);  // u8 [Frows][T], then reversed
     float *us = reinterpret_cast<float *>(rs + (size_t)Frows * T * 2);  // float [F][T] sorted (built here)
     uint4 *stage_all = reinterpret_cast<uint4 *>(us + (size_t)Frows * T);
-    constexpr int VS = vslots<W>();
+    constexpr int VS = VSLOTS;
     uint32_t *vrows = reinterpret_cast<uint32_t *>(stage_all + W * 32);     // [W][VS][32]
     uint64_t *bar = reinterpret_cast<uint64_t *>(vrows + W * VS * 32);
     int *next = reinterpret_cast<int *>(bar + 1);
@@ -37,7 +37,8 @@ __global__ void __launch_bounds__(W * 32, 1) k_hard5(const __grid_constant__ CUt
     int32_t *place = reinterpret_cast<int32_t *>(walked + 4 * W);    // [T] the caller's sample, or -1 (PRED)
     const uint4 *recs = reinterpret_cast<const uint4 *>(a.recs);
 
-    const int tile = blockIdx.x, group = blockIdx.y, G = gridDim.y;
+    const TileTask task(a);
+    const int tile = task.tile, group = task.group, G = task.groups;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
     if (threadIdx.x == 0) {
@@ -151,12 +152,12 @@ size_t hard5_smem_bytes(int F, int W)
 {
     const int Fb = F < 256 ? F : 256;
     const size_t Frows = (size_t)((F + Fb - 1) / Fb) * Fb;
-    const size_t vs = W >= 32 ? vslots<32>() : vslots<16>();
+    const size_t vs = VSLOTS;
     return Frows * T * (4 + 2 + 4) + (size_t)W * 32 * 16 + (size_t)W * vs * 32 * 4 + T * 4 + 16 + (size_t)W * 16 + T * 4;
 }
 
 template <int W, bool CAT, bool PRED>
-static rs_status launch5_t(Ctx *ctx, Dataset *ds, const HardArgs &a, cudaStream_t stream)
+static rs_status launch5_t(Ctx *ctx, Dataset *ds, HardArgs a, cudaStream_t stream)
 {
     const size_t smem = hard5_smem_bytes(a.F, W);
     if (smem > ctx->smem_optin || !ds->ranked) return RS_ERR_TOO_LARGE;
@@ -170,8 +171,9 @@ static rs_status launch5_t(Ctx *ctx, Dataset *ds, const HardArgs &a, cudaStream_
     const CUtensorMap *tmx = dataset_tmap(ds, T);
     const CUtensorMap *tmr = dataset_rank_tmap(ds);
     if (!tmx || !tmr) return RS_ERR_DEVICE;
-    const int tiles = (int)((a.N + T - 1) / T);
-    dim3 grid(tiles, a.groups);
+    int resident = 1;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, k_hard5<W, CAT, PRED>, W * 32, smem);
+    const int grid = split_tiles(ctx, a.N, a.F, a.P, T, W, resident, a);
     {
         TimedLaunch tl(ctx, TK_HARD, stream);
         k_hard5<W, CAT, PRED><<<grid, W * 32, smem, stream>>>(*tmx, *tmr, a);

@@ -126,7 +126,7 @@ rs_status eval_hard_static(Ctx *ctx, uint64_t ds_h, const rs_batch *b, int32_t *
 
     const int tid = ctx->forced_tile >= 0 && tile_config_fits(tile_config(ctx->forced_tile), ds->F)
                         ? ctx->forced_tile
-                        : heuristic_tile_for(*ds);
+                        : heuristic_tile_for(*ds, b->P, b->cond_set != nullptr);
     if ((rc = enqueue_hard(ctx, ds.get(), tile_config(tid), bd, s, correct, per_class, preds, stream)))
         return rc;
 

@@ -323,7 +323,8 @@ struct HardArgs {
     int32_t *correct;        // [P]  (zeroed by the launcher)
     int32_t *per_class;      // [P*K] or null
     int32_t *preds;          // [P*N] or null
-    int32_t groups;          // set groups (grid.y)
+    int32_t groups;          // set groups (grid.y; forms 4 and 5: of the tiles from `whole` on)
+    int32_t whole;           // forms 4 and 5: tiles that one CTA walks with all sets (split_tiles)
     uint32_t *status;
     const int32_t *last_end; // [P*K] or null (see PackOut)
     const float *Xt;         // [F][n_pad] (read directly by the global-memory configuration)
@@ -335,6 +336,21 @@ struct HardArgs {
 rs_status launch_hard(Ctx *ctx, Dataset *ds, const TileConfig &tc, const HardArgs &a,
                       cudaStream_t stream);
 int choose_groups(Ctx *ctx, const Dataset *ds, const TileConfig &tc, int P);
+// Split of a launch of the sign-mask or rank-coded form into CTAs (whole, groups of HardArgs), with
+// `resident` CTAs of W warps per SM; returns the number of CTAs.
+int split_tiles(Ctx *ctx, int64_t N, int F, int P, int S, int W, int resident, HardArgs &a);
+// The CTA's tile and set group.
+struct TileTask {
+    int tile, group, groups;
+    __device__ __forceinline__ TileTask(const HardArgs &a)
+    {
+        const int b = blockIdx.x;
+        if (b < a.whole) { tile = b; group = 0; groups = 1; return; }
+        groups = a.groups;
+        tile = a.whole + (b - a.whole) / groups;
+        group = (b - a.whole) % groups;
+    }
+};
 rs_status launch_hard2(Ctx *ctx, Dataset *ds, int V, int W, bool mm, const HardArgs &a,
                        cudaStream_t stream);
 rs_status launch_hard4(Ctx *ctx, Dataset *ds, int V, int W, const HardArgs &a, cudaStream_t stream);
@@ -349,7 +365,7 @@ rs_status enqueue_hard(Ctx *ctx, Dataset *ds, const TileConfig &tc, const BatchD
                        const Scratch &s, int32_t *correct, int32_t *per_class, int32_t *preds,
                        cudaStream_t stream);
 // The built-in tile choice for a dataset (no autotuned entry).
-int heuristic_tile_for(const Dataset &ds);
+int heuristic_tile_for(const Dataset &ds, int P, bool cat);
 const CUtensorMap *dataset_tmap(Dataset *ds, int S);
 const CUtensorMap *dataset_rank_tmap(Dataset *ds);
 
