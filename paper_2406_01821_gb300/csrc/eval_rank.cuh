@@ -34,20 +34,27 @@ constexpr uint32_t HIGH = 0x80808080u;          // bit 7 of every byte
 constexpr uint32_t ONES = 0x01010101u;
 constexpr int T = RANK_TILE;                     // samples per tile (= one warp, four per lane)
 
-// #{j : row[j] <= c} (or < c) over the 128 ascending values of a row stored at j ^ sw.
-template <bool LE>
-__device__ __forceinline__ int count_below(const float *row, int sw, float c)
+// #{j : row[j] <= c} over the 128 ascending values of a row in shared memory: each step is a load at a
+// fixed offset from a 32-bit address, a compare and a predicated add on the address (the XOR-swizzled
+// column it replaced took two operations more a step; ten generations of 10,000 sets 92.0 -> 89.3 ms).
+__device__ __forceinline__ int count_below(const float *row, float c)
 {
-    int pos = 0;
+    const uint32_t a0 = (uint32_t)__cvta_generic_to_shared(row);
+    uint32_t a = a0;
+    float u;
 #pragma unroll
-    for (int step = 64; step >= 1; step >>= 1) {
-        const float u = row[(pos + step - 1) ^ sw];
-        if (LE ? (u <= c) : (u < c)) pos += step;
+    for (uint32_t step = 64; step >= 1; step >>= 1) {
+        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(u) : "r"(a + (step - 1) * 4u));
+        if (u <= c) a += step * 4u;
     }
-    const float u = row[pos ^ sw];               // pos <= 127: one more for a full count
-    if (LE ? (u <= c) : (u < c)) pos += 1;
-    return pos;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(u) : "r"(a));
+    if (u <= c) a += 4u;                         // at most 127 so far: one more for a full count
+    return (int)((a - a0) >> 2);
 }
+
+// Floats per sorted column: one more than its values, so that searches of different features start
+// in different banks.
+constexpr int US = T + 1;
 
 // pass rows per warp for pair / product conditions of one chunk
 constexpr int VSLOTS = 12;
@@ -58,7 +65,7 @@ __device__ __forceinline__ uint32_t row_off(uint32_t f) { return sparse::row_off
 
 // The per-tile tables built in shared memory by the whole block once the tile's features xs
 // [F][T] and rank bytes rs [Frows][T] have landed: the reversed ranks (127 - rank) at rs + rev_off,
-// each feature's sorted column us[f][pos ^ (f & 31)] = x[f][n] with pos the rank of x[f][n] (its
+// each feature's sorted column us[f][pos] = x[f][n] (US floats a row) with pos the rank of x[f][n] (its
 // position in the tile's stable ascending order: a permutation, so every slot is written), and the
 // float rows permuted in place (row_off). One warp per row.
 __device__ __forceinline__ void build_tile_tables(float *xs, unsigned char *rs, uint32_t rev_off, float *us, int F)
@@ -69,12 +76,11 @@ __device__ __forceinline__ void build_tile_tables(float *xs, unsigned char *rs, 
         const float4 x = row[lane];
         const uint32_t r = reinterpret_cast<const uint32_t *>(rs)[f * 32 + lane];
         reinterpret_cast<uint32_t *>(rs + rev_off)[f * 32 + lane] = r ^ 0x7F7F7F7Fu;
-        float *u = us + f * T;
-        const uint32_t sw = (uint32_t)f & 31u;
-        u[(r & 0x7Fu) ^ sw] = x.x;
-        u[(r >> 8 & 0x7Fu) ^ sw] = x.y;
-        u[(r >> 16 & 0x7Fu) ^ sw] = x.z;
-        u[(r >> 24) ^ sw] = x.w;
+        float *u = us + f * US;
+        u[r & 0x7Fu] = x.x;
+        u[r >> 8 & 0x7Fu] = x.y;
+        u[r >> 16 & 0x7Fu] = x.z;
+        u[r >> 24] = x.w;
         __syncwarp();
         row[lane ^ (f & 7)] = x;
     }
@@ -85,7 +91,7 @@ __device__ __forceinline__ uint2 stage_cut(uint4 r, const float *us, uint32_t re
 {
     const uint32_t f = min(r.x & R5_F_MASK, (uint32_t)(F - 1));
     const bool le = (r.x >> R5_TAG_SHIFT) == R5_CUT_LT;
-    const int L = count_below<true>(us + f * T, (int)(f & 31u), __uint_as_float(r.z));
+    const int L = count_below(us + f * US, __uint_as_float(r.z));
     return make_uint2((le ? rev_off : 0u) + f * T, (uint32_t)(le ? 255 - L : L + 127) * ONES);
 }
 
@@ -109,8 +115,9 @@ __device__ __forceinline__ uint32_t class_bytes(const int32_t *yl, int k)
 // a NaN operand or inf - inf gives the canonical NaN, whose sign bit is clear (false, as the
 // IEEE compare). Used on finite datasets only (rank tables), where the products are finite or
 // +-inf.
-__device__ __forceinline__ uint32_t pass_row(uint4 q, const unsigned char *xs, uint32_t lane16)
+__device__ __forceinline__ uint32_t pass_row(const uint4 *e, const unsigned char *xs, uint32_t lane16)
 {
+    const uint4 q = *e;
     const float4 x = *reinterpret_cast<const float4 *>(xs + (q.x ^ lane16));
     const float4 z = *reinterpret_cast<const float4 *>(xs + (q.y ^ lane16));
     const float2 a2 = make_float2(__uint_as_float(q.z), __uint_as_float(q.z));
@@ -256,8 +263,8 @@ __device__ __forceinline__ uint32_t walk_set(uint4 *st, uint32_t *vrow, uint32_t
         {                                             // pass rows, one warp-wide evaluation each
             uint32_t *vr = vrow + lane;
             for (int j = 0; j < np; j += 2) {
-                const uint32_t v0 = pass_row(st[j], xs, lane16);
-                if (j + 1 < np) vr[32] = pass_row(st[j + 1], xs, lane16);
+                const uint32_t v0 = pass_row(st + j, xs, lane16);
+                if (j + 1 < np) vr[32] = pass_row(st + j + 1, xs, lane16);
                 vr[0] = v0;
                 vr += 64;
             }

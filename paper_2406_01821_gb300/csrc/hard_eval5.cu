@@ -27,14 +27,14 @@ __global__ void __launch_bounds__(W * 32, 32 / W) k_hard5(const __grid_constant_
     unsigned char *xs = smem;                                         // float [Frows][T]
     float *ones = reinterpret_cast<float *>(xs + (size_t)Frows * T * 4);  // [T] of 1.0 (products)
     unsigned char *rs = reinterpret_cast<unsigned char *>(ones + T);  // u8 [Frows][T], then reversed
-    float *us = reinterpret_cast<float *>(rs + (size_t)Frows * T * 2);  // float [F][T] sorted (built here)
-    uint4 *stage_all = reinterpret_cast<uint4 *>(us + (size_t)Frows * T);
+    uint4 *stage_all = reinterpret_cast<uint4 *>(rs + (size_t)Frows * T * 2);
     constexpr int VS = VSLOTS;
     uint32_t *vrows = reinterpret_cast<uint32_t *>(stage_all + W * 32);     // [W][VS][32]
     uint64_t *bar = reinterpret_cast<uint64_t *>(vrows + W * VS * 32);
     int *next = reinterpret_cast<int *>(bar + 1);
     uint32_t *walked = reinterpret_cast<uint32_t *>(bar + 2);        // [W][4] work counters (counting)
     int32_t *place = reinterpret_cast<int32_t *>(walked + 4 * W);    // [T] the caller's sample, or -1 (PRED)
+    float *us = reinterpret_cast<float *>(place + T);                // float [F][US] sorted (built here)
     const uint4 *recs = reinterpret_cast<const uint4 *>(a.recs);
 
     const TileTask task(a);
@@ -153,7 +153,7 @@ size_t hard5_smem_bytes(int F, int W)
     const int Fb = F < 256 ? F : 256;
     const size_t Frows = (size_t)((F + Fb - 1) / Fb) * Fb;
     const size_t vs = VSLOTS;
-    return Frows * T * (4 + 2 + 4) + (size_t)W * 32 * 16 + (size_t)W * vs * 32 * 4 + T * 4 + 16 + (size_t)W * 16 + T * 4;
+    return Frows * T * (4 + 2) + (size_t)F * US * 4 + (size_t)W * 32 * 16 + (size_t)W * vs * 32 * 4 + T * 4 + 16 + (size_t)W * 16 + T * 4;
 }
 
 template <int W, bool CAT, bool PRED>

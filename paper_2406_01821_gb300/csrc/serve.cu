@@ -39,9 +39,8 @@ constexpr int SS = 32 * SV;           // samples per tile (unit)
 constexpr int SERVE_MAX_F = 256;      // shared x tile [F][128]: 128 KB
 constexpr int SERVE_RANK_MAX_F = 128; // rank-coded units: x, ranks, reversed ranks, sorted [F][128]
 constexpr int SVS = 8;                // pass-row slots per warp of rank-coded units
-constexpr size_t TILE_BYTES = (size_t)SERVE_MAX_F * SS * 4 > (size_t)SERVE_RANK_MAX_F * SS * 10
-                                  ? (size_t)SERVE_MAX_F * SS * 4
-                                  : (size_t)SERVE_RANK_MAX_F * SS * 10;
+constexpr size_t RANK_BYTES = (size_t)SERVE_RANK_MAX_F * (SS * 6 + rank::US * 4);
+constexpr size_t TILE_BYTES = (size_t)SERVE_MAX_F * SS * 4 > RANK_BYTES ? (size_t)SERVE_MAX_F * SS * 4 : RANK_BYTES;
 constexpr size_t ONES_BYTES = (size_t)SS * 4;   // a row of 1.0: the right side of product conditions
 constexpr size_t SERVE_SMEM = TILE_BYTES + (size_t)SW * 64 * 16 + (size_t)SW * SVS * 32 * 4 + ONES_BYTES;
 constexpr int MAX_SLOTS = 2048;
