@@ -148,10 +148,13 @@ struct Dataset {
     int64_t N = 0, n_pad = 0;
     int32_t F = 0, K = 0;
     bool finite = false;          // no NaN or infinity in X
+    // one allocation that starts at Xt:
     float *Xt = nullptr;          // [F][n_pad], samples grouped by label (stable), zero padded
     int32_t *y = nullptr;         // [n_pad] labels in that order, -1 for padding
     int32_t *perm = nullptr;      // [N] caller index of sorted position
     int32_t *inv = nullptr;       // [N] sorted position of caller index
+    uint32_t *flags = nullptr;    // [F] 0: the feature holds category codes 0..63 only
+    int32_t ncode = 0;            // features with flag 0
     std::vector<int64_t> class_count;
     std::map<int, CUtensorMap> tmaps;   // keyed by samples per tile
     // Rank table (finite datasets with F <= RANK_MAX_F), per 128-sample tile and feature f:

@@ -4,6 +4,7 @@
 #include <cudaTypedefs.h>
 
 #include "rs_internal.cuh"
+#include "block_scan.cuh"
 #include "dataset_lru.h"
 #include "tma.cuh"
 
@@ -216,61 +217,73 @@ namespace {
 constexpr int REG_BLOCK = 1024;
 
 // Per block of REG_BLOCK samples: label histogram and each sample's rank among earlier samples
-// of the same label in the block (a stable order within the block).
+// of the same label in the block (a stable order within the block). The lanes of a warp that share a
+// label find each other with one match; the warps add to the block's counts in turn. (A loop over
+// the earlier samples of the block, as before, took 25 us on 300,000 samples; this takes 5.)
 __global__ void k_label_rank(const int32_t *y, int64_t N, int K, int32_t *blk_count,
                              int32_t *rank, uint32_t *status)
 {
-    extern __shared__ int32_t sh[];
-    int32_t *ys = sh;                 // [REG_BLOCK]
-    int32_t *hist = sh + REG_BLOCK;   // [K]
+    extern __shared__ int32_t hist[];  // [K]
     const int64_t n = (int64_t)blockIdx.x * REG_BLOCK + threadIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int k = threadIdx.x; k < K; k += blockDim.x) hist[k] = 0;
     int lab = -1;
     if (n < N) {
         lab = y[n];
         if (lab < 0 || lab >= K) { atomicOr(status, ST_BAD_LABEL); lab = -1; }
     }
-    ys[threadIdx.x] = lab;
+    const uint32_t same = __match_any_sync(0xFFFFFFFFu, lab);
+    const int within = __popc(same & ((1u << lane) - 1u));
+    int base = 0;
+    for (int w = 0; w < REG_BLOCK / 32; ++w) {
+        __syncthreads();
+        if (w != warp) continue;
+        if (lab >= 0) base = hist[lab];
+        __syncwarp();
+        if (lab >= 0 && within == 0) hist[lab] = base + __popc(same);
+    }
     __syncthreads();
-    if (lab >= 0) atomicAdd(&hist[lab], 1);
-    int r = 0;
-    for (int i = 0; i < (int)threadIdx.x; ++i) r += (ys[i] == lab);
-    if (n < N) rank[n] = r;
-    __syncthreads();
+    if (n < N) rank[n] = base + within;
     for (int k = threadIdx.x; k < K; k += blockDim.x)
         blk_count[(int64_t)blockIdx.x * K + k] = hist[k];
 }
 
-// One thread per label: exclusive offsets of every block within the label-grouped order.
+// One CTA per label: exclusive offsets of every block within the label-grouped order.
 __global__ void k_label_offsets(int32_t *blk_count, int64_t nblk, int K, int64_t *class_total)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= K) return;
-    int64_t run = 0;
-    for (int64_t b = 0; b < nblk; ++b) {
-        int32_t c = blk_count[b * K + k];
-        blk_count[b * K + k] = (int32_t)run;
-        run += c;
+    const int k = blockIdx.x;
+    int run = 0;
+    for (int64_t b0 = 0; b0 < nblk; b0 += blockDim.x) {
+        const int64_t b = b0 + threadIdx.x;
+        const int c = b < nblk ? blk_count[b * K + k] : 0;
+        int total;
+        const int before = block_exclusive_scan(c, &total);
+        if (b < nblk) blk_count[b * K + k] = run + before;
+        run += total;
     }
-    class_total[k] = run;
+    if (threadIdx.x == 0) class_total[k] = run;
 }
 
 __global__ void k_class_start(const int64_t *class_total, int K, int64_t *class_start)
 {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        int64_t run = 0;
-        for (int k = 0; k < K; ++k) { class_start[k] = run; run += class_total[k]; }
+    int run = 0;
+    for (int k0 = 0; k0 < K; k0 += blockDim.x) {
+        const int k = k0 + threadIdx.x;
+        int total;
+        const int before = block_exclusive_scan(k < K ? (int)class_total[k] : 0, &total);
+        if (k < K) class_start[k] = run + before;
+        run += total;
     }
 }
 
-__global__ void k_label_scatter(const int32_t *y, int64_t N, int K, const int32_t *blk_off,
+__global__ void k_label_scatter(const int32_t *y, int64_t N, int64_t n_pad, int K, const int32_t *blk_off,
                                 const int64_t *class_start, const int32_t *rank, int32_t *perm,
-                                int32_t *inv, int32_t *y_sorted)
+                                int32_t *inv, int32_t *y_sorted, const uint32_t *status)
 {
     const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
+    if (n >= n_pad || *status) return;
+    if (n >= N) { y_sorted[n] = -1; return; }
     const int lab = y[n];
-    if (lab < 0 || lab >= K) return;
     const int64_t blk = n / REG_BLOCK;
     const int64_t pos = class_start[lab] + blk_off[blk * K + lab] + rank[n];
     perm[pos] = (int32_t)n;
@@ -278,95 +291,135 @@ __global__ void k_label_scatter(const int32_t *y, int64_t N, int K, const int32_
     y_sorted[pos] = lab;
 }
 
-// Xt[f][m] = X[perm[m]][f] for m < N, 0 for the padding; 32x32 tiles through shared memory.
-__global__ void k_transpose_gather(const float *X, int64_t N, int F, int64_t n_pad,
-                                   const int32_t *perm, float *Xt)
+// Positions of a warp's 128 keys (lane l: the keys of samples l + 32 v) in ascending order, equal keys
+// in sample order. The keys alone are sorted, by a bitonic network with lane l holding places 4 l ..
+// 4 l + 3, and each key is then looked up in the sorted column: seven search steps cost less than
+// carrying the sample number through the network as 64-bit keys (28 stages of two shuffles and a
+// 64-bit compare-exchange). Equal keys find the same place and are told apart by a match.
+// sorted: the warp's 128 words.
+__device__ __forceinline__ void rank_column(const uint32_t (&key)[4], uint32_t *sorted, int lane, uint32_t (&pos)[4])
 {
-    __shared__ float tile[32][33];
-    const int64_t m0 = (int64_t)blockIdx.x * 32;
-    const int f0 = blockIdx.y * 32;
-    const int tx = threadIdx.x, ty = threadIdx.y;   // 32 x 8
-    for (int j = ty; j < 32; j += 8) {
-        const int64_t m = m0 + j;
-        const int f = f0 + tx;
-        float v = 0.f;
-        if (m < N && f < F) v = X[(int64_t)perm[m] * F + f];
-        tile[j][tx] = v;
-    }
-    __syncthreads();
-    for (int j = ty; j < 32; j += 8) {
-        const int f = f0 + j;
-        const int64_t m = m0 + tx;
-        if (f < F && m < n_pad) Xt[(int64_t)f * n_pad + m] = tile[tx][j];
-    }
-}
-
-__global__ void k_nonfinite(const float *x, int64_t n, uint32_t *flag)
-{
-    bool bad = false;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        bad |= !isfinite(x[i]);
-    if (__any_sync(0xFFFFFFFFu, bad) && (threadIdx.x & 31) == 0) atomicOr(flag, 1u);
-}
-
-// Rank table of one 128-sample tile and feature per warp: the position of each value in the
-// tile's ascending order, equal values in sample order (-0 before +0: any order within a group of
-// equal values keeps the group contiguous, which is all the cut tests need). The evaluators
-// rebuild the sorted column from it in shared memory (one scatter), so it is the only table kept
-// beside the features. The warp sorts the keys (value order, then sample) with a bitonic network,
-// lane l holding elements 4l .. 4l+3, and scatters each element's final place back to its sample.
-__global__ void k_rank_tiles(const float *Xt, int64_t n_pad, int F, uint8_t *Rk)
-{
-    __shared__ uint8_t pos_of[8][RANK_TILE];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int f = blockIdx.y * (blockDim.x >> 5) + wib;
-    if (f >= F) return;
-    const int64_t t = blockIdx.x;
-    const float4 x4 = *reinterpret_cast<const float4 *>(Xt + (int64_t)f * n_pad + t * RANK_TILE + 4 * lane);
-    const float xv[4] = {x4.x, x4.y, x4.z, x4.w};
-    unsigned long long a[4];
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-        const uint32_t u = __float_as_uint(xv[v]);
-        const uint32_t key = (u & 0x80000000u) ? ~u : (u | 0x80000000u);   // float order (finite data)
-        a[v] = ((unsigned long long)key << 32) | (uint32_t)(4 * lane + v);
-    }
+    uint32_t a[4] = {key[0], key[1], key[2], key[3]};
 #pragma unroll
     for (int k = 2; k <= RANK_TILE; k <<= 1) {
 #pragma unroll
         for (int j = k >> 1; j > 0; j >>= 1) {
             if (j >= 4) {                            // partners in lane ^ (j / 4), same slot
+                const bool low = ((4 * lane & j) == 0) == ((4 * lane & k) == 0);
 #pragma unroll
                 for (int v = 0; v < 4; ++v) {
-                    const int e = 4 * lane + v;
-                    const unsigned long long o = __shfl_xor_sync(0xFFFFFFFFu, a[v], j >> 2);
-                    const bool take_min = ((e & j) == 0) == ((e & k) == 0);
-                    a[v] = take_min ? (o < a[v] ? o : a[v]) : (o > a[v] ? o : a[v]);
+                    const uint32_t o = __shfl_xor_sync(0xFFFFFFFFu, a[v], j >> 2);
+                    a[v] = low ? min(a[v], o) : max(a[v], o);
                 }
             } else {                                 // partners within the lane
 #pragma unroll
                 for (int v = 0; v < 4; ++v) {
                     if (v & j) continue;
-                    const int w = v | j;
                     const bool asc = ((4 * lane + v) & k) == 0;
-                    const unsigned long long lo = a[v] < a[w] ? a[v] : a[w], hi = a[v] < a[w] ? a[w] : a[v];
+                    const uint32_t lo = min(a[v], a[v | j]), hi = max(a[v], a[v | j]);
                     a[v] = asc ? lo : hi;
-                    a[w] = asc ? hi : lo;
+                    a[v | j] = asc ? hi : lo;
                 }
             }
         }
     }
-#pragma unroll
-    for (int v = 0; v < 4; ++v) pos_of[wib][(uint32_t)a[v]] = (uint8_t)(4 * lane + v);
+    reinterpret_cast<uint4 *>(sorted)[lane] = make_uint4(a[0], a[1], a[2], a[3]);
+    const uint32_t next = __shfl_down_sync(0xFFFFFFFFu, a[0], 1);
+    const bool ties = __any_sync(0xFFFFFFFFu, a[0] == a[1] || a[1] == a[2] || a[2] == a[3] || (lane < 31 && a[3] == next));
     __syncwarp();
-    const uint32_t w = *reinterpret_cast<const uint32_t *>(&pos_of[wib][4 * lane]);
-    reinterpret_cast<uint32_t *>(Rk + (int64_t)f * n_pad + t * RANK_TILE)[lane] = w;
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+        uint32_t p = 0;
+#pragma unroll
+        for (uint32_t step = RANK_TILE / 2; step >= 1; step >>= 1)
+            if (sorted[p + step - 1] < key[v]) p += step;
+        pos[v] = p;
+    }
+    if (!ties) return;
+    __syncwarp();
+    reinterpret_cast<uint4 *>(sorted)[lane] = make_uint4(0u, 0u, 0u, 0u);      // now: keys seen per place
+    __syncwarp();
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+        const uint32_t same = __match_any_sync(0xFFFFFFFFu, pos[v]);
+        const uint32_t seen = sorted[pos[v]], within = __popc(same & ((1u << lane) - 1u));
+        __syncwarp();
+        if (within == 0) sorted[pos[v]] = seen + __popc(same);
+        __syncwarp();
+        pos[v] += seen + within;
+    }
 }
 
-__global__ void k_fill_i32(int32_t *p, int64_t n, int32_t v)
+// One 128-sample tile of 32 features: Xt[f][m] = X[perm[m]][f] (0 for the padding), the tile's rank
+// table (with Rk; finite data), and per feature whether it holds a non-finite value (bit 0) or one
+// that is no category code 0..63 (bit 1). The rows are gathered into shared memory, so that the
+// transpose, the rank sort and the tests read X once and Xt not at all: 300,007 x 96 in one pass where
+// a transpose (83 us), a test (21 us) and a sort (338 us) took three: 173 us. Bound by instruction
+// issue and shared-memory latency in the sort (260 MB of traffic are 38 us).
+constexpr int REG_WARPS = 8;
+__global__ void __launch_bounds__(REG_WARPS * 32) k_register_tile(const float *X, int64_t N, int F, int64_t n_pad,
+                                                                  const int32_t *perm, float *Xt, uint8_t *Rk,
+                                                                  uint32_t *flags, const uint32_t *status)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) p[i] = v;
+    __shared__ float tile[RANK_TILE][33];
+    __shared__ __align__(16) uint32_t sorted[REG_WARPS][RANK_TILE];
+    __shared__ __align__(4) uint8_t place[REG_WARPS][RANK_TILE];
+    if (*status) return;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t m0 = (int64_t)blockIdx.x * RANK_TILE;
+    const int f0 = blockIdx.y * 32;
+    constexpr int ROWS = RANK_TILE / REG_WARPS;
+    {
+        const int64_t m = m0 + w * ROWS + (lane % ROWS);
+        const int src = m < N ? perm[m] : -1;
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) {
+            const int s = __shfl_sync(0xFFFFFFFFu, src, r);
+            tile[w * ROWS + r][lane] = (s >= 0 && f0 + lane < F) ? X[(int64_t)s * F + f0 + lane] : 0.f;
+        }
+    }
+    __syncthreads();
+    for (int c = w; c < 32 && f0 + c < F; c += REG_WARPS) {
+        const int f = f0 + c;
+        float *out = Xt + (int64_t)f * n_pad + m0 + lane;
+        uint32_t key[4], pos[4];
+        bool odd = false, plain = false;
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const float x = tile[lane + 32 * v][c];
+            out[32 * v] = x;
+            odd |= !isfinite(x);
+            plain |= !(x >= 0.f && x <= 63.f && x == truncf(x));
+            const uint32_t u = __float_as_uint(x);
+            key[v] = (u & 0x80000000u) ? ~u : (u | 0x80000000u);               // float order
+        }
+        const uint32_t fl = (__any_sync(0xFFFFFFFFu, odd) ? 1u : 0u) | (__any_sync(0xFFFFFFFFu, plain) ? 2u : 0u);
+        if (lane == 0 && (fl & ~__ldcg(flags + f))) atomicOr(flags + f, fl);
+        if (!Rk) continue;
+        rank_column(key, sorted[w], lane, pos);
+        __syncwarp();
+#pragma unroll
+        for (int v = 0; v < 4; ++v) place[w][lane + 32 * v] = (uint8_t)pos[v];
+        __syncwarp();
+        reinterpret_cast<uint32_t *>(Rk + (int64_t)f * n_pad + m0)[lane] = reinterpret_cast<const uint32_t *>(place[w])[lane];
+    }
+}
+
+// status[1]: some value is not finite; status[2]: features that hold category codes only.
+__global__ void k_register_summary(const uint32_t *flags, int F, uint32_t *status)
+{
+    int odd = 0, codes = 0;
+    for (int f = threadIdx.x; f < F; f += blockDim.x) {
+        odd |= flags[f] & 1u;
+        codes += flags[f] == 0u;
+    }
+    odd = __syncthreads_or(odd);
+    int total;
+    block_exclusive_scan(codes, &total);
+    if (threadIdx.x == 0) {
+        status[1] = odd;
+        status[2] = total;
+    }
 }
 
 }  // namespace
@@ -434,97 +487,91 @@ const CUtensorMap *dataset_tmap(Dataset *ds, int S)
 
 // Build the device copy of dataset d (N, F, K and n_pad set) from X and y (host or device per
 // `mem`): feature-major Xt grouped by label, labels, permutation and inverse, class counts, the
-// finite flag and, for finite data of at most RANK_MAX_F features, the rank table.
+// finite flag and, for finite data of at most RANK_MAX_F features, the rank table. The dataset is one
+// allocation (and one for the rank table), the temporary arrays another; the host waits once, at the
+// end: every kernel after the label check does nothing when a label was out of range.
 static rs_status build_device(Dataset &d, const float *X, const int32_t *y, int32_t mem, cudaStream_t stream)
 {
     const int64_t N = d.N;
     const int32_t F = d.F, K = d.K;
     const int64_t nblk = (N + REG_BLOCK - 1) / REG_BLOCK;
+    const bool rank_tables = F <= RANK_MAX_F;
 
-    float *Xd = nullptr;
-    int32_t *yd = nullptr, *blk = nullptr, *rank = nullptr;
-    int64_t *ctot = nullptr, *cstart = nullptr;
-    uint32_t *st = nullptr;
+    char *own = nullptr, *tmp = nullptr;
     rs_status rc = RS_OK;
-    auto cleanup = [&] {
-        if (mem == RS_MEM_HOST) { cudaFree(Xd); cudaFree(yd); }
-        cudaFree(blk); cudaFree(rank); cudaFree(ctot); cudaFree(cstart); cudaFree(st);
-    };
-    auto release = [&] {              // the dataset's own arrays, after a failure
-        cudaFree(d.Xt); cudaFree(d.y); cudaFree(d.perm); cudaFree(d.inv); cudaFree(d.Rk);
-        d.Xt = nullptr; d.y = nullptr; d.perm = nullptr; d.inv = nullptr; d.Rk = nullptr;
+    auto fail = [&] {                 // everything taken so far
+        cudaFree(own); cudaFree(tmp); cudaFree(d.Rk);
+        d.Xt = nullptr; d.y = nullptr; d.perm = nullptr; d.inv = nullptr; d.flags = nullptr; d.Rk = nullptr;
     };
 #define REG_CUDA(call)                                      \
     do {                                                    \
         cudaError_t e_ = (call);                            \
         if (e_ != cudaSuccess) {                            \
             rc = cuda_fail(e_, #call);                      \
-            cleanup();                                      \
-            release();                                      \
+            fail();                                         \
             return rc;                                      \
         }                                                   \
     } while (0)
 
+    const auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+    size_t at = 0;
+    const auto take = [&](size_t bytes) { const size_t o = at; at += up(bytes); return o; };
+    const size_t o_x = take(sizeof(float) * (size_t)d.n_pad * F), o_y = take(sizeof(int32_t) * (size_t)d.n_pad),
+                 o_perm = take(sizeof(int32_t) * (size_t)N), o_inv = take(sizeof(int32_t) * (size_t)N),
+                 o_flags = take(sizeof(uint32_t) * (size_t)F);
+    REG_CUDA(cudaMalloc(&own, at));
+    d.Xt = reinterpret_cast<float *>(own + o_x);
+    d.y = reinterpret_cast<int32_t *>(own + o_y);
+    d.perm = reinterpret_cast<int32_t *>(own + o_perm);
+    d.inv = reinterpret_cast<int32_t *>(own + o_inv);
+    d.flags = reinterpret_cast<uint32_t *>(own + o_flags);
+    if (rank_tables) REG_CUDA(cudaMalloc(&d.Rk, (size_t)d.n_pad * F));
+    at = 0;
+    // the status words and the class counts, read back together
+    const size_t o_st = take(16 + sizeof(int64_t) * (size_t)K), o_start = take(sizeof(int64_t) * (size_t)K),
+                 o_blk = take(sizeof(int32_t) * (size_t)nblk * K), o_rank = take(sizeof(int32_t) * (size_t)N);
+    const size_t o_xd = mem == RS_MEM_HOST ? take(sizeof(float) * (size_t)N * F) : 0,
+                 o_yd = mem == RS_MEM_HOST ? take(sizeof(int32_t) * (size_t)N) : 0;
+    REG_CUDA(cudaMalloc(&tmp, at));
+    uint32_t *st = reinterpret_cast<uint32_t *>(tmp + o_st);
+    int64_t *ctot = reinterpret_cast<int64_t *>(tmp + o_st + 16), *cstart = reinterpret_cast<int64_t *>(tmp + o_start);
+    int32_t *blk = reinterpret_cast<int32_t *>(tmp + o_blk), *rank = reinterpret_cast<int32_t *>(tmp + o_rank);
+    const float *Xd = X;
+    const int32_t *yd = y;
     if (mem == RS_MEM_HOST) {
-        REG_CUDA(cudaMalloc(&Xd, sizeof(float) * N * F));
-        REG_CUDA(cudaMalloc(&yd, sizeof(int32_t) * N));
-        REG_CUDA(cudaMemcpyAsync(Xd, X, sizeof(float) * N * F, cudaMemcpyHostToDevice, stream));
-        REG_CUDA(cudaMemcpyAsync(yd, y, sizeof(int32_t) * N, cudaMemcpyHostToDevice, stream));
-    } else {
-        Xd = const_cast<float *>(X);
-        yd = const_cast<int32_t *>(y);
+        REG_CUDA(cudaMemcpyAsync(tmp + o_xd, X, sizeof(float) * (size_t)N * F, cudaMemcpyHostToDevice, stream));
+        REG_CUDA(cudaMemcpyAsync(tmp + o_yd, y, sizeof(int32_t) * (size_t)N, cudaMemcpyHostToDevice, stream));
+        Xd = reinterpret_cast<const float *>(tmp + o_xd);
+        yd = reinterpret_cast<const int32_t *>(tmp + o_yd);
     }
-    REG_CUDA(cudaMalloc(&d.Xt, sizeof(float) * d.n_pad * F));
-    REG_CUDA(cudaMalloc(&d.y, sizeof(int32_t) * d.n_pad));
-    REG_CUDA(cudaMalloc(&d.perm, sizeof(int32_t) * N));
-    REG_CUDA(cudaMalloc(&d.inv, sizeof(int32_t) * N));
-    REG_CUDA(cudaMalloc(&blk, sizeof(int32_t) * nblk * K));
-    REG_CUDA(cudaMalloc(&rank, sizeof(int32_t) * N));
-    REG_CUDA(cudaMalloc(&ctot, sizeof(int64_t) * K));
-    REG_CUDA(cudaMalloc(&cstart, sizeof(int64_t) * K));
-    REG_CUDA(cudaMalloc(&st, sizeof(uint32_t)));
-    REG_CUDA(cudaMemsetAsync(st, 0, sizeof(uint32_t), stream));
-    k_fill_i32<<<(unsigned)((d.n_pad + 255) / 256), 256, 0, stream>>>(d.y, d.n_pad, -1);
-    k_label_rank<<<(unsigned)nblk, REG_BLOCK, sizeof(int32_t) * (REG_BLOCK + K), stream>>>(
-        yd, N, K, blk, rank, st);
+    REG_CUDA(cudaMemsetAsync(st, 0, 16, stream));
+    REG_CUDA(cudaMemsetAsync(d.flags, 0, sizeof(uint32_t) * (size_t)F, stream));
+    k_label_rank<<<(unsigned)nblk, REG_BLOCK, sizeof(int32_t) * K, stream>>>(yd, N, K, blk, rank, st);
+    k_label_offsets<<<K, 1024, 0, stream>>>(blk, nblk, K, ctot);
+    k_class_start<<<1, 1024, 0, stream>>>(ctot, K, cstart);
+    k_label_scatter<<<(unsigned)((d.n_pad + 255) / 256), 256, 0, stream>>>(yd, N, d.n_pad, K, blk, cstart, rank, d.perm,
+                                                                           d.inv, d.y, st);
+    const dim3 tg((unsigned)(d.n_pad / RANK_TILE), (unsigned)((F + 31) / 32));
+    k_register_tile<<<tg, REG_WARPS * 32, 0, stream>>>(Xd, N, F, d.n_pad, d.perm, d.Xt, d.Rk, d.flags, st);
+    k_register_summary<<<1, 1024, 0, stream>>>(d.flags, F, st);
     REG_CUDA(cudaGetLastError());
-    uint32_t hst = 0;
-    // labels must be valid before they are used as scatter positions
-    REG_CUDA(cudaMemcpyAsync(&hst, st, sizeof(uint32_t), cudaMemcpyDeviceToHost, stream));
+    std::vector<char> back(16 + sizeof(int64_t) * (size_t)K);
+    REG_CUDA(cudaMemcpyAsync(back.data(), st, back.size(), cudaMemcpyDeviceToHost, stream));
     REG_CUDA(cudaStreamSynchronize(stream));
-    if (hst) {
-        cleanup();
-        set_error("dataset rejected: %s", status_text(hst).c_str());
-        release();
+    uint32_t hst[4];
+    std::memcpy(hst, back.data(), sizeof(hst));
+    if (hst[0]) {
+        set_error("dataset rejected: %s", status_text(hst[0]).c_str());
+        fail();
         return RS_ERR_INVALID;
     }
-    k_label_offsets<<<(K + 127) / 128, 128, 0, stream>>>(blk, nblk, K, ctot);
-    k_class_start<<<1, 32, 0, stream>>>(ctot, K, cstart);
-    k_label_scatter<<<(unsigned)((N + 255) / 256), 256, 0, stream>>>(yd, N, K, blk, cstart, rank,
-                                                                      d.perm, d.inv, d.y);
-    dim3 tg((unsigned)(d.n_pad / 32), (unsigned)((F + 31) / 32));
-    k_transpose_gather<<<tg, dim3(32, 8), 0, stream>>>(Xd, N, F, d.n_pad, d.perm, d.Xt);
-    REG_CUDA(cudaGetLastError());
-    REG_CUDA(cudaMemsetAsync(st, 0, sizeof(uint32_t), stream));
-    k_nonfinite<<<1024, 256, 0, stream>>>(d.Xt, d.n_pad * F, st);
-    REG_CUDA(cudaGetLastError());
-    uint32_t nonfinite = 0;
-    REG_CUDA(cudaMemcpyAsync(&nonfinite, st, sizeof(uint32_t), cudaMemcpyDeviceToHost, stream));
     d.class_count.resize(K);
-    REG_CUDA(cudaMemcpyAsync(d.class_count.data(), ctot, sizeof(int64_t) * K,
-                             cudaMemcpyDeviceToHost, stream));
-    REG_CUDA(cudaStreamSynchronize(stream));
-    d.finite = nonfinite == 0;
-    if (d.finite && F <= RANK_MAX_F) {
-        // rank table for the rank-coded evaluator (1 byte per value)
-        REG_CUDA(cudaMalloc(&d.Rk, (size_t)d.n_pad * F));
-        dim3 rg((unsigned)(d.n_pad / RANK_TILE), (unsigned)((F + 7) / 8));
-        k_rank_tiles<<<rg, 256, 0, stream>>>(d.Xt, d.n_pad, F, d.Rk);
-        REG_CUDA(cudaGetLastError());
-        REG_CUDA(cudaStreamSynchronize(stream));
-        d.ranked = true;
-    }
-    cleanup();
+    std::memcpy(d.class_count.data(), back.data() + 16, sizeof(int64_t) * (size_t)K);
+    d.finite = hst[1] == 0;
+    d.ncode = (int32_t)hst[2];
+    d.ranked = d.finite && rank_tables;
+    if (!d.ranked && d.Rk) { cudaFree(d.Rk); d.Rk = nullptr; }
+    cudaFree(tmp);
 #undef REG_CUDA
     return RS_OK;
 }
@@ -537,12 +584,9 @@ static size_t dataset_device_bytes(const Dataset &d)
 
 static void free_device(Dataset &d)
 {
-    cudaFree(d.Xt);
-    cudaFree(d.y);
-    cudaFree(d.perm);
-    cudaFree(d.inv);
+    cudaFree(d.Xt);                  // the start of the dataset's own allocation
     cudaFree(d.Rk);
-    d.Xt = nullptr; d.y = nullptr; d.perm = nullptr; d.inv = nullptr; d.Rk = nullptr;
+    d.Xt = nullptr; d.y = nullptr; d.perm = nullptr; d.inv = nullptr; d.flags = nullptr; d.Rk = nullptr;
     std::lock_guard<std::mutex> lk(d.mu);
     d.tmaps.clear();                 // tensor maps hold the device addresses
     d.rmap_ok = false;
@@ -757,10 +801,8 @@ void preload_dataset_kernels()
     cudaFuncGetAttributes(&fa, k_label_offsets);
     cudaFuncGetAttributes(&fa, k_class_start);
     cudaFuncGetAttributes(&fa, k_label_scatter);
-    cudaFuncGetAttributes(&fa, k_transpose_gather);
-    cudaFuncGetAttributes(&fa, k_nonfinite);
-    cudaFuncGetAttributes(&fa, k_rank_tiles);
-    cudaFuncGetAttributes(&fa, k_fill_i32);
+    cudaFuncGetAttributes(&fa, k_register_tile);
+    cudaFuncGetAttributes(&fa, k_register_summary);
 }
 
 }  // namespace rs
