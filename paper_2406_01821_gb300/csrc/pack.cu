@@ -118,24 +118,40 @@ __device__ void rewrite_lin(float a, float t, int op, float &v0, float &v1)
     }
 }
 
-// Pack v2 records: one thread per rule.
-__global__ void k_pack_rules2(BatchDev b, int F, int K, int S, int form, Rec *recs_out, uint32_t *status)
+// Every rule is packed by RULE_LANES neighbouring lanes, a condition each at a time: the loads and
+// rewrites of a rule's conditions overlap instead of following one another. This lane's rule.
+constexpr int RULE_LANES = 8;
+struct RuleLane {
+    int r, sub, c0, c1, cls;
+    bool live;                 // the rule exists and its offsets and length are sound
+    __device__ RuleLane(const BatchDev &b, int K, int block, uint32_t *status)
+    {
+        r = (int)(((int64_t)block * blockDim.x + threadIdx.x) / RULE_LANES);
+        sub = threadIdx.x % RULE_LANES;
+        live = r < b.R;
+        c0 = c1 = cls = 0;
+        if (!live) return;
+        c0 = b.rule_cond_off[r];
+        c1 = b.rule_cond_off[r + 1];
+        cls = b.rule_class[r];
+        if (c0 < 0 || c1 < c0 || c1 > b.C) { atomicOr(status, ST_BAD_OFFSETS); live = false; }
+        else if (c1 - c0 > 0xFFF) { atomicOr(status, ST_TOO_LARGE); live = false; }
+        else if (cls < 0 || cls >= K) { atomicOr(status, ST_BAD_CLASS); cls = 0; }
+        if (!live) c1 = c0 = 0;
+    }
+};
+
+// Pack v2 / v4 records.
+__device__ void pack_rule2(const BatchDev &b, int F, int K, int S, int form, Rec *recs_out, uint32_t *status, int block)
 {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b.dR) { b.R = *b.dR; b.C = *b.dC; }
-    if (r >= b.R) return;
-    const int c0 = b.rule_cond_off[r], c1 = b.rule_cond_off[r + 1];
-    if (c0 < 0 || c1 < c0 || c1 > b.C) { atomicOr(status, ST_BAD_OFFSETS); return; }
-    if (c1 - c0 > 0xFFF) { atomicOr(status, ST_TOO_LARGE); return; }
-    int cls = b.rule_class[r];
-    if (cls < 0 || cls >= K) { atomicOr(status, ST_BAD_CLASS); cls = 0; }
+    const RuleLane rl(b, K, block, status);
     uint4 *out = reinterpret_cast<uint4 *>(recs_out);
-    const uint32_t len = (uint32_t)(c1 - c0);
+    const uint32_t len = (uint32_t)(rl.c1 - rl.c0);
     const uint32_t row16 = (uint32_t)S / 4;   // 16-byte units per feature row
     const auto row = [&](int f) { return (uint32_t)f * row16 | (form == 4 ? (uint32_t)f & 7u : 0u); };
-    for (int c = c0; c < c1; ++c) {
+    for (int c = rl.c0 + rl.sub; c < rl.c1; c += RULE_LANES) {
         const int f = b.cond_f[c], g = b.cond_g[c], op = b.cond_op[c];
-        uint32_t w0 = len << LEN_SHIFT, w1 = (uint32_t)cls << CLS_SHIFT;
+        uint32_t w0 = len << LEN_SHIFT, w1 = (uint32_t)rl.cls << CLS_SHIFT;
         float v0 = 0.f, v1 = __uint_as_float(0x7F800000u);   // never true
         if (f < 0 || f >= F || g < -1 || g >= F) {
             atomicOr(status, ST_BAD_FEATURE);
@@ -144,11 +160,11 @@ __global__ void k_pack_rules2(BatchDev b, int F, int K, int S, int form, Rec *re
         } else if (g < 0 && form == 4) {
             // cut form: x > c  <=>  sign(fl(+-x - c')) clear with c' = nextup(+-c)
             uint32_t kind;
-            float c0, c1;
-            rewrite_threshold(b.cond_a[c], b.cond_t[c], op, kind, c0, c1);
+            float k0, k1;
+            rewrite_threshold(b.cond_a[c], b.cond_t[c], op, kind, k0, k1);
             const float pinf = __uint_as_float(0x7F800000u);
-            if (kind == KIND_GT) { v0 = 1.f; v1 = -nextafterf(c0, pinf); }
-            else if (kind == KIND_LT) { v0 = -1.f; v1 = -nextafterf(-c0, pinf); }
+            if (kind == KIND_GT) { v0 = 1.f; v1 = -nextafterf(k0, pinf); }
+            else if (kind == KIND_LT) { v0 = -1.f; v1 = -nextafterf(-k0, pinf); }
             else { rewrite_lin(b.cond_a[c], b.cond_t[c], op, v0, v1); w0 |= GENERAL_BIT; }
             w0 |= row(f);
         } else if (g < 0) {
@@ -161,11 +177,10 @@ __global__ void k_pack_rules2(BatchDev b, int F, int K, int S, int form, Rec *re
             w0 |= row(lf) | PAIR_BIT;
             w1 |= row(rg);
         }
-        if (form == 4 && c == c1 - 1) w1 |= END4_BIT;
+        if (form == 4 && c == rl.c1 - 1) w1 |= END4_BIT;
         out[c] = make_uint4(w0, w1, __float_as_uint(v0), __float_as_uint(v1));
     }
 }
-
 
 // Order buckets of the counting sort of sets by cost (k_order, and k_pack_sets for one-block batches).
 constexpr int ORDER_BUCKETS = 1024;
@@ -208,82 +223,102 @@ __device__ void scan_buckets(int *hist)
 }
 
 // Offsets, default class and first empty rule of set p (an empty rule fires for every sample
-// still unclaimed, so the set effectively ends there with that class as its default). Returns
-// the set's cost (its record count).
-__device__ int pack_one_set(const BatchDev &b, int K, int p, SetInfo *sets, int32_t *last_end, uint32_t *status)
+// still unclaimed, so the set effectively ends there with that class as its default), by one warp, a
+// rule a lane. le: the warp's LAST_END_MAX_K words of shared memory. Returns the set's cost (its
+// record count).
+__device__ int pack_one_set(const BatchDev &b, int K, int p, int lane, int *le, SetInfo *sets, int32_t *last_end,
+                            uint32_t *status)
 {
+    constexpr uint32_t FULL = 0xFFFFFFFFu;
     SetInfo si{0, 0, 0, 0};
     const int rb = b.set_rule_off[p], re = b.set_rule_off[p + 1];
     int d = b.set_default[p];
-    if (d < 0 || d >= K) { atomicOr(status, ST_BAD_CLASS); d = 0; }
+    if (d < 0 || d >= K) { if (lane == 0) atomicOr(status, ST_BAD_CLASS); d = 0; }
     si.deflt = d;
-    if (rb < 0 || re < rb || re > b.R) {
-        atomicOr(status, ST_BAD_OFFSETS);
-        sets[p] = si;
-        return 0;
-    }
-    int c_begin = 0, c_end = 0;
-    bool ok = true;
+    bool ok = rb >= 0 && re >= rb && re <= b.R;
     if (last_end)
-        for (int k = 0; k < K; ++k) last_end[(int64_t)p * K + k] = 0;
-    for (int r = rb; r < re; ++r) {
-        const int c0 = b.rule_cond_off[r], c1 = b.rule_cond_off[r + 1];
-        if (c0 < 0 || c1 < c0 || c1 > b.C) { ok = false; break; }
-        if (c1 - c0 > 0xFFF) { atomicOr(status, ST_TOO_LARGE); ok = false; break; }
-        if (r == rb) { c_begin = c0; c_end = c0; }
-        const int cls = b.rule_class[r];
-        if (cls < 0 || cls >= K) { atomicOr(status, ST_BAD_CLASS); ok = false; break; }
-        if (c1 == c0) { si.deflt = cls; break; }   // empty rule: fires on everything left
-        c_end = c1;
-        if (last_end) last_end[(int64_t)p * K + cls] = c1 - c_begin;
+        for (int k = lane; k < K; k += 32) le[k] = 0;
+    __syncwarp();
+    int c_begin = 0, c_end = 0;
+    bool open = ok;                          // no empty and no unsound rule so far
+    for (int r0 = rb; open && r0 < re; r0 += 32) {
+        const int r = r0 + lane;
+        int c0 = 0, c1 = 1, cls = 0;
+        bool bad = false;
+        if (r < re) {
+            c0 = b.rule_cond_off[r];
+            c1 = b.rule_cond_off[r + 1];
+            cls = b.rule_class[r];
+            bad = c0 < 0 || c1 < c0 || c1 > b.C;
+            if (!bad && c1 - c0 > 0xFFF) { atomicOr(status, ST_TOO_LARGE); bad = true; }
+            if (!bad && (cls < 0 || cls >= K)) { atomicOr(status, ST_BAD_CLASS); bad = true; }
+        }
+        if (r0 == rb) c_begin = c_end = __shfl_sync(FULL, c0, 0);
+        const uint32_t bads = __ballot_sync(FULL, bad), stops = __ballot_sync(FULL, bad || c1 == c0);
+        const int n = stops ? __ffs(stops) - 1 : min(32, re - r0);         // rules before the stop
+        if (lane < n && last_end) atomicMax(&le[cls], c1 - c_begin);
+        if (n > 0) c_end = __shfl_sync(FULL, c1, n - 1);
+        if (stops) {
+            open = false;
+            if ((bads >> n) & 1u) ok = false;
+            else si.deflt = __shfl_sync(FULL, cls, n);   // empty rule: fires on everything left
+        }
     }
+    __syncwarp();
     if (!ok) {
-        atomicOr(status, ST_BAD_OFFSETS);
+        if (lane == 0) atomicOr(status, ST_BAD_OFFSETS);
         c_begin = c_end = 0;
-        if (last_end)
-            for (int k = 0; k < K; ++k) last_end[(int64_t)p * K + k] = 0;
-    } else if (last_end) {
+    }
+    if (last_end) {
         // for the default class d: the end of the last rule of any other class (after it every rule
         // left names d, and so does the default: every sample still unclaimed counts for d)
         int m = 0;
-        for (int k = 0; k < K; ++k)
-            if (k != si.deflt) m = max(m, last_end[(int64_t)p * K + k]);
-        last_end[(int64_t)p * K + si.deflt] = m;
+        for (int k = lane; k < K; k += 32)
+            if (k != si.deflt) m = max(m, le[k]);
+        m = __reduce_max_sync(FULL, m);
+        for (int k = lane; k < K; k += 32) last_end[(int64_t)p * K + k] = ok ? (k == si.deflt ? m : le[k]) : 0;
+        __syncwarp();
     }
     si.rec_begin = c_begin;
     si.rec_end = c_end;
     si.cost = c_end - c_begin;
-    sets[p] = si;
+    if (lane == 0) sets[p] = si;
     return si.cost;
 }
 
-// One thread per set: the set's descriptor, and zeroed counts (correct[p], per_class[p][*]) when
-// the output pointers are given. With `order_here` (a batch of at most one block) the block also
-// sorts the sets by cost, which otherwise k_order does in a launch of its own.
-__global__ void k_pack_sets(BatchDev b, int K, PackOut o, bool order_here)
+constexpr int PACK_BLOCK = 1024;             // a warp per set, RULE_LANES lanes per rule
+constexpr int ORDER_HERE_SETS = 64;          // sets up to which one block packs and also sorts them
+
+// The set part of the packing, one warp per set: the set's descriptor, and zeroed counts (correct[p],
+// per_class[p][*]) when the output pointers are given. With `order_here` one block takes all sets and
+// also sorts them by cost, which otherwise k_order does in a launch of its own.
+__device__ void pack_sets(const BatchDev &b, int K, const PackOut &o, bool order_here)
 {
     __shared__ int hist[ORDER_BUCKETS];
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b.dR) { b.R = *b.dR; b.C = *b.dC; }
-    if (p == 0) {
+    __shared__ int le[PACK_BLOCK / 32][LAST_END_MAX_K];
+    __shared__ int cost_of[ORDER_HERE_SETS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = PACK_BLOCK / 32;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
         if (b.set_rule_off[0] != 0 || b.set_rule_off[b.P] != b.R ||
             b.rule_cond_off[0] != 0 || b.rule_cond_off[b.R] != b.C)
             atomicOr(o.status, ST_BAD_OFFSETS);
     }
-    int cost = 0;
-    if (p < b.P) {
-        if (o.correct) o.correct[p] = 0;
+    const int p0 = order_here ? warp : blockIdx.x * warps + warp;
+    for (int p = p0; p < b.P; p += order_here ? warps : b.P) {
+        if (lane == 0 && o.correct) o.correct[p] = 0;
         if (o.per_class)
-            for (int k = 0; k < K; ++k) o.per_class[(int64_t)p * K + k] = 0;
-        cost = pack_one_set(b, K, p, o.sets, o.last_end, o.status);
+            for (int k = lane; k < K; k += 32) o.per_class[(int64_t)p * K + k] = 0;
+        const int cost = pack_one_set(b, K, p, lane, le[warp], o.sets, o.last_end, o.status);
+        if (order_here && lane == 0) cost_of[p] = cost;
     }
     if (!order_here) return;   // uniform over the launch
+    const int p = threadIdx.x;
     for (int i = threadIdx.x; i < ORDER_BUCKETS; i += blockDim.x) hist[i] = 0;
     __syncthreads();
-    if (p < b.P) atomicAdd(&hist[order_bucket(cost)], 1);
+    if (p < b.P) atomicAdd(&hist[order_bucket(cost_of[p])], 1);
     __syncthreads();
     scan_buckets(hist);
-    if (p < b.P) o.order[atomicAdd(&hist[order_bucket(cost)], 1)] = p;
+    if (p < b.P) o.order[atomicAdd(&hist[order_bucket(cost_of[p])], 1)] = p;
 }
 
 // Kind of a condition in format v5, decided with the same tests as rewrite_threshold (without its
@@ -304,52 +339,56 @@ __device__ uint32_t kind5(const BatchDev &b, int c, int F)
     return up ? R5_CUT_GT : R5_CUT_LT;
 }
 
-// Pack v5 records, one thread per rule: the cuts, the pairs and the remaining conditions (a
-// conjunction does not depend on the order of its conditions); the rule's last record carries
-// the end-of-rule flag and the rule class.
-__global__ void k_pack_rules5(BatchDev b, int F, int K, Rec *recs_out, uint32_t *status)
+// Pack v5 records: the cuts, the pairs and the remaining conditions of each rule (a conjunction does
+// not depend on the order of its conditions); the rule's last record carries the end-of-rule flag
+// and the rule class.
+__device__ void pack_rule5(const BatchDev &b, int F, int K, Rec *recs_out, uint32_t *status, int block)
 {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b.dR) { b.R = *b.dR; b.C = *b.dC; }
-    if (r >= b.R) return;
-    const int c0 = b.rule_cond_off[r], c1 = b.rule_cond_off[r + 1];
-    if (c0 < 0 || c1 < c0 || c1 > b.C) { atomicOr(status, ST_BAD_OFFSETS); return; }
-    if (c1 - c0 > 0xFFF) { atomicOr(status, ST_TOO_LARGE); return; }
-    int cls = b.rule_class[r];
-    if (cls < 0 || cls >= K) { atomicOr(status, ST_BAD_CLASS); cls = 0; }
+    constexpr uint32_t FULL = 0xFFFFFFFFu;
+    const RuleLane rl(b, K, block, status);
+    const int shift = (threadIdx.x & 31) / RULE_LANES * RULE_LANES;
+    const uint32_t mine = ((1u << RULE_LANES) - 1u) << shift, before = (1u << (threadIdx.x & 31)) - 1u;
+    const auto is_cut = [](uint32_t k) { return k == R5_CUT_GT || k == R5_CUT_LT; };
     uint4 *out = reinterpret_cast<uint4 *>(recs_out);
     int ncut = 0, npair = 0;
-    for (int c = c0; c < c1; ++c) {
-        const uint32_t k = kind5(b, c, F);
-        ncut += (k == R5_CUT_GT || k == R5_CUT_LT);
-        npair += (k == R5_PAIR);
+    for (int c0 = rl.c0; __any_sync(FULL, c0 < rl.c1); c0 += RULE_LANES) {
+        const int c = c0 + rl.sub;
+        const uint32_t k = c < rl.c1 ? kind5(b, c, F) : R5_NONE;
+        ncut += __popc(__ballot_sync(FULL, is_cut(k)) & mine);
+        npair += __popc(__ballot_sync(FULL, k == R5_PAIR) & mine);
     }
-    int qc = c0, qp = c0 + ncut, qg = c0 + ncut + npair;
+    int qc = rl.c0, qp = rl.c0 + ncut, qg = rl.c0 + ncut + npair;
     const float pinf = __uint_as_float(0x7F800000u);
-    for (int c = c0; c < c1; ++c) {
-        const uint32_t k = kind5(b, c, F);
+    for (int c0 = rl.c0; __any_sync(FULL, c0 < rl.c1); c0 += RULE_LANES) {
+        const int c = c0 + rl.sub;
+        const bool here = c < rl.c1;
+        const uint32_t k = here ? kind5(b, c, F) : R5_NONE;
+        const uint32_t cuts = __ballot_sync(FULL, is_cut(k)) & mine, pairs = __ballot_sync(FULL, k == R5_PAIR) & mine;
+        const uint32_t rest = __ballot_sync(FULL, here) & mine & ~(cuts | pairs);
+        const int q = is_cut(k) ? qc + __popc(cuts & before) : (k == R5_PAIR ? qp + __popc(pairs & before)
+                                                                            : qg + __popc(rest & before));
+        qc += __popc(cuts);
+        qp += __popc(pairs);
+        qg += __popc(rest);
+        if (!here) continue;
         const int f = b.cond_f[c], g = b.cond_g[c], op = b.cond_op[c];
-        int q;
         uint4 rec;
-        if (k == R5_CUT_GT || k == R5_CUT_LT) {
+        if (is_cut(k)) {
             uint32_t kind;
             float cut, unused;
             rewrite_threshold(b.cond_a[c], b.cond_t[c], op, kind, cut, unused);
             // x < c  <=>  x <= nextdown(c) for non-NaN x: both cut kinds then count tile values <= w2
             if (k == R5_CUT_LT) cut = nextafterf(cut, __uint_as_float(0xFF800000u));
             rec = make_uint4((k << R5_TAG_SHIFT) | (uint32_t)f, 0u, __float_as_uint(cut), 0u);
-            q = qc++;
         } else if (k == R5_PAIR) {
             const int lf = op == 0 ? f : g, rg = op == 0 ? g : f;
             const float a = op == 0 ? b.cond_a[c] : b.cond_b[c];
             const float bb = op == 0 ? b.cond_b[c] : b.cond_a[c];
             rec = make_uint4((R5_PAIR << R5_TAG_SHIFT) | (uint32_t)lf, (uint32_t)rg, __float_as_uint(a),
                              __float_as_uint(bb));
-            q = qp++;
         } else if (k == R5_SET) {
             const uint64_t set = b.cond_set[c];
             rec = make_uint4((R5_SET << R5_TAG_SHIFT) | (uint32_t)f, 0u, (uint32_t)set, (uint32_t)(set >> 32));
-            q = qg++;
         } else {
             float v0 = 0.f, v1 = pinf;   // never true
             uint32_t rf = 0;
@@ -357,25 +396,17 @@ __global__ void k_pack_rules5(BatchDev b, int F, int K, Rec *recs_out, uint32_t 
             else if (op != 0 && op != 1) atomicOr(status, ST_BAD_OP);
             else { rewrite_lin(b.cond_a[c], b.cond_t[c], op, v0, v1); rf = (uint32_t)f; }
             rec = make_uint4((R5_GEN << R5_TAG_SHIFT) | rf, 0u, __float_as_uint(v0), __float_as_uint(v1));
-            q = qg++;
         }
-        if (q == c1 - 1) rec.x |= R5_END_BIT | ((uint32_t)cls << R5_CLS_SHIFT);
+        if (q == rl.c1 - 1) rec.x |= R5_END_BIT | ((uint32_t)rl.cls << R5_CLS_SHIFT);
         out[q] = rec;
     }
 }
 
-// One thread per rule: build the records of its conditions.
-__global__ void k_pack_rules(BatchDev b, int F, int K, Rec *recs, uint32_t *status)
+// Pack v1 records.
+__device__ void pack_rule1(const BatchDev &b, int F, int K, Rec *recs, uint32_t *status, int block)
 {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b.dR) { b.R = *b.dR; b.C = *b.dC; }
-    if (r >= b.R) return;
-    const int c0 = b.rule_cond_off[r], c1 = b.rule_cond_off[r + 1];
-    if (c0 < 0 || c1 < c0 || c1 > b.C) { atomicOr(status, ST_BAD_OFFSETS); return; }
-    if (c1 - c0 > 0xFFF) { atomicOr(status, ST_TOO_LARGE); return; }    // rule length is 12 bits
-    int cls = b.rule_class[r];
-    if (cls < 0 || cls >= K) { atomicOr(status, ST_BAD_CLASS); cls = 0; }
-    for (int c = c0; c < c1; ++c) {
+    const RuleLane rl(b, K, block, status);
+    for (int c = rl.c0 + rl.sub; c < rl.c1; c += RULE_LANES) {
         const int f = b.cond_f[c], g = b.cond_g[c], op = b.cond_op[c];
         Rec rec;
         uint32_t kind = KIND_NEVER;
@@ -399,15 +430,30 @@ __global__ void k_pack_rules(BatchDev b, int F, int K, Rec *recs, uint32_t *stat
         } else {                   // a*x[f] < b*x[g]  <=>  b*x[g] > a*x[f]
             kind = KIND_PAIR; rf = g; rg = f; v0 = b.cond_b[c]; v1 = b.cond_a[c];
         }
-        const uint32_t last = (c == c1 - 1) ? 1u : 0u;
-        const uint32_t skip = (uint32_t)min(c1 - 1 - c, 0xFFFF);
-        rec.meta = kind | (last << 3) | ((uint32_t)cls << 4) | (skip << 16);
+        const uint32_t last = (c == rl.c1 - 1) ? 1u : 0u;
+        const uint32_t skip = (uint32_t)min(rl.c1 - 1 - c, 0xFFFF);
+        rec.meta = kind | (last << 3) | ((uint32_t)rl.cls << 4) | (skip << 16);
         rec.f = (uint16_t)rf;
         rec.g = (uint16_t)rg;
         rec.v0 = v0;
         rec.v1 = v1;
         recs[c] = rec;
     }
+}
+
+// Sets and rules in one launch: blocks [0, set_blocks) the sets, the others the rules, which depend on
+// nothing the sets write. As two launches with a thread per set and per rule, each walking its rules or
+// conditions one load after another, packing took 15 us of the paper-shape call's 38; 7 us so.
+template <int VER>
+__global__ void __launch_bounds__(PACK_BLOCK) k_pack(BatchDev b, int F, int K, int S, PackOut o, int set_blocks,
+                                                     bool order_here)
+{
+    if (b.dR) { b.R = *b.dR; b.C = *b.dC; }
+    if ((int)blockIdx.x < set_blocks) { pack_sets(b, K, o, order_here); return; }
+    const int block = (int)blockIdx.x - set_blocks;
+    if (VER == 5) pack_rule5(b, F, K, o.recs, o.status, block);
+    else if (VER == 1) pack_rule1(b, F, K, o.recs, o.status, block);
+    else pack_rule2(b, F, K, S, VER, o.recs, o.status, block);
 }
 
 // Single-CTA counting sort of sets by cost, most expensive first (bucketed; the order only
@@ -428,22 +474,18 @@ __global__ void k_order(const SetInfo *sets, int P, int32_t *order)
 
 int launch_pack(const BatchDev &b, int F, int K, int S, int ver, const PackOut &o, cudaStream_t stream)
 {
-    int n = 0;
-    constexpr int SET_BLOCK = 256;
-    const bool order_here = o.order && b.P <= SET_BLOCK;
-    if (b.P > 0) { k_pack_sets<<<(b.P + SET_BLOCK - 1) / SET_BLOCK, SET_BLOCK, 0, stream>>>(b, K, o, order_here); ++n; }
-    if (b.R > 0 && ver == 5) {
-        k_pack_rules5<<<(b.R + 127) / 128, 128, 0, stream>>>(b, F, K, o.recs, o.status);
-        ++n;
-    } else if (b.R > 0 && ver >= 2) {
-        k_pack_rules2<<<(b.R + 127) / 128, 128, 0, stream>>>(b, F, K, S, ver == 4 ? 4 : 2, o.recs, o.status);
-        ++n;
-    } else if (b.R > 0) {
-        k_pack_rules<<<(b.R + 127) / 128, 128, 0, stream>>>(b, F, K, o.recs, o.status);
-        ++n;
-    }
-    if (b.P > 0 && o.order && !order_here) { k_order<<<1, 1024, 0, stream>>>(o.sets, b.P, o.order); ++n; }
-    return n;
+    const bool order_here = o.order && b.P <= ORDER_HERE_SETS;
+    const int set_blocks = b.P == 0 ? 0 : (order_here ? 1 : (b.P + PACK_BLOCK / 32 - 1) / (PACK_BLOCK / 32));
+    const int rule_blocks = (int)(((int64_t)b.R * RULE_LANES + PACK_BLOCK - 1) / PACK_BLOCK);
+    const int grid = set_blocks + rule_blocks;
+    if (grid == 0) return 0;
+    if (ver == 5) k_pack<5><<<grid, PACK_BLOCK, 0, stream>>>(b, F, K, S, o, set_blocks, order_here);
+    else if (ver == 4) k_pack<4><<<grid, PACK_BLOCK, 0, stream>>>(b, F, K, S, o, set_blocks, order_here);
+    else if (ver >= 2) k_pack<2><<<grid, PACK_BLOCK, 0, stream>>>(b, F, K, S, o, set_blocks, order_here);
+    else k_pack<1><<<grid, PACK_BLOCK, 0, stream>>>(b, F, K, S, o, set_blocks, order_here);
+    if (b.P == 0 || !o.order || order_here) return 1;
+    k_order<<<1, 1024, 0, stream>>>(o.sets, b.P, o.order);
+    return 2;
 }
 
 // --------------------------------------------------------------- exhaustive rewrite self-check
@@ -505,10 +547,10 @@ rs_status selftest_rewrite(const float *a_h, const float *t_h, const int8_t *op_
 void preload_pack_kernels()
 {
     cudaFuncAttributes fa;
-    cudaFuncGetAttributes(&fa, k_pack_rules);
-    cudaFuncGetAttributes(&fa, k_pack_rules2);
-    cudaFuncGetAttributes(&fa, k_pack_rules5);
-    cudaFuncGetAttributes(&fa, k_pack_sets);
+    cudaFuncGetAttributes(&fa, k_pack<1>);
+    cudaFuncGetAttributes(&fa, k_pack<2>);
+    cudaFuncGetAttributes(&fa, k_pack<4>);
+    cudaFuncGetAttributes(&fa, k_pack<5>);
     cudaFuncGetAttributes(&fa, k_order);
 }
 
