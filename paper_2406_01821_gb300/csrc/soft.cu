@@ -63,33 +63,6 @@ struct __align__(16) SoftRec {
                       // bits of its category set (0..31 in a, 32..63 in bt)
 };
 
-__global__ void k_pack_soft(BatchDev b, int F, int K, SoftRec *recs, uint32_t *status, int32_t *work_counter)
-{
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c == 0) work_counter[0] = work_counter[SOFT_NEXT_FF_LEN] = work_counter[SOFT_NEXT_FF] = 0;
-    if (b.dR) { b.R = *b.dR; b.C = *b.dC; }
-    if (c >= b.C) return;
-    const int f = b.cond_f[c], g = b.cond_g[c], op = b.cond_op[c];
-    SoftRec r{0, 0, 0, 0.f, 0.f};
-    if (f < 0 || f >= F || g < -1 || g >= F) atomicOr(status, ST_BAD_FEATURE);
-    else if (op == RS_OP_IN && b.cond_set && g == -1) {
-        const uint64_t set = b.cond_set[c];
-        r.meta = 4u;
-        r.f = (uint16_t)f;
-        r.a = __uint_as_float((uint32_t)set);
-        r.bt = __uint_as_float((uint32_t)(set >> 32));
-    } else if (op != 0 && op != 1) atomicOr(status, ST_BAD_OP);
-    else {
-        r.meta = (g >= 0 ? 1u : 0u) | (op == 1 ? 2u : 0u);
-        r.f = (uint16_t)f;
-        r.g = (uint16_t)(g >= 0 ? g : 0);
-        r.a = b.cond_a[c];
-        r.bt = g >= 0 ? b.cond_b[c] : b.cond_t[c];
-    }
-    recs[c] = r;
-}
-
-// Validation of the set/rule structure (one thread per set).
 // Single-CTA counting sort of the sets by size (rules + conditions, most first), so that the
 // warps of one CTA group walk sets of similar length. Malformed offsets count as size 0 (the
 // check kernel rejects the batch).
@@ -115,33 +88,75 @@ __global__ void k_soft_order(BatchDev b, int32_t *order)
     for (int p = threadIdx.x; p < b.P; p += blockDim.x) order[atomicAdd(&hist[bucket(p)], 1)] = p;
 }
 
-__global__ void k_check_sets_soft(BatchDev b, int K, uint32_t *status, int32_t *maxima, int maxR,
-                                  int maxC)
+// Validation of set p's structure by one warp, a rule a lane.
+__device__ void check_set_soft(const BatchDev &b, int p, int lane, int K, uint32_t *status, int32_t *maxima, int maxR,
+                               int maxC)
 {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b.dR) { b.R = *b.dR; b.C = *b.dC; }
-    if (p == 0) {
-        if (b.set_rule_off[0] != 0 || b.set_rule_off[b.P] != b.R ||
-            b.rule_cond_off[0] != 0 || b.rule_cond_off[b.R] != b.C)
-            atomicOr(status, ST_BAD_OFFSETS);
-    }
-    if (p >= b.P) return;
     const int rb = b.set_rule_off[p], re = b.set_rule_off[p + 1];
     const int d = b.set_default[p];
-    if (d < 0 || d >= K) atomicOr(status, ST_BAD_CLASS);
-    if (rb < 0 || re < rb || re > b.R) { atomicOr(status, ST_BAD_OFFSETS); return; }
-    if (re - rb > SOFT_MAX_RULES) { atomicOr(status, ST_TOO_LARGE); return; }
-    for (int r = rb; r < re; ++r) {
+    if (lane == 0 && (d < 0 || d >= K)) atomicOr(status, ST_BAD_CLASS);
+    if (rb < 0 || re < rb || re > b.R) { if (lane == 0) atomicOr(status, ST_BAD_OFFSETS); return; }
+    if (re - rb > SOFT_MAX_RULES) { if (lane == 0) atomicOr(status, ST_TOO_LARGE); return; }
+    bool bad = false;
+    for (int r = rb + lane; r < re; r += 32) {
         const int c0 = b.rule_cond_off[r], c1 = b.rule_cond_off[r + 1];
-        if (c0 < 0 || c1 < c0 || c1 > b.C) { atomicOr(status, ST_BAD_OFFSETS); return; }
+        bad |= c0 < 0 || c1 < c0 || c1 > b.C;
         const int cls = b.rule_class[r];
         if (cls < 0 || cls >= K) atomicOr(status, ST_BAD_CLASS);
     }
+    if (__any_sync(FULL, bad)) { if (lane == 0) atomicOr(status, ST_BAD_OFFSETS); return; }
+    if (lane != 0) return;
     const int nc = re > rb ? b.rule_cond_off[re] - b.rule_cond_off[rb] : 0;
     if (nc > SOFT_MAX_CONDS || re - rb > maxR || nc > maxC) atomicOr(status, ST_TOO_LARGE);
     atomicMax(&maxima[0], re - rb);
     atomicMax(&maxima[1], nc);
 }
+
+// The record of condition c.
+__device__ void pack_soft_one(const BatchDev &b, int c, int F, SoftRec *recs, uint32_t *status)
+{
+    const int f = b.cond_f[c], g = b.cond_g[c], op = b.cond_op[c];
+    SoftRec r{0, 0, 0, 0.f, 0.f};
+    if (f < 0 || f >= F || g < -1 || g >= F) atomicOr(status, ST_BAD_FEATURE);
+    else if (op == RS_OP_IN && b.cond_set && g == -1) {
+        const uint64_t set = b.cond_set[c];
+        r.meta = 4u;
+        r.f = (uint16_t)f;
+        r.a = __uint_as_float((uint32_t)set);
+        r.bt = __uint_as_float((uint32_t)(set >> 32));
+    } else if (op != 0 && op != 1) atomicOr(status, ST_BAD_OP);
+    else {
+        r.meta = (g >= 0 ? 1u : 0u) | (op == 1 ? 2u : 0u);
+        r.f = (uint16_t)f;
+        r.g = (uint16_t)(g >= 0 ? g : 0);
+        r.a = b.cond_a[c];
+        r.bt = g >= 0 ? b.cond_b[c] : b.cond_t[c];
+    }
+    recs[c] = r;
+}
+
+// One launch: blocks [0, set_blocks) validate the sets, a warp each; the others pack the conditions
+// and reset the call's counters. (A thread per set walking its rules took 12 us in a launch of its own.)
+constexpr int SOFT_PREP_BLOCK = 256;
+__global__ void k_soft_prep(BatchDev b, int F, int K, SoftRec *recs, uint32_t *status, int32_t *counters,
+                            int32_t *maxima, int maxR, int maxC, int set_blocks)
+{
+    if (b.dR) { b.R = *b.dR; b.C = *b.dC; }
+    if ((int)blockIdx.x < set_blocks) {
+        const int p = (int)((blockIdx.x * SOFT_PREP_BLOCK + threadIdx.x) >> 5);
+        if (blockIdx.x == 0 && threadIdx.x == 0 &&
+            (b.set_rule_off[0] != 0 || b.set_rule_off[b.P] != b.R || b.rule_cond_off[0] != 0 ||
+             b.rule_cond_off[b.R] != b.C))
+            atomicOr(status, ST_BAD_OFFSETS);
+        if (p < b.P) check_set_soft(b, p, threadIdx.x & 31, K, status, maxima, maxR, maxC);
+        return;
+    }
+    const int64_t c = (int64_t)(blockIdx.x - set_blocks) * SOFT_PREP_BLOCK + threadIdx.x;
+    if (c == 0) counters[0] = counters[SOFT_NEXT_FF_LEN] = counters[SOFT_NEXT_FF] = 0;
+    if (recs && c < b.C) pack_soft_one(b, (int)c, F, recs, status);
+}
+
+static int soft_set_blocks(int P) { return (int)(((int64_t)P * 32 + SOFT_PREP_BLOCK - 1) / SOFT_PREP_BLOCK); }
 
 // log(1 + e) for 0 <= e <= 1 as e p(e), with p the polynomial of degree 8 of least maximum
 // relative error against log1p(e) / e on [0, 1] (Remez exchange, 3.0e-8 before its coefficients
@@ -1605,14 +1620,11 @@ static rs_status soft_run(Ctx *ctx, const SoftArgs &s, int known_maxR, int known
     }
     const bool known = known_maxR > 0;
     repeat = repeat && pre && known;
-    if (!repeat) {
-        RS_CUDA(cudaMemsetAsync(next, 0, sizeof(int32_t) * SOFT_NEXT_N, stream));
-        k_check_sets_soft<<<(P + 255) / 256, 256, 0, stream>>>(b, s.K, s.status, next + 1,
-                                                               known ? known_maxR : SOFT_MAX_RULES,
-                                                               known ? known_maxC : SOFT_MAX_CONDS);
-        count_launch(ctx);
-    }
-    k_pack_soft<<<(unsigned)((Ccap + 255) / 256), 256, 0, stream>>>(b, s.F, s.K, recs, s.status, next);
+    if (!repeat) RS_CUDA(cudaMemsetAsync(next, 0, sizeof(int32_t) * SOFT_NEXT_N, stream));
+    const int set_blocks = repeat ? 0 : soft_set_blocks(P);
+    k_soft_prep<<<set_blocks + (unsigned)((Ccap + SOFT_PREP_BLOCK - 1) / SOFT_PREP_BLOCK), SOFT_PREP_BLOCK, 0, stream>>>(
+        b, s.F, s.K, recs, s.status, next, next + 1, known ? known_maxR : SOFT_MAX_RULES,
+        known ? known_maxC : SOFT_MAX_CONDS, set_blocks);
     count_launch(ctx);
     if (!repeat) {
         k_soft_order<<<1, 1024, 0, stream>>>(b, order);
@@ -1786,7 +1798,8 @@ rs_status soft_validate(Ctx *ctx, const SoftArgs &a, int *maxR, int *maxC, cudaS
     int32_t *maxima = nullptr;
     RS_CUDA(dev_alloc_async(&maxima, sizeof(int32_t) * 4, stream));
     RS_CUDA(cudaMemsetAsync(maxima, 0, sizeof(int32_t) * 4, stream));
-    k_check_sets_soft<<<(b.P + 255) / 256, 256, 0, stream>>>(b, a.K, a.status, maxima, SOFT_MAX_RULES, SOFT_MAX_CONDS);
+    k_soft_prep<<<soft_set_blocks(b.P), SOFT_PREP_BLOCK, 0, stream>>>(b, a.F, a.K, nullptr, a.status, nullptr, maxima,
+                                                                      SOFT_MAX_RULES, SOFT_MAX_CONDS, soft_set_blocks(b.P));
     count_launch(ctx);
     uint32_t *hs = host_status_slot();
     if (!hs) { cudaFreeAsync(maxima, stream); return RS_ERR_OOM; }
@@ -1835,8 +1848,7 @@ void preload_soft_kernels()
     cudaFuncGetAttributes(&fa, k_soft_ff<true, false>);
     cudaFuncGetAttributes(&fa, k_soft_ff<false, true>);
     cudaFuncGetAttributes(&fa, k_soft_ff<true, true>);
-    cudaFuncGetAttributes(&fa, k_check_sets_soft);
-    cudaFuncGetAttributes(&fa, k_pack_soft);
+    cudaFuncGetAttributes(&fa, k_soft_prep);
     cudaFuncGetAttributes(&fa, k_soft_order);
     cudaFuncGetAttributes(&fa, k_soft_reduce_grad);
     cudaFuncGetAttributes(&fa, k_soft_reduce_loss);
