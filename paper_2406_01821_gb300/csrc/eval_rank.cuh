@@ -57,7 +57,7 @@ __device__ __forceinline__ int count_below(const float *row, float c)
 constexpr int US = T + 1;
 
 // pass rows per warp for pair / product conditions of one chunk
-constexpr int VSLOTS = 12;
+constexpr int VSLOTS = 12, VSLOTS_CAT = 10;
 constexpr uint32_t NOOP_K = 127u * ONES;     // constant - rank never has bit 7 set: never fails
 
 // A staged row offset of the float tile (eval_sparse.cuh).
@@ -68,7 +68,12 @@ __device__ __forceinline__ uint32_t row_off(uint32_t f) { return sparse::row_off
 // each feature's sorted column us[f][pos] = x[f][n] (US floats a row) with pos the rank of x[f][n] (its
 // position in the tile's stable ascending order: a permutation, so every slot is written), and the
 // float rows permuted in place (row_off). One warp per row.
-__device__ __forceinline__ void build_tile_tables(float *xs, unsigned char *rs, uint32_t rev_off, float *us, int F)
+// With code_of (a row number per feature, CODE_NONE for none): the code rows of features that hold
+// category codes only, two words a lane: {nibble v = high three bits of sample v's code, byte v = 1 <<
+// its low three bits}.
+constexpr uint32_t CODE_NONE = 0xFFu;
+__device__ __forceinline__ void build_tile_tables(float *xs, unsigned char *rs, uint32_t rev_off, float *us, int F,
+                                                  const unsigned char *code_of = nullptr, uint2 *codes = nullptr)
 {
     const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
     for (int f = threadIdx.x >> 5; f < F; f += warps) {
@@ -81,6 +86,16 @@ __device__ __forceinline__ void build_tile_tables(float *xs, unsigned char *rs, 
         u[r >> 8 & 0x7Fu] = x.y;
         u[r >> 16 & 0x7Fu] = x.z;
         u[r >> 24] = x.w;
+        if (code_of && code_of[f] != CODE_NONE) {
+            const uint32_t c[4] = {(uint32_t)x.x, (uint32_t)x.y, (uint32_t)x.z, (uint32_t)x.w};
+            uint2 w = make_uint2(0u, 0u);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                w.x |= (c[v] >> 3 & 7u) << (4 * v);
+                w.y |= (1u << (c[v] & 7u)) << (8 * v);
+            }
+            codes[code_of[f] * 32 + lane] = w;
+        }
         __syncwarp();
         row[lane ^ (f & 7)] = x;
     }
@@ -132,13 +147,25 @@ __device__ __forceinline__ uint32_t pass_row(const uint4 *e, const unsigned char
     return __byte_perm(s01, s23, 0x5410);
 }
 
-// Pass row of a membership condition, staged as {row_off of f, -, set bits 0..31, set
+// Pass row of a membership condition, staged as {row_off of f, code row or
+// CODE_NONE, set bits 0..31, set
 // bits 32..63}: 0xFF in byte v where the lane's sample v holds a category code in the set.
 __device__ __forceinline__ uint32_t set_row(uint4 q, const unsigned char *xs, uint32_t lane16)
 {
     const float4 x = *reinterpret_cast<const float4 *>(xs + (q.x ^ lane16));
     return (category_member(x.x, q.z, q.w) ? 0x000000FFu : 0u) | (category_member(x.y, q.z, q.w) ? 0x0000FF00u : 0u) |
            (category_member(x.z, q.z, q.w) ? 0x00FF0000u : 0u) | (category_member(x.w, q.z, q.w) ? 0xFF000000u : 0u);
+}
+
+// The same from the feature's code row: the set's byte that holds a sample's code is picked by its
+// high bits, four samples at once (a byte permute of the set's eight bytes), its bit by its low ones;
+// a byte with that bit set carries into bit 7. Three operations where the floats take about forty.
+__device__ __forceinline__ uint32_t code_row(uint4 q, const uint2 *codes, int lane)
+{
+    const uint2 w = codes[q.y * 32u + lane];
+    uint32_t m;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(m) : "r"(q.z), "r"(q.w), "r"(w.x));
+    return (m & w.y) + 0x7F7F7F7Fu;
 }
 
 // One group of four staged records with end-of-rule flags M (bit u: record u ends its rule).
@@ -211,7 +238,8 @@ __device__ __forceinline__ uint32_t walk_set(uint4 *st, uint32_t *vrow, uint32_t
                                              const uint4 *recs, int rb, int nrec, const float *us,
                                              uint32_t rev_off, int F, int kmine, const unsigned char *rl,
                                              const unsigned char *xs, uint32_t ones_off, const int32_t *yl,
-                                             uint32_t claimed, int deflt, WalkCount &wc, int &more)
+                                             uint32_t claimed, int deflt, WalkCount &wc, int &more,
+                                             const unsigned char *code_of = nullptr, const uint2 *codes = nullptr)
 {
     static_assert(VS <= 16, "pair table and staged records share the warp's 512-byte stage");
     const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
@@ -254,7 +282,7 @@ __device__ __forceinline__ uint32_t walk_set(uint4 *st, uint32_t *vrow, uint32_t
         } else if (CAT && ((sm >> lane) & 1u)) {
             const uint32_t slot = np + __popc(sm & ((1u << lane) - 1u));
             const uint32_t f = min(raw.x & R5_F_MASK, (uint32_t)(F - 1));
-            st[slot] = make_uint4(row_off(f), 0u, raw.z, raw.w);
+            st[slot] = make_uint4(row_off(f), code_of ? code_of[f] : CODE_NONE, raw.z, raw.w);
             sr = make_uint2(vrow_off + 128u * slot, FULL);
         } else if (lane >= cnt || tag == R5_NONE) {
             sr = make_uint2(0u, NOOP_K);
@@ -269,7 +297,10 @@ __device__ __forceinline__ uint32_t walk_set(uint4 *st, uint32_t *vrow, uint32_t
                 vr += 64;
             }
             if (CAT)
-                for (int j = np; j < np + __popc(sm); ++j) vrow[j * 32 + lane] = set_row(st[j], xs, lane16);
+                for (int j = np; j < np + __popc(sm); ++j) {
+                    const uint4 q = st[j];
+                    vrow[j * 32 + lane] = q.y != CODE_NONE ? code_row(q, codes, lane) : set_row(q, xs, lane16);
+                }
         }
         __syncwarp();
         s8[lane] = sr;

@@ -1,5 +1,7 @@
 // Rank-coded batch evaluator (record format v5); the method and the device code are described in
 // eval_rank.cuh.
+#include <algorithm>
+
 #include "rs_internal.cuh"
 #include "eval_rank.cuh"
 #include "tma.cuh"
@@ -28,13 +30,16 @@ __global__ void __launch_bounds__(W * 32, 32 / W) k_hard5(const __grid_constant_
     float *ones = reinterpret_cast<float *>(xs + (size_t)Frows * T * 4);  // [T] of 1.0 (products)
     unsigned char *rs = reinterpret_cast<unsigned char *>(ones + T);  // u8 [Frows][T], then reversed
     uint4 *stage_all = reinterpret_cast<uint4 *>(rs + (size_t)Frows * T * 2);
-    constexpr int VS = VSLOTS;
+    constexpr int VS = CAT ? VSLOTS_CAT : VSLOTS;
     uint32_t *vrows = reinterpret_cast<uint32_t *>(stage_all + W * 32);     // [W][VS][32]
     uint64_t *bar = reinterpret_cast<uint64_t *>(vrows + W * VS * 32);
     int *next = reinterpret_cast<int *>(bar + 1);
     uint32_t *walked = reinterpret_cast<uint32_t *>(bar + 2);        // [W][4] work counters (counting)
     int32_t *place = reinterpret_cast<int32_t *>(walked + 4 * W);    // [T] the caller's sample, or -1 (PRED)
-    float *us = reinterpret_cast<float *>(place + T);                // float [F][US] sorted (built here)
+    // CAT: the code rows [a.code_rows][32] and each feature's row
+    uint2 *codes = reinterpret_cast<uint2 *>(place + T);
+    unsigned char *code_of = reinterpret_cast<unsigned char *>(codes + (CAT ? a.code_rows * 32 : 0));
+    float *us = reinterpret_cast<float *>(code_of + (CAT ? (F + 3) / 4 * 4 : 0));   // float [F][US] sorted (built here)
     const uint4 *recs = reinterpret_cast<const uint4 *>(a.recs);
 
     const TileTask task(a);
@@ -55,6 +60,16 @@ __global__ void __launch_bounds__(W * 32, 32 / W) k_hard5(const __grid_constant_
             tma_load_2d(rs + (size_t)b * Fb * T, &tmr, tile * T, b * Fb, bar);
         }
     }
+    if (CAT && warp == W - 1) {                    // number the features that hold category codes only
+        int n = 0;
+        for (int f0 = 0; f0 < F; f0 += 32) {
+            const bool code = f0 + lane < F && a.flags[f0 + lane] == 0u;
+            const uint32_t b = __ballot_sync(FULL, code);
+            const int row = n + __popc(b & ((1u << lane) - 1u));
+            if (f0 + lane < F) code_of[f0 + lane] = code && row < a.code_rows ? (unsigned char)row : (unsigned char)CODE_NONE;
+            n += __popc(b);
+        }
+    }
     const int32_t *yl = a.y + (int64_t)tile * T + lane * 4;   // n_pad is a multiple of T
     const int64_t t_last = min((int64_t)tile * T + T, a.N) - 1;
     const int kmin = a.y[(int64_t)tile * T], kmax = a.y[t_last];
@@ -68,7 +83,11 @@ __global__ void __launch_bounds__(W * 32, 32 / W) k_hard5(const __grid_constant_
         return;
     }
     const uint32_t rev_off = (uint32_t)Frows * T;
-    build_tile_tables(reinterpret_cast<float *>(xs), rs, rev_off, us, F);
+    if (CAT) {
+        build_tile_tables(reinterpret_cast<float *>(xs), rs, rev_off, us, F, code_of, codes);
+    } else {
+        build_tile_tables(reinterpret_cast<float *>(xs), rs, rev_off, us, F);
+    }
     if (threadIdx.x < T) {
         ones[threadIdx.x] = 1.f;
         const int64_t n = (int64_t)tile * T + threadIdx.x;
@@ -107,7 +126,7 @@ __global__ void __launch_bounds__(W * 32, 32 / W) k_hard5(const __grid_constant_
         uint32_t hit;
         if (PRED) {
             const uint32_t pred = walk_set<false, VS, CAT, true>(st, vr, vr_off, lane, recs, rb, nrec, us, rev_off, F, -2, rl,
-                                                                 xs, ones_off, yl, claimed0, si.deflt, wc, more);
+                                                                 xs, ones_off, yl, claimed0, si.deflt, wc, more, CAT ? code_of : nullptr, codes);
             const int4 to = *reinterpret_cast<const int4 *>(place + 4 * lane);
             int32_t *out = a.preds + (int64_t)p * a.N;
             if (to.x >= 0) out[to.x] = (int32_t)(pred & 0xFFu);
@@ -118,10 +137,10 @@ __global__ void __launch_bounds__(W * 32, 32 / W) k_hard5(const __grid_constant_
             hit = ~(((d & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | d) & HIGH & ~claimed0;
         } else if (uniform) {
             hit = walk_set<true, VS, CAT>(st, vr, vr_off, lane, recs, rb, nrec, us, rev_off, F, kmin, rl, xs, ones_off, yl,
-                                          claimed0, si.deflt, wc, more);
+                                          claimed0, si.deflt, wc, more, CAT ? code_of : nullptr, codes);
         } else {
             hit = walk_set<false, VS, CAT>(st, vr, vr_off, lane, recs, rb, nrec, us, rev_off, F, -2, rl, xs, ones_off, yl,
-                                           claimed0, si.deflt, wc, more);
+                                           claimed0, si.deflt, wc, more, CAT ? code_of : nullptr, codes);
         }
         if (a.walked && lane == 0) {           // the warp's own slots: no atomics
             uint32_t *wk = walked + 4 * warp;
@@ -159,8 +178,18 @@ size_t hard5_smem_bytes(int F, int W)
 template <int W, bool CAT, bool PRED>
 static rs_status launch5_t(Ctx *ctx, Dataset *ds, HardArgs a, cudaStream_t stream)
 {
-    const size_t smem = hard5_smem_bytes(a.F, W);
+    size_t smem = hard5_smem_bytes(a.F, W);
     if (smem > ctx->smem_optin || !ds->ranked) return RS_ERR_TOO_LARGE;
+    if (CAT) {
+        // fewer pass-row slots make room for the code rows: all of them, or as many as keep the CTAs
+        // per SM that the kernel has without them (features beyond them are tested on their floats)
+        const size_t most = 2 * (smem + 1024) <= ctx->smem_optin + 1024 && W == 16 ? (ctx->smem_optin + 1024) / 2 - 1024
+                                                                                 : ctx->smem_optin;
+        smem -= (size_t)W * (VSLOTS - VSLOTS_CAT) * 128;
+        smem += (size_t)(a.F + 3) / 4 * 4;
+        a.code_rows = (int32_t)std::min<size_t>({(size_t)ds->ncode, (size_t)CODE_NONE, (most - smem) / 256});
+        smem += (size_t)a.code_rows * 256;
+    }
     static std::once_flag once;
     static cudaError_t attr_err = cudaSuccess;
     std::call_once(once, [&] {

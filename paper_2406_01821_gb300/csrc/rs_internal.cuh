@@ -332,6 +332,8 @@ struct HardArgs {
     const int32_t *last_end; // [P*K] or null (see PackOut)
     const float *Xt;         // [F][n_pad] (read directly by the global-memory configuration)
     bool cat;                // the records may hold membership tests
+    const uint32_t *flags;   // [F] 0: the feature holds category codes only
+    int32_t code_rows;       // rank-coded form with membership tests: features with a code row
     unsigned long long *walked;  // [4] or null: records, rows, rule ends, (set, tile) walks summed
                                  // over the rank-coded evaluator's walks (work-counting contexts)
 };

@@ -188,3 +188,44 @@ def test_serving(ctx, orc):
         assert e.value.code == -6
     finally:
         ctx.dataset_destroy(dsw)
+
+
+@pytest.mark.parametrize("F,ncat", [(12, 8), (120, 120), (63, 40)])
+def test_code_rows_and_float_rows(orc, F, ncat):
+    """Membership tests on columns of codes 0..63 only (tested by their code rows, as many as fit)
+    beside columns with one value that is no code (a fraction, 64, -1: tested on their floats), in
+    both warp counts of the rank-coded form, with and without predictions."""
+    import torch
+    from paper_2406_01821_gb300 import build, rs
+    build.build()
+    rng = np.random.default_rng(F)
+    N, K = 1500, 3
+    X = rng.standard_normal((N, F)).astype(np.float32)
+    X[:, :ncat] = rng.integers(0, 64, (N, ncat))
+    X[rng.integers(0, N), 0] = 2.5
+    X[rng.integers(0, N), 1] = 64.0
+    X[rng.integers(0, N), 2] = -1.0
+    X[rng.integers(0, N, 20), 3] = -0.0
+    y = rng.integers(0, K, N).astype(np.int32)
+
+    def cond():
+        f = int(rng.integers(0, F))
+        if f < ncat and rng.random() < 0.8:
+            size = int(rng.choice([1, 8, 32, 60, 64]))
+            return (f, -1, synth.IN, 0.0, 0.0, 0.0, [int(k) for k in rng.choice(64, size, replace=False)])
+        return (f, -1, int(rng.integers(0, 2)), 1.0, 0.0, float(rng.choice(X[:, f])))
+
+    sets = [[(int(rng.integers(0, K)), [cond() for _ in range(int(rng.integers(1, 5)))])
+             for _ in range(int(rng.integers(1, 20)))] for _ in range(90)]
+    b = synth.from_lists(sets, rng.integers(0, K, len(sets)).tolist())
+    want = orc.eval_hard(X, y, K, b, want_preds=True)
+    with rs.Context(0) as ctx:
+        ds = ctx.dataset(X, y, K)
+        db = rs.DeviceBatch.from_host(b)
+        for tile in (21, 22):
+            ctx.set_tile_config(tile)
+            for preds in (False, True):
+                got = ctx.eval_hard(ds, db, K, N, preds=preds)
+                torch.cuda.synchronize()
+                for g, w in zip(got, want):
+                    assert g is None or np.array_equal(g.cpu().numpy(), w)
