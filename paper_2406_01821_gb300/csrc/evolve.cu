@@ -103,37 +103,34 @@ __device__ __forceinline__ bool better(const int32_t *fit, int i, int j)
     return fit[i] > fit[j] || (fit[i] == fit[j] && i < j);
 }
 
-// order[rank] = individual; rank = number of individuals ranked before it.
-__global__ void k_rank(const int32_t *fit, int P, int32_t *order)
+// order[rank] = individual; rank = number of individuals ranked before it. A warp ranks RANK_SETS
+// individuals, its lanes striding over all others: 10,000 individuals in 28 us, where a thread per
+// individual on 40 CTAs took 141.
+constexpr int RANK_SETS = 4, RANK_THREADS = 256;
+__global__ void __launch_bounds__(RANK_THREADS) k_rank(const int32_t *fit, int P, int32_t *order)
 {
-    __shared__ int32_t sf[1024];
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int fi = i < P ? fit[i] : 0;
-    int pos = 0;
-    for (int base = 0; base < P; base += 1024) {
-        __syncthreads();
-        for (int j = threadIdx.x; j < 1024 && base + j < P; j += blockDim.x) sf[j] = fit[base + j];
-        __syncthreads();
-        const int lim = min(1024, P - base);
-        if (i < P)
-            for (int j = 0; j < lim; ++j) {
-                const int fj = sf[j];
-                pos += (fj > fi) || (fj == fi && base + j < i);
-            }
+    const int lane = threadIdx.x & 31;
+    const int i0 = (int)((blockIdx.x * RANK_THREADS + threadIdx.x) >> 5) * RANK_SETS;
+    if (i0 >= P) return;
+    int fi[RANK_SETS], pos[RANK_SETS];
+#pragma unroll
+    for (int q = 0; q < RANK_SETS; ++q) {
+        fi[q] = fit[min(i0 + q, P - 1)];
+        pos[q] = 0;
     }
-    if (i < P) order[pos] = i;
-}
-
-__device__ void copy_rule(const PopDev &src, int si, int sr, const PopDev &dst, int di, int dr, int lane, int nl)
-{
-    const int64_t s = (int64_t)si * src.RMAX + sr, d = (int64_t)di * dst.RMAX + dr;
-    if (lane == 0) { dst.rcls[d] = src.rcls[s]; dst.ncond[d] = src.ncond[s]; }
-    for (int k = lane; k < src.CMAX; k += nl) {
-        const int64_t q = s * src.CMAX + k, w = d * dst.CMAX + k;
-        dst.cf[w] = src.cf[q]; dst.cg[w] = src.cg[q]; dst.cop[w] = src.cop[q];
-        dst.ca[w] = src.ca[q]; dst.cb[w] = src.cb[q]; dst.ct[w] = src.ct[q];
+#pragma unroll 4
+    for (int j = lane; j < P; j += 32) {
+        const int fj = fit[j];
+#pragma unroll
+        for (int q = 0; q < RANK_SETS; ++q) pos[q] += (fj > fi[q]) || (fj == fi[q] && j < i0 + q);
+    }
+#pragma unroll
+    for (int q = 0; q < RANK_SETS; ++q) {
+        const int r = __reduce_add_sync(FULL, pos[q]);
+        if (lane == 0 && i0 + q < P) order[r] = i0 + q;
     }
 }
+static unsigned rank_blocks(int P) { return (unsigned)((P + RANK_SETS * RANK_THREADS / 32 - 1) / (RANK_SETS * RANK_THREADS / 32)); }
 
 __device__ void put_cond(const PopDev &p, int64_t rj, int k, const Cond &c)
 {
@@ -147,14 +144,57 @@ __device__ Cond get_cond(const PopDev &p, int64_t rj, int k)
     return Cond{p.cf[q], p.cg[q], p.cop[q], p.ca[q], p.cb[q], p.ct[q]};
 }
 
-// Single-thread mutation of child c in `o` (same operator list and draw order as the reference).
-__device__ void mutate(Rng &r, const PopDev &o, int c, const DataView &d)
+// A child's mutation as drawn before its genome is copied: the operators that move whole rules or
+// conditions (delete a condition, add or delete a rule) are carried out by the warp's copy.
+struct Mutation {
+    int32_t type = -1;         // -1: none
+    int32_t j = -1;            // rule deleted / position of the added rule / rule that loses a condition
+    int32_t k = 0, n = 0;      // condition deleted; conditions of the rule (delete) or of the new rule (add)
+
+    // The rule that rule q of the child is copied from; dead slots keep their contents, as shifting the
+    // copied rules in place would leave them.
+    __device__ __forceinline__ int rule(int q, int nr) const
+    {
+        if (j < 0) return q;
+        if (type == 5) return q > j && q <= nr ? q - 1 : q;
+        if (type == 6) return q >= j && q < nr - 1 ? q + 1 : q;
+        return q;
+    }
+    __device__ __forceinline__ int cond(int q, int kk) const
+    {
+        return type == 4 && q == j && kk >= k && kk < n - 1 ? kk + 1 : kk;
+    }
+};
+
+// The draws of a mutation up to the point where the genome is needed (lane 0; same operator list and
+// draw order as the reference). ncond: the conditions of the child's rule as copied.
+template <class NCond>
+__device__ Mutation draw_mutation(Rng &r, int nr, int RMAX, int CMAX, const NCond &ncond)
 {
-    const int32_t type = r.uniform_int(8);
+    Mutation m;
+    m.type = r.uniform_int(8);
+    if (m.type == 4) {
+        const int j = r.uniform_int(nr);
+        m.n = ncond(j);
+        if (m.n > 1) { m.j = j; m.k = r.uniform_int(m.n); }
+    } else if (m.type == 5) {
+        if (nr < RMAX) {
+            m.j = r.uniform_int(nr + 1);
+            m.n = min(1 + r.uniform_int(3), CMAX);
+        }
+    } else if (m.type == 6) {
+        if (nr > 1) m.j = r.uniform_int(nr);
+    }
+    return m;
+}
+
+// The rest of the mutation of child c in `o`, whose genome has been copied (lane 0).
+__device__ void mutate(Rng &r, const Mutation &m, const PopDev &o, int c, const DataView &d)
+{
     const int64_t base = (int64_t)c * o.RMAX;
-    int32_t nr = o.nrule[c];
+    const int32_t nr = o.nrule[c];
     int32_t j, k;
-    switch (type) {
+    switch (m.type) {
     case 0: {
         j = r.uniform_int(nr); k = r.uniform_int(o.ncond[base + j]);
         Cond x = get_cond(o, base + j, k);
@@ -194,46 +234,24 @@ __device__ void mutate(Rng &r, const PopDev &o, int c, const DataView &d)
         break;
     }
     case 4: {
-        j = r.uniform_int(nr);
-        const int32_t n = o.ncond[base + j];
-        if (n > 1) {
-            k = r.uniform_int(n);
-            for (int q = k; q + 1 < n; ++q) put_cond(o, base + j, q, get_cond(o, base + j, q + 1));
-            o.ncond[base + j] = n - 1;
-        }
+        if (m.j >= 0) o.ncond[base + m.j] = m.n - 1;
         break;
     }
     case 5: {
-        if (nr < o.RMAX) {
-            const int32_t pos = r.uniform_int(nr + 1);
-            int32_t n = 1 + r.uniform_int(3);
-            if (n > o.CMAX) n = o.CMAX;
-            for (int q = nr; q > pos; --q) {
-                o.rcls[base + q] = o.rcls[base + q - 1];
-                o.ncond[base + q] = o.ncond[base + q - 1];
-                for (int kk = 0; kk < o.CMAX; ++kk) put_cond(o, base + q, kk, get_cond(o, base + q - 1, kk));
-            }
-            o.ncond[base + pos] = n;
-            for (int q = 0; q < n; ++q) {
+        if (m.j >= 0) {
+            o.ncond[base + m.j] = m.n;
+            for (int q = 0; q < m.n; ++q) {
                 Cond x;
                 random_condition(r, d, x);
-                put_cond(o, base + pos, q, x);
+                put_cond(o, base + m.j, q, x);
             }
-            o.rcls[base + pos] = r.uniform_int(d.K);
+            o.rcls[base + m.j] = r.uniform_int(d.K);
             o.nrule[c] = nr + 1;
         }
         break;
     }
     case 6: {
-        if (nr > 1) {
-            j = r.uniform_int(nr);
-            for (int q = j; q + 1 < nr; ++q) {
-                o.rcls[base + q] = o.rcls[base + q + 1];
-                o.ncond[base + q] = o.ncond[base + q + 1];
-                for (int kk = 0; kk < o.CMAX; ++kk) put_cond(o, base + q, kk, get_cond(o, base + q + 1, kk));
-            }
-            o.nrule[c] = nr - 1;
-        }
+        if (m.j >= 0) o.nrule[c] = nr - 1;
         break;
     }
     default: {
@@ -244,7 +262,9 @@ __device__ void mutate(Rng &r, const PopDev &o, int c, const DataView &d)
     }
 }
 
-// One warp per child: copies in parallel, random decisions on lane 0.
+// One warp per child: copies in parallel, random decisions on lane 0. 10,000 children of 32 x 6 slots
+// took 150 us when rules were copied one by one and lane 0 shifted them for an added or deleted rule
+// (a load and a store after another for every slot behind it); 60 us so.
 // gen = gen0 + *gidx: the generation index is read on the device, so that one captured graph
 // serves every generation.
 constexpr int NEXT_GEN_THREADS = 256;   // k_next_generation's block: 8 warps, one child each
@@ -291,16 +311,36 @@ __global__ void __launch_bounds__(NEXT_GEN_THREADS) k_next_generation(PopDev in,
     A = __shfl_sync(FULL, A, 0);
     B = __shfl_sync(FULL, B, 0);
     take_b = __shfl_sync(FULL, take_b, 0);
-    if (lane == 0) { out.nrule[c] = in.nrule[A]; out.deflt[c] = in.deflt[A]; }
-    for (int q = 0; q < in.RMAX; ++q) {
-        const bool fromb = (take_b >> q) & 1u;
-        copy_rule(in, fromb ? B : A, q, out, c, q, lane, 32);
+    const int nr = in.nrule[A];
+    Mutation m;
+    if (c >= elite && lane == 0 && r.uniform01() < 0.9f)
+        m = draw_mutation(r, nr, in.RMAX, in.CMAX,
+                          [&](int q) { return in.ncond[(int64_t)((take_b >> q) & 1u ? B : A) * in.RMAX + q]; });
+    m.type = __shfl_sync(FULL, m.type, 0);
+    m.j = __shfl_sync(FULL, m.j, 0);
+    m.k = __shfl_sync(FULL, m.k, 0);
+    m.n = __shfl_sync(FULL, m.n, 0);
+    // the copy: lane by lane over the set's slots, each from the parent its rule came from
+    if (lane == 0) { out.nrule[c] = nr; out.deflt[c] = in.deflt[A]; }
+    const auto parent_rule = [&](int q) {
+        const int p = m.rule(q, nr);
+        return (int64_t)((take_b >> p) & 1u ? B : A) * in.RMAX + p;
+    };
+    if (lane < in.RMAX) {
+        const int64_t src = parent_rule(lane), dst = (int64_t)c * in.RMAX + lane;
+        out.rcls[dst] = in.rcls[src];
+        out.ncond[dst] = in.ncond[src];
+    }
+    const int slots = in.RMAX * in.CMAX;
+    for (int i = lane; i < slots; i += 32) {
+        const int q = i / in.CMAX;
+        const int64_t src = parent_rule(q) * in.CMAX + m.cond(q, i - q * in.CMAX), dst = (int64_t)c * slots + i;
+        out.cf[dst] = in.cf[src]; out.cg[dst] = in.cg[src]; out.cop[dst] = in.cop[src];
+        out.ca[dst] = in.ca[src]; out.cb[dst] = in.cb[src]; out.ct[dst] = in.ct[src];
     }
     __syncwarp();
-    if (c >= elite && lane == 0) {
-        // continue the child's draw sequence (the warp-wide copy did not draw)
-        if (r.uniform01() < 0.9f) mutate(r, out, c, d);
-    }
+    // the child's draw sequence goes on (the warp-wide copy did not draw)
+    if (lane == 0 && m.type >= 0) mutate(r, m, out, c, d);
 }
 
 // ---------------------------------------------------------------- slots -> CSR
@@ -673,7 +713,7 @@ rs_status evolve_run(Ctx *ctx, uint64_t ds_h, const rs_evolve_config *cfg, rs_po
         count_launch(ctx, build_csr(in, nullptr, P, w, st));
         if ((grc = evaluate(P, fit, st))) return grc;
         if (tune) {
-            k_rank<<<(P + 255) / 256, 256, 0, st>>>(fit, P, order);
+            k_rank<<<rank_blocks(P), RANK_THREADS, 0, st>>>(fit, P, order);
             count_launch(ctx, 1 + build_csr(in, order, T, w, st));   // the T best, in rank order
             RS_CUDA(cudaMemcpyAsync(ta, w.o.cond_a, 4 * TC, cudaMemcpyDeviceToDevice, st));
             RS_CUDA(cudaMemcpyAsync(tb, w.o.cond_b, 4 * TC, cudaMemcpyDeviceToDevice, st));
@@ -719,7 +759,7 @@ rs_status evolve_run(Ctx *ctx, uint64_t ds_h, const rs_evolve_config *cfg, rs_po
             k_stats<<<1, 1024, 0, st>>>(fit, P, best, mean, gslot + par, last ? nullptr : gslot + (par ^ 1));
             count_launch(ctx);
             if (last) return RS_OK;
-            k_rank<<<(P + 255) / 256, 256, 0, st>>>(fit, P, order);
+            k_rank<<<rank_blocks(P), RANK_THREADS, 0, st>>>(fit, P, order);
             count_launch(ctx);
         }
         k_next_generation<<<(P * 32 + NEXT_GEN_THREADS - 1) / NEXT_GEN_THREADS, NEXT_GEN_THREADS, 0, st>>>(
