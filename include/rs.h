@@ -100,7 +100,7 @@ rs_status rs_check(rs_ctx *ctx, void *stream);
  *   N >= 1, 1 <= F <= RS_MAX_FEATURES, 1 <= K <= RS_MAX_CLASSES
  * The library keeps its own copy (feature-major, samples grouped by label); the caller may free X
  * and y when the call returns. Device memory held: 4 bytes per value and 12 per sample (labels,
- * order), N rounded up to 256, plus for finite data with F <= 160 one byte per value (the rank of
+ * order), N rounded up to 256, plus for finite data with F <= 128 one byte per value (the rank of
  * each value within its 128-sample tile, for the rank-coded evaluator).
  * Errors: RS_ERR_INVALID (sizes, a label out of range), RS_ERR_OOM.
  * On success *ds_out receives a non-zero handle.
@@ -408,9 +408,10 @@ rs_status rs_tile_config_info(int32_t id, int32_t *samples_per_tile, int32_t *wa
                               int32_t *samples_per_lane);
 /* Evaluator form of configuration `id`: 1 condition at a time; 2 rule at a time; 3 rule at a
  * time with the margin minimum; 4 sign-mask conjunction (finite datasets, else runs as 3);
- * 5 rank-coded cuts (datasets with rank tables: finite and at most 160 features; else runs as
- * 4, then 3). Form 4 produces counts only, form 5 predictions too for up to 256 classes: other
- * calls that ask for predictions run as 3.
+ * 5 rank-coded cuts (finite datasets of at most 128 features, 63 with 16 warps; on other finite
+ * datasets of at most 256 features the same walk on the features themselves; else runs as 4,
+ * then 3). Form 4 produces counts only, form 5 predictions too for up to 256 classes: other calls
+ * that ask for predictions run as 3.
  * The other configurations stage a feature tile in shared memory and need F small enough for
  * it; configuration 23 (form 1) reads the features from global memory and takes any F. */
 rs_status rs_tile_config_form(int32_t id, int32_t *form);

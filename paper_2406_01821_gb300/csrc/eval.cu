@@ -114,22 +114,22 @@ static std::string tune_key(const Dataset &ds, const rs_batch *b)
 
 static int heuristic_tile(const Dataset &ds, int P, bool cat)
 {
-    // Datasets with rank tables: the rank-coded evaluator. Two CTAs of 16 warps where both fit an SM
-    // (up to 63 features): one stages its tile while the other walks (46 sets on 470,000 x 30: 201 us
-    // against 256 with one CTA of 32 warps; 800 sets: 1859 and 1873). Wider: one CTA of 32 warps,
-    // or of 16 where the tables leave no room for 32 (129 < F < 155: 800 sets on 100,000 x 150, 721 us
-    // against 760 with the sign-mask form). A few sets cannot pay for the tables of wide tiles: up
-    // to 32, the sign-mask form in small CTAs (16 sets on 470,000 x 106: 190 us against 257; at 46 sets
-    // 306 and 296).
-    if (ds.ranked) {
-        const size_t s16 = hard5_smem_bytes(ds.F, 16), s32 = hard5_smem_bytes(ds.F, 32), most = 227 * 1024;
-        if (2 * (s16 + 1024) <= most + 1024) return 21;
-        if (P <= 32 && !cat && tile_config_fits(tile_config(16), ds.F)) return 16;
-        if (s32 <= most) return 22;
-        if (s16 <= most) return 21;
+    // Finite data of at most 256 features: the rank-coded walk where 32 warps find room for its tables
+    // (up to 128 features), else the direct walk. Two CTAs of 16 warps where both fit an SM: one stages
+    // its tile while the other walks. The rank-coded walk in two CTAs (up to 63 features) is the faster
+    // for few sets and as fast for many (46 sets on 470,000 x 30: 201 us against 256 with one CTA of 32
+    // warps; 800 sets: 1859 and 1873). On wider data two CTAs only hold the direct walk (up to 157
+    // features), which pays as long as building the tables would weigh more than walking faster with
+    // them: 46 sets on 470,000 x 106, 236 us against 280; 64: 282 and 306; 100: 398 and 386.
+    // Membership tests keep the rank-coded walk, whose code rows test them.
+    if (ds.finite && direct_smem_bytes(ds.F, 32) <= 227 * 1024) {
+        if (ds.ranked && rank_tables_fit(ds.F, 16)) return 21;
+        const bool two = 2 * (direct_smem_bytes(ds.F, 16) + 1024) <= 228 * 1024;
+        return two && P <= 64 && !(cat && ds.ranked && rank_tables_fit(ds.F, 32)) ? 21 : 22;
     }
-    // Else the 32-warp sign-mask form (margin-minimum form on non-finite data), then smaller tiles for
-    // wide data, and for data too wide for any shared tile the configuration reading global memory.
+    // Else the 32-warp margin-minimum form on non-finite data, then smaller tiles for wide data (the
+    // sign-mask form where it is finite), and for data too wide for any shared tile the configuration
+    // reading global memory.
     static const int prefs[] = {22, 21, 18, 16, 20, 3, 5, 23};
     for (int id : prefs)
         if (tile_config_fits(tile_config(id), ds.F)) return id;
@@ -271,7 +271,7 @@ rs_status enqueue_hard(Ctx *ctx, Dataset *ds, const TileConfig &tc_in, const Bat
     // batches with membership conditions run the forms that evaluate them (rank-coded or v1)
     const TileConfig &tc = bd.cond_set ? categorical_config(tc_in, *ds, preds != nullptr) : tc_in;
     const int ver = effective_version(tc, *ds, preds != nullptr);
-    const int pack_ver = ver == 5 ? 5 : (ver == 4 ? 4 : (ver >= 2 ? 2 : 1));
+    const int pack_ver = ver >= 5 ? 5 : (ver == 4 ? 4 : (ver >= 2 ? 2 : 1));
     count_launch(ctx, launch_pack(bd, ds->F, ds->K, tc.S(), pack_ver, po, stream));
     RS_CUDA(cudaGetLastError());
     HardArgs a{};

@@ -110,6 +110,35 @@ __device__ __forceinline__ uint2 stage_cut(uint4 r, const float *us, uint32_t re
     return make_uint2((le ? rev_off : 0u) + f * T, (uint32_t)(le ? 255 - L : L + 127) * ONES);
 }
 
+// The direct walk (finite datasets without rank tables: more than RANK_MAX_F features, or tables that
+// do not fit) takes the same records in the same chunks, but tests a cut on the float row: with s =
+// +-1 the sign of s x + n is set exactly where the cut fails,
+//     '>':  x - c' < 0, c' the float above c        (s = 1,  n = -c')
+//     '<=': c - x < 0                               (s = -1, n = c)
+// for finite x (a difference of equal floats is +0; n = -0 is made +0), one fused multiply-add a sample,
+// and the four signs are gathered into one word. No search, no tables: 12 instructions and a 512-byte
+// row read a cut against 7 and a 128-byte one, so the rank-coded walk stays the faster where it fits
+// (600 sets on 150,001 samples: 1.34 ms at F = 128, the direct walk 1.59 at F = 233, where the sign-mask
+// form takes 1.95). Staged: {row_off of f | le, n}.
+__device__ __forceinline__ uint2 stage_cut_direct(uint4 r, int F)
+{
+    const uint32_t f = min(r.x & R5_F_MASK, (uint32_t)(F - 1));
+    const bool le = (r.x >> R5_TAG_SHIFT) == R5_CUT_LT;
+    const float c = __uint_as_float(r.z);
+    const float n = (le ? c : -nextafterf(c, __uint_as_float(0x7F800000u))) + 0.f;
+    return make_uint2(row_off(f) | (le ? 1u : 0u), __float_as_uint(n));
+}
+
+__device__ __forceinline__ uint32_t cut_word(uint32_t off, uint32_t n, const unsigned char *xs, uint32_t lane16)
+{
+    const float4 x = *reinterpret_cast<const float4 *>(xs + ((off & ~15u) ^ lane16));
+    const float s = __uint_as_float(0x3F800000u | off << 31), b = __uint_as_float(n);
+    const float d0 = __fmaf_rn(s, x.x, b), d1 = __fmaf_rn(s, x.y, b), d2 = __fmaf_rn(s, x.z, b), d3 = __fmaf_rn(s, x.w, b);
+    const uint32_t s01 = __byte_perm(__float_as_uint(d0), __float_as_uint(d1), 0x0073);
+    const uint32_t s23 = __byte_perm(__float_as_uint(d2), __float_as_uint(d3), 0x0073);
+    return __byte_perm(s01, s23, 0x5410);
+}
+
 // Bit 7 of byte v where the lane's sample v (labels yl[0..3]) has label k. Only tiles that hold
 // more than one label need it, so the labels are read again instead of kept in registers.
 __device__ __forceinline__ uint32_t class_bytes(const int32_t *yl, int k)
@@ -233,7 +262,8 @@ struct Decode5 {
 };
 
 // Returns the hit bits; `more` receives the lane's hits of the sparse tail that are not in them.
-template <bool UNI, int VS, bool CAT, bool PRED = false>
+// DIRECT: the direct walk (us, rl and rev_off unused, vrow_off relative to xs).
+template <bool UNI, int VS, bool CAT, bool PRED = false, bool DIRECT = false>
 __device__ __forceinline__ uint32_t walk_set(uint4 *st, uint32_t *vrow, uint32_t vrow_off, int lane,
                                              const uint4 *recs, int rb, int nrec, const float *us,
                                              uint32_t rev_off, int F, int kmine, const unsigned char *rl,
@@ -271,7 +301,7 @@ __device__ __forceinline__ uint32_t walk_set(uint4 *st, uint32_t *vrow, uint32_t
         // A pair or product condition gets a pass-row slot and a pair-table entry.
         const uint32_t cls = (raw.x >> R5_CLS_SHIFT) & 0xFFFu;
         const uint32_t ew = PRED ? cls * ONES : (UNI ? ((int)cls == kmine ? 0xFFFFFFFFu : 0u) : cls);
-        uint2 sr = stage_cut(raw, us, rev_off, F);
+        uint2 sr = DIRECT ? stage_cut_direct(raw, F) : stage_cut(raw, us, rev_off, F);
         const int np = __popc(pm);
         if ((pm >> lane) & 1u) {
             const uint32_t slot = __popc(pm & ((1u << lane) - 1u));
@@ -285,7 +315,7 @@ __device__ __forceinline__ uint32_t walk_set(uint4 *st, uint32_t *vrow, uint32_t
             st[slot] = make_uint4(row_off(f), code_of ? code_of[f] : CODE_NONE, raw.z, raw.w);
             sr = make_uint2(vrow_off + 128u * slot, FULL);
         } else if (lane >= cnt || tag == R5_NONE) {
-            sr = make_uint2(0u, NOOP_K);
+            sr = DIRECT ? make_uint2(0u, 0x7F800000u) : make_uint2(0u, NOOP_K);     // +inf: never fails
         }
         __syncwarp();
         {                                             // pass rows, one warp-wide evaluation each
@@ -310,11 +340,21 @@ __device__ __forceinline__ uint32_t walk_set(uint4 *st, uint32_t *vrow, uint32_t
         for (int g = 0; g < cnt; g += 4) {
             const uint4 ra = *reinterpret_cast<const uint4 *>(s8 + g);
             const uint4 rc = *reinterpret_cast<const uint4 *>(s8 + g + 2);
-            const uint32_t e0 = ra.y - *reinterpret_cast<const uint32_t *>(rl + ra.x);
-            const uint32_t e1 = ra.w - *reinterpret_cast<const uint32_t *>(rl + ra.z);
-            const uint32_t e2 = rc.y - *reinterpret_cast<const uint32_t *>(rl + rc.x);
-            const uint32_t e3 = rc.w - *reinterpret_cast<const uint32_t *>(rl + rc.z);
-            const uint32_t e[4] = {e0, e1, e2, e3};
+            uint32_t e[4];
+            if (DIRECT) {
+                const uint32_t rows = (pm | sm) >> g;
+                const uint32_t off[4] = {ra.x, ra.z, rc.x, rc.z}, val[4] = {ra.y, ra.w, rc.y, rc.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (rows & (1u << u)) e[u] = ~*reinterpret_cast<const uint32_t *>(xs + off[u] + 4 * lane);
+                    else e[u] = cut_word(off[u], val[u], xs, lane16);
+                }
+            } else {
+                e[0] = ra.y - *reinterpret_cast<const uint32_t *>(rl + ra.x);
+                e[1] = ra.w - *reinterpret_cast<const uint32_t *>(rl + ra.z);
+                e[2] = rc.y - *reinterpret_cast<const uint32_t *>(rl + rc.x);
+                e[3] = rc.w - *reinterpret_cast<const uint32_t *>(rl + rc.z);
+            }
             const uint32_t *swg = sw + g;
             switch ((ends >> g) & 0xFu) {
 #define RS_GROUP4(M) case M: group4<M, UNI, PRED>(e, swg, yl, fail, claimed, hit); break;

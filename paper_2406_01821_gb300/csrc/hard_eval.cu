@@ -277,14 +277,25 @@ constexpr int kNumConfigs = sizeof(kConfigs) / sizeof(kConfigs[0]);
 
 int tile_config_count() { return kNumConfigs; }
 
+// Whether 32 warps of the rank-coded form find room on an SM with their tables: one CTA of 32 or two of
+// 16 (one CTA of 16 warps alone is slower than the direct walk).
+bool rank_tables_fit(int F, int W)
+{
+    const size_t s = hard5_smem_bytes(F, W);
+    return W >= 32 ? s <= 227 * 1024 : 2 * (s + 1024) <= 228 * 1024;
+}
+
+// The form a configuration runs as: its own, or DIRECT_VERSION (rank-coded configurations on finite
+// datasets whose rank tables do not exist or do not fit), 4 (neither fits), 3 (non-finite data).
 int effective_version(const TileConfig &tc, const Dataset &ds, bool preds)
 {
     if (tc.ver >= 4 && !ds.finite) return 3;              // same V and W exist for version 3
-    const bool ranked = tc.ver == 5 && ds.ranked && hard5_smem_bytes(ds.F, tc.W) <= 227 * 1024;
-    // the rank-coded form writes predictions as bytes; the sign-mask form writes none
-    if (tc.ver >= 4 && preds && !(ranked && ds.K <= 256)) return 3;
-    if (tc.ver == 5 && !ranked) return 4;
-    return tc.ver;
+    int ver = tc.ver;
+    if (ver == 5 && !(ds.ranked && rank_tables_fit(ds.F, tc.W)))
+        ver = direct_smem_bytes(ds.F, tc.W) <= 227 * 1024 ? DIRECT_VERSION : 4;
+    // these walks write predictions as bytes; the sign-mask form writes none
+    if (preds && (ver == 4 || (ver >= 5 && ds.K > 256))) return 3;
+    return ver;
 }
 
 const TileConfig &tile_config(int id) { return kConfigs[id]; }
@@ -293,7 +304,7 @@ const TileConfig &tile_config(int id) { return kConfigs[id]; }
 // another form is replaced by the first v1 configuration that fits the dataset.
 const TileConfig &categorical_config(const TileConfig &tc, const Dataset &ds, bool preds)
 {
-    if (tc.ver == 1 || effective_version(tc, ds, preds) == 5) return tc;
+    if (tc.ver == 1 || effective_version(tc, ds, preds) >= 5) return tc;
     for (int id : {0, 5, 23})
         if (tile_config_fits(kConfigs[id], ds.F)) return kConfigs[id];
     return kConfigs[23];
@@ -315,7 +326,7 @@ rs_status launch_hard(Ctx *ctx, Dataset *ds, const TileConfig &tc, const HardArg
     // correct and per_class were zeroed by the packing (k_pack_sets), which every call runs first
     if (a.P == 0) return RS_OK;
     const int ver = effective_version(tc, *ds, a.preds != nullptr);
-    if (ver == 5) return launch_hard5(ctx, ds, tc.W, a, stream);
+    if (ver >= 5) return launch_hard5(ctx, ds, tc.W, ver == DIRECT_VERSION, a, stream);
     if (ver == 4) return launch_hard4(ctx, ds, tc.V, tc.W, a, stream);
     if (ver >= 2) return launch_hard2(ctx, ds, tc.V, tc.W, ver == 3, a, stream);
     switch (tc.id) {

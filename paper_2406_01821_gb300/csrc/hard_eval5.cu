@@ -3,6 +3,7 @@
 #include <algorithm>
 
 #include "rs_internal.cuh"
+#include "eval_core.cuh"
 #include "eval_rank.cuh"
 #include "tma.cuh"
 
@@ -17,7 +18,8 @@ constexpr uint64_t TMA_WAIT_LIMIT_NS = 2000000000ull;
 // four scattered 4-byte stores a lane, which L2 gathers (the store adds 10 to 20 us to 200 sets on
 // 100,000 samples). The predicted classes of a lane's samples are the bytes of one word; the walk has
 // no class-tail stop, and hits are the bytes equal to the label's.
-template <int W, bool CAT, bool PRED>
+// DIRECT: the direct walk on datasets without rank tables (tmr unused).
+template <int W, bool CAT, bool PRED, bool DIRECT>
 __global__ void __launch_bounds__(W * 32, 32 / W) k_hard5(const __grid_constant__ CUtensorMap tmx,
                                                   const __grid_constant__ CUtensorMap tmr, HardArgs a)
 {
@@ -29,7 +31,7 @@ __global__ void __launch_bounds__(W * 32, 32 / W) k_hard5(const __grid_constant_
     unsigned char *xs = smem;                                         // float [Frows][T]
     float *ones = reinterpret_cast<float *>(xs + (size_t)Frows * T * 4);  // [T] of 1.0 (products)
     unsigned char *rs = reinterpret_cast<unsigned char *>(ones + T);  // u8 [Frows][T], then reversed
-    uint4 *stage_all = reinterpret_cast<uint4 *>(rs + (size_t)Frows * T * 2);
+    uint4 *stage_all = reinterpret_cast<uint4 *>(rs + (DIRECT ? 0 : (size_t)Frows * T * 2));
     constexpr int VS = CAT ? VSLOTS_CAT : VSLOTS;
     uint32_t *vrows = reinterpret_cast<uint32_t *>(stage_all + W * 32);     // [W][VS][32]
     uint64_t *bar = reinterpret_cast<uint64_t *>(vrows + W * VS * 32);
@@ -37,7 +39,7 @@ __global__ void __launch_bounds__(W * 32, 32 / W) k_hard5(const __grid_constant_
     uint32_t *walked = reinterpret_cast<uint32_t *>(bar + 2);        // [W][4] work counters (counting)
     int32_t *place = reinterpret_cast<int32_t *>(walked + 4 * W);    // [T] the caller's sample, or -1 (PRED)
     // CAT: the code rows [a.code_rows][32] and each feature's row
-    uint2 *codes = reinterpret_cast<uint2 *>(place + T);
+    uint2 *codes = reinterpret_cast<uint2 *>(place + T);       // (rank-coded form)
     unsigned char *code_of = reinterpret_cast<unsigned char *>(codes + (CAT ? a.code_rows * 32 : 0));
     float *us = reinterpret_cast<float *>(code_of + (CAT ? (F + 3) / 4 * 4 : 0));   // float [F][US] sorted (built here)
     const uint4 *recs = reinterpret_cast<const uint4 *>(a.recs);
@@ -54,13 +56,13 @@ __global__ void __launch_bounds__(W * 32, 32 / W) k_hard5(const __grid_constant_
     if (threadIdx.x < 4 * W) walked[threadIdx.x] = 0;
     __syncthreads();
     if (threadIdx.x == 0) {
-        mbar_arrive_expect_tx(bar, (uint32_t)Frows * T * 5u);
+        mbar_arrive_expect_tx(bar, (uint32_t)Frows * T * (DIRECT ? 4u : 5u));
         for (int b = 0; b < nbox; ++b) {
             tma_load_2d(xs + (size_t)b * Fb * T * 4, &tmx, tile * T, b * Fb, bar);
-            tma_load_2d(rs + (size_t)b * Fb * T, &tmr, tile * T, b * Fb, bar);
+            if (!DIRECT) tma_load_2d(rs + (size_t)b * Fb * T, &tmr, tile * T, b * Fb, bar);
         }
     }
-    if (CAT && warp == W - 1) {                    // number the features that hold category codes only
+    if (CAT && !DIRECT && warp == W - 1) {         // number the features that hold category codes only
         int n = 0;
         for (int f0 = 0; f0 < F; f0 += 32) {
             const bool code = f0 + lane < F && a.flags[f0 + lane] == 0u;
@@ -83,7 +85,9 @@ __global__ void __launch_bounds__(W * 32, 32 / W) k_hard5(const __grid_constant_
         return;
     }
     const uint32_t rev_off = (uint32_t)Frows * T;
-    if (CAT) {
+    if (DIRECT) {
+        core::permute_rows<4>(reinterpret_cast<float *>(xs), F);
+    } else if (CAT) {
         build_tile_tables(reinterpret_cast<float *>(xs), rs, rev_off, us, F, code_of, codes);
     } else {
         build_tile_tables(reinterpret_cast<float *>(xs), rs, rev_off, us, F);
@@ -120,13 +124,13 @@ __global__ void __launch_bounds__(W * 32, 32 / W) k_hard5(const __grid_constant_
                              : si.rec_end - si.rec_begin;
 
         uint32_t *vr = vrows + warp * VS * 32;
-        const uint32_t vr_off = (uint32_t)(reinterpret_cast<unsigned char *>(vr) - rs);
+        const uint32_t vr_off = (uint32_t)(reinterpret_cast<unsigned char *>(vr) - (DIRECT ? xs : rs));
         WalkCount wc;
         int more;
         uint32_t hit;
         if (PRED) {
-            const uint32_t pred = walk_set<false, VS, CAT, true>(st, vr, vr_off, lane, recs, rb, nrec, us, rev_off, F, -2, rl,
-                                                                 xs, ones_off, yl, claimed0, si.deflt, wc, more, CAT ? code_of : nullptr, codes);
+            const uint32_t pred = walk_set<false, VS, CAT, true, DIRECT>(st, vr, vr_off, lane, recs, rb, nrec, us, rev_off, F, -2, rl,
+                                                                 xs, ones_off, yl, claimed0, si.deflt, wc, more, CAT && !DIRECT ? code_of : nullptr, codes);
             const int4 to = *reinterpret_cast<const int4 *>(place + 4 * lane);
             int32_t *out = a.preds + (int64_t)p * a.N;
             if (to.x >= 0) out[to.x] = (int32_t)(pred & 0xFFu);
@@ -136,11 +140,11 @@ __global__ void __launch_bounds__(W * 32, 32 / W) k_hard5(const __grid_constant_
             const uint32_t d = pred ^ label4;      // a byte of 0: a hit
             hit = ~(((d & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | d) & HIGH & ~claimed0;
         } else if (uniform) {
-            hit = walk_set<true, VS, CAT>(st, vr, vr_off, lane, recs, rb, nrec, us, rev_off, F, kmin, rl, xs, ones_off, yl,
-                                          claimed0, si.deflt, wc, more, CAT ? code_of : nullptr, codes);
+            hit = walk_set<true, VS, CAT, false, DIRECT>(st, vr, vr_off, lane, recs, rb, nrec, us, rev_off, F, kmin, rl, xs, ones_off, yl,
+                                          claimed0, si.deflt, wc, more, CAT && !DIRECT ? code_of : nullptr, codes);
         } else {
-            hit = walk_set<false, VS, CAT>(st, vr, vr_off, lane, recs, rb, nrec, us, rev_off, F, -2, rl, xs, ones_off, yl,
-                                           claimed0, si.deflt, wc, more, CAT ? code_of : nullptr, codes);
+            hit = walk_set<false, VS, CAT, false, DIRECT>(st, vr, vr_off, lane, recs, rb, nrec, us, rev_off, F, -2, rl, xs, ones_off, yl,
+                                           claimed0, si.deflt, wc, more, CAT && !DIRECT ? code_of : nullptr, codes);
         }
         if (a.walked && lane == 0) {           // the warp's own slots: no atomics
             uint32_t *wk = walked + 4 * warp;
@@ -167,20 +171,31 @@ __global__ void __launch_bounds__(W * 32, 32 / W) k_hard5(const __grid_constant_
 
 }  // namespace
 
-size_t hard5_smem_bytes(int F, int W)
+// Shared memory but for the tables: stages, pass rows, the ones row, the barrier, counters and places.
+static size_t hard5_fixed_bytes(int W)
 {
-    const int Fb = F < 256 ? F : 256;
-    const size_t Frows = (size_t)((F + Fb - 1) / Fb) * Fb;
-    const size_t vs = VSLOTS;
-    return Frows * T * (4 + 2) + (size_t)F * US * 4 + (size_t)W * 32 * 16 + (size_t)W * vs * 32 * 4 + T * 4 + 16 + (size_t)W * 16 + T * 4;
+    return (size_t)W * 32 * 16 + (size_t)W * VSLOTS * 32 * 4 + T * 4 + 16 + (size_t)W * 16 + T * 4;
 }
 
-template <int W, bool CAT, bool PRED>
+static size_t tma_rows(int F)
+{
+    const int Fb = F < 256 ? F : 256;
+    return (size_t)((F + Fb - 1) / Fb) * Fb;
+}
+
+size_t hard5_smem_bytes(int F, int W)
+{
+    return tma_rows(F) * T * (4 + 2) + (size_t)F * US * 4 + hard5_fixed_bytes(W);
+}
+
+size_t direct_smem_bytes(int F, int W) { return tma_rows(F) * T * 4 + hard5_fixed_bytes(W); }
+
+template <int W, bool CAT, bool PRED, bool DIRECT>
 static rs_status launch5_t(Ctx *ctx, Dataset *ds, HardArgs a, cudaStream_t stream)
 {
-    size_t smem = hard5_smem_bytes(a.F, W);
-    if (smem > ctx->smem_optin || !ds->ranked) return RS_ERR_TOO_LARGE;
-    if (CAT) {
+    size_t smem = DIRECT ? direct_smem_bytes(a.F, W) : hard5_smem_bytes(a.F, W);
+    if (smem > ctx->smem_optin || !(DIRECT ? ds->finite : ds->ranked)) return RS_ERR_TOO_LARGE;
+    if (CAT && !DIRECT) {
         // fewer pass-row slots make room for the code rows: all of them, or as many as keep the CTAs
         // per SM that the kernel has without them (features beyond them are tested on their floats)
         const size_t most = 2 * (smem + 1024) <= ctx->smem_optin + 1024 && W == 16 ? (ctx->smem_optin + 1024) / 2 - 1024
@@ -193,34 +208,39 @@ static rs_status launch5_t(Ctx *ctx, Dataset *ds, HardArgs a, cudaStream_t strea
     static std::once_flag once;
     static cudaError_t attr_err = cudaSuccess;
     std::call_once(once, [&] {
-        attr_err = cudaFuncSetAttribute(k_hard5<W, CAT, PRED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        attr_err = cudaFuncSetAttribute(k_hard5<W, CAT, PRED, DIRECT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)ctx->smem_optin);
     });
     if (attr_err != cudaSuccess) return cuda_fail(attr_err, "cudaFuncSetAttribute(k_hard5)");
     const CUtensorMap *tmx = dataset_tmap(ds, T);
-    const CUtensorMap *tmr = dataset_rank_tmap(ds);
+    const CUtensorMap *tmr = DIRECT ? tmx : dataset_rank_tmap(ds);
     if (!tmx || !tmr) return RS_ERR_DEVICE;
     int resident = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, k_hard5<W, CAT, PRED>, W * 32, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, k_hard5<W, CAT, PRED, DIRECT>, W * 32, smem);
     const int grid = split_tiles(ctx, a.N, a.F, a.P, T, W, resident, a);
     {
         TimedLaunch tl(ctx, TK_HARD, stream);
-        k_hard5<W, CAT, PRED><<<grid, W * 32, smem, stream>>>(*tmx, *tmr, a);
+        k_hard5<W, CAT, PRED, DIRECT><<<grid, W * 32, smem, stream>>>(*tmx, *tmr, a);
     }
     RS_CUDA(cudaGetLastError());
     count_launch(ctx);
     return RS_OK;
 }
 
-rs_status launch_hard5(Ctx *ctx, Dataset *ds, int W, const HardArgs &a, cudaStream_t stream)
+template <int W, bool DIRECT>
+static rs_status launch5_w(Ctx *ctx, Dataset *ds, const HardArgs &a, cudaStream_t stream)
+{
+    if (a.preds) return a.cat ? launch5_t<W, true, true, DIRECT>(ctx, ds, a, stream)
+                              : launch5_t<W, false, true, DIRECT>(ctx, ds, a, stream);
+    return a.cat ? launch5_t<W, true, false, DIRECT>(ctx, ds, a, stream)
+                 : launch5_t<W, false, false, DIRECT>(ctx, ds, a, stream);
+}
+
+rs_status launch_hard5(Ctx *ctx, Dataset *ds, int W, bool direct, const HardArgs &a, cudaStream_t stream)
 {
     if (a.P == 0) return RS_OK;
-    if (a.preds) {
-        if (W == 16) return a.cat ? launch5_t<16, true, true>(ctx, ds, a, stream) : launch5_t<16, false, true>(ctx, ds, a, stream);
-        if (W == 32) return a.cat ? launch5_t<32, true, true>(ctx, ds, a, stream) : launch5_t<32, false, true>(ctx, ds, a, stream);
-    }
-    if (W == 16) return a.cat ? launch5_t<16, true, false>(ctx, ds, a, stream) : launch5_t<16, false, false>(ctx, ds, a, stream);
-    if (W == 32) return a.cat ? launch5_t<32, true, false>(ctx, ds, a, stream) : launch5_t<32, false, false>(ctx, ds, a, stream);
+    if (W == 16) return direct ? launch5_w<16, true>(ctx, ds, a, stream) : launch5_w<16, false>(ctx, ds, a, stream);
+    if (W == 32) return direct ? launch5_w<32, true>(ctx, ds, a, stream) : launch5_w<32, false>(ctx, ds, a, stream);
     return RS_ERR_INVALID;
 }
 
@@ -229,14 +249,22 @@ rs_status launch_hard5(Ctx *ctx, Dataset *ds, int W, const HardArgs &a, cudaStre
 void preload_hard5_kernels()
 {
     cudaFuncAttributes fa;
-    cudaFuncGetAttributes(&fa, k_hard5<16, false, false>);
-    cudaFuncGetAttributes(&fa, k_hard5<16, false, true>);
-    cudaFuncGetAttributes(&fa, k_hard5<16, true, false>);
-    cudaFuncGetAttributes(&fa, k_hard5<16, true, true>);
-    cudaFuncGetAttributes(&fa, k_hard5<32, false, false>);
-    cudaFuncGetAttributes(&fa, k_hard5<32, false, true>);
-    cudaFuncGetAttributes(&fa, k_hard5<32, true, false>);
-    cudaFuncGetAttributes(&fa, k_hard5<32, true, true>);
+    cudaFuncGetAttributes(&fa, k_hard5<16, false, false, false>);
+    cudaFuncGetAttributes(&fa, k_hard5<16, false, false, true>);
+    cudaFuncGetAttributes(&fa, k_hard5<16, false, true, false>);
+    cudaFuncGetAttributes(&fa, k_hard5<16, false, true, true>);
+    cudaFuncGetAttributes(&fa, k_hard5<16, true, false, false>);
+    cudaFuncGetAttributes(&fa, k_hard5<16, true, false, true>);
+    cudaFuncGetAttributes(&fa, k_hard5<16, true, true, false>);
+    cudaFuncGetAttributes(&fa, k_hard5<16, true, true, true>);
+    cudaFuncGetAttributes(&fa, k_hard5<32, false, false, false>);
+    cudaFuncGetAttributes(&fa, k_hard5<32, false, false, true>);
+    cudaFuncGetAttributes(&fa, k_hard5<32, false, true, false>);
+    cudaFuncGetAttributes(&fa, k_hard5<32, false, true, true>);
+    cudaFuncGetAttributes(&fa, k_hard5<32, true, false, false>);
+    cudaFuncGetAttributes(&fa, k_hard5<32, true, false, true>);
+    cudaFuncGetAttributes(&fa, k_hard5<32, true, true, false>);
+    cudaFuncGetAttributes(&fa, k_hard5<32, true, true, true>);
 }
 
 }  // namespace rs

@@ -195,7 +195,7 @@ struct TileConfig {
     int S() const { return 32 * V; }
 };
 constexpr int RANK_TILE = 128;    // samples per rank tile (ranks fit in 7 bits)
-constexpr int RANK_MAX_F = 160;   // widest dataset given rank tables
+constexpr int RANK_MAX_F = 128;   // widest dataset given rank tables (the widest whose tables fit 32 warps)
 int tile_config_count();
 const TileConfig &tile_config(int id);
 // Largest F a configuration can stage (its x tile must fit in shared memory).
@@ -359,10 +359,13 @@ struct TileTask {
 rs_status launch_hard2(Ctx *ctx, Dataset *ds, int V, int W, bool mm, const HardArgs &a,
                        cudaStream_t stream);
 rs_status launch_hard4(Ctx *ctx, Dataset *ds, int V, int W, const HardArgs &a, cudaStream_t stream);
-rs_status launch_hard5(Ctx *ctx, Dataset *ds, int W, const HardArgs &a, cudaStream_t stream);
+rs_status launch_hard5(Ctx *ctx, Dataset *ds, int W, bool direct, const HardArgs &a, cudaStream_t stream);
 // Shared memory of the v5 evaluator for F features and W warps.
 size_t hard5_smem_bytes(int F, int W);
+size_t direct_smem_bytes(int F, int W);   // and of its direct walk
 // The evaluator version a configuration runs as for this dataset and output choice.
+bool rank_tables_fit(int F, int W);
+constexpr int DIRECT_VERSION = 6;
 int effective_version(const TileConfig &tc, const Dataset &ds, bool preds);
 const TileConfig &categorical_config(const TileConfig &tc, const Dataset &ds, bool preds);
 // Enqueue packing + evaluation of a device batch with the given scratch.

@@ -46,7 +46,7 @@ constexpr size_t SERVE_SMEM = TILE_BYTES + (size_t)SW * 64 * 16 + (size_t)SW * S
 constexpr int MAX_SLOTS = 2048;
 constexpr int GROUP_SETS = 128;       // sets per unit: four per warp
 constexpr int GROUP_SETS_RANKED = 256;  // rank-coded units: their tile staging is heavier
-constexpr int SERVE_RANK_MIN_P = 64;    // smaller requests keep the sign-mask units
+constexpr int SERVE_RANK_MIN_P = 64;    // smaller requests take direct units
 constexpr int SPARE_SMS = 4;          // left to the packing kernels of new requests
 constexpr uint64_t IDLE_NS = 20000000ull;   // persistent kernel idle limit: 20 ms
 // claim word: epoch (24 bits) | next unit (20 bits) | units (20 bits)
@@ -88,9 +88,10 @@ __device__ __forceinline__ uint64_t now_ns()
     return t;
 }
 
-// One unit on a dataset with rank tables: stage the tile's x and ranks, build its reversed ranks
-// and sorted columns, then walk sets [set0, set1) with the rank-coded evaluator.
-__device__ __forceinline__ void serve_unit_ranked(const ReqDesc &d, int tile, int set0, int set1,
+// One unit on a finite dataset: stage the tile's x (and ranks: build its reversed ranks and sorted
+// columns; DIRECT: permute its rows), then walk sets [set0, set1) with the rank-coded or the direct walk.
+template <bool DIRECT>
+__device__ __forceinline__ void serve_unit_walk(const ReqDesc &d, int tile, int set0, int set1,
                                                   unsigned char *smem, uint4 *st, uint32_t *vr, uint32_t ones_off,
                                                   int *s_next)
 {
@@ -102,21 +103,23 @@ __device__ __forceinline__ void serve_unit_ranked(const ReqDesc &d, int tile, in
     const int64_t col0 = (int64_t)tile * T;
     for (int i = threadIdx.x; i < F * (T / 4); i += blockDim.x) {
         const int f = i / (T / 4), c4 = i % (T / 4);
-        reinterpret_cast<float4 *>(xs)[i] = *reinterpret_cast<const float4 *>(d.Xt + (int64_t)f * d.n_pad + col0 + 4 * c4);
+        reinterpret_cast<float4 *>(xs)[DIRECT ? i ^ (f & 7) : i] = *reinterpret_cast<const float4 *>(d.Xt + (int64_t)f * d.n_pad + col0 + 4 * c4);
     }
-    for (int i = threadIdx.x; i < F * (T / 16); i += blockDim.x) {
-        const int f = i / (T / 16), c16 = i % (T / 16);
-        reinterpret_cast<uint4 *>(rs)[i] = *reinterpret_cast<const uint4 *>(d.Rk + (int64_t)f * d.n_pad + col0 + 16 * c16);
+    if (!DIRECT) {
+        for (int i = threadIdx.x; i < F * (T / 16); i += blockDim.x) {
+            const int f = i / (T / 16), c16 = i % (T / 16);
+            reinterpret_cast<uint4 *>(rs)[i] = *reinterpret_cast<const uint4 *>(d.Rk + (int64_t)f * d.n_pad + col0 + 16 * c16);
+        }
+        __syncthreads();
+        build_tile_tables(reinterpret_cast<float *>(xs), rs, (uint32_t)F * T, us, F);
     }
-    __syncthreads();
-    build_tile_tables(reinterpret_cast<float *>(xs), rs, (uint32_t)F * T, us, F);
     const int32_t *yl = d.y + col0 + lane * 4;
     const int64_t t_last = min(col0 + T, d.N) - 1;
     const int kmin = d.y[col0], kmax = d.y[t_last];
     const bool uniform = kmin == kmax;
     const uint32_t claimed0 = class_bytes(yl, -1);
     const uint32_t rev_off = (uint32_t)F * T;
-    const uint32_t vr_off = (uint32_t)(reinterpret_cast<unsigned char *>(vr) - rs);
+    const uint32_t vr_off = (uint32_t)(reinterpret_cast<unsigned char *>(vr) - (DIRECT ? xs : rs));
     const unsigned char *rl = rs + lane * 4;
     __syncthreads();
     while (true) {
@@ -135,16 +138,18 @@ __device__ __forceinline__ void serve_unit_ranked(const ReqDesc &d, int tile, in
         uint32_t hit;
         rank::WalkCount wc;                 // not reported by the serving kernel
         int more;
-        if (d.cat)
+        if (!DIRECT && d.cat)           // membership tests are served by rank-coded units only
             hit = uniform ? walk_set<true, SVS, true>(st, vr, vr_off, lane, d.recs, rb, nrec, us, rev_off, F, kmin,
                                                       rl, xs, ones_off, yl, claimed0, deflt, wc, more)
                           : walk_set<false, SVS, true>(st, vr, vr_off, lane, d.recs, rb, nrec, us, rev_off, F, -2,
                                                        rl, xs, ones_off, yl, claimed0, deflt, wc, more);
         else
-            hit = uniform ? walk_set<true, SVS, false>(st, vr, vr_off, lane, d.recs, rb, nrec, us, rev_off, F, kmin,
-                                                       rl, xs, ones_off, yl, claimed0, deflt, wc, more)
-                          : walk_set<false, SVS, false>(st, vr, vr_off, lane, d.recs, rb, nrec, us, rev_off, F, -2,
-                                                        rl, xs, ones_off, yl, claimed0, deflt, wc, more);
+            hit = uniform ? walk_set<true, SVS, false, false, DIRECT>(st, vr, vr_off, lane, d.recs, rb, nrec, us, rev_off,
+                                                                      F, kmin, rl, xs, ones_off, yl, claimed0, deflt, wc,
+                                                                      more)
+                          : walk_set<false, SVS, false, false, DIRECT>(st, vr, vr_off, lane, d.recs, rb, nrec, us, rev_off,
+                                                                       F, -2, rl, xs, ones_off, yl, claimed0, deflt, wc,
+                                                                       more);
         const int hits = __reduce_add_sync(FULL, __popc(hit) + more);
         if (lane == 0 && hits) atomicAdd(&d.correct[p], hits);
         if (d.per_class) {
@@ -241,8 +246,10 @@ __global__ void __launch_bounds__(SW * 32, 1) k_serve(ServeArgs a)
         const ReqDesc &d = sd;       // shared: keeps the descriptor out of registers
         const int tile = unit / d.groups, grp = unit % d.groups;
         const int set0 = grp * d.gsets, set1 = min(d.P, set0 + d.gsets);
-        if (d.ranked) {
-            serve_unit_ranked(d, tile, set0, set1, smem, st, vrows + warp * SVS * 32, ones_off, &s_next);
+        if (d.finite) {
+            uint32_t *vr = vrows + warp * SVS * 32;
+            if (d.ranked) serve_unit_walk<false>(d, tile, set0, set1, smem, st, vr, ones_off, &s_next);
+            else serve_unit_walk<true>(d, tile, set0, set1, smem, st, vr, ones_off, &s_next);
             __syncthreads();
             if (threadIdx.x == 0) {
                 __threadfence();
@@ -260,8 +267,7 @@ __global__ void __launch_bounds__(SW * 32, 1) k_serve(ServeArgs a)
         const int nvec = d.F * (SS / 4);
         for (int i = threadIdx.x; i < nvec; i += blockDim.x) {
             const int f = i / (SS / 4), c4 = i % (SS / 4);
-            // the sign-mask form reads permuted rows (eval_sparse.cuh), the general form plain ones
-            reinterpret_cast<float4 *>(xs)[d.finite ? i ^ (f & 7) : i] =
+            reinterpret_cast<float4 *>(xs)[i] =
                 *reinterpret_cast<const float4 *>(d.Xt + (int64_t)f * d.n_pad + col0 + 4 * c4);
         }
         const int64_t n0 = col0 + lane * SV;
@@ -289,23 +295,13 @@ __global__ void __launch_bounds__(SW * 32, 1) k_serve(ServeArgs a)
                 si.rec_begin = t.x; si.rec_end = t.y; si.deflt = t.z; si.cost = t.w;
             }
             bool hit[SV];
-            int more = 0;
-            if (d.finite) {
-                uint32_t h[SV];
-                int re = si.rec_end;
-                if (uniform && d.last_end)
-                    re = min(si.rec_begin + __ldcg(d.last_end + (int64_t)p * d.K + kmin), re);
-                core::eval_set_sign<SV>(d.recs, si.rec_begin, re, st, smem, lane, si.deflt, y, d.y + n0, uniform, kmin, h,
-                                        more);
-#pragma unroll
-                for (int v = 0; v < SV; ++v) hit[v] = h[v] != 0u;
-            } else {
+            {
                 int pred[SV];
                 core::eval_set<SV>(d.recs, si.rec_begin, si.rec_end, st, xl, lane, si.deflt, valid, pred);
 #pragma unroll
                 for (int v = 0; v < SV; ++v) hit[v] = pred[v] == y[v];
             }
-            int hits = __reduce_add_sync(core::FULL, more);
+            int hits = 0;
 #pragma unroll
             for (int v = 0; v < SV; ++v) hits += __popc(__ballot_sync(core::FULL, hit[v]));
             if (lane == 0 && hits) atomicAdd(&d.correct[p], hits);
@@ -908,7 +904,7 @@ bool CudaBackend::admit(Request &r)
     cudaMemsetAsync(r.d_status, 0, 4, s->sstream);
     const bool finite = r.ds->finite;
     const bool ranked = serve_ranked(*r.ds, r.P, r.cat);
-    count_launch(s->ctx, launch_pack(bd, r.ds->F, r.K, SS, ranked ? 5 : (finite ? 4 : 2), po, s->sstream));
+    count_launch(s->ctx, launch_pack(bd, r.ds->F, r.K, SS, finite ? 5 : 2, po, s->sstream));
     ReqDesc d{};
     d.Xt = r.ds->Xt; d.y = r.ds->y; d.N = r.ds->N; d.n_pad = r.ds->n_pad; d.F = r.ds->F; d.K = r.K;
     d.recs = reinterpret_cast<const uint4 *>(po.recs); d.sets = po.sets; d.order = po.order;

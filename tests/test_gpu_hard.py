@@ -543,12 +543,13 @@ def test_measured_pipe_rates():
     assert all(v > 0 for v in r.values()), r
 
 
-@pytest.mark.parametrize("F,K,cat", [(3, 2, False), (9, 40, False), (128, 5, False), (16, 3, True)])
+@pytest.mark.parametrize("F,K,cat", [(3, 2, False), (9, 40, False), (100, 300, False), (128, 5, False), (16, 3, True),
+                                     (200, 4, False), (256, 2, False), (170, 3, True)])
 def test_sparse_tail_of_the_walks(orc, F, K, cat):
     """Sets whose first rules leave 0 to 40 samples of a 128-sample tile unclaimed, followed by rules
     that straddle the 32-record windows (up to 100 conditions), with pairs, ties, both
     comparisons, products and membership tests, on tiles of one label and of several: the
-    rank-coded and the sign-mask forms and the serving units."""
+    rank-coded, direct and sign-mask walks, their predictions, and the serving units."""
     import torch
     from paper_2406_01821_gb300 import build, rs
     build.build()
@@ -582,14 +583,18 @@ def test_sparse_tail_of_the_walks(orc, F, K, cat):
             long_rule = (int(rng.integers(0, K)), easy * (tail - 1) + [cond()])
             sets.append(head + rules[:7] + [long_rule] + rules[7:])
     b = synth.from_lists(sets, rng.integers(0, K, len(sets)).tolist())
-    oc, opc, _ = orc.eval_hard(X, y, K, b)
+    oc, opc, opr = orc.eval_hard(X, y, K, b, want_preds=True)
     with rs.Context(0) as ctx:
         ds = ctx.dataset(X, y, K)
         for tile in (16, 17, 18, 19, 20, 21, 22):
             ctx.set_tile_config(tile)
-            c, pc, _ = ctx.eval_hard(ds, rs.DeviceBatch.from_host(b), K)
-            torch.cuda.synchronize()
-            assert np.array_equal(c.cpu().numpy(), oc) and np.array_equal(pc.cpu().numpy(), opc)
+            for preds in (False, True):
+                c, pc, pr = ctx.eval_hard(ds, rs.DeviceBatch.from_host(b), K, N, preds=preds)
+                torch.cuda.synchronize()
+                assert np.array_equal(c.cpu().numpy(), oc) and np.array_equal(pc.cpu().numpy(), opc)
+                assert pr is None or np.array_equal(pr.cpu().numpy(), opr)
+        if cat and F > 128:
+            return                               # served by rank-coded units only
         t = ctx.submit(ds, rs.HostBatch(b))
         c, pc, _ = ctx.poll(t, b.P, K, timeout_us=30_000_000)
         assert np.array_equal(c, oc) and np.array_equal(pc, opc)
