@@ -48,7 +48,12 @@ constexpr int GROUP_SETS = 128;       // sets per unit: four per warp
 constexpr int GROUP_SETS_RANKED = 256;  // rank-coded units: their tile staging is heavier
 constexpr int SERVE_RANK_MIN_P = 64;    // smaller requests take direct units
 constexpr int SPARE_SMS = 4;          // left to the packing kernels of new requests
-constexpr uint64_t IDLE_NS = 20000000ull;   // persistent kernel idle limit: 20 ms
+// Persistent kernel idle limit: 2 ms without a claim and with no unit being walked anywhere. The first
+// CTA that finds it so closes the kernel for all: a CTA that left alone would be missing from the work
+// that keeps the others alive. Units that arrive then wait for the scheduler's next launch. While it
+// idles the kernel holds nearly every SM: with a limit of 20 ms, 72 requests of 27 ms kept the GPU
+// from the process's other streams for 47.
+constexpr uint64_t IDLE_NS = 2000000ull;
 // claim word: epoch (24 bits) | next unit (20 bits) | units (20 bits)
 constexpr int CW_NEXT = 20, CW_EPOCH = 40;
 constexpr unsigned long long CW_MASK = (1ull << 20) - 1;
@@ -75,7 +80,9 @@ struct ServeArgs {
     unsigned long long *claims;             // [MAX_SLOTS] claim words
     const volatile int32_t *active;         // [MAX_SLOTS] active slots (a hint; claims decide)
     const volatile int32_t *nactive;
-    unsigned int *rr;                       // round-robin cursor
+    unsigned long long *last_claim;         // globaltimer of the latest claim
+    int32_t *busy;                          // CTAs that hold or are taking a unit
+    int32_t *closed;                        // set once: nothing is claimed any more, every CTA leaves
     int32_t *done;                          // [MAX_SLOTS] units finished per slot
     volatile unsigned long long *host_flag; // mapped host memory [MAX_SLOTS]: finished epoch
     const volatile int32_t *stop;           // mapped host memory
@@ -178,6 +185,7 @@ __global__ void __launch_bounds__(SW * 32, 1) k_serve(ServeArgs a)
     __shared__ ReqDesc sd;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint4 *st = stage_all + warp * 64;
+    if (threadIdx.x == 0) *reinterpret_cast<volatile unsigned long long *>(a.last_claim) = now_ns();
 
     while (true) {
         if (warp == 0) {
@@ -186,7 +194,6 @@ __global__ void __launch_bounds__(SW * 32, 1) k_serve(ServeArgs a)
             // is not held behind a large one. The lanes read 32 claim words at a time; the chosen
             // request is taken by compare-and-swap (a lost race rescans).
             int slot = -1, unit = -1;
-            uint64_t idle0 = 0;
             while (true) {
                 // host-written words: lane 0 reads them, so every lane takes the same branches
                 if (__shfl_sync(core::FULL, lane == 0 ? *a.stop : 0, 0)) break;
@@ -207,9 +214,15 @@ __global__ void __launch_bounds__(SW * 32, 1) k_serve(ServeArgs a)
                 if (best != 0xFFFFFFFFu) {
                     const int i = (int)(best & 0x7FFu);
                     int got = -1, sl = -1;
+                    bool closed = false;
                     if (lane == 0) {
                         sl = a.active[i];
-                        if (sl >= 0 && sl < MAX_SLOTS) {
+                        // busy is raised before the flag is read, and the flag set before busy is read: a
+                        // closing CTA sees this one or is seen by it
+                        atomicAdd(a.busy, 1);
+                        __threadfence();
+                        closed = *reinterpret_cast<volatile int32_t *>(a.closed) != 0;
+                        if (!closed && sl >= 0 && sl < MAX_SLOTS) {
                             unsigned long long w = *reinterpret_cast<volatile unsigned long long *>(a.claims + sl);
                             while (((w >> CW_NEXT) & CW_MASK) < (w & CW_MASK)) {
                                 const unsigned long long old = atomicCAS(a.claims + sl, w, w + (1ull << CW_NEXT));
@@ -218,13 +231,26 @@ __global__ void __launch_bounds__(SW * 32, 1) k_serve(ServeArgs a)
                             }
                         }
                     }
+                    if (lane == 0) {
+                        if (got < 0) atomicSub(a.busy, 1);
+                        else *reinterpret_cast<volatile unsigned long long *>(a.last_claim) = now_ns();
+                    }
+                    if (__shfl_sync(core::FULL, closed ? 1 : 0, 0)) break;
                     got = __shfl_sync(core::FULL, got, 0);
                     if (got >= 0) { slot = __shfl_sync(core::FULL, sl, 0); unit = got; break; }
                     continue;                   // the request filled up meanwhile: rescan
                 }
-                const uint64_t tn = __shfl_sync(core::FULL, now_ns(), 0);
-                if (idle0 == 0) idle0 = tn;
-                else if (tn - idle0 > IDLE_NS) break;
+                int leave = 0;
+                if (lane == 0) {
+                    const unsigned long long last = *reinterpret_cast<volatile unsigned long long *>(a.last_claim);
+                    const unsigned long long tn = now_ns();
+                    leave = *reinterpret_cast<volatile int32_t *>(a.closed) != 0;
+                    if (!leave && tn > last && tn - last > IDLE_NS && *reinterpret_cast<volatile int32_t *>(a.busy) == 0) {
+                        atomicExch(a.closed, 1);
+                        leave = 1;
+                    }
+                }
+                if (__shfl_sync(core::FULL, leave, 0)) break;
                 __nanosleep(2000);
             }
             if (lane == 0) {
@@ -258,6 +284,7 @@ __global__ void __launch_bounds__(SW * 32, 1) k_serve(ServeArgs a)
                     __threadfence_system();
                     a.host_flag[slot] = d.epoch;
                 }
+                atomicSub(a.busy, 1);
             }
             __syncthreads();
             continue;
@@ -326,6 +353,7 @@ __global__ void __launch_bounds__(SW * 32, 1) k_serve(ServeArgs a)
                 __threadfence_system();
                 a.host_flag[slot] = d.epoch;
             }
+            atomicSub(a.busy, 1);
         }
         __syncthreads();
     }
@@ -417,7 +445,7 @@ struct Server {
     ReqDesc *d_table = nullptr;
     unsigned long long *d_claims = nullptr;
     int32_t *d_active = nullptr;           // [MAX_SLOTS + 1]: list, then its length
-    unsigned int *d_rr = nullptr;
+    unsigned long long *d_life = nullptr;  // last claim; busy and closed (ServeArgs)
     std::vector<int32_t> h_active;         // host copy of the active list
     cudaStream_t cstream = nullptr;        // completion copies
     int32_t *d_done = nullptr;
@@ -555,8 +583,7 @@ static rs_status server_start(Ctx *ctx, Server **out)
     if ((e = cudaMemset(s->d_claims, 0, sizeof(unsigned long long) * MAX_SLOTS))) return fail(e, "claims");
     if ((e = cudaMalloc(&s->d_active, sizeof(int32_t) * (MAX_SLOTS + 1)))) return fail(e, "active");
     if ((e = cudaMemset(s->d_active, 0, sizeof(int32_t) * (MAX_SLOTS + 1)))) return fail(e, "active");
-    if ((e = cudaMalloc(&s->d_rr, sizeof(unsigned int)))) return fail(e, "rr");
-    if ((e = cudaMemset(s->d_rr, 0, sizeof(unsigned int)))) return fail(e, "rr");
+    if ((e = cudaMalloc(&s->d_life, 16))) return fail(e, "idle words");
     if ((e = cudaMalloc(&s->d_done, sizeof(int32_t) * MAX_SLOTS))) return fail(e, "done");
     if ((e = cudaHostAlloc(&s->h_flag, sizeof(unsigned long long) * MAX_SLOTS, cudaHostAllocMapped))) return fail(e, "flags");
     if ((e = cudaHostAlloc(&s->h_stop, sizeof(int32_t), cudaHostAllocMapped))) return fail(e, "stop");
@@ -615,7 +642,7 @@ void server_shutdown(Ctx *ctx)
     cudaFree(s->d_table);
     cudaFree(s->d_claims);
     cudaFree(s->d_active);
-    cudaFree(s->d_rr);
+    cudaFree(s->d_life);
     cudaFree(s->d_done);
     for (auto &kv : s->pinned_free) cudaFreeHost(kv.second);
     for (cudaEvent_t e : s->event_pool) cudaEventDestroy(e);
@@ -950,7 +977,9 @@ void CudaBackend::launch_kernel()
 {
     // the descriptors and ring entries must be in place before the kernel starts
     cudaStreamWaitEvent(s->kstream, s->sch.active.back()->ev, 0);
-    ServeArgs a{s->d_table, s->d_claims, s->d_active, s->d_active + MAX_SLOTS, s->d_rr, s->d_done,
+    cudaMemsetAsync(s->d_life, 0, 16, s->kstream);
+    int32_t *words = reinterpret_cast<int32_t *>(s->d_life + 1);
+    ServeArgs a{s->d_table, s->d_claims, s->d_active, s->d_active + MAX_SLOTS, s->d_life, words, words + 1, s->d_done,
                 (volatile unsigned long long *)s->h_flag, (volatile int32_t *)s->h_stop};
     k_serve<<<s->grid, SW * 32, s->smem, s->kstream>>>(a);
     cudaEventRecord(s->kevent, s->kstream);
