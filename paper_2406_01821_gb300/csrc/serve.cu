@@ -44,8 +44,11 @@ constexpr size_t TILE_BYTES = (size_t)SERVE_MAX_F * SS * 4 > RANK_BYTES ? (size_
 constexpr size_t ONES_BYTES = (size_t)SS * 4;   // a row of 1.0: the right side of product conditions
 constexpr size_t SERVE_SMEM = TILE_BYTES + (size_t)SW * 64 * 16 + (size_t)SW * SVS * 32 * 4 + ONES_BYTES;
 constexpr int MAX_SLOTS = 2048;
-constexpr int GROUP_SETS = 128;       // sets per unit: four per warp
-constexpr int GROUP_SETS_RANKED = 256;  // rank-coded units: their tile staging is heavier
+// Sets per unit: as many as leave UNITS_MIN units to the request (two for every CTA), at most
+// GROUP_SETS_MAX, at least GROUP_SETS_MIN (rank-coded units, whose staging is heavier: _RANKED). Large
+// units lose less to their staging and to the last walks, which some warps of the CTA wait for: 72
+// mixed requests in 28.9 / 24.1 / 22.6 ms with direct units of at most 128 / 256 / 512 sets.
+constexpr int GROUP_SETS_MIN = 128, GROUP_SETS_MIN_RANKED = 256, GROUP_SETS_MAX = 512, UNITS_MIN = 296;
 constexpr int SERVE_RANK_MIN_P = 64;    // smaller requests take direct units
 constexpr int SPARE_SMS = 4;          // left to the packing kernels of new requests
 // Persistent kernel idle limit: 2 ms without a claim and with no unit being walked anywhere. The first
@@ -95,6 +98,13 @@ __device__ __forceinline__ uint64_t now_ns()
     return t;
 }
 
+// An asynchronous 16-byte copy into shared memory: a thread's copies are all in flight at once.
+__device__ __forceinline__ void copy16(void *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
 // One unit on a finite dataset: stage the tile's x (and ranks: build its reversed ranks and sorted
 // columns; DIRECT: permute its rows), then walk sets [set0, set1) with the rank-coded or the direct walk.
 template <bool DIRECT>
@@ -110,16 +120,18 @@ __device__ __forceinline__ void serve_unit_walk(const ReqDesc &d, int tile, int 
     const int64_t col0 = (int64_t)tile * T;
     for (int i = threadIdx.x; i < F * (T / 4); i += blockDim.x) {
         const int f = i / (T / 4), c4 = i % (T / 4);
-        reinterpret_cast<float4 *>(xs)[DIRECT ? i ^ (f & 7) : i] = *reinterpret_cast<const float4 *>(d.Xt + (int64_t)f * d.n_pad + col0 + 4 * c4);
+        copy16(reinterpret_cast<float4 *>(xs) + (DIRECT ? i ^ (f & 7) : i), d.Xt + (int64_t)f * d.n_pad + col0 + 4 * c4);
     }
     if (!DIRECT) {
         for (int i = threadIdx.x; i < F * (T / 16); i += blockDim.x) {
             const int f = i / (T / 16), c16 = i % (T / 16);
-            reinterpret_cast<uint4 *>(rs)[i] = *reinterpret_cast<const uint4 *>(d.Rk + (int64_t)f * d.n_pad + col0 + 16 * c16);
+            copy16(reinterpret_cast<uint4 *>(rs) + i, d.Rk + (int64_t)f * d.n_pad + col0 + 16 * c16);
         }
+        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
         build_tile_tables(reinterpret_cast<float *>(xs), rs, (uint32_t)F * T, us, F);
     }
+    if (DIRECT) asm volatile("cp.async.wait_all;" ::: "memory");
     const int32_t *yl = d.y + col0 + lane * 4;
     const int64_t t_last = min(col0 + T, d.N) - 1;
     const int kmin = d.y[col0], kmax = d.y[t_last];
@@ -375,9 +387,18 @@ bool serve_ranked(const Dataset &ds, int P, bool cat)
 {
     return ds.ranked && ds.F <= SERVE_RANK_MAX_F && (P >= SERVE_RANK_MIN_P || cat);
 }
+int serve_group_sets(const Dataset &ds, int P, bool cat)
+{
+    const int64_t tiles = (ds.N + SS - 1) / SS;
+    int g = GROUP_SETS_MAX;
+    const int least = serve_ranked(ds, P, cat) ? GROUP_SETS_MIN_RANKED : GROUP_SETS_MIN;
+    while (g > least && tiles * ((P + g - 1) / g) < UNITS_MIN) g /= 2;
+    return g;
+}
+
 int64_t serve_groups(const Dataset &ds, int P, bool cat)
 {
-    const int g = serve_ranked(ds, P, cat) ? GROUP_SETS_RANKED : GROUP_SETS;
+    const int g = serve_group_sets(ds, P, cat);
     return std::max<int64_t>(1, (P + g - 1) / g);
 }
 
@@ -940,7 +961,7 @@ bool CudaBackend::admit(Request &r)
     d.epoch = r.ticket & 0xFFFFFFull;
     d.Rk = ranked ? r.ds->Rk : nullptr;
     d.ranked = ranked ? 1 : 0;
-    d.gsets = ranked ? GROUP_SETS_RANKED : GROUP_SETS;
+    d.gsets = serve_group_sets(*r.ds, r.P, r.cat);
     d.last_end = po.last_end;
     d.cat = r.cat ? 1 : 0;
     // a copy from pageable memory is staged before the call returns, so `d` may go out of scope
