@@ -108,7 +108,8 @@ rs_status rs_check(rs_ctx *ctx, void *stream);
 rs_status rs_dataset_create(rs_ctx *ctx, const float *X, const int32_t *y, int64_t N, int32_t F,
                             int32_t K, int32_t mem, void *stream, uint64_t *ds_out);
 /*
- * Unregister a dataset and free its device copy (and its host copy under a dataset budget). The
+ * Unregister a dataset and free its device copy (and its host copy under a dataset budget; up to
+ * 256 MiB of freed dataset memory stays with the context for the next registration). The
  * device's queued work completes first, so no call enqueued earlier on any stream still reads it.
  * Errors: RS_ERR_NOT_FOUND (unknown handle); RS_ERR_INVALID while the dataset is in use: a call on
  * it is running in another thread, or a serving request on it has not been polled yet (queued,

@@ -147,6 +147,13 @@ rs_status rs_create(const rs_config *cfg, rs_ctx **out)
             delete ctx;
             return rc;
         }
+        if (rs_status rc = dataset_pool_create(ctx)) {
+            dataset_pool_destroy(ctx);
+            cudaFree(ctx->d_sticky);
+            cudaFree(ctx->d_walked);
+            delete ctx;
+            return rc;
+        }
         // keep freed stream-ordered scratch in the pool instead of returning it to the OS
         cudaMemPool_t pool;
         if (cudaDeviceGetDefaultMemPool(&pool, c.device) == cudaSuccess) {
@@ -183,6 +190,7 @@ rs_status rs_destroy(rs_ctx *ctx)
         for (auto id : ids) dataset_destroy(ctx, id, true);   // serving is shut down: nothing reads them
         release_dataset_events(ctx);
         ctx->graphs.clear();
+        dataset_pool_destroy(ctx);
         cudaFree(ctx->d_sticky);
         cudaFree(ctx->d_walked);
         delete ctx;

@@ -217,6 +217,8 @@ struct Profiler {
     double ms[2] = {0, 0};
 };
 
+constexpr uint64_t DATASET_POOL_KEEP = 256ull << 20;
+
 struct Ctx {
     int device = 0;
     uint32_t flags = 0;
@@ -238,6 +240,12 @@ struct Ctx {
     uint32_t *d_sticky = nullptr;            // async-mode sticky device status
     unsigned char *static_scratch = nullptr; // device address of rs_eval_hard_static's fixed array
     unsigned long long *d_walked = nullptr;  // [4] walked-work counters (RS_CTX_COUNT_WORK contexts)
+    // Memory of the datasets and of their registration: a pool of the context's own that keeps up to
+    // DATASET_POOL_KEEP bytes of freed memory mapped until the context is destroyed (mapping and
+    // unmapping 150 MB took 200 us of registering 300,007 x 96 and 130 of dropping it). Allocations
+    // and frees go through a stream of their own, waited for, so that the memory is usable on any.
+    cudaMemPool_t ds_pool = nullptr;
+    cudaStream_t ds_stream = nullptr;
     Profiler prof;
     struct Server *server = nullptr;
 };
@@ -260,6 +268,8 @@ struct DatasetUseMark {
     bool may_create = true;
     ~DatasetUseMark() { if (ds) mark_dataset_use(ctx, ds, stream, may_create); }
 };
+rs_status dataset_pool_create(Ctx *ctx);
+void dataset_pool_destroy(Ctx *ctx);
 // Free the context's spare events and every dataset's marks (context teardown).
 void release_dataset_events(Ctx *ctx);
 

@@ -485,12 +485,50 @@ const CUtensorMap *dataset_tmap(Dataset *ds, int S)
     return &res.first->second;
 }
 
+rs_status dataset_pool_create(Ctx *ctx)
+{
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = ctx->device;
+    RS_CUDA(cudaMemPoolCreate(&ctx->ds_pool, &props));
+    uint64_t keep = DATASET_POOL_KEEP;
+    RS_CUDA(cudaMemPoolSetAttribute(ctx->ds_pool, cudaMemPoolAttrReleaseThreshold, &keep));
+    RS_CUDA(cudaStreamCreateWithFlags(&ctx->ds_stream, cudaStreamNonBlocking));
+    return RS_OK;
+}
+
+void dataset_pool_destroy(Ctx *ctx)
+{
+    if (ctx->ds_stream) {
+        cudaStreamSynchronize(ctx->ds_stream);
+        cudaStreamDestroy(ctx->ds_stream);
+    }
+    if (ctx->ds_pool) cudaMemPoolDestroy(ctx->ds_pool);
+    ctx->ds_stream = nullptr;
+    ctx->ds_pool = nullptr;
+}
+
+template <class T>
+static cudaError_t ds_alloc(Ctx *ctx, T **p, size_t bytes)
+{
+    const cudaError_t e = cudaMallocFromPoolAsync(reinterpret_cast<void **>(p), bytes, ctx->ds_pool, ctx->ds_stream);
+    if (e != cudaSuccess) { *p = nullptr; return e; }
+    return cudaStreamSynchronize(ctx->ds_stream);
+}
+
+// The caller has seen to it that no device work uses p any more.
+static void ds_free(Ctx *ctx, void *p)
+{
+    if (p) cudaFreeAsync(p, ctx->ds_stream);
+}
+
 // Build the device copy of dataset d (N, F, K and n_pad set) from X and y (host or device per
 // `mem`): feature-major Xt grouped by label, labels, permutation and inverse, class counts, the
 // finite flag and, for finite data of at most RANK_MAX_F features, the rank table. The dataset is one
 // allocation (and one for the rank table), the temporary arrays another; the host waits once, at the
 // end: every kernel after the label check does nothing when a label was out of range.
-static rs_status build_device(Dataset &d, const float *X, const int32_t *y, int32_t mem, cudaStream_t stream)
+static rs_status build_device(Ctx *ctx, Dataset &d, const float *X, const int32_t *y, int32_t mem, cudaStream_t stream)
 {
     const int64_t N = d.N;
     const int32_t F = d.F, K = d.K;
@@ -500,7 +538,8 @@ static rs_status build_device(Dataset &d, const float *X, const int32_t *y, int3
     char *own = nullptr, *tmp = nullptr;
     rs_status rc = RS_OK;
     auto fail = [&] {                 // everything taken so far
-        cudaFree(own); cudaFree(tmp); cudaFree(d.Rk);
+        cudaStreamSynchronize(stream);
+        ds_free(ctx, own); ds_free(ctx, tmp); ds_free(ctx, d.Rk);
         d.Xt = nullptr; d.y = nullptr; d.perm = nullptr; d.inv = nullptr; d.flags = nullptr; d.Rk = nullptr;
     };
 #define REG_CUDA(call)                                      \
@@ -519,20 +558,20 @@ static rs_status build_device(Dataset &d, const float *X, const int32_t *y, int3
     const size_t o_x = take(sizeof(float) * (size_t)d.n_pad * F), o_y = take(sizeof(int32_t) * (size_t)d.n_pad),
                  o_perm = take(sizeof(int32_t) * (size_t)N), o_inv = take(sizeof(int32_t) * (size_t)N),
                  o_flags = take(sizeof(uint32_t) * (size_t)F);
-    REG_CUDA(cudaMalloc(&own, at));
+    REG_CUDA(ds_alloc(ctx, &own, at));
     d.Xt = reinterpret_cast<float *>(own + o_x);
     d.y = reinterpret_cast<int32_t *>(own + o_y);
     d.perm = reinterpret_cast<int32_t *>(own + o_perm);
     d.inv = reinterpret_cast<int32_t *>(own + o_inv);
     d.flags = reinterpret_cast<uint32_t *>(own + o_flags);
-    if (rank_tables) REG_CUDA(cudaMalloc(&d.Rk, (size_t)d.n_pad * F));
+    if (rank_tables) REG_CUDA(ds_alloc(ctx, &d.Rk, (size_t)d.n_pad * F));
     at = 0;
     // the status words and the class counts, read back together
     const size_t o_st = take(16 + sizeof(int64_t) * (size_t)K), o_start = take(sizeof(int64_t) * (size_t)K),
                  o_blk = take(sizeof(int32_t) * (size_t)nblk * K), o_rank = take(sizeof(int32_t) * (size_t)N);
     const size_t o_xd = mem == RS_MEM_HOST ? take(sizeof(float) * (size_t)N * F) : 0,
                  o_yd = mem == RS_MEM_HOST ? take(sizeof(int32_t) * (size_t)N) : 0;
-    REG_CUDA(cudaMalloc(&tmp, at));
+    REG_CUDA(ds_alloc(ctx, &tmp, at));
     uint32_t *st = reinterpret_cast<uint32_t *>(tmp + o_st);
     int64_t *ctot = reinterpret_cast<int64_t *>(tmp + o_st + 16), *cstart = reinterpret_cast<int64_t *>(tmp + o_start);
     int32_t *blk = reinterpret_cast<int32_t *>(tmp + o_blk), *rank = reinterpret_cast<int32_t *>(tmp + o_rank);
@@ -570,8 +609,8 @@ static rs_status build_device(Dataset &d, const float *X, const int32_t *y, int3
     d.finite = hst[1] == 0;
     d.ncode = (int32_t)hst[2];
     d.ranked = d.finite && rank_tables;
-    if (!d.ranked && d.Rk) { cudaFree(d.Rk); d.Rk = nullptr; }
-    cudaFree(tmp);
+    if (!d.ranked && d.Rk) { ds_free(ctx, d.Rk); d.Rk = nullptr; }
+    ds_free(ctx, tmp);
 #undef REG_CUDA
     return RS_OK;
 }
@@ -582,10 +621,10 @@ static size_t dataset_device_bytes(const Dataset &d)
            (d.Rk ? (size_t)d.n_pad * d.F : 0);
 }
 
-static void free_device(Dataset &d)
+static void free_device(Ctx *ctx, Dataset &d)
 {
-    cudaFree(d.Xt);                  // the start of the dataset's own allocation
-    cudaFree(d.Rk);
+    ds_free(ctx, d.Xt);              // the start of the dataset's own allocation
+    ds_free(ctx, d.Rk);
     d.Xt = nullptr; d.y = nullptr; d.perm = nullptr; d.inv = nullptr; d.flags = nullptr; d.Rk = nullptr;
     std::lock_guard<std::mutex> lk(d.mu);
     d.tmaps.clear();                 // tensor maps hold the device addresses
@@ -676,7 +715,7 @@ static void make_room(Ctx *ctx, size_t need, uint64_t keep)
     for (uint64_t h : v) {
         Dataset &d = *ctx->datasets[h];
         drop_graphs(ctx, h);
-        free_device(d);
+        free_device(ctx, d);
         d.resident = false;
         d.unmarked_use = false;
         ctx->ds_resident -= std::min(ctx->ds_resident, d.dev_bytes);
@@ -717,7 +756,7 @@ rs_status dataset_create(Ctx *ctx, const float *X, const int32_t *y, int64_t N, 
         if (e == cudaSuccess) e = cudaMemcpy(ds->hy.data(), y, sizeof(int32_t) * (size_t)N, kind);
         if (e != cudaSuccess) return cuda_fail(e, "dataset host copy");
     }
-    const rs_status rc = build_device(*ds, X, y, mem, stream);
+    const rs_status rc = build_device(ctx, *ds, X, y, mem, stream);
     if (rc) return rc;
     ds->dev_bytes = dataset_device_bytes(*ds);
     std::lock_guard<std::mutex> lk(ctx->mu);
@@ -743,7 +782,7 @@ rs_status use_dataset(Ctx *ctx, uint64_t h, std::shared_ptr<Dataset> *out)
         rs_status rc = device_guard(ctx);
         if (rc) return rc;
         make_room(ctx, d.dev_bytes, h);
-        if ((rc = build_device(d, d.hX.data(), d.hy.data(), RS_MEM_HOST, nullptr))) return rc;
+        if ((rc = build_device(ctx, d, d.hX.data(), d.hy.data(), RS_MEM_HOST, nullptr))) return rc;
         d.resident = true;
         ctx->ds_resident += d.dev_bytes;
         ++ctx->ds_rebuilds;
@@ -788,7 +827,7 @@ rs_status dataset_destroy(Ctx *ctx, uint64_t h, bool force)
         ds->inflight.clear();
     }
     RS_CUDA(cudaDeviceSynchronize());
-    free_device(*ds);
+    free_device(ctx, *ds);
     return RS_OK;
 }
 
