@@ -1,4 +1,4 @@
-// The sparse tail of a walk, shared by the rank-coded and the sign-mask evaluators.
+// The sparse tail of a walk, shared by the rank-coded, the direct and the sign-mask evaluators.
 //
 // The first rules claim most samples (each of the ragged workload's claims an eighth of
 // what is left), so that a set's last chunks are walked for a handful of samples: once at most

@@ -264,7 +264,7 @@ __device__ void mutate(Rng &r, const Mutation &m, const PopDev &o, int c, const 
 
 // One warp per child: copies in parallel, random decisions on lane 0. 10,000 children of 32 x 6 slots
 // took 150 us when rules were copied one by one and lane 0 shifted them for an added or deleted rule
-// (a load and a store after another for every slot behind it); 60 us so.
+// (a load and a store after another for every slot behind it); 64 us so.
 // gen = gen0 + *gidx: the generation index is read on the device, so that one captured graph
 // serves every generation.
 constexpr int NEXT_GEN_THREADS = 256;   // k_next_generation's block: 8 warps, one child each

@@ -376,7 +376,8 @@ int choose_groups(Ctx *ctx, const Dataset *ds, const TileConfig &tc, int P)
 // 64 + F / 3 sets (measured: 7 us at F = 30, 9 us at F = 106 against 0.09 us a set and tile with one
 // 32-warp CTA per SM), so that tiles are given to one CTA each as long as they fill whole waves of
 // the SMs' CTA slots; only the tiles left over are split into set groups, as many as make the last
-// waves shortest. 512 sets on 782 tiles: 442 us with every tile in four groups (21 waves), 300 us so.
+// waves shortest. 512 sets on 782 tiles of 32 features:
+// 442 us with every tile in four groups (21 waves), 405 us so, in two CTAs of 16 warps an SM.
 int split_tiles(Ctx *ctx, int64_t N, int F, int P, int S, int W, int resident, HardArgs &a)
 {
     const int64_t tiles = (N + S - 1) / S, slots = (int64_t)ctx->sm_count * std::max(1, resident);

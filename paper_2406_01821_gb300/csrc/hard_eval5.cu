@@ -1,4 +1,4 @@
-// Rank-coded batch evaluator (record format v5); the method and the device code are described in
+// Rank-coded batch evaluator and direct walk (record format v5); the method and the device code are described in
 // eval_rank.cuh.
 #include <algorithm>
 

@@ -89,7 +89,7 @@ constexpr uint32_t GENERAL_BIT = 1u << 31;
 // v4 only, in w1: the last record of its rule. v4 row offsets carry the row's permutation (f & 7).
 constexpr uint32_t END4_BIT = 1u << 31;
 
-// Record format v5 (rank-coded evaluator): per rule its threshold cuts, its pair conditions and
+// Record format v5 (rank-coded evaluator and direct walk): per rule its threshold cuts, its pair conditions and
 // its remaining product conditions, one record per condition (same positions as the conditions).
 // w0 = tag << 29 | end-of-rule << 28 | rule class << 16 (last record of a rule) | feature.
 //   cut:     x[f] > w2 (R5_CUT_GT) or x[f] <= w2 (R5_CUT_LT: x[f] < c stored as w2 = nextdown(c))
@@ -190,7 +190,8 @@ struct TileConfig {
     int ver;     // 1: condition-at-a-time evaluator, 2: rule-at-a-time (record v2),
                  // 3: rule-at-a-time with the margin-minimum conjunction,
                  // 4: sign-mask conjunction for finite datasets (falls back to 3 otherwise)
-                 // 5: rank-coded cuts for ranked datasets (falls back to 4, then 3)
+                 // 5: rank-coded cuts for ranked datasets, else (finite data) the same records walked
+                 //    directly on the floats (DIRECT_VERSION; falls back to 4, then 3)
     bool gmem = false;   // form 1 reading features from global memory (no shared tile: any F)
     int S() const { return 32 * V; }
 };
@@ -337,7 +338,7 @@ struct HardArgs {
     int32_t *per_class;      // [P*K] or null
     int32_t *preds;          // [P*N] or null
     int32_t groups;          // set groups (grid.y; forms 4 and 5: of the tiles from `whole` on)
-    int32_t whole;           // forms 4 and 5: tiles that one CTA walks with all sets (split_tiles)
+    int32_t whole;           // forms 4, 5 and the direct walk: tiles that one CTA walks with all sets (split_tiles)
     uint32_t *status;
     const int32_t *last_end; // [P*K] or null (see PackOut)
     const float *Xt;         // [F][n_pad] (read directly by the global-memory configuration)

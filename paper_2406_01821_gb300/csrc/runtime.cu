@@ -517,11 +517,15 @@ static cudaError_t ds_alloc(Ctx *ctx, T **p, size_t bytes)
     return cudaStreamSynchronize(ctx->ds_stream);
 }
 
-// The caller has seen to it that no device work uses p any more.
+// The caller has seen to it that no device work uses p any more. The pool gives memory beyond
+// DATASET_POOL_KEEP back to the driver when its stream is next waited for: ds_settle, after the last
+// free of an operation, so that a dropped dataset's memory is there for any other allocator.
 static void ds_free(Ctx *ctx, void *p)
 {
     if (p) cudaFreeAsync(p, ctx->ds_stream);
 }
+
+static void ds_settle(Ctx *ctx) { cudaStreamSynchronize(ctx->ds_stream); }
 
 // Build the device copy of dataset d (N, F, K and n_pad set) from X and y (host or device per
 // `mem`): feature-major Xt grouped by label, labels, permutation and inverse, class counts, the
@@ -540,6 +544,7 @@ static rs_status build_device(Ctx *ctx, Dataset &d, const float *X, const int32_
     auto fail = [&] {                 // everything taken so far
         cudaStreamSynchronize(stream);
         ds_free(ctx, own); ds_free(ctx, tmp); ds_free(ctx, d.Rk);
+        ds_settle(ctx);
         d.Xt = nullptr; d.y = nullptr; d.perm = nullptr; d.inv = nullptr; d.flags = nullptr; d.Rk = nullptr;
     };
 #define REG_CUDA(call)                                      \
@@ -611,6 +616,7 @@ static rs_status build_device(Ctx *ctx, Dataset &d, const float *X, const int32_
     d.ranked = d.finite && rank_tables;
     if (!d.ranked && d.Rk) { ds_free(ctx, d.Rk); d.Rk = nullptr; }
     ds_free(ctx, tmp);
+    ds_settle(ctx);
 #undef REG_CUDA
     return RS_OK;
 }
@@ -625,6 +631,7 @@ static void free_device(Ctx *ctx, Dataset &d)
 {
     ds_free(ctx, d.Xt);              // the start of the dataset's own allocation
     ds_free(ctx, d.Rk);
+    ds_settle(ctx);
     d.Xt = nullptr; d.y = nullptr; d.perm = nullptr; d.inv = nullptr; d.flags = nullptr; d.Rk = nullptr;
     std::lock_guard<std::mutex> lk(d.mu);
     d.tmaps.clear();                 // tensor maps hold the device addresses

@@ -5,8 +5,8 @@
 // allow, uploads and packs each one, writes its descriptor into a device table and publishes it in
 // the device list of active requests with a claim word (epoch | next unit | units). One persistent
 // kernel, kept alive while work arrives, lets each CTA claim a unit -- a 128-sample tile of the
-// request's dataset times a group of up to 128 of its sets -- from the active requests in
-// round-robin order (processor sharing: a small request does not wait behind a large one), load
+// request's dataset times a group of up to 512 of its sets -- from the active requests (shortest
+// remaining work first: a small request does not wait behind a large one), load
 // the tile into shared memory, evaluate those sets on it and add exact counts. The CTA finishing
 // a request's last unit raises the request's flag in mapped host memory; the scheduler then copies
 // the counts back on its own stream and frees the slot and its memory. Requests admitted while
@@ -381,8 +381,7 @@ size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 // Requests on datasets with rank tables use the rank-coded evaluator when they have enough sets
 // to amortise its tile staging (x, ranks and sorted columns, and one search per cut and tile).
-// Requests with membership conditions always take them (the sign-mask units have no membership
-// test).
+// Requests with membership conditions take them whatever their size where the dataset has tables.
 bool serve_ranked(const Dataset &ds, int P, bool cat)
 {
     return ds.ranked && ds.F <= SERVE_RANK_MAX_F && (P >= SERVE_RANK_MIN_P || cat);

@@ -150,3 +150,34 @@ def test_serving_request_pins_its_dataset(orc):
         assert ctx.dataset_stats()["rebuilds"] == rebuilds      # it was never evicted
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("reject", (False, True))
+def test_dropped_dataset_memory_is_given_back(reject):
+    """A context keeps at most 256 MiB of dropped datasets' memory mapped (rs.h); the rest is free for
+    any other allocator once the dropping (or rejecting) call has returned. 64 MiB allow for what the
+    calls load for the first time and other processes' noise; the dataset and its scratch take 0.65 GiB."""
+    import torch
+    from paper_2406_01821_gb300 import build, rs
+    build.build()
+    ctx = rs.Context(0)
+    try:
+        n, f = 1 << 20, 128
+        X = torch.zeros((n, f), device="cuda")
+        y = torch.zeros(n, dtype=torch.int32, device="cuda")
+        if reject:
+            y[n // 2] = 7                          # not a class of K = 2
+        small = ctx.dataset(np.zeros((300, 4), np.float32), np.zeros(300, np.int32), 2)
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        if reject:
+            with pytest.raises(rs.RsError):
+                ctx.dataset(X, y, 2)
+        else:
+            ds = ctx.dataset(X, y, 2)
+            assert before - torch.cuda.mem_get_info()[0] >= 4 * n * f
+            ctx.dataset_destroy(ds)
+        assert before - torch.cuda.mem_get_info()[0] <= (256 + 64) << 20
+        ctx.dataset_destroy(small)
+    finally:
+        ctx.close()
