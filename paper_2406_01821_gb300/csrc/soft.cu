@@ -888,7 +888,7 @@ __device__ __forceinline__ void cond_grads(const SoftWarp &m, int ci, int nconds
 // Forward (and adjoint) of a set of R rules over one group of 64 NV samples: lane l holds samples
 // n0 + 2 NV l + i (bit i of valid: the sample exists). tm: the warp's tensor-memory base
 // (staged-tile adjoint). Returns true, having added nothing, when some sample's p_y is below e^-64
-// (or not a number): the group's bit is then set, and k_soft_ff evaluates it in float-float after
+// or something is not a number: the group's bit is then set, and k_soft_ff evaluates it in float-float after
 // this kernel.
 template <bool BWD, bool CAT, bool TILE, int NV>
 __device__ __forceinline__ bool soft_group(const SoftKArgs &a, const SoftWarp &m, int p, int R, int nconds, int deflt,
@@ -952,12 +952,13 @@ __device__ __forceinline__ bool soft_group(const SoftKArgs &a, const SoftWarp &m
         c0 = c1;
     }
     add_class(deflt, U);
-    // every q_r went into p_y or 1 - p_y: a NaN anywhere shows in one of them
+    // every q_r went into p_y or 1 - p_y: a NaN anywhere shows in one of them (looked for beyond the
+    // data's end too, where the features are zeros: a NaN times a weight of 0 would spoil the sums)
     bool big = false;
 #pragma unroll
     for (int i = 0; i < NV; ++i)
-        big |= (((valid >> (2 * i)) & 1u) && !(py.v[i].x >= SOFT_P_MIN && po.v[i].x >= 0.f)) ||
-               (((valid >> (2 * i + 1)) & 1u) && !(py.v[i].y >= SOFT_P_MIN && po.v[i].y >= 0.f));
+        big |= !(py.v[i].x >= (((valid >> (2 * i)) & 1u) ? SOFT_P_MIN : 0.f) && po.v[i].x >= 0.f) ||
+               !(py.v[i].y >= (((valid >> (2 * i + 1)) & 1u) ? SOFT_P_MIN : 0.f) && po.v[i].y >= 0.f);
     if (BWD && TILE) tmem_wait_put();
     if (__any_sync(FULL, big)) return true;
     // -log p_y; near 1 from 1 - p_y, which is its own sum of positive terms
@@ -1153,9 +1154,8 @@ __global__ void __launch_bounds__(SOFT_W * 32) k_soft(SoftKArgs a)
 }
 
 // The same evaluation with the warps of a team on as many neighbouring sets (in size order) over
-// the same chunk: the features of each 64-sample group are staged once per team in shared memory
-// (double-buffered asynchronous copies), so condition loads are shared-memory reads. Per-set
-// results are identical to k_soft (same per-sample arithmetic and summation order).
+// the same chunk, four samples a lane: the features of each group of 128 are staged once per team in
+// shared memory (double-buffered asynchronous copies), so condition loads are shared-memory reads.
 constexpr int SOFT_TW_MIN = 4, SOFT_TW_MAX = 16;   // warps per CTA (and sets per team) of the staged-tile kernel
 constexpr int SOFT_GT = 64 * SOFT_NV_TILE;    // samples per group of the staged-tile kernel
 constexpr int SOFT_TILE_STATIC = 256;   // bytes kept for the kernel's static shared memory

@@ -387,3 +387,31 @@ def test_soft_linear_domain_edges(ctx, orc, N, F, P, R, C, K, tau):
     check_against_oracle(got, ref)
     assert np.allclose(got["probs"], ref["probs"], rtol=RTOL, atol=1e-30)
     assert np.array_equal(got["loss_fwd"], got["loss"])
+
+
+@pytest.mark.parametrize("N,F,P,R,C,far,tau", [
+    (1003, 6, 30, (2, 12), (1, 5), 0.03, 0.05),     # scattered, a last group of odd size
+    (130, 130, 5, (2, 6), (1, 4), 0.2, 0.05),       # the per-warp kernel
+    (9001, 4, 3, (2, 30), (1, 3), 0.5, 0.02),       # many groups to a task
+    (257, 3, 200, (2, 3), (1, 2), 1.0, 0.02),       # every sample far
+])
+def test_soft_far_samples_and_ragged_end(ctx, orc, N, F, P, R, C, far, tau):
+    """Samples far outside the thresholds' range, scattered among others, whose groups are left to the
+    float-float pass; and a set that meets its samples at small margins but the zeros beyond the data's
+    end at margins whose exponentials overflow."""
+    X, y = synth.gaussian_mixture(N, F, 2, 23)
+    b = synth.random_rulesets(synth.quantile_table(X), 2, P, R, C, 23, pair_prob=0.0)
+    rng = np.random.default_rng(23)
+    X[rng.random(N) < far] *= np.float32(30.0)
+    X[:, F - 1] = (20.0 + 0.05 * rng.standard_normal(N)).astype(np.float32)
+    r = b.set_rule_off[-2]
+    c = b.rule_cond_off[r]
+    if b.rule_cond_off[r + 1] - c > 1:
+        b.cond_f[c:c + 2], b.cond_op[c:c + 2], b.cond_a[c:c + 2] = (F - 1, 0), 0, 1.0
+        b.cond_t[c:c + 2] = 20.0, -20.0
+    b = reachable(b)
+    dl = rng.uniform(0.5, 2, b.P)
+    got = soft_gpu(ctx, X, y, 2, b, tau, dl, probs=True)
+    ref = orc.soft(X, y, 2, b, tau, dloss=dl, want_probs=True, want_mag=True)
+    check_against_oracle(got, ref)
+    assert np.allclose(got["probs"], ref["probs"], rtol=RTOL, atol=1e-30)
