@@ -145,7 +145,7 @@ def executed_work(prof, batch, N):
 
 def source_hash():
     h = hashlib.sha256()
-    for f in ("hard_eval.cu", "hard_eval4.cu", "hard_eval5.cu", "eval_rank.cuh", "eval_core.cuh", "pack.cu",
+    for f in ("hard_eval.cu", "hard_eval4.cu", "hard_eval5.cu", "eval_rank.cuh", "eval_sparse.cuh", "eval_core.cuh", "pack.cu",
               "rs_internal.cuh", "tma.cuh"):
         with open(os.path.join(ROOT, "paper_2406_01821_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
@@ -433,9 +433,9 @@ def soft_transcendentals(batch, N):
     condition and sample an exp and a log1p (log-sigmoid) and an exp (sigmoid of -u); per rule and
     sample an expm1 and a log (log(1 - q)) forward and again in the adjoint, an exp (the gradient
     of lq), two log-sum-exps (exp + log1p each) in the adjoint and one forward for rules of the
-    sample's class (counted for every rule: an upper bound on the forward share). The kernels do
-    fewer per rule: the adjoint reuses the forward's log(1 - q) and runs one of its two
-    log-sum-exps (the other only adds log(1 - q))."""
+    sample's class (counted for every rule: an upper bound on the forward share). The kernels work in
+    the linear domain and execute fewer: an exponential per condition and sample forward, an
+    exponential and a reciprocal in the adjoint, and a few reciprocals per rule."""
     return N * (3 * batch.C + 11 * batch.R)
 
 
