@@ -49,11 +49,18 @@ constexpr int SOFT_G = 32 * SOFT_V;
 // float-float list, list items taken
 constexpr int SOFT_NEXT_FF_LEN = 3, SOFT_NEXT_FF = 4, SOFT_NEXT_N = 8;
 
-// Floats of a warp's shared arrays: lu [maxR + 1][G], acc [maxC][4], and lq [maxR][G] when the
-// class probabilities are written.
-__host__ __device__ constexpr size_t soft_per_warp(int maxR, int maxC, bool with_lq)
+// Floats of a float-float warp's shared arrays: acc [maxC][4], and lu [maxR + 1][32] and lq [maxR][32]
+// when the class probabilities are written.
+__host__ __device__ constexpr size_t soft_ff_floats(int maxR, int maxC, bool probs)
 {
-    return (size_t)(maxR + 1) * SOFT_G + (size_t)maxC * 4 + (with_lq ? (size_t)maxR * SOFT_G : 0);
+    return (size_t)maxC * 4 + (probs ? (size_t)(2 * maxR + 1) * 32 : 0);
+}
+
+// Largest sets the entry points take: four times these floats fit an SM's shared memory (the size of an
+// earlier layout of the per-warp arrays, kept as the limit; the present ones are smaller).
+__host__ constexpr size_t soft_limit_floats(int maxR, int maxC, bool probs)
+{
+    return (size_t)(maxR + 1) * SOFT_G + (size_t)maxC * 4 + (probs ? (size_t)maxR * SOFT_G : 0);
 }
 
 struct __align__(16) SoftRec {
@@ -296,8 +303,8 @@ struct SoftKArgs {
 struct XView {
     const float *col;
     int64_t stride;
-    // x[f] of the lane's sample v (32 v samples after its first)
-    __device__ __forceinline__ float operator()(int f, int v) const { return col[(int64_t)f * stride + 32 * v]; }
+    // x[f] of the lane's sample
+    __device__ __forceinline__ float operator()(int f) const { return col[(int64_t)f * stride]; }
 };
 
 // ------------------------------------------------------------------ float-float arithmetic
@@ -375,14 +382,45 @@ __device__ __forceinline__ ff ff_log_unit(float y)
     return ff_add_f(kl, logf(m));
 }
 
-// The signed scaled margin u = s * (a * x[f] - rhs) / tau of condition rc for the lane's sample
-// v, in float-float: the products are exact (a float times a float), 1/tau is a float-float.
-__device__ __forceinline__ ff margin_ff(const SoftKArgs &a, const SoftRec &rc, const XView &x, int v)
+// A condition's record with the lane's feature values (xg: the second feature of a pair).
+struct CondIn {
+    SoftRec rc;
+    float xf, xg;
+};
+
+__device__ __forceinline__ CondIn load_cond(const SoftKArgs &a, int c, const XView &x)
 {
-    const ff lhs = ff_two_prod(rc.a, x(rc.f, v));
-    const ff rhs = (rc.meta & 1u) ? ff_two_prod(rc.bt, x(rc.g, v)) : ff{rc.bt, 0.f};
+    CondIn t;
+    t.rc = a.recs[c];
+    t.xf = x(t.rc.f);
+    t.xg = x((t.rc.meta & 1u) ? t.rc.g : t.rc.f);
+    return t;
+}
+
+// f(condition) for c0 <= c < c1 in order, the loads of FF_BATCH conditions issued before the first of
+// them is used.
+constexpr int FF_BATCH = 4;
+template <class Fn>
+__device__ __forceinline__ void each_cond(const SoftKArgs &a, int c0, int c1, const XView &x, Fn f)
+{
+    for (int c = c0; c < c1; c += FF_BATCH) {
+        CondIn t[FF_BATCH];
+#pragma unroll
+        for (int i = 0; i < FF_BATCH; ++i) t[i] = load_cond(a, min(c + i, c1 - 1), x);
+#pragma unroll
+        for (int i = 0; i < FF_BATCH; ++i)
+            if (c + i < c1) f(t[i]);
+    }
+}
+
+// The signed scaled margin u = s * (a * x[f] - rhs) / tau of a condition for the lane's sample, in
+// float-float: the products are exact (a float times a float), 1/tau is a float-float.
+__device__ __forceinline__ ff margin_ff(const SoftKArgs &a, const CondIn &t)
+{
+    const ff lhs = ff_two_prod(t.rc.a, t.xf);
+    const ff rhs = (t.rc.meta & 1u) ? ff_two_prod(t.rc.bt, t.xg) : ff{t.rc.bt, 0.f};
     ff u = ff_mul(ff_add(lhs, ff_neg(rhs)), ff{a.inv_tau, a.inv_tau_lo});
-    if (rc.meta & 2u) u = ff_neg(u);
+    if (t.rc.meta & 2u) u = ff_neg(u);
     return u;
 }
 
@@ -394,20 +432,19 @@ __device__ __forceinline__ ff log_sigmoid_ff(ff u, float &l1pe)
     return u.hi < 0.f ? ff_add_f(u, -l1pe) : ff{-l1pe, 0.f};
 }
 
-// log q of one rule for the lane's sample v in float-float (membership tests: 0 or -inf).
+// log q of one rule for the lane's sample in float-float (membership tests: 0 or -inf).
 template <bool CAT>
-__device__ ff rule_logq_ff(const SoftKArgs &a, int c0, int c1, const XView &x, int v)
+__device__ ff rule_logq_ff(const SoftKArgs &a, int c0, int c1, const XView &x)
 {
     ff s{0.f, 0.f};
-    for (int c = c0; c < c1; ++c) {
-        const SoftRec rc = a.recs[c];
-        if (CAT && (rc.meta & 4u)) {
-            if (!category_member(x(rc.f, v), __float_as_uint(rc.a), __float_as_uint(rc.bt))) s = {-INFINITY, 0.f};
-            continue;
+    each_cond(a, c0, c1, x, [&](const CondIn &t) {
+        if (CAT && (t.rc.meta & 4u)) {
+            if (!category_member(t.xf, __float_as_uint(t.rc.a), __float_as_uint(t.rc.bt))) s = {-INFINITY, 0.f};
+            return;
         }
         float l1pe;
-        s = ff_add(s, log_sigmoid_ff(margin_ff(a, rc, x, v), l1pe));
-    }
+        s = ff_add(s, log_sigmoid_ff(margin_ff(a, t), l1pe));
+    });
     return s;
 }
 
@@ -418,7 +455,7 @@ __device__ ff rule_logq_ff(const SoftKArgs &a, int c0, int c1, const XView &x, i
 // log-sum-exp of -u_c with the largest term factored out. A rule of holding membership tests
 // only has q = 1 exactly and log(1 - q) = -inf.
 template <bool CAT>
-__device__ ff rule_log1mq_ff(const SoftKArgs &a, int c0, int c1, const XView &x, int v, ff lq)
+__device__ ff rule_log1mq_ff(const SoftKArgs &a, int c0, int c1, const XView &x, ff lq)
 {
     if (lq.hi == -INFINITY) return {0.f, 0.f};
     const float lqf = ff_f(lq);
@@ -426,19 +463,17 @@ __device__ ff rule_log1mq_ff(const SoftKArgs &a, int c0, int c1, const XView &x,
     if (lqf < -0.69314718f) return {log1pf(-expf(lqf)), 0.f};
     if (lqf < -0x1p-24f) return ff_log_unit(-expm1f(lqf));
     ff m{INFINITY, 0.f};
-    for (int c = c0; c < c1; ++c) {
-        const SoftRec rc = a.recs[c];
-        if (CAT && (rc.meta & 4u)) continue;
-        const ff u = margin_ff(a, rc, x, v);
+    each_cond(a, c0, c1, x, [&](const CondIn &t) {
+        if (CAT && (t.rc.meta & 4u)) return;
+        const ff u = margin_ff(a, t);
         if (ff_less(u, m)) m = u;
-    }
+    });
     if (m.hi == INFINITY) return {-INFINITY, 0.f};
     float acc = 0.f;
-    for (int c = c0; c < c1; ++c) {
-        const SoftRec rc = a.recs[c];
-        if (CAT && (rc.meta & 4u)) continue;
-        acc += expf(ff_f(ff_add(m, ff_neg(margin_ff(a, rc, x, v)))));
-    }
+    each_cond(a, c0, c1, x, [&](const CondIn &t) {
+        if (CAT && (t.rc.meta & 4u)) return;
+        acc += expf(ff_f(ff_add(m, ff_neg(margin_ff(a, t)))));
+    });
     return ff_add_f(ff_neg(m), logf(acc));
 }
 
@@ -463,95 +498,89 @@ __device__ __forceinline__ void reduce_pair(float2 g0, float2 g1, int ci0, bool 
     }
 }
 
-// Class probabilities of the sample in slot `sl` (lane + 32 v) of the group from its per-rule log q
-// and log "no earlier rule fired" (lq, lu; lu[R] for the default).
-template <int V>
-__device__ __forceinline__ void write_probs(const SoftKArgs &a, int p, int rb, int R, int deflt, int64_t n0, int sl,
-                                            float (*lq)[32 * V], float (*lu)[32 * V])
+// Class probabilities of the lane's sample n from its per-rule log q and log "no earlier rule fired"
+// (lq, lu; lu[R] for the default).
+__device__ __forceinline__ void write_probs(const SoftKArgs &a, int p, int rb, int R, int deflt, int64_t n, int lane,
+                                            float (*lq)[32], float (*lu)[32])
 {
-    const int64_t orig = a.perm[n0 + sl];
+    const int64_t orig = a.perm[n];
     for (int k = 0; k < a.K; ++k) {
-        float lpk = (deflt == k) ? lu[R][sl] : -INFINITY;
+        float lpk = (deflt == k) ? lu[R][lane] : -INFINITY;
         for (int j = 0; j < R; ++j)
-            if (a.rule_class[rb + j] == k) lpk = log_add(lpk, lq[j][sl] + lu[j][sl]);
+            if (a.rule_class[rb + j] == k) lpk = log_add(lpk, lq[j][lane] + lu[j][lane]);
         a.probs[((int64_t)p * a.N + orig) * a.K + k] = expf(lpk);
     }
 }
 
-// soft_group in float-float arithmetic, one sample of each lane at a time (all lanes walk the same
+// soft_group in float-float arithmetic, one sample n to a lane (all lanes walk the same
 // rules and conditions, so the gradient butterflies stay warp-wide). Forward: log q_r and
 // log(1 - q_r) of every rule, lu and log p_y accumulated in float-float. Adjoint: lu_r recovered
 // backwards as lu_{r+1} - log(1 - q_r) (exact to float-float precision; from the saved value at
 // the first rule with q_r = 1, after which lu is -inf), the S and T recursions in float-float, and
 // d ell / d u_c = -+exp(lq_r + lu_r + lT_{r+1} or lS_{r+1} - lp_y + log sigmoid(-u_c)) formed in the
-// exponent. Per-set sums keep the float path's fixed order: the loss in the caller's Kahan sum,
-// the gradients through the same butterfly and lanes.
-template <bool BWD, bool CAT, int V>
-__device__ __forceinline__ void soft_group_ff(const SoftKArgs &a, int p, int rb, int R, int cb, int deflt, int64_t n0,
-                                           uint32_t valid, const XView &x, float (*lq)[32 * V],
-                                           float (*lu)[32 * V], float (*acc)[4], int lane, float &loss_s,
-                                           float &loss_c)
+// exponent. Per-set sums keep a fixed order: the loss in the caller's Kahan sum, the gradients
+// through one butterfly per two conditions and fixed lanes. lq, lu: only with class probabilities.
+template <bool BWD, bool CAT>
+__device__ __forceinline__ void soft_group_ff(const SoftKArgs &a, int p, int rb, int R, int cb, int deflt, int64_t n,
+                                           bool ok, const XView &x, float (*lq)[32], float (*lu)[32],
+                                           float (*acc)[4], int lane, float &loss_s, float &loss_c)
 {
-    for (int v = 0; v < V; ++v) {
-        const bool ok = (valid >> v) & 1u;
-        const int yv = ok ? a.y[n0 + lane + 32 * v] : -1;
-        const int sl = lane + 32 * v;
-        // ---------------- forward
-        ff lur{0.f, 0.f}, lpy{-INFINITY, 0.f}, lu_fin{0.f, 0.f};
-        int jinf = R;                          // first rule with q = 1 (log(1 - q) = -inf)
-        for (int j = 0; j < R; ++j) {
-            const int r = rb + j;
-            const int c0 = a.rule_cond_off[r], c1 = a.rule_cond_off[r + 1];
-            const ff lqj = rule_logq_ff<CAT>(a, c0, c1, x, v);
-            const ff l1q = rule_log1mq_ff<CAT>(a, c0, c1, x, v, lqj);
-            if (a.rule_class[r] == yv) lpy = ff_log_add(lpy, ff_add(lqj, lur));
-            if (lq) lq[j][sl] = lqj.hi;
-            lu[j][sl] = lur.hi;
-            if (l1q.hi == -INFINITY && jinf == R) { jinf = j; lu_fin = lur; }
-            lur = ff_add(lur, l1q);
-        }
-        lu[R][sl] = lur.hi;
-        if (deflt == yv) lpy = ff_log_add(lpy, lur);
-        if (ok) kadd_loss(loss_s, loss_c, -ff_f(lpy));
-        if (a.probs && ok) write_probs<V>(a, p, rb, R, deflt, n0, sl, lq, lu);   // this lane's own slot
-        if (!BWD) continue;
-        // ---------------- adjoint
-        ff lS = deflt == yv ? ff{0.f, 0.f} : ff{-INFINITY, 0.f};
-        ff lT = deflt == yv ? ff{-INFINITY, 0.f} : ff{0.f, 0.f};
-        ff lu_next = lur;
-        for (int j = R - 1; j >= 0; --j) {
-            const int r = rb + j;
-            const int cls = a.rule_class[r];
-            const int c0 = a.rule_cond_off[r], c1 = a.rule_cond_off[r + 1];
-            const ff lqj = rule_logq_ff<CAT>(a, c0, c1, x, v);
-            const ff l1q = rule_log1mq_ff<CAT>(a, c0, c1, x, v, lqj);
-            const ff luj = j > jinf ? ff{-INFINITY, 0.f} : (j == jinf ? lu_fin : ff_add(lu_next, ff_neg(l1q)));
-            lu_next = luj;
-            const bool same = cls == yv;
-            const ff lw = same ? lT : lS;
-            const bool zero = !ok || lw.hi == -INFINITY || lqj.hi == -INFINITY || luj.hi == -INFINITY;
-            const ff G = ff_add(ff_add(ff_add(lqj, luj), lw), ff_neg(lpy));
-            const float sign = same ? -1.f : 1.f;
-            lS = ff_log_add(same ? lqj : ff{-INFINITY, 0.f}, ff_add(l1q, lS));
-            lT = ff_log_add(same ? ff{-INFINITY, 0.f} : lqj, ff_add(l1q, lT));
-            for (int c = c0; c < c1; c += 2) {
-                const bool has1 = c + 1 < c1;
-                float2 g[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+    const int yv = ok ? a.y[n] : -1;
+    // ---------------- forward
+    ff lur{0.f, 0.f}, lpy{-INFINITY, 0.f}, lu_fin{0.f, 0.f};
+    int jinf = R;                          // first rule with q = 1 (log(1 - q) = -inf)
+    for (int j = 0; j < R; ++j) {
+        const int r = rb + j;
+        const int c0 = a.rule_cond_off[r], c1 = a.rule_cond_off[r + 1];
+        const ff lqj = rule_logq_ff<CAT>(a, c0, c1, x);
+        const ff l1q = rule_log1mq_ff<CAT>(a, c0, c1, x, lqj);
+        if (a.rule_class[r] == yv) lpy = ff_log_add(lpy, ff_add(lqj, lur));
+        if (lq) { lq[j][lane] = lqj.hi; lu[j][lane] = lur.hi; }
+        if (l1q.hi == -INFINITY && jinf == R) { jinf = j; lu_fin = lur; }
+        lur = ff_add(lur, l1q);
+    }
+    if (lq) lu[R][lane] = lur.hi;
+    if (deflt == yv) lpy = ff_log_add(lpy, lur);
+    if (ok) kadd_loss(loss_s, loss_c, -ff_f(lpy));
+    if (lq && ok) write_probs(a, p, rb, R, deflt, n, lane, lq, lu);   // this lane's own slots
+    if (!BWD) return;
+    // ---------------- adjoint
+    ff lS = deflt == yv ? ff{0.f, 0.f} : ff{-INFINITY, 0.f};
+    ff lT = deflt == yv ? ff{-INFINITY, 0.f} : ff{0.f, 0.f};
+    ff lu_next = lur;
+    for (int j = R - 1; j >= 0; --j) {
+        const int r = rb + j;
+        const int cls = a.rule_class[r];
+        const int c0 = a.rule_cond_off[r], c1 = a.rule_cond_off[r + 1];
+        const ff lqj = rule_logq_ff<CAT>(a, c0, c1, x);
+        const ff l1q = rule_log1mq_ff<CAT>(a, c0, c1, x, lqj);
+        const ff luj = j > jinf ? ff{-INFINITY, 0.f} : (j == jinf ? lu_fin : ff_add(lu_next, ff_neg(l1q)));
+        lu_next = luj;
+        const bool same = cls == yv;
+        const ff lw = same ? lT : lS;
+        const bool zero = !ok || lw.hi == -INFINITY || lqj.hi == -INFINITY || luj.hi == -INFINITY;
+        const ff G = ff_add(ff_add(ff_add(lqj, luj), lw), ff_neg(lpy));
+        const float sign = same ? -1.f : 1.f;
+        lS = ff_log_add(same ? lqj : ff{-INFINITY, 0.f}, ff_add(l1q, lS));
+        lT = ff_log_add(same ? ff{-INFINITY, 0.f} : lqj, ff_add(l1q, lT));
+        for (int c = c0; c < c1; c += 2) {
+            const bool has1 = c + 1 < c1;
+            const CondIn t[2] = {load_cond(a, c, x), load_cond(a, has1 ? c + 1 : c, x)};
+            float2 g[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    if (i == 1 && !has1) break;
-                    const SoftRec rc = a.recs[c + i];
-                    if ((CAT && (rc.meta & 4u)) || zero) continue;
-                    const ff u = margin_ff(a, rc, x, v);
-                    float l1pe;
-                    log_sigmoid_ff(u, l1pe);
-                    const ff lsn = u.hi > 0.f ? ff_add_f(ff_neg(u), -l1pe) : ff{-l1pe, 0.f};   // log sigmoid(-u)
-                    const float sg = (rc.meta & 2u) ? -1.f : 1.f;
-                    const float du = sign * expf(ff_f(ff_add(G, lsn))) * sg * a.inv_tau;
-                    g[i] = make_float2(du * x(rc.f, v), (rc.meta & 1u) ? -du * x(rc.g, v) : -du);
-                }
-                reduce_pair(g[0], g[1], c - cb, has1, acc, lane);
+            for (int i = 0; i < 2; ++i) {
+                if (i == 1 && !has1) break;
+                const SoftRec &rc = t[i].rc;
+                if ((CAT && (rc.meta & 4u)) || zero) continue;
+                const ff u = margin_ff(a, t[i]);
+                float l1pe;
+                log_sigmoid_ff(u, l1pe);
+                const ff lsn = u.hi > 0.f ? ff_add_f(ff_neg(u), -l1pe) : ff{-l1pe, 0.f};   // log sigmoid(-u)
+                const float sg = (rc.meta & 2u) ? -1.f : 1.f;
+                const float du = sign * expf(ff_f(ff_add(G, lsn))) * sg * a.inv_tau;
+                g[i] = make_float2(du * t[i].xf, (rc.meta & 1u) ? -du * t[i].xg : -du);
             }
+            reduce_pair(g[0], g[1], c - cb, has1, acc, lane);
         }
     }
 }
@@ -1273,11 +1302,16 @@ __global__ void __maxnreg__(128) k_soft_tile(SoftKArgs a, int F)
 }
 
 // The float-float pass: the CTAs take the (set, chunk) tasks that the main kernel listed, SOFT_W warps
-// to a task: warp i evaluates every SOFT_W-th of the groups whose bits the main kernel set (those it
-// left out) in float-float (soft_group_ff), its loss and gradient sums Kahan-summed in group order;
-// the warps' sums are added to the task's partials in warp order, so that results do not depend on
-// the order of the list. Runs after the main kernel on the same stream; features are read from
-// global memory.
+// to a task: warp i evaluates every SOFT_W-th 32 samples of the groups whose bits the main kernel set
+// (those it left out) in float-float (soft_group_ff), its loss and gradient sums Kahan-summed in their
+// order; the warps' sums are added to the task's partials in warp order, so that results do not depend
+// on the order of the list. Runs after the main kernel on the same stream; features are read from
+// global memory. What bounds it is the chain of one warp's conditions (a record, its features, the
+// arithmetic, one after another), hence the batched loads (each_cond) and one sample to a lane, four
+// warps to a group of 128. With two samples to a lane, one after the
+// other, and each condition's loads on their own, 88 us for the class probabilities of 48 sets on
+// 20,000 x 30 and 228 us for the adjoint of 64 on 100,000 x 32 where a few samples of every group lie
+// far out; 48 and 122 us so (twice the CTAs or batches of two loads were no faster).
 template <bool BWD, bool CAT>
 __global__ void __launch_bounds__(SOFT_W * 32) k_soft_ff(SoftKArgs a)
 {
@@ -1287,13 +1321,11 @@ __global__ void __launch_bounds__(SOFT_W * 32) k_soft_ff(SoftKArgs a)
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (*a.status) return;
     const int items = a.next[SOFT_NEXT_FF_LEN];
-    const size_t per_warp = soft_per_warp(a.maxR, a.maxC, a.probs != nullptr);
+    const size_t per_warp = soft_ff_floats(a.maxR, a.maxC, a.probs != nullptr);
     float *base_w = sm + per_warp * w;
-    float(*lu)[SOFT_G] = reinterpret_cast<float(*)[SOFT_G]>(base_w);
-    float(*acc)[4] = reinterpret_cast<float(*)[4]>(base_w + (size_t)(a.maxR + 1) * SOFT_G);
-    float(*lq)[SOFT_G] = a.probs ? reinterpret_cast<float(*)[SOFT_G]>(base_w + (size_t)(a.maxR + 1) * SOFT_G +
-                                                                    (size_t)a.maxC * 4)
-                                 : nullptr;
+    float(*acc)[4] = reinterpret_cast<float(*)[4]>(base_w);
+    float(*lu)[32] = a.probs ? reinterpret_cast<float(*)[32]>(base_w + (size_t)a.maxC * 4) : nullptr;
+    float(*lq)[32] = a.probs ? lu + a.maxR + 1 : nullptr;
     while (true) {
         __syncthreads();
         if (threadIdx.x == 0) s_item = atomicAdd(a.next + SOFT_NEXT_FF, 1);
@@ -1315,18 +1347,15 @@ __global__ void __launch_bounds__(SOFT_W * 32) k_soft_ff(SoftKArgs a)
         const int64_t s1 = min(s0 + a.chunk, a.N);
         const uint32_t *fbits = a.ffbits + task * a.ff_wpt;
         uint32_t fw = 0;
-        int k = 0;                                     // 64-sample groups of marked groups so far
-        for (int64_t nb = s0; nb < s1; nb += SOFT_G) {
+        int k = 0;                                     // 32-sample pieces of marked groups so far
+        for (int64_t nb = s0; nb < s1; nb += 32) {
             const int gi = (int)((nb - s0) / a.group);
             if ((nb - s0) % (32 * a.group) == 0) fw = fbits[gi >> 5];
             if (!((fw >> (gi & 31)) & 1u)) continue;
             if ((k++ & (SOFT_W - 1)) != w) continue;
-            uint32_t valid = 0;
-#pragma unroll
-            for (int v = 0; v < SOFT_V; ++v) valid |= (nb + lane + 32 * v < s1 ? 1u : 0u) << v;
-            const XView x{a.Xt + nb + lane, a.n_pad};
-            soft_group_ff<BWD, CAT, SOFT_V>(a, p, rb, re - rb, cb, deflt, nb, valid, x, lq, lu, acc, lane, loss_s,
-                                            loss_c);
+            const int64_t n = nb + lane;
+            soft_group_ff<BWD, CAT>(a, p, rb, re - rb, cb, deflt, n, n < s1, XView{a.Xt + n, a.n_pad}, lq, lu, acc,
+                                    lane, loss_s, loss_c);
         }
         float ls = loss_s;
 #pragma unroll
@@ -1339,11 +1368,10 @@ __global__ void __launch_bounds__(SOFT_W * 32) k_soft_ff(SoftKArgs a)
             a.part_loss[task] += t;
         }
         if (BWD) {
-            const float(*acc0)[4] = reinterpret_cast<const float(*)[4]>(sm + (size_t)(a.maxR + 1) * SOFT_G);
             for (int i = threadIdx.x; i < (ce - cb); i += SOFT_W * 32) {
                 float ga = 0.f, gbt = 0.f;
                 for (int v = 0; v < SOFT_W; ++v) {
-                    const float *t = reinterpret_cast<const float *>(acc0) + per_warp * v + 4 * (size_t)i;
+                    const float *t = sm + per_warp * v + 4 * (size_t)i;
                     ga += t[0];
                     gbt += t[2];
                 }
@@ -1677,13 +1705,14 @@ static rs_status soft_run(Ctx *ctx, const SoftArgs &s, int known_maxR, int known
         }
     }
     k.pslots = k.probs ? std::min(k.K, k.maxR + 1) : 0;
-    const size_t smem_ff = sizeof(float) * soft_per_warp(k.maxR, k.maxC, k.probs != nullptr) * SOFT_W;
+    const size_t smem_ff = sizeof(float) * soft_ff_floats(k.maxR, k.maxC, k.probs != nullptr) * SOFT_W;
     const size_t smem = soft_main_bytes(k.maxR, k.maxC, bwd, false, k.pslots) * SOFT_W;
     const size_t per_warp = soft_main_bytes(k.maxR, k.maxC, bwd, true, k.pslots);
     // the staged-tile kernel when its smallest per-CTA footprint (and two feature tiles) fits
     const size_t smem_tile = soft_team_bytes(SOFT_TW_MIN, per_warp, s.F);
     const bool tiled = s.F <= 128 && smem_tile + SOFT_TILE_STATIC <= ctx->smem_optin;
-    if (rc == RS_OK && (smem > ctx->smem_optin || smem_ff > ctx->smem_optin)) {
+    const size_t limit = sizeof(float) * soft_limit_floats(k.maxR, k.maxC, k.probs != nullptr) * SOFT_W;
+    if (rc == RS_OK && (smem > ctx->smem_optin || limit > ctx->smem_optin)) {
         rc = RS_ERR_TOO_LARGE;
         set_error("soft evaluation: sets too large for shared memory");
     }
