@@ -141,9 +141,11 @@ __device__ __forceinline__ uint32_t cut_word(uint32_t off, uint32_t n, const uns
 
 // Bit 7 of byte v where the lane's sample v (labels yl[0..3]) has label k. Only tiles that hold
 // more than one label need it, so the labels are read again instead of kept in registers.
+// LIVE: see sparse::load_label.
+template <bool LIVE = false>
 __device__ __forceinline__ uint32_t class_bytes(const int32_t *yl, int k)
 {
-    const int4 y = __ldg(reinterpret_cast<const int4 *>(yl));
+    const int4 y = sparse::load_label<LIVE>(reinterpret_cast<const int4 *>(yl));
     return ((y.x == k) ? 0x80u : 0u) | ((y.y == k) ? 0x8000u : 0u) | ((y.z == k) ? 0x800000u : 0u) |
            ((y.w == k) ? 0x80000000u : 0u);
 }
@@ -199,7 +201,7 @@ __device__ __forceinline__ uint32_t code_row(uint4 q, const uint2 *codes, int la
 
 // One group of four staged records with end-of-rule flags M (bit u: record u ends its rule).
 // PRED: the class words are the class in every byte, and hit holds the predicted classes, a byte a sample.
-template <uint32_t M, bool UNI, bool PRED>
+template <uint32_t M, bool UNI, bool PRED, bool LIVE>
 __device__ __forceinline__ void group4(const uint32_t (&e)[4], const uint32_t *sw, const int32_t *yl,
                                        uint32_t &fail, uint32_t &claimed, uint32_t &hit)
 {
@@ -217,7 +219,7 @@ __device__ __forceinline__ void group4(const uint32_t (&e)[4], const uint32_t *s
                 asm("prmt.b32 %0, %1, 0, 0xBA98;" : "=r"(m) : "r"(newly));
                 hit = (w & m) | (hit & ~m);
             } else if (UNI) hit |= newly & w;
-            else hit |= newly & class_bytes(yl, (int)w);
+            else hit |= newly & class_bytes<LIVE>(yl, (int)w);
             claimed |= newly;
             fail = claimed;
         }
@@ -263,7 +265,7 @@ struct Decode5 {
 
 // Returns the hit bits; `more` receives the lane's hits of the sparse tail that are not in them.
 // DIRECT: the direct walk (us, rl and rev_off unused, vrow_off relative to xs).
-template <bool UNI, int VS, bool CAT, bool PRED = false, bool DIRECT = false>
+template <bool UNI, int VS, bool CAT, bool PRED = false, bool DIRECT = false, bool LIVE = false>
 __device__ __forceinline__ uint32_t walk_set(uint4 *st, uint32_t *vrow, uint32_t vrow_off, int lane,
                                              const uint4 *recs, int rb, int nrec, const float *us,
                                              uint32_t rev_off, int F, int kmine, const unsigned char *rl,
@@ -357,7 +359,7 @@ __device__ __forceinline__ uint32_t walk_set(uint4 *st, uint32_t *vrow, uint32_t
             }
             const uint32_t *swg = sw + g;
             switch ((ends >> g) & 0xFu) {
-#define RS_GROUP4(M) case M: group4<M, UNI, PRED>(e, swg, yl, fail, claimed, hit); break;
+#define RS_GROUP4(M) case M: group4<M, UNI, PRED, LIVE>(e, swg, yl, fail, claimed, hit); break;
             RS_GROUP4(0) RS_GROUP4(1) RS_GROUP4(2) RS_GROUP4(3) RS_GROUP4(4) RS_GROUP4(5) RS_GROUP4(6)
             RS_GROUP4(7) RS_GROUP4(8) RS_GROUP4(9) RS_GROUP4(10) RS_GROUP4(11) RS_GROUP4(12)
             RS_GROUP4(13) RS_GROUP4(14) RS_GROUP4(15)
@@ -373,7 +375,7 @@ __device__ __forceinline__ uint32_t walk_set(uint4 *st, uint32_t *vrow, uint32_t
         if (live <= sparse::MAX && ends) {                   // from the first rule not finished yet
             const int tail = cnt - (32 - __clz(ends));
             wc.records += c0 - tail;
-            more = sparse::tail<4, UNI, CAT, PRED>(sw, recs, rb, c0 - tail, nrec, lane, kmine, xs, yl, claimed, deflt, hit, wc,
+            more = sparse::tail<4, UNI, CAT, PRED, LIVE>(sw, recs, rb, c0 - tail, nrec, lane, kmine, xs, yl, claimed, deflt, hit, wc,
                                              Decode5{F, ones_off});
             return hit;
         }
@@ -382,7 +384,7 @@ __device__ __forceinline__ uint32_t walk_set(uint4 *st, uint32_t *vrow, uint32_t
     if (PRED) return hit;
     const uint32_t left = ~claimed & HIGH;
     if (UNI) hit |= (deflt == kmine) ? left : 0u;
-    else hit |= left & class_bytes(yl, deflt);
+    else hit |= left & class_bytes<LIVE>(yl, deflt);
     return hit;
 }
 

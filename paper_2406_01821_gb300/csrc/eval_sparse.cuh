@@ -21,6 +21,12 @@ constexpr uint32_t FULL = 0xFFFFFFFFu;
 // 92.2 / 92.5 / 92.5 ms.
 constexpr int MAX = 20;
 
+// A dataset's label. LIVE: read through L2 in a kernel that may outlive the dataset at this address: an
+// evicted dataset's memory can hold another one's labels while the serving kernel runs on, and a line of
+// the read-only or L1 cache would then be stale.
+template <bool LIVE, class T>
+__device__ __forceinline__ T load_label(const T *p) { return LIVE ? __ldcg(p) : __ldg(p); }
+
 // Work a walk did: records, pair / product / membership conditions and rule ends (profiling counters).
 struct WalkCount {
     uint32_t records = 0, rows = 0, ends = 0;
@@ -49,7 +55,7 @@ struct Rec {
 // instructions a window, against about 500 and 140 for a dense chunk. Returns the lane's hits (UNI);
 // otherwise they go to the samples' words. PRED (four samples a lane): `hit` holds the predicted
 // classes, a byte a sample, and receives those of the tail through 32 words after the list.
-template <int V, bool UNI, bool CAT, bool PRED, class Decode>
+template <int V, bool UNI, bool CAT, bool PRED, bool LIVE = false, class Decode>
 __device__ __forceinline__ int tail(uint32_t *list, const uint4 *recs, int rb, int c0, int nrec, int lane, int kmine,
                                     const unsigned char *xs, const int32_t *yl, uint32_t claimed, int deflt,
                                     uint32_t &hit, WalkCount &wc, const Decode &decode)
@@ -116,7 +122,7 @@ __device__ __forceinline__ int tail(uint32_t *list, const uint4 *recs, int rb, i
             if (first & K) ++hits;
         } else {
             const int k = __shfl_sync(FULL, r.cls, fired ? __ffs(first) - 1 : 0);
-            give_back(__ballot_sync(FULL, fired != 0u && k == __ldg(yl - V * lane + (at >> 2))));
+            give_back(__ballot_sync(FULL, fired != 0u && k == load_label<LIVE>(yl - V * lane + (at >> 2))));
         }
         const uint32_t stay = __ballot_sync(FULL, lane < n && fired == 0u);
         if (__popc(stay) != n) {                       // close the list's gaps
@@ -134,7 +140,7 @@ __device__ __forceinline__ int tail(uint32_t *list, const uint4 *recs, int rb, i
         return 0;
     }
     if (UNI) return hits + (lane < n && deflt == kmine ? 1 : 0);
-    give_back(__ballot_sync(FULL, lane < n && deflt == __ldg(yl - V * lane + (at >> 2))));
+    give_back(__ballot_sync(FULL, lane < n && deflt == load_label<LIVE>(yl - V * lane + (at >> 2))));
     return 0;
 }
 

@@ -134,9 +134,9 @@ __device__ __forceinline__ void serve_unit_walk(const ReqDesc &d, int tile, int 
     if (DIRECT) asm volatile("cp.async.wait_all;" ::: "memory");
     const int32_t *yl = d.y + col0 + lane * 4;
     const int64_t t_last = min(col0 + T, d.N) - 1;
-    const int kmin = d.y[col0], kmax = d.y[t_last];
+    const int kmin = __ldcg(d.y + col0), kmax = __ldcg(d.y + t_last);
     const bool uniform = kmin == kmax;
-    const uint32_t claimed0 = class_bytes(yl, -1);
+    const uint32_t claimed0 = class_bytes<true>(yl, -1);
     const uint32_t rev_off = (uint32_t)F * T;
     const uint32_t vr_off = (uint32_t)(reinterpret_cast<unsigned char *>(vr) - (DIRECT ? xs : rs));
     const unsigned char *rl = rs + lane * 4;
@@ -158,17 +158,19 @@ __device__ __forceinline__ void serve_unit_walk(const ReqDesc &d, int tile, int 
         rank::WalkCount wc;                 // not reported by the serving kernel
         int more;
         if (!DIRECT && d.cat)           // membership tests are served by rank-coded units only
-            hit = uniform ? walk_set<true, SVS, true>(st, vr, vr_off, lane, d.recs, rb, nrec, us, rev_off, F, kmin,
-                                                      rl, xs, ones_off, yl, claimed0, deflt, wc, more)
-                          : walk_set<false, SVS, true>(st, vr, vr_off, lane, d.recs, rb, nrec, us, rev_off, F, -2,
-                                                       rl, xs, ones_off, yl, claimed0, deflt, wc, more);
+            hit = uniform ? walk_set<true, SVS, true, false, false, true>(st, vr, vr_off, lane, d.recs, rb, nrec, us,
+                                                                          rev_off, F, kmin, rl, xs, ones_off, yl,
+                                                                          claimed0, deflt, wc, more)
+                          : walk_set<false, SVS, true, false, false, true>(st, vr, vr_off, lane, d.recs, rb, nrec, us,
+                                                                           rev_off, F, -2, rl, xs, ones_off, yl,
+                                                                           claimed0, deflt, wc, more);
         else
-            hit = uniform ? walk_set<true, SVS, false, false, DIRECT>(st, vr, vr_off, lane, d.recs, rb, nrec, us, rev_off,
-                                                                      F, kmin, rl, xs, ones_off, yl, claimed0, deflt, wc,
-                                                                      more)
-                          : walk_set<false, SVS, false, false, DIRECT>(st, vr, vr_off, lane, d.recs, rb, nrec, us, rev_off,
-                                                                       F, -2, rl, xs, ones_off, yl, claimed0, deflt, wc,
-                                                                       more);
+            hit = uniform ? walk_set<true, SVS, false, false, DIRECT, true>(st, vr, vr_off, lane, d.recs, rb, nrec, us,
+                                                                            rev_off, F, kmin, rl, xs, ones_off, yl,
+                                                                            claimed0, deflt, wc, more)
+                          : walk_set<false, SVS, false, false, DIRECT, true>(st, vr, vr_off, lane, d.recs, rb, nrec, us,
+                                                                             rev_off, F, -2, rl, xs, ones_off, yl,
+                                                                             claimed0, deflt, wc, more);
         const int hits = __reduce_add_sync(FULL, __popc(hit) + more);
         if (lane == 0 && hits) atomicAdd(&d.correct[p], hits);
         if (d.per_class) {
@@ -176,7 +178,7 @@ __device__ __forceinline__ void serve_unit_walk(const ReqDesc &d, int tile, int 
                 if (lane == 0 && hits) atomicAdd(&d.per_class[(int64_t)p * d.K + kmin], hits);
             } else {
                 for (int k = kmin; k <= kmax; ++k) {
-                    const int c = __reduce_add_sync(FULL, __popc(hit & class_bytes(yl, k)));
+                    const int c = __reduce_add_sync(FULL, __popc(hit & class_bytes<true>(yl, k)));
                     if (lane == 0 && c) atomicAdd(&d.per_class[(int64_t)p * d.K + k], c);
                 }
             }
@@ -275,8 +277,8 @@ __global__ void __launch_bounds__(SW * 32, 1) k_serve(ServeArgs a)
         const int slot = s_slot, unit = s_unit;
         if (slot < 0) return;
         __threadfence();
-        // Descriptors and per-request buffers are reused while this kernel lives: read them
-        // through L2 (.cg), never from a possibly stale L1 line.
+        // Descriptors, per-request buffers and, after an eviction, dataset memory are reused while this
+        // kernel lives: read them through L2 (.cg), never from a possibly stale L1 line.
         if (threadIdx.x < (int)(sizeof(ReqDesc) / 16))
             reinterpret_cast<int4 *>(&sd)[threadIdx.x] =
                 __ldcg(reinterpret_cast<const int4 *>(a.table + slot) + threadIdx.x);
@@ -307,18 +309,18 @@ __global__ void __launch_bounds__(SW * 32, 1) k_serve(ServeArgs a)
         for (int i = threadIdx.x; i < nvec; i += blockDim.x) {
             const int f = i / (SS / 4), c4 = i % (SS / 4);
             reinterpret_cast<float4 *>(xs)[i] =
-                *reinterpret_cast<const float4 *>(d.Xt + (int64_t)f * d.n_pad + col0 + 4 * c4);
+                __ldcg(reinterpret_cast<const float4 *>(d.Xt + (int64_t)f * d.n_pad + col0 + 4 * c4));
         }
         const int64_t n0 = col0 + lane * SV;
         int y[SV];
         bool valid[SV];
 #pragma unroll
         for (int v = 0; v < SV; ++v) {
-            y[v] = d.y[n0 + v];
+            y[v] = __ldcg(d.y + n0 + v);
             valid[v] = y[v] >= 0;
         }
         const int64_t t_last = min(col0 + SS, d.N) - 1;
-        const int kmin = d.y[col0], kmax = d.y[t_last];
+        const int kmin = __ldcg(d.y + col0), kmax = __ldcg(d.y + t_last);
         const bool uniform = kmin == kmax;
         __syncthreads();
         const float *xl = xs + lane * SV;

@@ -152,6 +152,48 @@ def test_serving_request_pins_its_dataset(orc):
         ctx.close()
 
 
+@pytest.mark.parametrize("finite", (True, False))
+def test_eviction_under_a_live_serving_kernel(orc, finite):
+    """Two datasets of one shape and different labels take each other's place in device memory while
+    requests on a third keep the serving kernel running: every request is counted with its own
+    dataset's labels and features."""
+    from paper_2406_01821_gb300 import rs
+    ctx = _budget_ctx()
+    try:
+        Xc, yc = synth.gaussian_mixture(200_000, 32, 4, 80)
+        bc = synth.random_rulesets(synth.quantile_table(Xc[:4000]), 4, 2000, (32, 64), (4, 8), 81)
+        third = ctx.dataset(Xc, yc, 4)
+        base = ctx.dataset_stats()["resident_bytes"]
+        pair = []
+        for i, share in enumerate(((0.2, 0.3, 0.5), (0.6, 0.3, 0.1))):
+            X, _, b = _data(i)
+            y = np.random.default_rng(82 + i).choice(K, N, p=share).astype(np.int32)
+            if not finite:
+                X[::37, 3] = np.nan
+            pair.append((X, y, b, orc.eval_hard(X, y, K, b)))
+        dss = [ctx.dataset(pair[0][0], pair[0][1], K)]
+        one = ctx.dataset_stats()["resident_bytes"] - base
+        ctx.set_dataset_budget(base + one + one // 2)
+        dss.append(ctx.dataset(pair[1][0], pair[1][1], K))
+        assert ctx.dataset_stats()["resident"] == 2
+        dbc = rs.DeviceBatch.from_host(bc)
+        backlog = [ctx.submit(third, dbc) for _ in range(24)]
+        for rnd in range(12):
+            i = rnd & 1
+            _, _, b, want = pair[i]
+            out = ctx.poll(ctx.submit(dss[i], rs.HostBatch(b)), b.P, K, timeout_us=60_000_000)
+            assert np.array_equal(out[0], want[0]), rnd
+            assert np.array_equal(out[1], want[1].reshape(-1, K)), rnd
+        assert ctx.dataset_stats()["rebuilds"] >= 11
+        assert ctx.poll(backlog[-1], bc.P, 4, timeout_us=0) is None     # the kernel was busy throughout
+        counts = [ctx.poll(t, bc.P, 4, timeout_us=60_000_000)[0] for t in backlog]
+        c, _, _ = ctx.eval_hard(third, rs.HostBatch(bc), 4)
+        for got in counts:
+            assert np.array_equal(got, c)
+    finally:
+        ctx.close()
+
+
 @pytest.mark.parametrize("reject", (False, True))
 def test_dropped_dataset_memory_is_given_back(reject):
     """A context keeps at most 256 MiB of dropped datasets' memory mapped (rs.h); the rest is free for
