@@ -667,7 +667,9 @@ static bool reap_marks(Ctx *ctx, Dataset &d)
 void mark_dataset_use(Ctx *ctx, Dataset *ds, cudaStream_t stream, bool may_create)
 {
     std::lock_guard<std::mutex> lk(ctx->mu);
-    if (!ctx->ds_budget) return;
+    // without a host copy it is never evicted; with one it is marked under no budget too: a budget set
+    // while the call's work is still queued must not take its memory
+    if (!ctx->ds_budget && ds->hy.empty()) return;
     reap_marks(ctx, *ds);
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) { cudaGetLastError(); cap = cudaStreamCaptureStatusActive; }

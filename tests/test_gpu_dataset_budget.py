@@ -152,6 +152,36 @@ def test_serving_request_pins_its_dataset(orc):
         ctx.close()
 
 
+def test_work_queued_without_a_budget_is_waited_for(orc):
+    """A dataset with a host copy, used by an asynchronous call while no budget is set: a budget set
+    before that work has run does not take the memory from under it."""
+    import torch
+    from paper_2406_01821_gb300 import rs
+    ctx = _budget_ctx(flags=rs.CTX_ASYNC)
+    try:
+        (X, y, b), (X2, y2, _) = _data(0), _data(1)
+        want = orc.eval_hard(X, y, K, b)
+        ds = ctx.dataset(X, y, K)
+        ctx.set_dataset_budget(0)
+        db = rs.DeviceBatch.from_host(b)
+        stream = torch.cuda.Stream()
+        c = torch.empty(b.P, dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
+        with torch.cuda.stream(stream):
+            torch.cuda._sleep(200_000_000)         # some 0.1 s before the call's kernels
+        ctx.eval_hard(ds, db, K, out=(c, None, None), stream=stream)
+        ctx.set_dataset_budget(1)
+        assert not stream.query() and ctx.dataset_stats()["evictions"] == 0
+        other = ctx.dataset(X2, y2, K)             # would take the evicted dataset's place
+        rs.check(rs.lib().rs_check(ctx.h, rs._stream_ptr(stream)))
+        assert np.array_equal(c.cpu().numpy(), want[0])
+        ctx.dataset_destroy(other)
+        ctx.set_dataset_budget(1)                  # the work has completed: evicted now
+        assert ctx.dataset_stats()["evictions"] == 1
+    finally:
+        ctx.close()
+
+
 @pytest.mark.parametrize("finite", (True, False))
 def test_eviction_under_a_live_serving_kernel(orc, finite):
     """Two datasets of one shape and different labels take each other's place in device memory while
