@@ -27,6 +27,7 @@
 #include "eval_core.cuh"
 #include "eval_rank.cuh"
 #include "rs_internal.cuh"
+#include "serve_close.h"
 #include "serve_sched.h"
 
 namespace rs {
@@ -84,11 +85,18 @@ struct ServeArgs {
     const volatile int32_t *active;         // [MAX_SLOTS] active slots (a hint; claims decide)
     const volatile int32_t *nactive;
     unsigned long long *last_claim;         // globaltimer of the latest claim
-    int32_t *busy;                          // CTAs that hold or are taking a unit
-    int32_t *closed;                        // set once: nothing is claimed any more, every CTA leaves
+    int32_t *life;                          // CTAs that hold or are taking a unit, and the closed bit (serve_close.h)
     int32_t *done;                          // [MAX_SLOTS] units finished per slot
     volatile unsigned long long *host_flag; // mapped host memory [MAX_SLOTS]: finished epoch
     const volatile int32_t *stop;           // mapped host memory
+};
+
+// The life word on device atomics.
+struct LifeWord {
+    int32_t *p;
+    __device__ __forceinline__ int add(int d) { return atomicAdd(p, d); }
+    __device__ __forceinline__ int cas(int e, int d) { return atomicCAS(p, e, d); }
+    __device__ __forceinline__ int load() { return *reinterpret_cast<volatile int32_t *>(p); }
 };
 
 __device__ __forceinline__ uint64_t now_ns()
@@ -199,6 +207,7 @@ __global__ void __launch_bounds__(SW * 32, 1) k_serve(ServeArgs a)
     __shared__ ReqDesc sd;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint4 *st = stage_all + warp * 64;
+    LifeWord word{a.life};
     if (threadIdx.x == 0) *reinterpret_cast<volatile unsigned long long *>(a.last_claim) = now_ns();
 
     while (true) {
@@ -231,11 +240,7 @@ __global__ void __launch_bounds__(SW * 32, 1) k_serve(ServeArgs a)
                     bool closed = false;
                     if (lane == 0) {
                         sl = a.active[i];
-                        // busy is raised before the flag is read, and the flag set before busy is read: a
-                        // closing CTA sees this one or is seen by it
-                        atomicAdd(a.busy, 1);
-                        __threadfence();
-                        closed = *reinterpret_cast<volatile int32_t *>(a.closed) != 0;
+                        closed = !life::enter(word);
                         if (!closed && sl >= 0 && sl < MAX_SLOTS) {
                             unsigned long long w = *reinterpret_cast<volatile unsigned long long *>(a.claims + sl);
                             while (((w >> CW_NEXT) & CW_MASK) < (w & CW_MASK)) {
@@ -246,8 +251,8 @@ __global__ void __launch_bounds__(SW * 32, 1) k_serve(ServeArgs a)
                         }
                     }
                     if (lane == 0) {
-                        if (got < 0) atomicSub(a.busy, 1);
-                        else *reinterpret_cast<volatile unsigned long long *>(a.last_claim) = now_ns();
+                        if (got >= 0) *reinterpret_cast<volatile unsigned long long *>(a.last_claim) = now_ns();
+                        else if (!closed) life::leave(word);
                     }
                     if (__shfl_sync(core::FULL, closed ? 1 : 0, 0)) break;
                     got = __shfl_sync(core::FULL, got, 0);
@@ -258,11 +263,7 @@ __global__ void __launch_bounds__(SW * 32, 1) k_serve(ServeArgs a)
                 if (lane == 0) {
                     const unsigned long long last = *reinterpret_cast<volatile unsigned long long *>(a.last_claim);
                     const unsigned long long tn = now_ns();
-                    leave = *reinterpret_cast<volatile int32_t *>(a.closed) != 0;
-                    if (!leave && tn > last && tn - last > IDLE_NS && *reinterpret_cast<volatile int32_t *>(a.busy) == 0) {
-                        atomicExch(a.closed, 1);
-                        leave = 1;
-                    }
+                    leave = life::closed(word) || (tn > last && tn - last > IDLE_NS && life::close(word));
                 }
                 if (__shfl_sync(core::FULL, leave, 0)) break;
                 __nanosleep(2000);
@@ -298,7 +299,7 @@ __global__ void __launch_bounds__(SW * 32, 1) k_serve(ServeArgs a)
                     __threadfence_system();
                     a.host_flag[slot] = d.epoch;
                 }
-                atomicSub(a.busy, 1);
+                life::leave(word);
             }
             __syncthreads();
             continue;
@@ -367,7 +368,7 @@ __global__ void __launch_bounds__(SW * 32, 1) k_serve(ServeArgs a)
                 __threadfence_system();
                 a.host_flag[slot] = d.epoch;
             }
-            atomicSub(a.busy, 1);
+            life::leave(word);
         }
         __syncthreads();
     }
@@ -467,7 +468,7 @@ struct Server {
     ReqDesc *d_table = nullptr;
     unsigned long long *d_claims = nullptr;
     int32_t *d_active = nullptr;           // [MAX_SLOTS + 1]: list, then its length
-    unsigned long long *d_life = nullptr;  // last claim; busy and closed (ServeArgs)
+    unsigned long long *d_life = nullptr;  // last claim; life word (ServeArgs)
     std::vector<int32_t> h_active;         // host copy of the active list
     cudaStream_t cstream = nullptr;        // completion copies
     int32_t *d_done = nullptr;
@@ -1000,9 +1001,9 @@ void CudaBackend::launch_kernel()
     // the descriptors and ring entries must be in place before the kernel starts
     cudaStreamWaitEvent(s->kstream, s->sch.active.back()->ev, 0);
     cudaMemsetAsync(s->d_life, 0, 16, s->kstream);
-    int32_t *words = reinterpret_cast<int32_t *>(s->d_life + 1);
-    ServeArgs a{s->d_table, s->d_claims, s->d_active, s->d_active + MAX_SLOTS, s->d_life, words, words + 1, s->d_done,
-                (volatile unsigned long long *)s->h_flag, (volatile int32_t *)s->h_stop};
+    ServeArgs a{s->d_table, s->d_claims, s->d_active, s->d_active + MAX_SLOTS, s->d_life,
+                reinterpret_cast<int32_t *>(s->d_life + 1), s->d_done, (volatile unsigned long long *)s->h_flag,
+                (volatile int32_t *)s->h_stop};
     k_serve<<<s->grid, SW * 32, s->smem, s->kstream>>>(a);
     cudaEventRecord(s->kevent, s->kstream);
     count_launch(s->ctx);
