@@ -489,11 +489,11 @@ rs_status rs_selftest_log1p_unit(rs_ctx *ctx, const float *e, int32_t n, float *
 rs_status rs_selftest_log1m_exp(rs_ctx *ctx, const float *s, int32_t n, float *out);
 
 /*
- * Fault injection on the host: of the per-call device allocations of the evaluation paths
- * (rs_eval_hard, rs_eval_soft_fwd/bwd, serving admission), the next `skip` succeed and the `count`
- * after them fail as if the device were out of memory (process-wide; count 0 disarms). A call
- * whose allocation fails returns RS_ERR_OOM having released whatever it had taken; serving keeps
- * the request queued and admits it once allocations succeed again.
+ * Fault injection on the host: of the device allocations of dataset registration and of the calls
+ * of the evaluation paths (rs_eval_hard, rs_eval_soft_fwd/bwd, serving admission), the next `skip`
+ * succeed and the `count` after them fail as if the device were out of memory (process-wide;
+ * count 0 disarms). A call whose allocation fails returns RS_ERR_OOM having released whatever it
+ * had taken; serving keeps the request queued and admits it once allocations succeed again.
  */
 rs_status rs_inject_alloc_failures(int32_t skip, int32_t count);
 

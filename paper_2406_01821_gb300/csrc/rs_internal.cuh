@@ -28,8 +28,8 @@ rs_status cuda_fail(cudaError_t e, const char *what);
     } while (0)
 
 // Host-side fault injection (tests): rs_inject_alloc_failures(skip, count) lets the next `skip`
-// per-call device allocations of the evaluation paths succeed and makes the `count` after them
-// fail as if the device were out of memory.
+// device allocations of dataset registration and of the evaluation paths' calls succeed and makes the
+// `count` after them fail as if the device were out of memory.
 bool take_injected_alloc_failure();
 inline cudaError_t dev_alloc_async(void **p, size_t bytes, cudaStream_t stream)
 {

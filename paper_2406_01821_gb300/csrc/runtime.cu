@@ -512,7 +512,7 @@ void dataset_pool_destroy(Ctx *ctx)
 template <class T>
 static cudaError_t ds_alloc(Ctx *ctx, T **p, size_t bytes)
 {
-    const cudaError_t e = cudaMallocFromPoolAsync(reinterpret_cast<void **>(p), bytes, ctx->ds_pool, ctx->ds_stream);
+    const cudaError_t e = dev_alloc_pool_async(p, bytes, ctx->ds_pool, ctx->ds_stream);
     if (e != cudaSuccess) { *p = nullptr; return e; }
     return cudaStreamSynchronize(ctx->ds_stream);
 }
@@ -569,7 +569,6 @@ static rs_status build_device(Ctx *ctx, Dataset &d, const float *X, const int32_
     d.perm = reinterpret_cast<int32_t *>(own + o_perm);
     d.inv = reinterpret_cast<int32_t *>(own + o_inv);
     d.flags = reinterpret_cast<uint32_t *>(own + o_flags);
-    if (rank_tables) REG_CUDA(ds_alloc(ctx, &d.Rk, (size_t)d.n_pad * F));
     at = 0;
     // the status words and the class counts, read back together
     const size_t o_st = take(16 + sizeof(int64_t) * (size_t)K), o_start = take(sizeof(int64_t) * (size_t)K),
@@ -577,6 +576,13 @@ static rs_status build_device(Ctx *ctx, Dataset &d, const float *X, const int32_
     const size_t o_xd = mem == RS_MEM_HOST ? take(sizeof(float) * (size_t)N * F) : 0,
                  o_yd = mem == RS_MEM_HOST ? take(sizeof(int32_t) * (size_t)N) : 0;
     REG_CUDA(ds_alloc(ctx, &tmp, at));
+    // The rank table comes last and is not insisted on before the data is known to be finite: data that
+    // turns out not to be needs no memory for it.
+    cudaError_t rank_alloc = cudaSuccess;
+    if (rank_tables && (rank_alloc = ds_alloc(ctx, &d.Rk, (size_t)d.n_pad * F)) != cudaSuccess) {
+        if (rank_alloc != cudaErrorMemoryAllocation) REG_CUDA(rank_alloc);
+        cudaGetLastError();
+    }
     uint32_t *st = reinterpret_cast<uint32_t *>(tmp + o_st);
     int64_t *ctot = reinterpret_cast<int64_t *>(tmp + o_st + 16), *cstart = reinterpret_cast<int64_t *>(tmp + o_start);
     int32_t *blk = reinterpret_cast<int32_t *>(tmp + o_blk), *rank = reinterpret_cast<int32_t *>(tmp + o_rank);
@@ -613,6 +619,7 @@ static rs_status build_device(Ctx *ctx, Dataset &d, const float *X, const int32_
     std::memcpy(d.class_count.data(), back.data() + 16, sizeof(int64_t) * (size_t)K);
     d.finite = hst[1] == 0;
     d.ncode = (int32_t)hst[2];
+    if (d.finite) REG_CUDA(rank_alloc);
     d.ranked = d.finite && rank_tables;
     if (!d.ranked && d.Rk) { ds_free(ctx, d.Rk); d.Rk = nullptr; }
     ds_free(ctx, tmp);

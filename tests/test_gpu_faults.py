@@ -114,3 +114,27 @@ def test_serving_retries_admission_and_relaunches_after_idle(orc):
     finally:
         lib.rs_inject_alloc_failures(0, 0)
         c.close()
+
+
+@pytest.mark.parametrize("finite", (True, False))
+def test_registration_with_failing_allocations(ctx, orc, finite):
+    """The dataset, its temporary arrays and its rank table fail to be allocated in turn: RS_ERR_OOM, but
+    for the rank table of data that is not finite, which has none."""
+    from paper_2406_01821_gb300 import rs
+    X, y, K, b = small_case(4)
+    if not finite:
+        X[::41, 5] = np.inf
+    lib = rs.lib()
+    try:
+        for skip in range(3 if finite else 2):
+            lib.rs_inject_alloc_failures(skip, 1)
+            with pytest.raises(rs.RsError) as e:
+                ctx.dataset(X, y, K)
+            assert e.value.code == -3
+        lib.rs_inject_alloc_failures(3 if finite else 2, 1)
+        ds = ctx.dataset(X, y, K)
+        lib.rs_inject_alloc_failures(0, 0)
+        check_counts(ctx, orc, X, y, K, b, ds)
+        ctx.dataset_destroy(ds)
+    finally:
+        lib.rs_inject_alloc_failures(0, 0)
