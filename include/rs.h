@@ -99,17 +99,18 @@ rs_status rs_check(rs_ctx *ctx, void *stream);
  *   y      int32[N], labels in 0..K-1
  *   N >= 1, 1 <= F <= RS_MAX_FEATURES, 1 <= K <= RS_MAX_CLASSES
  * The library keeps its own copy (feature-major, samples grouped by label); the caller may free X
- * and y when the call returns. Device memory held: 4 bytes per value and 12 per sample (labels,
- * order), N rounded up to 256, plus for finite data with F <= 128 one byte per value (the rank of
- * each value within its 128-sample tile, for the rank-coded evaluator).
+ * and y when the call returns. Device memory held: 4 bytes per value, 12 per sample (labels,
+ * order) and 4 per feature, N rounded up to 256, plus for finite data with F <= 128 one byte per
+ * value (the rank of each value within its 128-sample tile, for the rank-coded evaluator).
  * Errors: RS_ERR_INVALID (sizes, a label out of range), RS_ERR_OOM.
  * On success *ds_out receives a non-zero handle.
  */
 rs_status rs_dataset_create(rs_ctx *ctx, const float *X, const int32_t *y, int64_t N, int32_t F,
                             int32_t K, int32_t mem, void *stream, uint64_t *ds_out);
 /*
- * Unregister a dataset and free its device copy (and its host copy under a dataset budget; up to
- * 256 MiB of freed dataset memory stays with the context for the next registration). The
+ * Unregister a dataset and free its device copy (and its host copy under a dataset budget). The
+ * context holds on to memory for its next registrations: what its datasets and freed dataset memory
+ * take together, up to 256 MiB (a smaller dataset budget: up to that), stays with it. The
  * device's queued work completes first, so no call enqueued earlier on any stream still reads it.
  * Errors: RS_ERR_NOT_FOUND (unknown handle); RS_ERR_INVALID while the dataset is in use: a call on
  * it is running in another thread, or a serving request on it has not been polled yet (queued,
@@ -133,7 +134,8 @@ rs_status rs_dataset_info(rs_ctx *ctx, uint64_t ds, int64_t *N, int32_t *F, int3
  * (an event on its stream); a dataset whose marked work is still pending (calls of asynchronous
  * contexts) is not chosen, and only work no mark covers (calls on a stream being captured) makes
  * an eviction wait for the whole device. rs_eval_hard_static, which allocates nothing, returns
- * RS_ERR_INVALID on an evicted dataset. Lowering the budget evicts at once.
+ * RS_ERR_INVALID on an evicted dataset. Lowering the budget evicts at once, and freed memory that the
+ * context holds on to beyond it goes back to the driver.
  */
 rs_status rs_set_dataset_budget(rs_ctx *ctx, uint64_t bytes);
 

@@ -241,8 +241,8 @@ struct Ctx {
     uint32_t *d_sticky = nullptr;            // async-mode sticky device status
     unsigned char *static_scratch = nullptr; // device address of rs_eval_hard_static's fixed array
     unsigned long long *d_walked = nullptr;  // [4] walked-work counters (RS_CTX_COUNT_WORK contexts)
-    // Memory of the datasets and of their registration: a pool of the context's own that keeps up to
-    // DATASET_POOL_KEEP bytes of freed memory mapped until the context is destroyed (mapping and
+    // Memory of the datasets and of their registration: a pool of the context's own that holds on to
+    // DATASET_POOL_KEEP bytes (a smaller dataset budget: to that) when datasets are dropped (mapping and
     // unmapping 150 MB took 200 us of registering 300,007 x 96 and 130 of dropping it). Allocations
     // and frees go through a stream of their own, waited for, so that the memory is usable on any.
     cudaMemPool_t ds_pool = nullptr;

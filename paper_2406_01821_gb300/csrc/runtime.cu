@@ -628,10 +628,11 @@ static rs_status build_device(Ctx *ctx, Dataset &d, const float *X, const int32_
     return RS_OK;
 }
 
-static size_t dataset_device_bytes(const Dataset &d)
+// Device bytes of a dataset: features, labels, order and its inverse, flags, rank table.
+static size_t dataset_device_bytes(int64_t N, int64_t n_pad, int32_t F, bool rank_table)
 {
-    return sizeof(float) * (size_t)d.n_pad * d.F + sizeof(int32_t) * ((size_t)d.n_pad + 2 * (size_t)d.N) +
-           (d.Rk ? (size_t)d.n_pad * d.F : 0);
+    return sizeof(float) * (size_t)n_pad * F + sizeof(int32_t) * ((size_t)n_pad + 2 * (size_t)N + (size_t)F) +
+           (rank_table ? (size_t)n_pad * F : 0);
 }
 
 static void free_device(Ctx *ctx, Dataset &d)
@@ -758,11 +759,8 @@ rs_status dataset_create(Ctx *ctx, const float *X, const int32_t *y, int64_t N, 
     {
         std::lock_guard<std::mutex> lk(ctx->mu);
         budget = ctx->ds_budget != 0;
-        if (budget) {                 // room for the largest form it can take (with a rank table)
-            const size_t upper = sizeof(float) * (size_t)ds->n_pad * F + sizeof(int32_t) * ((size_t)ds->n_pad + 2 * (size_t)N) +
-                                 (F <= RANK_MAX_F ? (size_t)ds->n_pad * F : 0);
-            make_room(ctx, upper, 0);
-        }
+        if (budget)                   // room for the largest form it can take (with a rank table)
+            make_room(ctx, dataset_device_bytes(N, ds->n_pad, F, F <= RANK_MAX_F), 0);
     }
     if (budget) {                     // the host copy an eviction rebuilds from
         ds->hX.resize((size_t)N * F);
@@ -774,7 +772,7 @@ rs_status dataset_create(Ctx *ctx, const float *X, const int32_t *y, int64_t N, 
     }
     const rs_status rc = build_device(ctx, *ds, X, y, mem, stream);
     if (rc) return rc;
-    ds->dev_bytes = dataset_device_bytes(*ds);
+    ds->dev_bytes = dataset_device_bytes(N, ds->n_pad, F, ds->Rk != nullptr);
     std::lock_guard<std::mutex> lk(ctx->mu);
     const uint64_t h = ctx->next_ds++;
     ds->last_use = ++ctx->ds_tick;
@@ -811,6 +809,9 @@ rs_status set_dataset_budget(Ctx *ctx, uint64_t bytes)
 {
     std::lock_guard<std::mutex> lk(ctx->mu);
     ctx->ds_budget = bytes;
+    // the pool keeps no more mapped than a budget allows
+    uint64_t keep = bytes ? std::min<uint64_t>(bytes, DATASET_POOL_KEEP) : DATASET_POOL_KEEP;
+    RS_CUDA(cudaMemPoolSetAttribute(ctx->ds_pool, cudaMemPoolAttrReleaseThreshold, &keep));
     // spare marks, so that calls that may not create one (the allocation-free entry) find one
     while (bytes && ctx->ds_events.size() < 32) {
         cudaEvent_t e = nullptr;
@@ -818,6 +819,7 @@ rs_status set_dataset_budget(Ctx *ctx, uint64_t bytes)
         ctx->ds_events.push_back(e);
     }
     make_room(ctx, 0, 0);
+    if (bytes) RS_CUDA(cudaMemPoolTrimTo(ctx->ds_pool, keep));
     return RS_OK;
 }
 

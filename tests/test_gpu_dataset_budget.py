@@ -224,6 +224,31 @@ def test_eviction_under_a_live_serving_kernel(orc, finite):
         ctx.close()
 
 
+def test_a_small_budget_holds_on_to_no_more(orc):
+    """Freed dataset memory that a context holds on to counts towards a budget below 256 MiB. 64 MiB
+    allow for the pool's granularity and other processes' noise; the dataset takes 0.25 GiB."""
+    import torch
+    from paper_2406_01821_gb300 import rs
+    ctx = _budget_ctx()
+    try:
+        X, y, b = _data(0)
+        want = orc.eval_hard(X, y, K, b)
+        small = ctx.dataset(X, y, K)
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        big = ctx.dataset(np.zeros((1 << 19, 96), np.float32), np.zeros(1 << 19, np.int32), 2)
+        assert before - torch.cuda.mem_get_info()[0] >= 4 * 96 << 19
+        ctx.eval_hard(small, rs.HostBatch(b), K)   # the more recent of the two
+        ctx.set_dataset_budget(16 << 20)           # evicts the large one
+        assert ctx.dataset_stats()["resident"] == 1
+        assert before - torch.cuda.mem_get_info()[0] <= 64 << 20
+        c, _, _ = ctx.eval_hard(small, rs.HostBatch(b), K)
+        assert np.array_equal(c, want[0])
+        ctx.dataset_destroy(big)
+    finally:
+        ctx.close()
+
+
 @pytest.mark.parametrize("reject", (False, True))
 def test_dropped_dataset_memory_is_given_back(reject):
     """A context keeps at most 256 MiB of dropped datasets' memory mapped (rs.h); the rest is free for
