@@ -14,6 +14,7 @@
 // Compiled without FMA contraction; every product is an explicit round-to-nearest multiply and
 // every compare is an IEEE ordered compare, so results equal the plain definition bit for bit.
 #include "rs_internal.cuh"
+#include "tile_split.h"
 #include "tma.cuh"
 
 namespace rs {
@@ -383,13 +384,7 @@ int split_tiles(Ctx *ctx, int64_t N, int F, int P, int S, int W, int resident, H
     const int64_t tiles = (N + S - 1) / S, slots = (int64_t)ctx->sm_count * std::max(1, resident);
     const int64_t rest = tiles % slots;
     a.whole = (int32_t)(tiles - rest);
-    a.groups = 1;
-    int64_t best = INT64_MAX;
-    for (int64_t g = 1; rest && g <= std::max(1, (P + W - 1) / W); ++g) {
-        const int64_t sets = (P + g - 1) / g;
-        const int64_t cost = (rest * g + slots - 1) / slots * (64 + F / 3 + (sets + W - 1) / W * W);
-        if (cost < best) { best = cost; a.groups = (int32_t)g; }
-    }
+    a.groups = (int32_t)split_groups(rest, slots, P, W, 64 + F / 3);
     return (int)(a.whole + rest * a.groups);
 }
 

@@ -130,8 +130,8 @@ rs_status launch4_t(Ctx *ctx, Dataset *ds, HardArgs a, cudaStream_t stream)
     if (attr_err != cudaSuccess) return cuda_fail(attr_err, "cudaFuncSetAttribute(k_hard4)");
     const CUtensorMap *tm = dataset_tmap(ds, 32 * V);
     if (!tm) return RS_ERR_DEVICE;
-    int resident = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, k_hard4<V, W>, W * 32, smem);
+    static std::atomic<uint64_t> asked{0};
+    const int resident = resident_ctas(asked, k_hard4<V, W>, W * 32, smem);
     const int grid = split_tiles(ctx, a.N, a.F, a.P, 32 * V, W, resident, a);
     {
         TimedLaunch tl(ctx, TK_HARD, stream);

@@ -215,8 +215,8 @@ static rs_status launch5_t(Ctx *ctx, Dataset *ds, HardArgs a, cudaStream_t strea
     const CUtensorMap *tmx = dataset_tmap(ds, T);
     const CUtensorMap *tmr = DIRECT ? tmx : dataset_rank_tmap(ds);
     if (!tmx || !tmr) return RS_ERR_DEVICE;
-    int resident = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, k_hard5<W, CAT, PRED, DIRECT>, W * 32, smem);
+    static std::atomic<uint64_t> asked{0};
+    const int resident = resident_ctas(asked, k_hard5<W, CAT, PRED, DIRECT>, W * 32, smem);
     const int grid = split_tiles(ctx, a.N, a.F, a.P, T, W, resident, a);
     {
         TimedLaunch tl(ctx, TK_HARD, stream);
