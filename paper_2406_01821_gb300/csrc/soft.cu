@@ -590,9 +590,11 @@ __device__ __forceinline__ void soft_group_ff(const SoftKArgs &a, int p, int rb,
 // with D = prod (1 + E) and z = D - 1,
 //     q = 1 / D,    1 - q = z / D    (taken as 1 - q itself where q < 1/2),
 // and z follows its own recursion z' = z + E D of positive terms, so that 1 - q keeps its relative
-// accuracy where q rounds to 1. D beyond 1.6e38 counts as q = 0 (an infinite D that meets an E of 0,
-// a margin beyond 87, turns into a NaN, and its group takes the float-float pass, as one does whose
-// margins are not numbers).
+// accuracy where q rounds to 1. D beyond 1.6e38 counts as q = 0. E enters D and z with the smallest
+// subnormal added, which only an E below 2^-124 notices (and 1 - q drops again): an infinite D stays
+// infinite when it meets an E that came out 0 (a margin beyond 87), where 0 x inf would make a NaN and
+// send the group to the float-float pass, whatever its p_y. (Accurate sets at a temperature of 0.02, 256
+// of 6 rules on 100,000 x 32: 25 ms with nearly every group there, 0.93 so.) A group whose margins are not numbers still goes there.
 // Everything after it is a sum of products of positive numbers as well: U_r = prod_{j<r} (1 - q_j),
 // p_y and 1 - p_y over the rules, S_r and T_r backwards (S_r = [same] q + (1 - q) S_{r+1}, T_r with
 // the other rules), and d ell / d log q_r = q_r U_r (S_{r+1} or -T_{r+1}) / p_y. No logarithm and no
@@ -612,11 +614,12 @@ __device__ __forceinline__ void soft_group_ff(const SoftKArgs &a, int p, int rb,
 // cost about 13 with its accumulator update. Forward + adjoint of 1024 sets x 32 rules x 4 conditions
 // on 262,144 samples: 139.7 ms in the log domain with two samples a lane (238 warp instructions per
 // condition and 64 samples), 70.3 ms so with U_r in tensor memory (123), 45.6 ms with E = e^-u in
-// place of e^-|u| and its sign and four samples a lane (72, issue slots 68 % busy at 16 warps an SM),
-// 44.6 ms with the caps taken off the forward's E.
+// place of e^-|u| and its sign and four samples a lane (72, issue slots 68 % busy at 16 warps an SM;
+// 44.6 without anything against inf x 0).
 constexpr int SOFT_SEG = 32;               // conditions per piece of a rule
 constexpr float SOFT_D_MAX = 1.6e38f;      // D from which q is 0 (above 2^126: its reciprocal is subnormal)
-constexpr float SOFT_E_MAX = 1e38f;        // E above which 1 / (1 + E) would come out 0
+constexpr float SOFT_E_MAX = 8e37f;        // cap of E in E / (1 + E), whose reciprocal comes out 0 above 2^126
+constexpr float SOFT_E_ADD = 1.4e-45f;     // the smallest subnormal: keeps E above 0 in D and z
 constexpr int SOFT_NV_TILE = 2, SOFT_NV = 1;    // float2 per lane: staged-tile and per-warp kernel
 constexpr int SOFT_CACHE = 4;              // conditions of a rule whose e the adjoint keeps in registers
 constexpr int SOFT_GROWS = 16;             // conditions per gradient table
@@ -710,6 +713,17 @@ __device__ __forceinline__ float rcp_ftz(float x)
 
 __device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
 
+// Products with subnormal operands and results taken as 0.
+__device__ __forceinline__ float2 mul2_ftz(float2 a, float2 b)
+{
+    float2 r;
+    asm("{\n\t.reg .b64 a, b, r;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmul.rn.ftz.f32x2 r, a, b;\n\t"
+        "mov.b64 {%0, %1}, r;\n\t}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+
 // Tensor memory as a per-warp array of Vec (2 NV columns each; a warp reaches its own 32 lanes).
 template <int NV>
 __device__ __forceinline__ void tmem_put(uint32_t at, const Vec<NV> &u)
@@ -790,8 +804,9 @@ struct SoftProd {
     {
 #pragma unroll
         for (int i = 0; i < NV; ++i) {
-            z[i] = __ffma2_rn(e.v[i], D[i], z[i]);
-            D[i] = __ffma2_rn(e.v[i], D[i], D[i]);
+            const float2 E = __fadd2_rn(e.v[i], f2(SOFT_E_ADD));
+            z[i] = __ffma2_rn(E, D[i], z[i]);
+            D[i] = __ffma2_rn(E, D[i], D[i]);
         }
     }
     // a membership test: its exact indicator
@@ -819,7 +834,7 @@ struct SoftProd {
             if (CAT && ((dead >> (2 * i)) & 2u)) r.y = 0.f;
             q.v[i] = r;
             // 1 - q rounded once where q < 1/2, else the quotient, which keeps a small 1 - q
-            w.v[i] = __fmul2_rn(z[i], r);
+            w.v[i] = mul2_ftz(z[i], r);                  // the added subnormals alone: 0
             const float2 v = __ffma2_rn(r, f2(-1.f), f2(1.f));
             if (r.x < 0.5f) w.v[i].x = v.x;
             if (r.y < 0.5f) w.v[i].y = v.y;
@@ -982,7 +997,7 @@ __device__ __forceinline__ bool soft_group(const SoftKArgs &a, const SoftWarp &m
     }
     add_class(deflt, U);
     // every q_r went into p_y or 1 - p_y: a NaN anywhere shows in one of them (looked for beyond the
-    // data's end too, where the features are zeros: a NaN times a weight of 0 would spoil the sums)
+    // data's end too, where a NaN times a weight of 0 would spoil the sums)
     bool big = false;
 #pragma unroll
     for (int i = 0; i < NV; ++i)

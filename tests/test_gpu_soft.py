@@ -415,3 +415,65 @@ def test_soft_far_samples_and_ragged_end(ctx, orc, N, F, P, R, C, far, tau):
     ref = orc.soft(X, y, 2, b, tau, dloss=dl, want_probs=True, want_mag=True)
     check_against_oracle(got, ref)
     assert np.allclose(got["probs"], ref["probs"], rtol=RTOL, atol=1e-30)
+
+
+def accurate_case(N, F, P, shift, seed):
+    """Well separated classes and sets that classify them: each rule tests one of four features whose
+    class means are `shift` apart, the first four rules two noise features beside it."""
+    rng = np.random.default_rng(seed)
+    y = rng.integers(0, 2, N).astype(np.int32)
+    X = rng.standard_normal((N, F)).astype(np.float32)
+    X[:, :4] += np.float32(shift) * y[:, None]
+    sets = []
+    for _ in range(P):
+        rules = []
+        for j in range(6):
+            c = j % 2
+            conds = [(int(rng.integers(0, 4)), -1, synth.GT if c else synth.LT, np.float32(1), 0.0,
+                      np.float32(shift * rng.uniform(0.35, 0.65)))]
+            for _ in range(2 if j < 4 else 0):
+                conds.append((int(rng.integers(4, F)), -1, int(rng.integers(0, 2)), np.float32(1), 0.0,
+                              np.float32(0.7 * rng.normal())))
+            rules.append((c, conds))
+        sets.append(rules)
+    return X, y, synth.from_lists(sets, [int(v) for v in rng.integers(0, 2, P)])
+
+
+@pytest.mark.parametrize("N,F,P,tau", [(1003, 8, 12, 0.03), (1003, 130, 7, 0.02), (517, 5, 20, 0.005)])
+def test_soft_sharp_accurate_sets_vs_oracle(ctx, orc, N, F, P, tau):
+    """Margins of hundreds of tau of both signs in one rule on samples that are classified well. Some
+    losses are far below 2^-53, where the oracle's own rounding near log 1 (a few units of 2^-53 a rule)
+    is all that it returns: `eps` allows for it, in the gradients times x / tau."""
+    X, y, b = accurate_case(N, F, P, 10.0, 31)
+    dl = np.random.default_rng(31).uniform(0.5, 2, b.P)
+    got = soft_gpu(ctx, X, y, 2, b, tau, dl, probs=True)
+    ref = orc.soft(X, y, 2, b, tau, dloss=dl, want_probs=True, want_mag=True)
+    eps = 64 * 2.0 ** -53
+    assert np.allclose(got["loss"], ref["loss"], rtol=RTOL, atol=eps)
+    for n in ("a", "b", "t"):
+        g, r, m = got["grad_" + n], ref["grad_" + n], ref["mag_" + n]
+        assert (np.abs(g - r) <= RTOL * np.maximum(np.abs(r), m) + eps * 2 * np.abs(X).max() / tau).all(), n
+    assert np.allclose(got["probs"], ref["probs"], rtol=RTOL, atol=1e-30)
+
+
+def test_soft_sharp_accurate_sets_take_the_float_path(ctx):
+    """The same at a temperature of 0.02 and of 0.5, where no exponential leaves float32's range: at most
+    four times as long (one group in the float-float pass takes more than ten times as long)."""
+    import torch
+    from paper_2406_01821_gb300 import rs
+    X, y, b = accurate_case(50_000, 32, 256, 10.0, 37)
+    ds = ctx.dataset(X, y, 2)
+    try:
+        db, dl = rs.DeviceBatch.from_host(b), torch.ones(b.P, device="cuda")
+        ms = {}
+        for tau in (0.5, 0.02):
+            for rep in range(5):
+                e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+                e[0].record()
+                ctx.soft_bwd(ds, db, tau, dl)
+                e[1].record()
+                torch.cuda.synchronize()
+                ms[tau] = min(ms.get(tau, 1e9), e[0].elapsed_time(e[1]))
+        assert ms[0.02] <= 4 * ms[0.5], ms
+    finally:
+        ctx.dataset_destroy(ds)
