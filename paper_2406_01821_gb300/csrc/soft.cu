@@ -397,22 +397,6 @@ __device__ __forceinline__ CondIn load_cond(const SoftKArgs &a, int c, const XVi
     return t;
 }
 
-// f(condition) for c0 <= c < c1 in order, the loads of FF_BATCH conditions issued before the first of
-// them is used.
-constexpr int FF_BATCH = 4;
-template <class Fn>
-__device__ __forceinline__ void each_cond(const SoftKArgs &a, int c0, int c1, const XView &x, Fn f)
-{
-    for (int c = c0; c < c1; c += FF_BATCH) {
-        CondIn t[FF_BATCH];
-#pragma unroll
-        for (int i = 0; i < FF_BATCH; ++i) t[i] = load_cond(a, min(c + i, c1 - 1), x);
-#pragma unroll
-        for (int i = 0; i < FF_BATCH; ++i)
-            if (c + i < c1) f(t[i]);
-    }
-}
-
 // The signed scaled margin u = s * (a * x[f] - rhs) / tau of a condition for the lane's sample, in
 // float-float: the products are exact (a float times a float), 1/tau is a float-float.
 __device__ __forceinline__ ff margin_ff(const SoftKArgs &a, const CondIn &t)
@@ -437,14 +421,15 @@ template <bool CAT>
 __device__ ff rule_logq_ff(const SoftKArgs &a, int c0, int c1, const XView &x)
 {
     ff s{0.f, 0.f};
-    each_cond(a, c0, c1, x, [&](const CondIn &t) {
+    for (int c = c0; c < c1; ++c) {
+        const CondIn t = load_cond(a, c, x);
         if (CAT && (t.rc.meta & 4u)) {
             if (!category_member(t.xf, __float_as_uint(t.rc.a), __float_as_uint(t.rc.bt))) s = {-INFINITY, 0.f};
-            return;
+            continue;
         }
         float l1pe;
         s = ff_add(s, log_sigmoid_ff(margin_ff(a, t), l1pe));
-    });
+    }
     return s;
 }
 
@@ -463,17 +448,19 @@ __device__ ff rule_log1mq_ff(const SoftKArgs &a, int c0, int c1, const XView &x,
     if (lqf < -0.69314718f) return {log1pf(-expf(lqf)), 0.f};
     if (lqf < -0x1p-24f) return ff_log_unit(-expm1f(lqf));
     ff m{INFINITY, 0.f};
-    each_cond(a, c0, c1, x, [&](const CondIn &t) {
-        if (CAT && (t.rc.meta & 4u)) return;
+    for (int c = c0; c < c1; ++c) {
+        const CondIn t = load_cond(a, c, x);
+        if (CAT && (t.rc.meta & 4u)) continue;
         const ff u = margin_ff(a, t);
         if (ff_less(u, m)) m = u;
-    });
+    }
     if (m.hi == INFINITY) return {-INFINITY, 0.f};
     float acc = 0.f;
-    each_cond(a, c0, c1, x, [&](const CondIn &t) {
-        if (CAT && (t.rc.meta & 4u)) return;
+    for (int c = c0; c < c1; ++c) {
+        const CondIn t = load_cond(a, c, x);
+        if (CAT && (t.rc.meta & 4u)) continue;
         acc += expf(ff_f(ff_add(m, ff_neg(margin_ff(a, t)))));
-    });
+    }
     return ff_add_f(ff_neg(m), logf(acc));
 }
 
@@ -594,7 +581,8 @@ __device__ __forceinline__ void soft_group_ff(const SoftKArgs &a, int p, int rb,
 // subnormal added, which only an E below 2^-124 notices (and 1 - q drops again): an infinite D stays
 // infinite when it meets an E that came out 0 (a margin beyond 87), where 0 x inf would make a NaN and
 // send the group to the float-float pass, whatever its p_y. (Accurate sets at a temperature of 0.02, 256
-// of 6 rules on 100,000 x 32: 25 ms with nearly every group there, 0.93 so.) A group whose margins are not numbers still goes there.
+// of 6 rules on 100,000 x 32: 25 ms with nearly every group there, 0.93 so.) A group whose margins are
+// not numbers still goes there.
 // Everything after it is a sum of products of positive numbers as well: U_r = prod_{j<r} (1 - q_j),
 // p_y and 1 - p_y over the rules, S_r and T_r backwards (S_r = [same] q + (1 - q) S_{r+1}, T_r with
 // the other rules), and d ell / d log q_r = q_r U_r (S_{r+1} or -T_{r+1}) / p_y. No logarithm and no
@@ -1321,12 +1309,12 @@ __global__ void __maxnreg__(128) k_soft_tile(SoftKArgs a, int F)
 // (those it left out) in float-float (soft_group_ff), its loss and gradient sums Kahan-summed in their
 // order; the warps' sums are added to the task's partials in warp order, so that results do not depend
 // on the order of the list. Runs after the main kernel on the same stream; features are read from
-// global memory. What bounds it is the chain of one warp's conditions (a record, its features, the
-// arithmetic, one after another), hence the batched loads (each_cond) and one sample to a lane, four
-// warps to a group of 128. With two samples to a lane, one after the
-// other, and each condition's loads on their own, 88 us for the class probabilities of 48 sets on
-// 20,000 x 30 and 228 us for the adjoint of 64 on 100,000 x 32 where a few samples of every group lie
-// far out; 48 and 122 us so (twice the CTAs or batches of two loads were no faster).
+// global memory, one sample to a lane. Few marked groups are bound by the chain of one warp's conditions
+// (a record, its features, the arithmetic, one after another), hence four warps to a group of 128; many
+// by the warps that an SM holds, so that as many CTAs run as fit. (Every group of 256 sets of 6 rules on
+// 100,000 x 32: 12.5 ms; with the loads of four conditions issued together, whose unrolled code is four
+// times as long, 25, and with 4 CTAs an SM, 33; the loads ahead gain nothing for few groups either: 145 us
+// with and without for the class probabilities of 48 sets on 20,000 x 30.)
 template <bool BWD, bool CAT>
 __global__ void __launch_bounds__(SOFT_W * 32) k_soft_ff(SoftKArgs a)
 {
@@ -1571,6 +1559,16 @@ static void launch_soft_kernel(Ctx *ctx, const SoftKArgs &k, bool tiled, bool bw
     }
 }
 
+// The float-float pass: as many CTAs as the SMs hold, or as there are tasks.
+template <bool BWD, bool CAT>
+static void launch_soft_ff(Ctx *ctx, const SoftKArgs &k, size_t smem, cudaStream_t stream)
+{
+    static std::atomic<uint64_t> asked{0};
+    const int resident = std::max(1, resident_ctas(asked, k_soft_ff<BWD, CAT>, SOFT_W * 32, smem));
+    const int64_t grid = std::min<int64_t>((int64_t)k.P * k.nchunks, (int64_t)ctx->sm_count * resident);
+    k_soft_ff<BWD, CAT><<<(unsigned)grid, SOFT_W * 32, smem, stream>>>(k);
+}
+
 // Words of the float-float group bits for P sets over N samples, for any chunking of at most
 // SOFT_MAX_CHUNKS chunks: chunks x ceil(groups per chunk / 32) <= N / 2048 + 2 * SOFT_MAX_CHUNKS.
 static size_t ff_words(int P, int64_t N)
@@ -1771,17 +1769,15 @@ static rs_status soft_run(Ctx *ctx, const SoftArgs &s, int known_maxR, int known
             if (b.cond_set) launch_soft_kernel<true>(ctx, k, tiled, bwd, s.F, smem, per_warp, sh, stream);
             else launch_soft_kernel<false>(ctx, k, tiled, bwd, s.F, smem, per_warp, sh, stream);
         }
-        {   // groups beyond float32's resolution (usually none: the kernel's warps exit at once)
-            const unsigned ffgrid = (unsigned)std::min<int64_t>((int64_t)P * k.nchunks, (int64_t)ctx->sm_count * 4);
-            if (b.cond_set) {
-                if (bwd) k_soft_ff<true, true><<<ffgrid, SOFT_W * 32, smem_ff, stream>>>(k);
-                else k_soft_ff<false, true><<<ffgrid, SOFT_W * 32, smem_ff, stream>>>(k);
-            } else {
-                if (bwd) k_soft_ff<true, false><<<ffgrid, SOFT_W * 32, smem_ff, stream>>>(k);
-                else k_soft_ff<false, false><<<ffgrid, SOFT_W * 32, smem_ff, stream>>>(k);
-            }
-            count_launch(ctx);
+        // groups beyond float32's resolution (usually none: the kernel's warps exit at once)
+        if (b.cond_set) {
+            if (bwd) launch_soft_ff<true, true>(ctx, k, smem_ff, stream);
+            else launch_soft_ff<false, true>(ctx, k, smem_ff, stream);
+        } else {
+            if (bwd) launch_soft_ff<true, false>(ctx, k, smem_ff, stream);
+            else launch_soft_ff<false, false>(ctx, k, smem_ff, stream);
         }
+        count_launch(ctx);
         if (bwd)                      // the gradients and (when asked) the loss in one launch
             k_soft_reduce_grad<<<P, 128, 0, stream>>>(part_ga, part_gbt, part_loss, nchunks, b.set_rule_off,
                                                      b.rule_cond_off, recs, P, Ccap, s.dloss,
