@@ -43,8 +43,8 @@ constexpr int SOFT_W = 4;                 // warps per CTA
 constexpr int SOFT_MAX_RULES = 64;        // rules per set held in shared memory
 constexpr int SOFT_MAX_CONDS = 512;       // conditions per set accumulated in shared memory
 constexpr int SOFT_MAX_CHUNKS = 128;
-constexpr int SOFT_V = 2;                 // samples per lane; a group is 32 * SOFT_V samples
-constexpr int SOFT_G = 32 * SOFT_V;
+constexpr int SOFT_G = 64;                // chunks are whole multiples of it
+constexpr int SOFT_FF_GROUP = 64;         // samples that go to the float-float pass together
 // the call's counters: tasks taken, [1..2] most rules / conditions of a set, length of the
 // float-float list, list items taken
 constexpr int SOFT_NEXT_FF_LEN = 3, SOFT_NEXT_FF = 4, SOFT_NEXT_N = 8;
@@ -289,9 +289,8 @@ struct SoftKArgs {
     const uint32_t *status;          // no work if non-zero (malformed batch)
     const int32_t *order;            // sets by decreasing size (schedule only; results do not depend on it)
     int32_t *fflist;                 // [nchunks * P]: tasks (ch * P + p) with groups left to the float-float pass
-    uint32_t *ffbits;                // [nchunks][P][ff_wpt]: bit g of a task: its group g is one of them
-    int32_t ff_wpt;                  // words per task (groups per chunk / 32, rounded up)
-    int32_t group;                   // samples per group of the main kernel (a bit of ffbits)
+    uint32_t *ffbits;                // [nchunks][P][ff_wpt]: bit g of a task: its g-th SOFT_FF_GROUP samples are among them
+    int32_t ff_wpt;                  // words per task (SOFT_FF_GROUPs per chunk / 32, rounded up)
     int32_t pslots;                  // class-probability slots per warp (0: not written)
     int32_t teams;                   // teams per CTA (staged-tile kernel)
     uint32_t tm_cols;                // tensor-memory columns of a CTA (staged-tile adjoint)
@@ -919,11 +918,11 @@ __device__ __forceinline__ void cond_grads(const SoftWarp &m, int ci, int nconds
 
 // Forward (and adjoint) of a set of R rules over one group of 64 NV samples: lane l holds samples
 // n0 + 2 NV l + i (bit i of valid: the sample exists). tm: the warp's tensor-memory base
-// (staged-tile adjoint). Returns true, having added nothing, when some sample's p_y is below e^-64
-// or something is not a number: the group's bit is then set, and k_soft_ff evaluates it in float-float after
-// this kernel.
+// (staged-tile adjoint). Returns a bit for each SOFT_FF_GROUP of its samples from which nothing was added,
+// since some sample's p_y in it is below e^-64 (all of them when something is not a number): the bits go
+// to the task's list, and k_soft_ff evaluates these samples in float-float after this kernel.
 template <bool BWD, bool CAT, bool TILE, int NV>
-__device__ __forceinline__ bool soft_group(const SoftKArgs &a, const SoftWarp &m, int p, int R, int nconds, int deflt,
+__device__ __forceinline__ uint32_t soft_group(const SoftKArgs &a, const SoftWarp &m, int p, int R, int nconds, int deflt,
                                            int64_t n0, uint32_t valid, const XPair<TILE, NV> &x, float nc, uint32_t tm,
                                            int lane, float &loss_s, float &loss_c)
 {
@@ -986,13 +985,24 @@ __device__ __forceinline__ bool soft_group(const SoftKArgs &a, const SoftWarp &m
     add_class(deflt, U);
     // every q_r went into p_y or 1 - p_y: a NaN anywhere shows in one of them (looked for beyond the
     // data's end too, where a NaN times a weight of 0 would spoil the sums)
-    bool big = false;
+    bool nan = false, far = false;
 #pragma unroll
-    for (int i = 0; i < NV; ++i)
-        big |= !(py.v[i].x >= (((valid >> (2 * i)) & 1u) ? SOFT_P_MIN : 0.f) && po.v[i].x >= 0.f) ||
-               !(py.v[i].y >= (((valid >> (2 * i + 1)) & 1u) ? SOFT_P_MIN : 0.f) && po.v[i].y >= 0.f);
+    for (int i = 0; i < NV; ++i) {
+        nan |= !(py.v[i].x >= 0.f && po.v[i].x >= 0.f) || !(py.v[i].y >= 0.f && po.v[i].y >= 0.f);
+        far |= (((valid >> (2 * i)) & 1u) && py.v[i].x < SOFT_P_MIN) ||
+               (((valid >> (2 * i + 1)) & 1u) && py.v[i].y < SOFT_P_MIN);
+    }
     if (BWD && TILE) tmem_wait_put();
-    if (__any_sync(FULL, big)) return true;
+    uint32_t left = 0;
+    {
+        constexpr uint32_t ALL = (1u << NV) - 1u;    // SOFT_FF_GROUP is 32 / NV lanes
+        const uint32_t f = __ballot_sync(FULL, far);
+        if (NV == 1) left = f ? 1u : 0u;
+        else left = ((f & 0xFFFFu) ? 1u : 0u) | ((f >> 16) ? 2u : 0u);
+        if (__any_sync(FULL, nan)) left = ALL;
+        if (left == ALL) return ALL;
+        if ((left >> (NV == 1 ? 0 : lane >> 4)) & 1u) valid = 0;     // finite: a weight of 0 leaves them out
+    }
     // -log p_y; near 1 from 1 - p_y, which is its own sum of positive terms
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
@@ -1019,7 +1029,7 @@ __device__ __forceinline__ bool soft_group(const SoftKArgs &a, const SoftWarp &m
                 }
             }
         }
-        return false;
+        return left;
     }
     // ---------------- adjoint
     __syncwarp();
@@ -1083,7 +1093,7 @@ __device__ __forceinline__ bool soft_group(const SoftKArgs &a, const SoftWarp &m
         for (int k = SOFT_CACHE - 1; k >= 0; --k)
             if (b0 + k < c1) cond_grads<CAT>(m, b0 + k, nconds, ce[k], G, x, lane);
     }
-    return false;
+    return left;
 }
 
 // Stage a set's records and rule ends for the warp (row: bytes of a staged feature row, or 1 for
@@ -1171,9 +1181,8 @@ __global__ void __launch_bounds__(SOFT_W * 32) k_soft(SoftKArgs a)
             const uint32_t valid = valid_mask<SOFT_NV>(s1 - n);
             // the dataset is padded to a multiple of 256 samples: every read stays inside it
             const XPair<false, SOFT_NV> x{reinterpret_cast<const char *>(a.Xt + n), a.n_pad * (int64_t)sizeof(float)};
-            if (soft_group<BWD, CAT, false, SOFT_NV>(a, m, p, R, nconds, a.set_default[p], nb, valid, x, nc, 0u, lane, loss_s,
-                                            loss_c))
-                fw |= 1u << (gi & 31);
+            fw |= soft_group<BWD, CAT, false, SOFT_NV>(a, m, p, R, nconds, a.set_default[p], nb, valid, x, nc, 0u, lane,
+                                                       loss_s, loss_c) << (gi & 31);
             if ((gi & 31) == 31 || nb + 64 * SOFT_NV >= s1) {
                 if (lane == 0) fbits[gi >> 5] = fw;
                 ff |= fw;
@@ -1281,10 +1290,10 @@ __global__ void __maxnreg__(128) k_soft_tile(SoftKArgs a, int F)
                 constexpr int NV = SOFT_NV_TILE;
                 const uint32_t valid = valid_mask<NV>(s1 - nb - 2 * NV * lane);
                 const XPair<true, NV> x{reinterpret_cast<const char *>(xbuf + (gi & 1) * F * SOFT_GT + 2 * NV * lane), 0};
-                if (soft_group<BWD, CAT, true, NV>(a, m, p, R, nconds, deflt, nb, valid, x, nc, tm, lane, loss_s, loss_c))
-                    fw |= 1u << (gi & 31);
-                if ((gi & 31) == 31 || gi + 1 == ngroups) {
-                    if (lane == 0) fbits[gi >> 5] = fw;
+                fw |= soft_group<BWD, CAT, true, NV>(a, m, p, R, nconds, deflt, nb, valid, x, nc, tm, lane, loss_s, loss_c)
+                      << (NV * gi & 31);
+                if ((NV * (gi + 1) & 31) == 0 || gi + 1 == ngroups) {
+                    if (lane == 0) fbits[NV * gi >> 5] = fw;
                     ff |= fw;
                     fw = 0;
                 }
@@ -1305,12 +1314,12 @@ __global__ void __maxnreg__(128) k_soft_tile(SoftKArgs a, int F)
 }
 
 // The float-float pass: the CTAs take the (set, chunk) tasks that the main kernel listed, SOFT_W warps
-// to a task: warp i evaluates every SOFT_W-th 32 samples of the groups whose bits the main kernel set
-// (those it left out) in float-float (soft_group_ff), its loss and gradient sums Kahan-summed in their
+// to a task: warp i evaluates every SOFT_W-th 32 samples of those whose bits the main kernel set
+// (SOFT_FF_GROUP samples each, left out there) in float-float (soft_group_ff), its loss and gradient sums Kahan-summed in their
 // order; the warps' sums are added to the task's partials in warp order, so that results do not depend
 // on the order of the list. Runs after the main kernel on the same stream; features are read from
 // global memory, one sample to a lane. Few marked groups are bound by the chain of one warp's conditions
-// (a record, its features, the arithmetic, one after another), hence four warps to a group of 128; many
+// (a record, its features, the arithmetic, one after another), hence four warps to a task; many
 // by the warps that an SM holds, so that as many CTAs run as fit. (Every group of 256 sets of 6 rules on
 // 100,000 x 32: 12.5 ms; with the loads of four conditions issued together, whose unrolled code is four
 // times as long, 25, and with 4 CTAs an SM, 33; the loads ahead gain nothing for few groups either: 145 us
@@ -1352,8 +1361,8 @@ __global__ void __launch_bounds__(SOFT_W * 32) k_soft_ff(SoftKArgs a)
         uint32_t fw = 0;
         int k = 0;                                     // 32-sample pieces of marked groups so far
         for (int64_t nb = s0; nb < s1; nb += 32) {
-            const int gi = (int)((nb - s0) / a.group);
-            if ((nb - s0) % (32 * a.group) == 0) fw = fbits[gi >> 5];
+            const int gi = (int)((nb - s0) / SOFT_FF_GROUP);
+            if ((nb - s0) % (32 * SOFT_FF_GROUP) == 0) fw = fbits[gi >> 5];
             if (!((fw >> (gi & 31)) & 1u)) continue;
             if ((k++ & (SOFT_W - 1)) != w) continue;
             const int64_t n = nb + lane;
@@ -1762,8 +1771,7 @@ static rs_status soft_run(Ctx *ctx, const SoftArgs &s, int known_maxR, int known
         }
         k.teams = sh.teams;
         k.tm_cols = (uint32_t)soft_tm_cols(sh.tw * sh.teams, k.maxR);
-        k.group = tiled ? SOFT_GT : 64 * SOFT_NV;
-        k.ff_wpt = (int32_t)(((k.chunk + k.group - 1) / k.group + 31) / 32);
+        k.ff_wpt = (int32_t)(((k.chunk + SOFT_FF_GROUP - 1) / SOFT_FF_GROUP + 31) / 32);
         {
             TimedLaunch tl(ctx, TK_SOFT, stream);
             if (b.cond_set) launch_soft_kernel<true>(ctx, k, tiled, bwd, s.F, smem, per_warp, sh, stream);
