@@ -352,20 +352,21 @@ struct HardArgs {
 rs_status launch_hard(Ctx *ctx, Dataset *ds, const TileConfig &tc, const HardArgs &a,
                       cudaStream_t stream);
 int choose_groups(Ctx *ctx, const Dataset *ds, const TileConfig &tc, int P);
-// CTAs of a kernel that an SM holds at once, by the driver's answer for this amount of dynamic shared
-// memory; `last` (one per kernel) keeps the latest, {bytes + 1, CTAs}: asking for each launch took 0.4
-// us of a call. The answer is a property of the kernel: the library runs on one kind of GPU only.
+// CTAs of a kernel that an SM holds at once, by the driver's answer for this launch shape; `last` (one per
+// kernel) keeps the latest, {bytes, threads, CTAs}: asking for each launch took 0.4 us of a call. The answer
+// is a property of the kernel: the library runs on one kind of GPU only.
 template <class Kernel>
 int resident_ctas(std::atomic<uint64_t> &last, Kernel kernel, int threads, size_t smem)
 {
+    const uint64_t shape = (uint64_t)smem << 32 | (uint64_t)threads << 16;
     const uint64_t known = last.load(std::memory_order_relaxed);
-    if (known >> 16 == smem + 1) return (int)(known & 0xFFFFu);
+    if (known >> 16 == shape >> 16) return (int)(known & 0xFFFFu);
     int n = 1;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem) != cudaSuccess) {
         cudaGetLastError();
         return 1;
     }
-    last.store((uint64_t)(smem + 1) << 16 | (uint64_t)n, std::memory_order_relaxed);
+    last.store(shape | (uint64_t)n, std::memory_order_relaxed);
     return n;
 }
 // Split of a launch of the sign-mask or rank-coded form into CTAs (whole, groups of HardArgs), with

@@ -18,11 +18,11 @@
 //                du/db = -s x_g / tau.
 // These are the formulas in logs; the float kernels evaluate them as products and sums of positive
 // numbers in the linear domain (see "the float path" below), whose relative errors do not grow with the
-// margins, and a group of samples in which some sample's p_y is below e^-64 (or is not a number) is
+// margins, and a group of samples in which some sample's p_y is below e^-32 (or is not a number) is
 // evaluated again in float-float logs (about 48 significant bits), with the margins formed exactly,
 // 1 - q_r taken as a log-sum-exp of -u_c when q_r rounds to 1, and each d ell / d u_c formed in the
-// exponent (soft_group_ff): there a probability comes near float32's range, and the exponentials of
-// margins of that size carry their rounding.
+// exponent (soft_group_ff): there the exponentials of margins of that size carry the margins' rounding
+// (2^-24 of 32 and more), and a probability comes near float32's range.
 //
 // Work: one warp owns a (rule set, sample chunk) pair and walks the chunk in groups of 64 or 128
 // samples (two or four neighbouring ones per lane), so each partial sum has a fixed summation order.
@@ -39,7 +39,8 @@ namespace rs {
 namespace {
 
 constexpr uint32_t FULL = 0xFFFFFFFFu;
-constexpr int SOFT_W = 4;                 // warps per CTA
+constexpr int SOFT_W = 4;                 // warps per CTA of the per-warp kernel
+constexpr int FF_W = 16, FF_W_PROBS = 8;  // and of the float-float pass, without and with class probabilities
 constexpr int SOFT_MAX_RULES = 64;        // rules per set held in shared memory
 constexpr int SOFT_MAX_CONDS = 512;       // conditions per set accumulated in shared memory
 constexpr int SOFT_MAX_CHUNKS = 128;
@@ -588,7 +589,7 @@ __device__ __forceinline__ void soft_group_ff(const SoftKArgs &a, int p, int rb,
 // log-sum-exp is left: per condition and sample one ex2 forward, and an ex2 and a reciprocal in the
 // adjoint, against two ex2, two degree-8 polynomials and a division before; relative errors grow
 // by a rounding per factor instead of an ulp of the log-probability. Underflow only meets terms
-// below 2^-126 of a sample whose p_y is at least e^-64 (others take the float-float pass).
+// below 2^-126 of a sample whose p_y is at least e^-32 (others take the float-float pass).
 // A rule of more than SOFT_SEG conditions is taken in pieces, q = q1 q2, 1 - q = w1 + q1 w2.
 //
 // What bounds it: instruction issue. A lane holds 2 NV neighbouring samples, so that a feature is one
@@ -611,7 +612,7 @@ constexpr int SOFT_NV_TILE = 2, SOFT_NV = 1;    // float2 per lane: staged-tile 
 constexpr int SOFT_CACHE = 4;              // conditions of a rule whose e the adjoint keeps in registers
 constexpr int SOFT_GROWS = 16;             // conditions per gradient table
 constexpr int SOFT_GPITCH = 288;           // bytes per table row: 32 lanes x 8, + 32 against bank conflicts
-constexpr float SOFT_P_MIN = 1.60381e-28f;   // e^-64: p_y below which a group is evaluated in float-float
+constexpr float SOFT_P_MIN = 1.26642e-14f;   // e^-32: p_y below which samples are evaluated in float-float
 constexpr int32_t SREC_THR = -1, SREC_SET = -2;  // SoftRec4.g of a threshold / membership record
 
 // A record staged for the warp's set: v = s (a x[f] - rhs) = a' x[f] + n' (x[g] for a pair).
@@ -919,7 +920,7 @@ __device__ __forceinline__ void cond_grads(const SoftWarp &m, int ci, int nconds
 // Forward (and adjoint) of a set of R rules over one group of 64 NV samples: lane l holds samples
 // n0 + 2 NV l + i (bit i of valid: the sample exists). tm: the warp's tensor-memory base
 // (staged-tile adjoint). Returns a bit for each SOFT_FF_GROUP of its samples from which nothing was added,
-// since some sample's p_y in it is below e^-64 (all of them when something is not a number): the bits go
+// since some sample's p_y in it is below e^-32 (all of them when something is not a number): the bits go
 // to the task's list, and k_soft_ff evaluates these samples in float-float after this kernel.
 template <bool BWD, bool CAT, bool TILE, int NV>
 __device__ __forceinline__ uint32_t soft_group(const SoftKArgs &a, const SoftWarp &m, int p, int R, int nconds, int deflt,
@@ -1313,24 +1314,26 @@ __global__ void __maxnreg__(128) k_soft_tile(SoftKArgs a, int F)
     }
 }
 
-// The float-float pass: the CTAs take the (set, chunk) tasks that the main kernel listed, SOFT_W warps
-// to a task: warp i evaluates every SOFT_W-th 32 samples of those whose bits the main kernel set
-// (SOFT_FF_GROUP samples each, left out there) in float-float (soft_group_ff), its loss and gradient sums Kahan-summed in their
-// order; the warps' sums are added to the task's partials in warp order, so that results do not depend
-// on the order of the list. Runs after the main kernel on the same stream; features are read from
-// global memory, one sample to a lane. Few marked groups are bound by the chain of one warp's conditions
-// (a record, its features, the arithmetic, one after another), hence four warps to a task; many
-// by the warps that an SM holds, so that as many CTAs run as fit. (Every group of 256 sets of 6 rules on
-// 100,000 x 32: 12.5 ms; with the loads of four conditions issued together, whose unrolled code is four
-// times as long, 25, and with 4 CTAs an SM, 33; the loads ahead gain nothing for few groups either: 145 us
-// with and without for the class probabilities of 48 sets on 20,000 x 30.)
+// The float-float pass: the CTAs take the (set, chunk) tasks that the main kernel listed, all warps of
+// a CTA on one task: warp i of W evaluates every W-th 32 samples of those whose bits the main kernel set
+// (SOFT_FF_GROUP samples each, left out there) in float-float (soft_group_ff), its loss and gradient sums
+// Kahan-summed in their order; the warps' sums are added to the task's partials in warp order, so that
+// results do not depend on the order of the list. Runs after the main kernel on the same stream; features
+// are read from global memory, one sample to a lane. Few marked samples are bound by the chain of one
+// warp's conditions (a record, its features, the arithmetic, one after another), hence FF_W = 16 warps to
+// a task (FF_W_PROBS = 8 for class probabilities, whose arrays leave room for fewer warps an SM); many by
+// the warps that an SM holds, so that as many CTAs run as fit. With 4 / 8 / 16 warps: class probabilities
+// of 48 sets on 20,000 x 30 (9 % of the samples marked) 231 / 187 / 226 us a call; the autograd step of 64
+// sets on 100,000 x 32 (two seeds; many marked samples in a few sets) 1.70 and 3.10 / 1.59 and 2.40 / 1.53
+// and 1.92 ms; nearly every sample of 256 sets of 6 rules on 100,000 x 32 10.5 / 11.0 / 10.5 ms (with the
+// loads of four conditions issued together, whose unrolled code is four times as long, twice that).
 template <bool BWD, bool CAT>
-__global__ void __launch_bounds__(SOFT_W * 32) k_soft_ff(SoftKArgs a)
+__global__ void __launch_bounds__(FF_W * 32, 2) k_soft_ff(SoftKArgs a)
 {
     extern __shared__ __align__(16) float sm[];
     __shared__ int s_item;
-    __shared__ float s_loss[SOFT_W];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    __shared__ float s_loss[FF_W];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
     if (*a.status) return;
     const int items = a.next[SOFT_NEXT_FF_LEN];
     const size_t per_warp = soft_ff_floats(a.maxR, a.maxC, a.probs != nullptr);
@@ -1364,7 +1367,7 @@ __global__ void __launch_bounds__(SOFT_W * 32) k_soft_ff(SoftKArgs a)
             const int gi = (int)((nb - s0) / SOFT_FF_GROUP);
             if ((nb - s0) % (32 * SOFT_FF_GROUP) == 0) fw = fbits[gi >> 5];
             if (!((fw >> (gi & 31)) & 1u)) continue;
-            if ((k++ & (SOFT_W - 1)) != w) continue;
+            if ((k++ & (W - 1)) != w) continue;
             const int64_t n = nb + lane;
             soft_group_ff<BWD, CAT>(a, p, rb, re - rb, cb, deflt, n, n < s1, XView{a.Xt + n, a.n_pad}, lq, lu, acc,
                                     lane, loss_s, loss_c);
@@ -1376,13 +1379,13 @@ __global__ void __launch_bounds__(SOFT_W * 32) k_soft_ff(SoftKArgs a)
         __syncthreads();
         if (threadIdx.x == 0) {
             float t = s_loss[0];
-            for (int i = 1; i < SOFT_W; ++i) t += s_loss[i];
+            for (int i = 1; i < W; ++i) t += s_loss[i];
             a.part_loss[task] += t;
         }
         if (BWD) {
-            for (int i = threadIdx.x; i < (ce - cb); i += SOFT_W * 32) {
+            for (int i = threadIdx.x; i < (ce - cb); i += W * 32) {
                 float ga = 0.f, gbt = 0.f;
-                for (int v = 0; v < SOFT_W; ++v) {
+                for (int v = 0; v < W; ++v) {
                     const float *t = sm + per_warp * v + 4 * (size_t)i;
                     ga += t[0];
                     gbt += t[2];
@@ -1570,12 +1573,14 @@ static void launch_soft_kernel(Ctx *ctx, const SoftKArgs &k, bool tiled, bool bw
 
 // The float-float pass: as many CTAs as the SMs hold, or as there are tasks.
 template <bool BWD, bool CAT>
-static void launch_soft_ff(Ctx *ctx, const SoftKArgs &k, size_t smem, cudaStream_t stream)
+static void launch_soft_ff(Ctx *ctx, const SoftKArgs &k, cudaStream_t stream)
 {
+    const int W = k.probs ? FF_W_PROBS : FF_W;
+    const size_t smem = sizeof(float) * soft_ff_floats(k.maxR, k.maxC, k.probs != nullptr) * W;
     static std::atomic<uint64_t> asked{0};
-    const int resident = std::max(1, resident_ctas(asked, k_soft_ff<BWD, CAT>, SOFT_W * 32, smem));
+    const int resident = std::max(1, resident_ctas(asked, k_soft_ff<BWD, CAT>, W * 32, smem));
     const int64_t grid = std::min<int64_t>((int64_t)k.P * k.nchunks, (int64_t)ctx->sm_count * resident);
-    k_soft_ff<BWD, CAT><<<(unsigned)grid, SOFT_W * 32, smem, stream>>>(k);
+    k_soft_ff<BWD, CAT><<<(unsigned)grid, W * 32, smem, stream>>>(k);
 }
 
 // Words of the float-float group bits for P sets over N samples, for any chunking of at most
@@ -1727,7 +1732,6 @@ static rs_status soft_run(Ctx *ctx, const SoftArgs &s, int known_maxR, int known
         }
     }
     k.pslots = k.probs ? std::min(k.K, k.maxR + 1) : 0;
-    const size_t smem_ff = sizeof(float) * soft_ff_floats(k.maxR, k.maxC, k.probs != nullptr) * SOFT_W;
     const size_t smem = soft_main_bytes(k.maxR, k.maxC, bwd, false, k.pslots) * SOFT_W;
     const size_t per_warp = soft_main_bytes(k.maxR, k.maxC, bwd, true, k.pslots);
     // the staged-tile kernel when its smallest per-CTA footprint (and two feature tiles) fits
@@ -1779,11 +1783,11 @@ static rs_status soft_run(Ctx *ctx, const SoftArgs &s, int known_maxR, int known
         }
         // groups beyond float32's resolution (usually none: the kernel's warps exit at once)
         if (b.cond_set) {
-            if (bwd) launch_soft_ff<true, true>(ctx, k, smem_ff, stream);
-            else launch_soft_ff<false, true>(ctx, k, smem_ff, stream);
+            if (bwd) launch_soft_ff<true, true>(ctx, k, stream);
+            else launch_soft_ff<false, true>(ctx, k, stream);
         } else {
-            if (bwd) launch_soft_ff<true, false>(ctx, k, smem_ff, stream);
-            else launch_soft_ff<false, false>(ctx, k, smem_ff, stream);
+            if (bwd) launch_soft_ff<true, false>(ctx, k, stream);
+            else launch_soft_ff<false, false>(ctx, k, stream);
         }
         count_launch(ctx);
         if (bwd)                      // the gradients and (when asked) the loss in one launch

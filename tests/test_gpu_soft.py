@@ -480,3 +480,31 @@ def test_soft_time_at_sharp_margins(ctx, shift, tau, most):
         assert ms[tau] <= most * ms[0.5], ms
     finally:
         ctx.dataset_destroy(ds)
+
+
+@pytest.mark.parametrize("F", [4, 130])
+def test_soft_small_label_probabilities_keep_their_bits(ctx, orc, F):
+    """Sets all of whose samples have p_y between e^-60 and e^-34, reached on two paths of about the same
+    probability: a rule of the label's class that fails by that many tau, and the default behind a rule of
+    the other class that holds by as many. The gradients are the paths' shares. In float32 a margin's
+    rounding (2^-24 of 34 to 60, in an exponent) makes 2e-6 to 4e-6 of a share, and each further step as
+    much again; in float-float the last float32 operations on quantities of order 1 (exponential, logarithm,
+    products, sums) are left: 16 units of 2^-24. Two samples a set, so that errors do not average out."""
+    rng = np.random.default_rng(41)
+    N, P = 2, 200
+    X = rng.uniform(0.5, 1.5, (N, F)).astype(np.float32)
+    y = np.ones(N, np.int32)
+    sets = []
+    for p in range(P):
+        u = rng.uniform(3.6, 5.8)                  # both margins, times tau = 0.1, at a feature of 1 (the mean)
+        a = np.float32(rng.uniform(0.02, 0.04))
+        sets.append([(1, [(0, -1, synth.GT, a, 0.0, np.float32(a + u))]),
+                     (0, [(1, -1, synth.LT, a, 0.0, np.float32(a + u + rng.uniform(-0.1, 0.1)))])])
+    b = synth.from_lists(sets, [1] * P)
+    got = soft_gpu(ctx, X, y, 2, b, 0.1, np.ones(P))
+    ref = orc.soft(X, y, 2, b, np.float32(0.1), dloss=np.ones(P), want_mag=True)
+    assert 34 < ref["loss"].min() and ref["loss"].max() < 60
+    for n in ("a", "t"):
+        err = np.abs(got["grad_" + n] - ref["grad_" + n])
+        assert (err <= 16 * 2.0 ** -24 * np.maximum(np.abs(ref["grad_" + n]), ref["mag_" + n])).all(), \
+            (n, float((err / ref["mag_" + n]).max()) * 2 ** 24)
