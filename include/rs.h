@@ -424,12 +424,14 @@ rs_status rs_tile_config_form(int32_t id, int32_t *form);
 rs_status rs_set_tile_config(rs_ctx *ctx, int32_t id);
 /* The configuration the next rs_eval_hard of `batch` on `ds` would use: the forced one
  * (rs_set_tile_config), else the tuned one for the batch's shape key (feature count, class count,
- * mean conditions per rule, log2 N, membership tests), else the built-in heuristic. */
+ * mean conditions per rule, log2 N, at most 64 sets or more, membership tests), else the built-in
+ * heuristic. */
 rs_status rs_tile_config_pick(rs_ctx *ctx, uint64_t ds, const rs_batch *batch, int32_t *id);
 /* Time every configuration on this dataset and batch (device pointers), record the fastest in the
  * context's table (and its JSON cache file) and return its id in *best. The cache file is read at
  * rs_create; a file that does not parse as a whole, or that names a configuration this library
- * does not have, is ignored (the heuristic applies until the tuner writes it again). */
+ * does not have, is ignored (the heuristic applies until the tuner writes it again); so are entries
+ * of earlier versions whose configurations ran other evaluators. */
 rs_status rs_autotune(rs_ctx *ctx, uint64_t ds, const rs_batch *batch, void *stream,
                       int32_t *best);
 

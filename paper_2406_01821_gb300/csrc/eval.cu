@@ -102,13 +102,20 @@ static rs_status stage_batch(const rs_batch *b, cudaStream_t stream, StagedBatch
 
 // ------------------------------------------------------------------------ tile configuration
 
+// Sets up to which the built-in choice for wide data is another (heuristic_tile).
+constexpr int TILE_FEW_SETS = 64;
+// Number of the configurations' meaning in the cache file: entries measured when an id ran another form
+// are not used (2: configurations 21 and 22 run the direct walk where the rank tables do not fit).
+constexpr int TUNE_FORMAT = 2;
+
 static std::string tune_key(const Dataset &ds, const rs_batch *b)
 {
     const double meanC = b->R > 0 ? (double)b->C / b->R : 0.0;
     const int cb = (int)std::lround(std::min(meanC, 16.0) * 2);   // half-condition buckets
     const int nb = (int)std::floor(std::log2((double)ds.N));
     std::ostringstream k;
-    k << "F" << ds.F << "|K" << ds.K << "|C" << cb << "|N" << nb << (b->cond_set ? "|cat" : "");
+    k << "v" << TUNE_FORMAT << "|F" << ds.F << "|K" << ds.K << "|C" << cb << "|N" << nb
+      << (b->P <= TILE_FEW_SETS ? "|few" : "|many") << (b->cond_set ? "|cat" : "");
     return k.str();
 }
 
@@ -125,7 +132,7 @@ static int heuristic_tile(const Dataset &ds, int P, bool cat)
     if (ds.finite && direct_smem_bytes(ds.F, 32) <= 227 * 1024) {
         if (ds.ranked && rank_tables_fit(ds.F, 16)) return 21;
         const bool two = 2 * (direct_smem_bytes(ds.F, 16) + 1024) <= 228 * 1024;
-        return two && P <= 64 && !(cat && ds.ranked && rank_tables_fit(ds.F, 32)) ? 21 : 22;
+        return two && P <= TILE_FEW_SETS && !(cat && ds.ranked && rank_tables_fit(ds.F, 32)) ? 21 : 22;
     }
     // Else the 32-warp margin-minimum form on non-finite data, then smaller tiles for wide data (the
     // sign-mask form where it is finite), and for data too wide for any shared tile the configuration

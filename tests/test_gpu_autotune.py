@@ -125,3 +125,27 @@ def test_valid_cache_entry_for_this_shape_is_used(tmp_path, work):
         ds = ctx.dataset(X, y, 5)
         assert ctx.tile_pick(ds, rs.DeviceBatch.from_host(b)) == other
         ctx.dataset_destroy(ds)
+
+
+def test_entries_of_other_sizes_and_versions_are_not_used(tmp_path):
+    """The built-in choice for wide data differs between few and many sets: an entry tuned with many does
+    not decide for few. A file written before the entries carried a version is read and not used."""
+    from paper_2406_01821_gb300 import build, rs
+    build.build()
+    X, y = synth.gaussian_mixture(3001, 140, 3, 32)
+    q = synth.quantile_table(X)
+    many, few = (synth.random_rulesets(q, 3, P, (1, 8), 4, 33) for P in (300, 40))
+    cache = tmp_path / "tune.json"
+    with rs.Context(0) as ctx:
+        ds = ctx.dataset(X, y, 3)
+        dm, df = rs.DeviceBatch.from_host(many), rs.DeviceBatch.from_host(few)
+        built_in = ctx.tile_pick(ds, dm), ctx.tile_pick(ds, df)
+    assert built_in[0] != built_in[1]
+    with rs.Context(0, autotune_cache=str(cache)) as ctx:
+        ds = ctx.dataset(X, y, 3)
+        best = ctx.autotune(ds, dm)
+        assert ctx.tile_pick(ds, dm) == best and ctx.tile_pick(ds, df) == built_in[1]
+    cache.write_text(json.dumps({"F140|K3|C8|N11": 5}))
+    with rs.Context(0, autotune_cache=str(cache)) as ctx:
+        ds = ctx.dataset(X, y, 3)
+        assert (ctx.tile_pick(ds, dm), ctx.tile_pick(ds, df)) == built_in
