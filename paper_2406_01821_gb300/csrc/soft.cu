@@ -424,7 +424,7 @@ __device__ ff rule_logq_ff(const SoftKArgs &a, int c0, int c1, const XView &x)
     for (int c = c0; c < c1; ++c) {
         const CondIn t = load_cond(a, c, x);
         if (CAT && (t.rc.meta & 4u)) {
-            if (!category_member(t.xf, __float_as_uint(t.rc.a), __float_as_uint(t.rc.bt))) s = {-INFINITY, 0.f};
+            if (!category_member(t.xf, __float_as_uint(t.rc.a), __float_as_uint(t.rc.bt))) s = ff_add(s, ff{-INFINITY, 0.f});
             continue;
         }
         float l1pe;
@@ -818,8 +818,8 @@ struct SoftProd {
             const float2 d = make_float2(min_nan(D[i].x, SOFT_D_MAX), min_nan(D[i].y, SOFT_D_MAX));
             float2 r = make_float2(rcp_ftz(d.x), rcp_ftz(d.y));
             r = __ffma2_rn(r, __ffma2_rn(__fmul2_rn(d, f2(-1.f)), r, f2(1.f)), r);
-            if (CAT && ((dead >> (2 * i)) & 1u)) r.x = 0.f;
-            if (CAT && ((dead >> (2 * i)) & 2u)) r.y = 0.f;
+            if (CAT && ((dead >> (2 * i)) & 1u)) r.x *= 0.f;     // a NaN stays
+            if (CAT && ((dead >> (2 * i)) & 2u)) r.y *= 0.f;
             q.v[i] = r;
             // 1 - q rounded once where q < 1/2, else the quotient, which keeps a small 1 - q
             w.v[i] = mul2_ftz(z[i], r);                  // the added subnormals alone: 0

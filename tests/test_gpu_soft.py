@@ -508,3 +508,26 @@ def test_soft_small_label_probabilities_keep_their_bits(ctx, orc, F):
         err = np.abs(got["grad_" + n] - ref["grad_" + n])
         assert (err <= 16 * 2.0 ** -24 * np.maximum(np.abs(ref["grad_" + n]), ref["mag_" + n])).all(), \
             (n, float((err / ref["mag_" + n]).max()) * 2 ** 24)
+
+
+@pytest.mark.parametrize("F", [6, 130])
+@pytest.mark.parametrize("test_first", [True, False])
+def test_soft_nan_margin_beside_a_failed_membership_test(ctx, orc, F, test_first):
+    """A margin that is not a number makes its set's loss NaN, whether or not a membership test of the same
+    rule fails for the sample and whichever comes first; sets without it are unaffected."""
+    rng = np.random.default_rng(43)
+    X = rng.standard_normal((300, F)).astype(np.float32)
+    X[:, 1] = rng.integers(0, 8, 300)
+    X[7, 0] = np.nan
+    X[7, 1] = 5.0
+    y = rng.integers(0, 2, 300).astype(np.int32)
+    member = (1, -1, synth.IN, 0.0, 0.0, 0.0, [0, 1, 2])              # fails for sample 7
+    on_nan = (0, -1, synth.GT, np.float32(1), 0.0, np.float32(0.1))
+    plain = (2, -1, synth.GT, np.float32(1), 0.0, np.float32(0.1))
+    conds = [member, on_nan] if test_first else [on_nan, member]
+    b = synth.from_lists([[(0, conds), (1, [plain])], [(0, [member, plain]), (1, [plain])]], [0, 0])
+    got = soft_gpu(ctx, X, y, 2, b, 0.3, np.ones(2))
+    ref = orc.soft(X, y, 2, b, 0.3, dloss=np.ones(2), want_mag=True)
+    assert np.isnan(ref["loss"][0]) and np.isfinite(ref["loss"][1])
+    assert np.isnan(got["loss"][0])
+    assert np.allclose(got["loss"][1], ref["loss"][1], rtol=RTOL, atol=0)
