@@ -339,6 +339,7 @@ def soft_leg(args, dev):
             "roofline": {"bound": "xu", "achieved": xu / (kern_ms / 1e3) / 1e12, "peak": xu_peak / 1e12,
                          "unit": "T transcendentals/s", "frac": xu / (kern_ms / 1e3) / xu_peak,
                          "transcendentals_per_pass": xu,
+                         "frac_executed": soft_executed_transcendentals(w.batch, w.N) / (kern_ms / 1e3) / xu_peak,
                          "peak_source": "measured: special-function unit ex2 stream (rs_measure_pipe_rates)"}}
 
 
@@ -437,6 +438,13 @@ def soft_transcendentals(batch, N):
     the linear domain and execute fewer: an exponential per condition and sample forward, an
     exponential and a reciprocal in the adjoint, and a few reciprocals per rule."""
     return N * (3 * batch.C + 11 * batch.R)
+
+
+def soft_executed_transcendentals(batch, N):
+    """What the kernels' linear-domain path executes on the special-function unit for rules of at most four
+    conditions: per condition and sample an exponential forward, an exponential and a reciprocal in the
+    adjoint; per rule and sample a reciprocal in each; per set and sample a logarithm and a reciprocal."""
+    return N * (3 * batch.C + 2 * batch.R + 2 * batch.P)
 
 
 def evolution_leg(args, dev, G: int = 200, arms: bool = True):

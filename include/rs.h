@@ -228,7 +228,8 @@ rs_status rs_eval_hard(rs_ctx *ctx, uint64_t ds, const rs_batch *batch, int32_t 
  *   loss[p] = (1/N) sum_n -log p_p(y_n | x_n)      float32[P]
  *   probs   float32[P*N*K] class probabilities at [(p*N + n)*K + k] (caller's sample order);
  *           may be NULL
- * Computed in float32 in the log domain. tau > 0.
+ * Computed in float32 on the probabilities themselves, for samples whose p_y is below e^-32 in
+ * pairs of float32 on their logs. tau > 0.
  */
 rs_status rs_eval_soft_fwd(rs_ctx *ctx, uint64_t ds, const rs_batch *batch, float tau,
                            float *loss, float *probs, void *stream);
@@ -480,15 +481,16 @@ rs_status rs_selftest_threshold_rewrite(rs_ctx *ctx, const float *a, const float
 
 /*
  * Self-check of the soft path's log(1 + e) for 0 <= e <= 1 (the term of every log-sigmoid and
- * log-sum-exp of Sec. 3's sigmoid relaxation): out[i] = the kernels' log1p(e[i]) for host arrays
+ * log-sum-exp of Sec. 3's sigmoid relaxation in the log form): out[i] = the kernels' log1p(e[i]) for host arrays
  * e, out of n entries, evaluated on the context's device.
  */
 rs_status rs_selftest_log1p_unit(rs_ctx *ctx, const float *e, int32_t n, float *out);
 
 /*
- * Self-check of the soft forward's log(1 - q) from log q (the log-probability that a rule does not
- * fire, Sec. 3's soft first-fire product): out[i] = the kernels' log(1 - e^s[i]) for host arrays s
- * (s <= 0; 0 gives -inf, -inf gives 0), n entries, evaluated on the context's device.
+ * log(1 - q) from log q (the log-probability that a rule does not fire, Sec. 3's soft first-fire
+ * product): out[i] = log(1 - e^s[i]) for host arrays s (s <= 0; 0 gives -inf, -inf gives 0), n
+ * entries, evaluated on the context's device. The kernels no longer form it so (rs_eval_soft_fwd);
+ * the entry point is kept for its callers.
  */
 rs_status rs_selftest_log1m_exp(rs_ctx *ctx, const float *s, int32_t n, float *out);
 

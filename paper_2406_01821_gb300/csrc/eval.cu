@@ -129,9 +129,9 @@ static int heuristic_tile(const Dataset &ds, int P, bool cat)
     // features), which pays as long as building the tables would weigh more than walking faster with
     // them: 46 sets on 470,000 x 106, 236 us against 280; 64: 282 and 306; 100: 398 and 386.
     // Membership tests keep the rank-coded walk, whose code rows test them.
-    if (ds.finite && direct_smem_bytes(ds.F, 32) <= 227 * 1024) {
+    if (ds.finite && direct_smem_bytes(ds.F, 32) <= SMEM_CTA) {
         if (ds.ranked && rank_tables_fit(ds.F, 16)) return 21;
-        const bool two = 2 * (direct_smem_bytes(ds.F, 16) + 1024) <= 228 * 1024;
+        const bool two = 2 * (direct_smem_bytes(ds.F, 16) + SMEM_RESERVED) <= SMEM_SM;
         return two && P <= TILE_FEW_SETS && !(cat && ds.ranked && rank_tables_fit(ds.F, 32)) ? 21 : 22;
     }
     // Else the 32-warp margin-minimum form on non-finite data, then smaller tiles for wide data (the

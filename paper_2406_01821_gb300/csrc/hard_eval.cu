@@ -283,7 +283,7 @@ int tile_config_count() { return kNumConfigs; }
 bool rank_tables_fit(int F, int W)
 {
     const size_t s = hard5_smem_bytes(F, W);
-    return W >= 32 ? s <= 227 * 1024 : 2 * (s + 1024) <= 228 * 1024;
+    return W >= 32 ? s <= SMEM_CTA : 2 * (s + SMEM_RESERVED) <= SMEM_SM;
 }
 
 // The form a configuration runs as: its own, or DIRECT_VERSION (rank-coded configurations on finite
@@ -293,7 +293,7 @@ int effective_version(const TileConfig &tc, const Dataset &ds, bool preds)
     if (tc.ver >= 4 && !ds.finite) return 3;              // same V and W exist for version 3
     int ver = tc.ver;
     if (ver == 5 && !(ds.ranked && rank_tables_fit(ds.F, tc.W)))
-        ver = direct_smem_bytes(ds.F, tc.W) <= 227 * 1024 ? DIRECT_VERSION : 4;
+        ver = direct_smem_bytes(ds.F, tc.W) <= SMEM_CTA ? DIRECT_VERSION : 4;
     // these walks write predictions as bytes; the sign-mask form writes none
     if (preds && (ver == 4 || (ver >= 5 && ds.K > 256))) return 3;
     return ver;
@@ -318,7 +318,7 @@ bool tile_config_fits(const TileConfig &tc, int F)
     const int Frows = ((F + Fb - 1) / Fb) * Fb;
     const size_t stage = (size_t)tc.W * (tc.ver >= 2 ? 64 : 32) * sizeof(Rec);
     const size_t smem = (size_t)Frows * tc.S() * sizeof(float) + stage + 16;
-    return smem <= 227 * 1024 && (tc.ver == 1 || (size_t)F * tc.S() / 4 < (1u << 18));
+    return smem <= SMEM_CTA && (tc.ver == 1 || (size_t)F * tc.S() / 4 < (1u << 18));
 }
 
 rs_status launch_hard(Ctx *ctx, Dataset *ds, const TileConfig &tc, const HardArgs &a,

@@ -198,8 +198,7 @@ static rs_status launch5_t(Ctx *ctx, Dataset *ds, HardArgs a, cudaStream_t strea
     if (CAT && !DIRECT) {
         // fewer pass-row slots make room for the code rows: all of them, or as many as keep the CTAs
         // per SM that the kernel has without them (features beyond them are tested on their floats)
-        const size_t most = 2 * (smem + 1024) <= ctx->smem_optin + 1024 && W == 16 ? (ctx->smem_optin + 1024) / 2 - 1024
-                                                                                 : ctx->smem_optin;
+        const size_t most = W == 16 && 2 * (smem + SMEM_RESERVED) <= SMEM_SM ? SMEM_SM / 2 - SMEM_RESERVED : SMEM_CTA;
         smem -= (size_t)W * (VSLOTS - VSLOTS_CAT) * 128;
         smem += (size_t)(a.F + 3) / 4 * 4;
         a.code_rows = (int32_t)std::min<size_t>({(size_t)ds->ncode, (size_t)CODE_NONE, (most - smem) / 256});

@@ -195,6 +195,8 @@ struct TileConfig {
     bool gmem = false;   // form 1 reading features from global memory (no shared tile: any F)
     int S() const { return 32 * V; }
 };
+// Shared memory of sm_103: a CTA's most, an SM's, and what each resident CTA takes of the latter beside its own.
+constexpr size_t SMEM_CTA = 227 * 1024, SMEM_SM = 228 * 1024, SMEM_RESERVED = 1024;
 constexpr int RANK_TILE = 128;    // samples per rank tile (ranks fit in 7 bits)
 constexpr int RANK_MAX_F = 128;   // widest dataset given rank tables (the widest whose tables fit 32 warps)
 int tile_config_count();

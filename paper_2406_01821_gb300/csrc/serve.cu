@@ -45,13 +45,13 @@ constexpr size_t TILE_BYTES = (size_t)SERVE_MAX_F * SS * 4 > RANK_BYTES ? (size_
 constexpr size_t ONES_BYTES = (size_t)SS * 4;   // a row of 1.0: the right side of product conditions
 constexpr size_t SERVE_SMEM = TILE_BYTES + (size_t)SW * 64 * 16 + (size_t)SW * SVS * 32 * 4 + ONES_BYTES;
 constexpr int MAX_SLOTS = 2048;
-// Sets per unit: as many as leave UNITS_MIN units to the request (two for every CTA), at most
+constexpr int SPARE_SMS = 4;          // left to the packing kernels of new requests
+// Sets per unit: as many as leave UNITS_MIN units to the request (two for every CTA of 152 SMs), at most
 // GROUP_SETS_MAX, at least GROUP_SETS_MIN (rank-coded units, whose staging is heavier: _RANKED). Large
 // units lose less to their staging and to the last walks, which some warps of the CTA wait for: 72
 // mixed requests in 28.9 / 24.1 / 22.6 ms with direct units of at most 128 / 256 / 512 sets.
-constexpr int GROUP_SETS_MIN = 128, GROUP_SETS_MIN_RANKED = 256, GROUP_SETS_MAX = 512, UNITS_MIN = 296;
+constexpr int GROUP_SETS_MIN = 128, GROUP_SETS_MIN_RANKED = 256, GROUP_SETS_MAX = 512, UNITS_MIN = 2 * (152 - SPARE_SMS);
 constexpr int SERVE_RANK_MIN_P = 64;    // smaller requests take direct units
-constexpr int SPARE_SMS = 4;          // left to the packing kernels of new requests
 // Persistent kernel idle limit: 2 ms without a claim and with no unit being walked anywhere. The first
 // CTA that finds it so closes the kernel for all: a CTA that left alone would be missing from the work
 // that keeps the others alive. Units that arrive then wait for the scheduler's next launch. While it

@@ -186,14 +186,14 @@ __device__ __forceinline__ float log1p_unit(float e)
 }
 
 // The hardware exponential (ex2.approx of x log2(e)) of a non-positive argument: for |x| up to about
-// 100 its relative error stays below a few 1e-6. Used by log1m_exp and by the class probabilities of
-// the float-float pass.
+// 100 its relative error stays below a few 1e-6. Used by the class probabilities of the float-float
+// pass and by log1m_exp.
 __device__ __forceinline__ float exp_np(float x) { return __expf(x); }
 
 // log(1 - e^s) for s <= 0: the log-probability that a rule whose conditions hold with
-// probability q = e^s does not fire (rs_selftest_log1m_exp; the kernels' float path works in the
-// linear domain). Both pieces are evaluated and one is selected (a warp's
-// samples fall on both sides):
+// probability q = e^s does not fire. For the entry point rs_selftest_log1m_exp only: the float path works
+// in the linear domain, the float-float pass has rule_log1mq_ff. Both pieces are evaluated and one is
+// selected:
 // * q <= e^(-1/2): log1p(-q) = -q a(q), a the degree-10 polynomial of least maximum relative
 //   error against -log1p(-q) / q on [0, e^(-1/2)] (Remez exchange; within 2 ulp given q). q comes
 //   from the hardware exponential, whose relative error (a few 1e-6 at most for the arguments
@@ -233,8 +233,7 @@ __device__ __forceinline__ float log1m_exp(float s)
     return t >= 0.5f ? ra : rb;
 }
 
-// The soft kernels' elementary functions evaluated on the device (test hooks): 0 = log1p_unit,
-// 1 = log1m_exp.
+// Elementary functions evaluated on the device (test hooks): 0 = log1p_unit, 1 = log1m_exp.
 __global__ void k_selftest_soft_math(const float *in, int n, float *out, int which)
 {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
@@ -283,7 +282,6 @@ struct SoftKArgs {
     float *part_loss;                // [nchunks][P]
     float *part_ga, *part_gbt;       // [nchunks][C]
     float *probs;                    // [P*N*K] or null
-    int32_t backward;
     int32_t *next;                   // [8] counters (SOFT_NEXT_*)
     int32_t maxR, maxC;              // shared-memory capacity per warp (rules, conditions)
     int64_t Ccap;                    // row stride of the gradient partials
@@ -297,9 +295,7 @@ struct SoftKArgs {
     uint32_t tm_cols;                // tensor-memory columns of a CTA (staged-tile adjoint)
 };
 
-// Feature access for one group of 64 samples: the lane's first sample column either in global
-// memory (x[f] at col[f * stride]) or in a staged shared-memory tile [F][64] (stride 64); its
-// second sample is 32 columns further.
+// Feature access of the float-float pass: the lane's sample column in global memory, x[f] at col[f * stride].
 struct XView {
     const float *col;
     int64_t stride;
@@ -589,7 +585,8 @@ __device__ __forceinline__ void soft_group_ff(const SoftKArgs &a, int p, int rb,
 // log-sum-exp is left: per condition and sample one ex2 forward, and an ex2 and a reciprocal in the
 // adjoint, against two ex2, two degree-8 polynomials and a division before; relative errors grow
 // by a rounding per factor instead of an ulp of the log-probability. Underflow only meets terms
-// below 2^-126 of a sample whose p_y is at least e^-32 (others take the float-float pass).
+// below 2^-126 of a sample whose p_y is at least e^-32 (others take the float-float pass), that is parts of
+// a gradient below 9e-25 x / tau, which count as 0.
 // A rule of more than SOFT_SEG conditions is taken in pieces, q = q1 q2, 1 - q = w1 + q1 w2.
 //
 // What bounds it: instruction issue. A lane holds 2 NV neighbouring samples, so that a feature is one
@@ -1709,7 +1706,6 @@ static rs_status soft_run(Ctx *ctx, const SoftArgs &s, int known_maxR, int known
     k.fflist = fflist;
     k.ffbits = ffbits;
     k.probs = s.probs;
-    k.backward = bwd;
     k.next = next;
     k.Ccap = Ccap;
     k.status = s.status;

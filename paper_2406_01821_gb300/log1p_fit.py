@@ -4,8 +4,8 @@ polynomial of least maximum relative error found by the Remez exchange in 50-dig
 multiply-adds) against float64:
 
 * `log1p_unit`: log(1 + e) on [0, 1] as e p(e), p of degree 8 fitted to log1p(e) / e.
-* `log1m_exp`: log(1 - e^s) for s <= 0, the log-probability that a rule with log q = s does not
-  fire, in two pieces split at s = -1/2:
+* `log1m_exp` (an entry point of its own; the kernels form 1 - q otherwise): log(1 - e^s) for s <= 0, the
+  log-probability that a rule with log q = s does not fire, in two pieces split at s = -1/2:
   - q = e^s <= e^(-1/2): log1p(-q) = -q a(q), a of degree 10 fitted to -log1p(-q) / q on
     [0, e^(-1/2)] (relative accuracy of log1p(-q) as q goes to 0);
   - t = -s < 1/2: log(1 - e^-t) = log t + t b(t), b of degree 3 fitted to
