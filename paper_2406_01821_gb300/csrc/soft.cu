@@ -1568,7 +1568,9 @@ static void launch_soft_kernel(Ctx *ctx, const SoftKArgs &k, bool tiled, bool bw
     }
 }
 
-// The float-float pass: as many CTAs as the SMs hold, or as there are tasks.
+// The float-float pass: as many CTAs as the SMs hold, or as there are tasks. The largest sets fit.
+static_assert(sizeof(float) * soft_ff_floats(SOFT_MAX_RULES, SOFT_MAX_CONDS, false) * FF_W <= SMEM_CTA - SOFT_TILE_STATIC &&
+              sizeof(float) * soft_ff_floats(SOFT_MAX_RULES, SOFT_MAX_CONDS, true) * FF_W_PROBS <= SMEM_CTA - SOFT_TILE_STATIC);
 template <bool BWD, bool CAT>
 static void launch_soft_ff(Ctx *ctx, const SoftKArgs &k, cudaStream_t stream)
 {

@@ -531,3 +531,17 @@ def test_soft_nan_margin_beside_a_failed_membership_test(ctx, orc, F, test_first
     assert np.isnan(ref["loss"][0]) and np.isfinite(ref["loss"][1])
     assert np.isnan(got["loss"][0])
     assert np.allclose(got["loss"][1], ref["loss"][1], rtol=RTOL, atol=0)
+
+
+def test_soft_largest_sets_in_the_float_float_pass(ctx, orc):
+    """Sets of 64 rules and 512 conditions, most samples far: the float-float pass with its largest shared
+    arrays, adjoint and class probabilities."""
+    X, y, _ = accurate_case(130, 8, 1, 3.0, 47)
+    b = synth.random_rulesets(synth.quantile_table(X), 2, 3, 64, 8, 47, pair_prob=0.3)
+    b.rule_class[b.set_rule_off[:-1]], b.rule_class[b.set_rule_off[:-1] + 1] = 0, 1
+    dl = np.ones(b.P)
+    got = soft_gpu(ctx, X, y, 2, b, 0.003, dl, probs=True)
+    ref = orc.soft(X, y, 2, b, np.float32(0.003), dloss=dl, want_probs=True, want_mag=True)
+    assert (ref["loss"] > 20).all()                # mean losses: samples beyond e^-32 in every group
+    check_against_oracle(got, ref)
+    assert np.allclose(got["probs"], ref["probs"], rtol=RTOL, atol=1e-30)
